@@ -174,8 +174,7 @@ typedef struct gx_explore_opts {
                                     skips find-or-put.  0 = off, 1..12 = 2^n, 0xFFFFFFFF =
                                     automatic (gx_default_opts): 2^9 unless the GPU-wide
                                     cache below is in use (together they measured slower);
-                                    2^6 with the queued 4-word kernel (region_passes), whose
-                                    CTAs then still fit 5 per SM */
+                                    2^6 for 4-word vectors, whose CTAs then still fit 5 per SM */
   float guided_scale;            /* GX_DL_GUIDED: score at which a state falls in the last
                                     bin (scores are predicted distances / max_dist); 0 = 1.0 */
   uint32_t watch;                /* 1 = safety check (Sec. 3: the negation of a safety property
@@ -205,30 +204,26 @@ typedef struct gx_explore_opts {
                                     (address-translation reach).  In a table above 64 GiB
                                     every hash round of a vector stays inside the 64 GiB
                                     span of its first bucket, so later rounds stay in the
-                                    pass's region too.  With more than one pass, 4-word
-                                    slots in 4- or 8-word buckets with one lane per bucket
-                                    run the level kernel with the successor queue (only the
-                                    pass's successors are probed, 32 at a time).  Results
-                                    do not depend on it.  0 = auto: the fewest passes whose
-                                    regions are at most 64 GiB (1 for tables up to 64 GiB) */
+                                    pass's region too.  Results do not depend on it.  0 = auto:
+                                    the fewest passes whose regions are at most 64 GiB (1 for
+                                    tables up to 64 GiB) */
   uint32_t global_cache_log2;    /* GPU-wide cache of recently seen vectors: 2^n
-                                    direct-mapped 64-bit entries in the workspace, cleared at
-                                    the start of each search and small enough to stay in L2.
-                                    An entry holds a vector exactly: 1- and 2-word vectors
-                                    as they are, 4-word vectors as their field bits packed
-                                    into 64 (no effect on 4-word vectors whose fields take
-                                    more than 64 bits).  A vector goes in after its
-                                    find-or-put found or inserted it, so a hit is a known
-                                    state and skips the table probe; most successors of a
-                                    level lead into the levels just before and after it.
-                                    0 = off, 1..26 = 2^n, 0xFFFFFFFF = automatic
-                                    (gx_default_opts): 2^23 entries (64 MiB) for 1- and
-                                    2-word vectors in tables of at least 2^26 slots with one
-                                    lane per bucket (group_lanes 1), else off.  Mid network:
-                                    0.36 bucket reads per successor and 18.9 ms, against 0.82
-                                    and 20.4 ms with the per-warp cache; small sizes
-                                    (2^14-2^18) are far slower, many warps writing the same
-                                    few lines */
+                                    direct-mapped entries in the workspace, cleared at the
+                                    start of each search and small enough to stay in L2.
+                                    An entry holds a vector exactly: its fields packed side by
+                                    side (b <= 64 bits; no effect on vectors with more) are
+                                    mixed by a bijection, n of the bits are the entry's index
+                                    and the other b - n are stored, in 16, 32 or 64 bits.  A
+                                    vector goes in after its find-or-put found or inserted it,
+                                    so a hit is a known state and skips the table probe; most
+                                    successors of a level lead into the levels just before and
+                                    after it.  0 = off, 1..26 = 2^n, 0xFFFFFFFF = automatic
+                                    (gx_default_opts): the most entries that take 64 MiB (2^25
+                                    for b <= 41, 2^24 for b <= 56, 2^23 above), in tables of at
+                                    least 2^26 slots with one lane per bucket (group_lanes 1),
+                                    for 4-word vectors only in one region pass; else off.  Mid
+                                    network (b = 40): 0.21 bucket reads per successor and
+                                    13.7 ms; with 2^23 entries 0.38 and 17.5 ms */
   uint32_t guided_fused;         /* GX_DL_GUIDED: 1 = score the states an iteration inserts
                                     inside its expansion kernel (each CTA keeps them in shared
                                     memory and scores 128 at a time on the tensor cores), 0 =

@@ -70,27 +70,24 @@ __global__ void __launch_bounds__(gx::kBlock) batch_init_kernel(const BatchArgs 
   for (int i = threadIdx.x; i < a.rounds; i += blockDim.x) muls[i] = a.muls.m[i];
   __syncthreads();
   const int net = blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5);
-  if (net >= a.n || (int)(threadIdx.x & 31) >= G) return;
+  if (net >= a.n || (threadIdx.x & 31) != 0) return;
   BNet& b = a.nets[net];
-  const Group<G> g;
   uint32_t v[W];
 #pragma unroll
   for (int w = 0; w < W; ++w) v[w] = b.init_vec[w];
   uint32_t probes = 0;
-  const int r = find_or_put<W, B, G>(b.table, b.log2nb, a.rounds, muls, v, g, probes);
-  if (g.glane == 0) {
-    if (r == FOP_INSERTED) store_vec<W>(b.frontier, v);
-    b.cur_begin = 0;
-    b.cur_end = 1;
-    b.next_end = 1;
-    b.transitions = b.dl_count = b.dl_sum = b.dl_xor = 0;
-    b.probes = probes;
-    b.error = r == FOP_INSERTED ? 0u : gx::ERR_TABLE_FULL;
-    b.active = r == FOP_INSERTED ? 1u : 0u;
-    b.first_dl = -1;
-    b.n_levels = 1;
-    b.levels[0] = 1;
-  }
+  const int r = find_or_put_state<W, B>(b.table, b.log2nb, a.rounds, muls, v, probes);
+  if (r == FOP_INSERTED) store_vec<W>(b.frontier, v);
+  b.cur_begin = 0;
+  b.cur_end = 1;
+  b.next_end = 1;
+  b.transitions = b.dl_count = b.dl_sum = b.dl_xor = 0;
+  b.probes = probes;
+  b.error = r == FOP_INSERTED ? 0u : gx::ERR_TABLE_FULL;
+  b.active = r == FOP_INSERTED ? 1u : 0u;
+  b.first_dl = -1;
+  b.n_levels = 1;
+  b.levels[0] = 1;
 }
 
 // One CTA: finish the level just expanded for every network, then lay out the
@@ -192,18 +189,17 @@ __global__ void __launch_bounds__(1024) batch_advance_kernel(const BatchArgs a, 
 // Networks have separate tables, so a hit is only valid for the network whose
 // vectors filled the cache: a warp clears its cache whenever it moves to a
 // chunk of another network.
-constexpr int kBatchCacheLog2 = 9;
+constexpr int kBatchCacheLog2 = 8;
 
 // The network a warp is working on, staged in shared memory when the warp
 // moves to it, so that its layout and table pointers take no registers in the
 // inner loop.
 struct WarpNet {
   NetBlobLayout lay;
-  const uint32_t* blob;
   uint32_t* table;
   unsigned long long* next_end;
   uint32_t* frontier;
-  uint64_t fmask, cur_begin;
+  uint64_t fmask, cur_begin, cur_end;
   int log2nb;
 };
 
@@ -219,9 +215,7 @@ struct SmemTarget {
   __device__ __forceinline__ uint64_t begin() const { return w->cur_begin; }
   __device__ __forceinline__ uint64_t region_mask() const { return 0; }
   __device__ __forceinline__ uint64_t region_bits() const { return 0; }
-  __device__ __forceinline__ unsigned long long* gcache() const { return nullptr; }
-  __device__ __forceinline__ uint64_t gcache_mask() const { return 0; }
-  __device__ __forceinline__ GKey gkey() const { return GKey{{64u, 64u, 64u}}; }
+  __device__ __forceinline__ gx::SeenCache gcache() const { return gx::SeenCache{}; }
 };
 
 // The batched kernel keeps a network index and chunk bounds besides the
@@ -232,34 +226,50 @@ struct BatchOcc {
   static constexpr int min_ctas = ExpandOcc<W, B, G>::min_ctas < 4 ? ExpandOcc<W, B, G>::min_ctas : 4;
 };
 
+constexpr int kWarpDescs = 32;  // processes whose descriptors a warp keeps in shared memory
+
+// Dynamic shared memory of the batched kernel, per warp: queues, staging, the
+// cache of seen vectors, the network and its processes' descriptors.
+template <int W>
+struct __align__(16) BatchSmem {
+  static constexpr int kWarps = gx::kBlock / 32;
+  static constexpr int kCache = W <= 2 ? (1 << kBatchCacheLog2) * W : 4;
+  WarpQueues<W, 32> queues[kWarps];
+  uint32_t stage[kWarps][kStage * W];
+  uint32_t cache[kWarps][kCache];
+  uint4 descs[kWarps][kWarpDescs];
+  WarpNet net[kWarps];
+  unsigned long long muls[kMaxRounds];
+};
+
 template <int W, int B, int G>
 __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch_expand_kernel(const BatchArgs a) {
-  // a fixed full-size grid: CTAs beyond what this iteration's chunks need leave
-  // before claiming (in the batch's long tail most iterations have few chunks)
-  if ((unsigned long long)blockIdx.x * (gx::kBlock / 32) >= __ldcg(a.prefix + a.n)) return;
-  __shared__ uint64_t muls[kMaxRounds];
-  for (int i = threadIdx.x; i < a.rounds; i += blockDim.x) muls[i] = a.muls.m[i];
-  __shared__ uint32_t stage_mem[gx::kBlock / 32][kStage * W];
-  constexpr int CW = W <= 2 ? W : 1;
-  __shared__ __align__(16) uint32_t cache_mem[gx::kBlock / 32][(1 << kBatchCacheLog2) * CW];
-  __shared__ WarpNet s_net[gx::kBlock / 32];
+  // a fixed full-size grid: CTAs beyond what this iteration's claims need leave
+  // before claiming (in the batch's long tail most iterations have few)
+  const unsigned long long total = __ldcg(a.prefix + a.n);
+  if ((unsigned long long)blockIdx.x * (gx::kBlock / 32) >= total) return;
+  extern __shared__ __align__(16) unsigned char bsm[];
+  BatchSmem<W>& S = *reinterpret_cast<BatchSmem<W>*>(bsm);
+  for (int i = threadIdx.x; i < a.rounds; i += blockDim.x) S.muls[i] = a.muls.m[i];
   __syncthreads();
-  WarpNet& wn = s_net[threadIdx.x >> 5];
-  const int lane = threadIdx.x & 31;
-  const Group<G> g;
-  WarpStage st{stage_mem[threadIdx.x >> 5], 0};
-  WarpCache cache{W <= 2 ? cache_mem[threadIdx.x >> 5] : nullptr, (1u << kBatchCacheLog2) - 1u};
-  int cached_net = -1;
-  __shared__ unsigned long long s_chunk[gx::kBlock / 32][2];  // [first, end) of the warp's chunk
-  unsigned long long* chunk_range = s_chunk[threadIdx.x >> 5];
-  constexpr int K = PerLane<G>::K;
-  const unsigned long long unit = __ldcg(a.unit);  // 1: one warp per state this iteration
-  while (true) {
+  const uint64_t* muls = reinterpret_cast<const uint64_t*>(S.muls);
+  const int wid = threadIdx.x >> 5;
+  const uint32_t lane = threadIdx.x & 31;
+  WarpNet& wn = S.net[wid];
+  uint4* descs = S.descs[wid];
+  WarpStage st{S.stage[wid], 0};
+  WarpCache cache{W <= 2 ? S.cache[wid] : nullptr, (1u << kBatchCacheLog2) - 1u};
+  const SmemTarget tg{&wn, a.rounds};
+  const uint32_t unit = (uint32_t)__ldcg(a.unit);  // states per claim this iteration
+  const uint32_t* t = nullptr;
+  auto claim = [&]() {
     unsigned long long c = 0;
     if (lane == 0) c = atomicAdd(a.claim, 1ull);
-    c = __shfl_sync(FULLMASK, c, 0);
-    if (c >= __ldcg(a.prefix + a.n)) break;  // chunks of this iteration, all networks
-    // the network whose chunks contain c: largest i with prefix[i] <= c
+    return __shfl_sync(FULLMASK, c, 0);
+  };
+  unsigned long long c = claim();
+  while (c < total) {
+    // the network whose claims contain c: largest i with prefix[i] <= c
     int lo = 0, hi = a.n - 1;
     while (lo < hi) {
       const int mid = (lo + hi + 1) >> 1;
@@ -267,82 +277,60 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
       else hi = mid - 1;
     }
     BNet& b = a.nets[lo];
-    if (lo != cached_net) {  // stage the network; the cache holds one network's vectors at a time
-      if (lane == 0) {
-        wn.lay = b.lay;
-        wn.blob = b.blob;
-        wn.table = b.table;
-        wn.next_end = &b.next_end;
-        wn.frontier = b.frontier;
-        wn.fmask = b.fmask;
-        wn.cur_begin = b.cur_begin;
-        wn.log2nb = b.log2nb;
-      }
-      if (W <= 2)
-        for (uint32_t i = lane; i < (1u << kBatchCacheLog2) * CW; i += 32) cache_mem[threadIdx.x >> 5][i] = 0u;
-      __syncwarp();
-      cached_net = lo;
-    }
-    const uint32_t* t = wn.blob;
-    const NetBlobLayout& L = wn.lay;
-    const SmemTarget tg{&wn, a.rounds};
+    const unsigned long long c0 = __ldcg(a.prefix + lo), c1 = __ldcg(a.prefix + lo + 1);
+    // stage the network; the cache holds one network's vectors at a time
+    t = b.blob;
     if (lane == 0) {
-      const uint64_t first = wn.cur_begin + (c - __ldcg(a.prefix + lo)) * unit;
-      const uint64_t end = b.cur_end;
-      chunk_range[0] = first;
-      chunk_range[1] = first + unit < end ? first + unit : end;
+      wn.lay = b.lay;
+      wn.table = b.table;
+      wn.next_end = &b.next_end;
+      wn.frontier = b.frontier;
+      wn.fmask = b.fmask;
+      wn.cur_begin = b.cur_begin;
+      wn.cur_end = b.cur_end;
+      wn.log2nb = b.log2nb;
     }
+    if (W <= 2)
+      for (uint32_t i = lane; i < (uint32_t)BatchSmem<W>::kCache; i += 32) S.cache[wid][i] = 0u;
     __syncwarp();
-    uint32_t trans = 0;  // per claim: below 2^32 (a state's successors are, and chunks stay far below)
+    const NetBlobLayout& L = wn.lay;
+    const bool staged = L.n_procs <= (uint32_t)kWarpDescs;
+    if (staged && lane < L.n_procs) descs[lane] = proc_desc(t, L, lane);
+    __syncwarp();
     uint32_t probes = 0, err = 0;
-    // Lane layout: one state per lane (unit > 1), or, in an iteration with few
-    // states, one state per warp (unit == 1): every lane holds the state and
-    // takes its successors l, l + 32, ... (found by index), so their
-    // find-or-puts overlap instead of forming one lane's chain.
-    static_assert(K == 1, "one successor per lane and round");
-    const bool wide = unit == 1;
-    for (uint64_t sub = chunk_range[0]; sub < chunk_range[1]; sub += 32) {
-      const uint64_t idx = wide ? sub : sub + lane;
-      const bool valid = idx < chunk_range[1];
-      uint32_t v[W];
-#pragma unroll
-      for (int w = 0; w < W; ++w) v[w] = 0;
-      if (valid) load_vec<W>(wn.frontier + (idx & wn.fmask) * W, v);
-      const uint32_t cnt = valid ? count_succ<W>(t, L, v) : 0u;
-      if (valid && (!wide || lane == 0)) {  // the lane that accounts for the state
-        trans += cnt;
-        if (cnt == 0) {
-          const uint64_t h = state_digest<W>(t, L, v);
-          atomicAdd(&b.dl_count, 1ull);
-          atomicAdd(&b.dl_sum, (unsigned long long)h);
-          atomicXor(&b.dl_xor, (unsigned long long)h);
-        }
-      }
-      uint32_t remaining = !wide ? cnt : (cnt > (uint32_t)lane ? (cnt - lane + 31) / 32 : 0u);
-      uint32_t kk = lane;  // wide: index of this lane's next successor
-      SuccIter it;
-      it.init();
-      while (__any_sync(FULLMASK, remaining != 0)) {
-        uint32_t s[K][W];
-        bool has[K];
-        has[0] = remaining != 0;
-        if (has[0]) {
-          if (wide) {
-            seek_succ<W>(t, L, v, kk, s[0]);
-            kk += 32;
-          } else {
-            next_succ<W>(it, t, L, v, s[0]);
+    unsigned long long trans = 0;
+    uint64_t pos = 0, end = 0;  // what is left of the claim
+    bool held = true;           // c is a claim of this network that has not been started
+    expand_states<W, B, G, 32>(
+        tg, muls, t, L, S.queues[wid], st, probes, err,
+        [&](uint32_t p) { return staged ? descs[p] : proc_desc(t, L, p); },
+        [&](uint64_t& at, uint32_t& m) {
+          m = 0;
+          if (pos == end) {
+            if (!held) c = claim();
+            held = c < c1;
+            if (!held) return;  // another network's, or none are left
+            pos = wn.cur_begin + (c - c0) * unit;
+            end = pos + unit < wn.cur_end ? pos + unit : wn.cur_end;
+            held = false;
           }
-          --remaining;
-        } else {
-#pragma unroll
-          for (int w = 0; w < W; ++w) s[0][w] = 0;
-        }
-        insert_lanes<W, B, G, K>(tg, muls, g, has, s, probes, err, st, cache);
-      }
-    }
+          at = pos;
+          m = end - pos < 32 ? (uint32_t)(end - pos) : 32u;
+          pos += m;
+        },
+        [](const uint32_t(&)[W]) {},
+        [&](const uint32_t(&v)[W], uint32_t n) {
+          trans += n;
+          if (n == 0) {
+            const uint64_t h = state_digest<W>(t, L, v);
+            atomicAdd(&b.dl_count, 1ull);
+            atomicAdd(&b.dl_sum, (unsigned long long)h);
+            atomicXor(&b.dl_xor, (unsigned long long)h);
+          }
+        },
+        [&](uint64_t, uint64_t hh, const uint32_t(&x)[W]) { return !(cache.base && cache.template seen<W>(hh, x)); });
     st.flush<W>(tg, err);
-    const unsigned long long tr = warp_sum((unsigned long long)trans);
+    const unsigned long long tr = warp_sum(trans);
     const unsigned long long pr = warp_sum((unsigned long long)probes);
     err = __reduce_or_sync(FULLMASK, err);
     if (lane == 0) {
@@ -350,6 +338,7 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
       if (pr) atomicAdd(&b.probes, pr);
       if (err) atomicOr(&b.error, err);
     }
+    __syncwarp();
   }
 }
 
@@ -361,12 +350,14 @@ namespace {
 struct BatchKernels {
   const void* init;
   const void* expand;
+  size_t smem;  // dynamic shared memory of expand
 };
 
 template <int W, int B, int G>
 BatchKernels batch_kernels() {
   return BatchKernels{reinterpret_cast<const void*>(&gxd::batch_init_kernel<W, B, G>),
-                      reinterpret_cast<const void*>(&gxd::batch_expand_kernel<W, B, G>)};
+                      reinterpret_cast<const void*>(&gxd::batch_expand_kernel<W, B, G>),
+                      sizeof(gxd::BatchSmem<W>)};
 }
 
 // (B, G) pairs built for batches; the autotuner picks among them.
@@ -511,7 +502,8 @@ gx_status build_graph(gx_batch* h, const BatchPlan& P, void* ws, int sms) {
   GB_CUDA(cudaGraphConditionalHandleCreate(&cond, g, 1, cudaGraphCondAssignDefault));
 
   int per_sm = 0;
-  GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, P.k.expand, kBlock, 0));
+  GB_CUDA(cudaFuncSetAttribute(P.k.expand, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.k.smem));
+  GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, P.k.expand, kBlock, P.k.smem));
   const int grid = sms * std::max(per_sm, 1);
 
   BatchArgs a{};
@@ -540,12 +532,12 @@ gx_status build_graph(gx_batch* h, const BatchPlan& P, void* ws, int sms) {
   GB_CUDA(cudaGraphAddMemsetNode(&mset, g, nullptr, 0, &mp));
 
   auto add_kernel = [&](cudaGraph_t gr, const cudaGraphNode_t* deps, size_t nd, const void* fn,
-                        dim3 grid, dim3 block, void** args, cudaGraphNode_t* out) -> cudaError_t {
+                        dim3 grid, dim3 block, size_t smem, void** args, cudaGraphNode_t* out) -> cudaError_t {
     cudaKernelNodeParams kp{};
     kp.func = const_cast<void*>(fn);
     kp.gridDim = grid;
     kp.blockDim = block;
-    kp.sharedMemBytes = 0;
+    kp.sharedMemBytes = (unsigned)smem;
     kp.kernelParams = args;
     return cudaGraphAddKernelNode(out, gr, deps, nd, &kp);
   };
@@ -556,9 +548,9 @@ gx_status build_graph(gx_batch* h, const BatchPlan& P, void* ws, int sms) {
 
   cudaGraphNode_t init, adv1;
   const int per_block = kBlock / 32;
-  GB_CUDA(add_kernel(g, &mset, 1, P.k.init, dim3((n + per_block - 1) / per_block), dim3(kBlock), args_a, &init));
+  GB_CUDA(add_kernel(g, &mset, 1, P.k.init, dim3((n + per_block - 1) / per_block), dim3(kBlock), 0, args_a, &init));
   GB_CUDA(add_kernel(g, &init, 1, reinterpret_cast<const void*>(&gxd::batch_advance_kernel), dim3(1),
-                     dim3(1024), args_adv1, &adv1));
+                     dim3(1024), 0, args_adv1, &adv1));
 
   cudaGraphNodeParams cp{};
   cp.type = cudaGraphNodeTypeConditional;
@@ -570,9 +562,9 @@ gx_status build_graph(gx_batch* h, const BatchPlan& P, void* ws, int sms) {
   cudaGraph_t body = cp.conditional.phGraph_out[0];
 
   cudaGraphNode_t ex, adv0;
-  GB_CUDA(add_kernel(body, nullptr, 0, P.k.expand, dim3(grid), dim3(kBlock), args_a, &ex));
+  GB_CUDA(add_kernel(body, nullptr, 0, P.k.expand, dim3(grid), dim3(kBlock), P.k.smem, args_a, &ex));
   GB_CUDA(add_kernel(body, &ex, 1, reinterpret_cast<const void*>(&gxd::batch_advance_kernel), dim3(1),
-                     dim3(1024), args_adv0, &adv0));
+                     dim3(1024), 0, args_adv0, &adv0));
   cudaGraphExec_t exec;
   GB_CUDA(cudaGraphInstantiate(&exec, g, 0));
   h->exec = exec;

@@ -148,6 +148,80 @@ __device__ __forceinline__ bool cas_slot(uint32_t* p, const uint32_t (&v)[W], ui
   }
 }
 
+// Hash of a state vector: two odd multiplications with the upper half folded
+// into the lower one between them (a bucket comes from one more, bucket_of, so
+// every bit of the vector reaches its top bits), without vec_hash's finaliser.
+// The low bits are left out for the hash-constant set's number; the caches of
+// seen vectors take their index from the upper half.
+constexpr uint64_t kSeqMask = kMaxRounds - 1;
+template <int W>
+__device__ __forceinline__ uint64_t state_hash(const uint32_t (&v)[W]) {
+  uint64_t x = v[0];
+  if constexpr (W >= 2) x |= (uint64_t)v[1] << 32;
+  if constexpr (W == 4) x += ((uint64_t)v[2] | ((uint64_t)v[3] << 32)) * 0xD6E8FEB86659FD93ull;
+  x *= 0xBF58476D1CE4E5B9ull;
+  x ^= x >> 32;
+  x *= 0x94D049BB133111EBull;
+  return x & ~kSeqMask;
+}
+
+// The bucket that hash-constant set k gives hash h.
+template <int B>
+__device__ __forceinline__ uint64_t seq_bucket(uint64_t h, uint32_t k, const uint64_t* __restrict__ muls, int log2nb) {
+  const uint64_t b = bucket_of(h, muls[0], log2nb);
+  return k == 0 ? b : bucket_in_span<B>(h, muls[k], log2nb, b);
+}
+
+// One bucket of B words read by one lane: FOP_FOUND, FOP_INSERTED, or -1 when
+// it is full of other vectors.
+template <int W, int B>
+__device__ __forceinline__ int bucket_step(uint32_t* __restrict__ bucket, const uint32_t (&v)[W]) {
+  constexpr int S = B / W;
+  uint32_t s[B];
+  load_words<B>(bucket, s);
+  bool match = false;
+  uint32_t cand = 0;  // slots that are empty or half-written
+#pragma unroll
+  for (int j = 0; j < S; ++j) {
+    bool eq = true, tagged = true;
+#pragma unroll
+    for (int w = 0; w < W; ++w) {
+      eq &= (s[j * W + w] == v[w]);
+      tagged &= (s[j * W + w] & kTag) != 0;
+    }
+    match |= eq;
+    if (!tagged) cand |= 1u << j;
+  }
+  if (match) return FOP_FOUND;
+  // claim the first candidate; on failure the CAS tells what the slot holds
+  while (cand) {
+    const int j = __ffs(cand) - 1;
+    uint32_t old[W];
+    if (cas_slot<W>(bucket + j * W, v, old)) return FOP_INSERTED;
+    bool eq = true;
+#pragma unroll
+    for (int w = 0; w < W; ++w) eq &= (old[w] == v[w]);
+    if (eq) return FOP_FOUND;
+    cand &= ~(1u << j);
+  }
+  return -1;
+}
+
+// Find-or-put of one state by one lane, bucket after bucket; `probes` is
+// increased by the number of buckets read.
+template <int W, int B>
+__device__ __forceinline__ int find_or_put_state(uint32_t* __restrict__ table, int log2nb, int rounds,
+                                                 const uint64_t* __restrict__ muls, const uint32_t (&v)[W],
+                                                 uint32_t& probes) {
+  const uint64_t h = state_hash<W>(v);
+  for (int k = 0; k < rounds; ++k) {
+    ++probes;
+    const int r = bucket_step<W, B>(table + seq_bucket<B>(h, k, muls, log2nb) * (uint64_t)B, v);
+    if (r >= 0) return r;
+  }
+  return FOP_FULL;
+}
+
 template <int G>
 struct Group {
   uint32_t mask;  // lanes of this group within the warp
@@ -179,14 +253,12 @@ struct Group {
 // FOP_FULL (no free slot under any of the `rounds` hash-constant sets), the
 // same value in every lane of the group.  `probes` of the group's first lane
 // is increased by the number of buckets read (once per bucket, not per lane).
-// With PRE, `pre` already holds this lane's part of the first bucket (read by
-// the caller, and counted there), so round 0 starts without a load.
 // find_or_put_hashed takes h = vec_hash(v) from the caller.
-template <int W, int B, int G, bool PRE>
+template <int W, int B, int G>
 __device__ __forceinline__ int find_or_put_hashed(uint32_t* __restrict__ table, int log2nb, int rounds,
                                                   const uint64_t* __restrict__ muls,
                                                   const uint32_t (&v)[W], const uint64_t h, const Group<G>& g,
-                                                  uint32_t& probes, const uint32_t (&pre)[(B / W / G) * W]) {
+                                                  uint32_t& probes) {
   constexpr int S = B / W;
   static_assert(S >= 1 && S % G == 0, "group size must divide the slots per bucket");
   constexpr int SPL = S / G;
@@ -196,13 +268,8 @@ __device__ __forceinline__ int find_or_put_hashed(uint32_t* __restrict__ table, 
     const uint64_t b = k == 0 ? b0 : bucket_in_span<B>(h, muls[k], log2nb, b0);
     uint32_t* lane_slots = table + b * (uint64_t)B + (uint64_t)g.glane * LW;
     uint32_t s[LW];
-    if (PRE && k == 0) {
-#pragma unroll
-      for (int i = 0; i < LW; ++i) s[i] = pre[i];
-    } else {
-      load_words<LW>(lane_slots, s);
-      probes += g.glane == 0;
-    }
+    load_words<LW>(lane_slots, s);
+    probes += g.glane == 0;
     bool match = false;
     uint32_t cand = 0;  // slots that are empty or half-written
 #pragma unroll
@@ -244,12 +311,89 @@ __device__ __forceinline__ int find_or_put_hashed(uint32_t* __restrict__ table, 
   return FOP_FULL;
 }
 
-template <int W, int B, int G, bool PRE>
-__device__ __forceinline__ int find_or_put_from(uint32_t* __restrict__ table, int log2nb, int rounds,
-                                                const uint64_t* __restrict__ muls,
-                                                const uint32_t (&v)[W], const Group<G>& g,
-                                                uint32_t& probes, const uint32_t (&pre)[(B / W / G) * W]) {
-  return find_or_put_hashed<W, B, G, PRE>(table, log2nb, rounds, muls, v, vec_hash<W>(v), g, probes, pre);
+// Buckets a group of G lanes has in flight: its items' loads are issued
+// together while a lane's share of them fits 16 registers.
+template <int W, int B, int G>
+constexpr int kLanesInFlight = 16 / (B / G) < 1 ? 1 : (16 / (B / G) < G ? 16 / (B / G) : G);
+
+// One bucket for every lane with `has` set, read by groups of G > 1 lanes; all
+// 32 lanes call it together and each gets its own vector's result (as
+// bucket_step; -1 without one).  The lanes of a group read their items' buckets
+// together, several in flight, and vote; every item's owner then claims the
+// first free slot itself, so the compare-and-swaps of a group's items overlap
+// instead of following one another.
+template <int W, int B, int G>
+__device__ __forceinline__ int bucket_step_lanes(uint32_t* __restrict__ table, bool has, uint64_t b,
+                                                 const uint32_t (&v)[W]) {
+  constexpr int S = B / W;
+  static_assert(G > 1 && S % G == 0, "group size must divide the slots per bucket");
+  constexpr int SPL = S / G;
+  constexpr int LW = SPL * W;
+  constexpr int CH = kLanesInFlight<W, B, G>;
+  const Group<G> g;
+  bool found = false;
+  int slot = S;  // first slot of the bucket that is empty or half-written
+#pragma unroll 1
+  for (int c = 0; c < G; c += CH) {
+    uint32_t s[CH][LW];
+    bool on[CH];
+#pragma unroll
+    for (int j = 0; j < CH; ++j) {
+      on[j] = g.template bcast<int>(has ? 1 : 0, g.base + c + j) != 0;
+      const uint64_t bj = g.template bcast<unsigned long long>(b, g.base + c + j);
+      if (on[j]) load_words<LW>(table + bj * (uint64_t)B + (uint64_t)g.glane * LW, s[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < CH; ++j) {
+      if (!on[j]) continue;  // the same in every lane of the group
+      uint32_t x[W];
+#pragma unroll
+      for (int w = 0; w < W; ++w) x[w] = g.template bcast<uint32_t>(v[w], g.base + c + j);
+      bool match = false;
+      int first = -1;
+#pragma unroll
+      for (int i = SPL - 1; i >= 0; --i) {
+        bool eq = true, tagged = true;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+          eq &= (s[j][i * W + w] == x[w]);
+          tagged &= (s[j][i * W + w] & kTag) != 0;
+        }
+        match |= eq;
+        if (!tagged) first = i;
+      }
+      const bool hit = g.any(match);
+      const uint32_t free_lanes = g.ballot(first >= 0);
+      int at = S;
+      if (free_lanes) {
+        const int leader = __ffs(free_lanes) - 1;
+        at = (leader - g.base) * SPL + g.template bcast<int>(first, leader);
+      }
+      if (g.glane == c + j) {
+        found = hit;
+        slot = at;
+      }
+    }
+  }
+  int r = -1;
+  if (has) {
+    if (found) r = FOP_FOUND;
+    // slots fill in order: from the first free one on, each compare-and-swap
+    // that fails tells what the slot holds -- this vector, or another one
+    for (; r < 0 && slot < S; ++slot) {
+      uint32_t old[W];
+      if (cas_slot<W>(table + b * (uint64_t)B + slot * W, v, old)) {
+        r = FOP_INSERTED;
+      } else {
+        bool eq = true;
+#pragma unroll
+        for (int w = 0; w < W; ++w) eq &= (old[w] == v[w]);
+        if (eq) r = FOP_FOUND;
+      }
+    }
+  }
+  __syncwarp();
+  return r;
 }
 
 template <int W, int B, int G>
@@ -257,8 +401,7 @@ __device__ __forceinline__ int find_or_put(uint32_t* __restrict__ table, int log
                                            const uint64_t* __restrict__ muls,
                                            const uint32_t (&v)[W], const Group<G>& g,
                                            uint32_t& probes) {
-  const uint32_t none[(B / W / G) * W] = {};
-  return find_or_put_from<W, B, G, false>(table, log2nb, rounds, muls, v, g, probes, none);
+  return find_or_put_hashed<W, B, G>(table, log2nb, rounds, muls, v, vec_hash<W>(v), g, probes);
 }
 
 // ---- vector fields

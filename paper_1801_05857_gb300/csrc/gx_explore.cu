@@ -42,6 +42,22 @@ void hash_multipliers(uint64_t* out, int n) {
   }
 }
 
+bool cache_layout(const Net& net, uint32_t log2_entries, SeenCache& c) {
+  uint32_t bits = 0;
+  if (!cache_key(net, c.word_at, bits)) return false;
+  c.shift = bits > log2_entries ? bits - log2_entries : 0;
+  c.mask = bits < 64 ? (1ull << bits) - 1 : ~0ull;
+  c.tag_mask = c.shift < 64 ? (1ull << c.shift) - 1 : ~0ull;
+  c.half = (bits + 1) / 2;
+  c.log2_bytes = cache_entry_log2(bits, log2_entries);
+  return true;
+}
+
+uint32_t auto_cache_log2(const Net& net) {
+  uint32_t at[3], bits = 0;
+  return cache_key(net, at, bits) ? cache_auto_log2(bits) : 0;
+}
+
 }  // namespace gx
 
 namespace gx {
@@ -227,15 +243,13 @@ struct Plan {
   uint64_t part_min = 0;   // smallest level that may use the partitioned path
   uint32_t regions = 1;    // passes per level of the direct path (region passes)
   uint64_t gcache = 0;     // entries of the GPU-wide cache of seen vectors (0 = off)
-  uint32_t gkey[3] = {64, 64, 64};  // key offsets of words 1..3 (4-word vectors)
+  uint64_t gcache_bytes = 0;
+  SeenCache seen{};        // its layout (base left out)
   uint32_t warp_log2 = 0;  // per-warp cache of seen vectors: 2^warp_log2 entries (0 = off)
   uint64_t off_ctl = 0, off_blob = 0, off_dl = 0, off_viol = 0, off_loop = 0, off_front = 0, off_table = 0;
   uint64_t off_hist = 0, off_off = 0, off_ptot = 0, off_tot = 0, off_succ = 0, off_gcache = 0;
   uint64_t total = 0;
   const KernelSet* ks = nullptr;
-  // the level kernel: ks->expand, or the queued second kernel with region passes
-  cudaError_t (*expand)(const ExpandArgs&, int, size_t, cudaStream_t) = nullptr;
-  const void* expand_fn = nullptr;
 };
 
 gx_status make_plan(const Net& net, const gx_explore_opts* o, Plan& P) {
@@ -294,25 +308,21 @@ gx_status make_plan(const Net& net, const gx_explore_opts* o, Plan& P) {
     while (P.regions < 16 && tbytes / P.regions > kAutoRegionBytes) P.regions *= 2;
   }
   if (P.regions > P.nb) P.regions = (uint32_t)P.nb;
-  // with region passes most generated successors fall outside the pass's region:
-  // the queued kernel (where it is a second one) probes only those inside it, 32 at a time
-  const bool queued = P.regions > 1 && P.ks->expand_queued;
-  P.expand = queued ? P.ks->expand_queued : P.ks->expand;
-  P.expand_fn = queued ? P.ks->expand_queued_fn : P.ks->expand_fn;
-  // the caches of seen vectors: auto = the GPU-wide one (2^23 entries) for 1- and
-  // 2-word vectors in tables of at least 2^26 slots with one lane per bucket (where it
-  // was measured), else the per-warp one (2^9)
-  // (4-word vectors use it only when their fields fit one 64-bit key)
-  const bool key_fits = P.W <= 2 || gx::cache_key_shifts(net, P.gkey);
-  if (o->global_cache_log2 == kAutoCache) {
-    if (P.W <= 2 && P.G == 1 && slots >= (1ull << 26)) P.gcache = 1ull << 23;
-  } else if (o->global_cache_log2) {
-    if (o->global_cache_log2 > 26) return fail(GX_ERR_INVALID, "global_cache_log2 must be at most 26");
-    if (key_fits) P.gcache = 1ull << o->global_cache_log2;
+  // the caches of seen vectors: auto = the GPU-wide one in tables of at least 2^26 slots
+  // with one lane per bucket (where it was measured), for vectors whose fields fit one
+  // 64-bit key, else the per-warp one (2^9).  4-word vectors: only in one pass (1.08e8-state
+  // irregular network, 4 GiB: 42 ms with it, 50 ms without; the memory-filling product
+  // network in two passes, 8 GiB: 231 ms with it, 186 ms without)
+  uint32_t glog = o->global_cache_log2;
+  if (glog == kAutoCache)
+    glog = P.G == 1 && slots >= (1ull << 26) && (P.W <= 2 || P.regions == 1) ? auto_cache_log2(net) : 0;
+  else if (glog > 26) return fail(GX_ERR_INVALID, "global_cache_log2 must be at most 26");
+  if (glog && cache_layout(net, glog, P.seen)) {
+    P.gcache = 1ull << glog;
+    P.gcache_bytes = P.gcache << P.seen.log2_bytes;
   }
-  // (the queued 4-word kernel: 2^6, whose 4 KiB per CTA leave room for 5 CTAs per SM;
-  // 2^9 took 4.55 s on the memory-scaled network, 2^6 3.52 s)
-  P.warp_log2 = o->warp_cache_log2 == kAutoCache ? (P.gcache ? 0u : queued ? 6u : 9u) : o->warp_cache_log2;
+  // (4-word vectors: 2^6, whose 4 KiB per CTA leave room for 5 CTAs per SM beside the queues)
+  P.warp_log2 = o->warp_cache_log2 == kAutoCache ? (P.gcache ? 0u : P.W == 4 ? 6u : 9u) : o->warp_cache_log2;
   P.cs = o->successor_buffer ? o->successor_buffer : std::min<uint64_t>(slots / 2, (1ull << 32) - 1);
   if (P.logp == 0) P.cs = 0;  // partitioned path off: no buffer
   if (P.cs >= (1ull << 32)) return fail(GX_ERR_INVALID, "successor_buffer must be below 2^32 vectors");
@@ -343,7 +353,7 @@ gx_status make_plan(const Net& net, const gx_explore_opts* o, Plan& P) {
   P.off_succ = off;
   off = align_up(off + 4ull * P.W * P.cs);
   P.off_gcache = off;
-  off = align_up(off + 8ull * P.gcache);
+  off = align_up(off + P.gcache_bytes);
   P.total = off;
   return GX_OK;
 }
@@ -420,7 +430,7 @@ gx_status build_loop_graph(gx_net* h, const Plan& P, Ctl* ctl, uint32_t* table, 
   const uint64_t words = (uint64_t)P.B * P.nb;
   constexpr uint64_t kPiece = 1ull << 30;  // words per memset node
   for (uint64_t w0 = 0; w0 < words; w0 += kPiece) GX_CUDA(add_memset(table + w0, std::min(kPiece, words - w0)));
-  if (eg.gcache) GX_CUDA(add_memset(eg.gcache, 2 * P.gcache));
+  if (eg.gcache.base) GX_CUDA(add_memset(eg.gcache.base, (P.gcache_bytes + 3) / 4));
   auto add_kernel = [&](cudaGraph_t gr, const cudaGraphNode_t* deps, size_t nd, const void* fn, dim3 gd, dim3 bd,
                         size_t sh, void** args, cudaGraphNode_t* out) -> cudaError_t {
     cudaKernelNodeParams kp{};
@@ -448,7 +458,7 @@ gx_status build_loop_graph(gx_net* h, const Plan& P, Ctl* ctl, uint32_t* table, 
   cudaGraphNode_t cnode;
   GX_CUDA(cudaGraphAddNode(&cnode, g, &start, nullptr, 1, &cp));
   cudaGraph_t body = cp.conditional.phGraph_out[0];
-  GX_CUDA(add_kernel(body, nullptr, 0, P.expand_fn, dim3((unsigned)grid), dim3(kBlock), smem, args_e, &ex));
+  GX_CUDA(add_kernel(body, nullptr, 0, P.ks->expand_fn, dim3((unsigned)grid), dim3(kBlock), smem, args_e, &ex));
   // region passes after the first: clear the claim counter, expand again
   for (uint32_t q = 1; q < P.regions; ++q) {
     ExpandArgs eq = region_pass(eg, P.regions, q);
@@ -461,7 +471,7 @@ gx_status build_loop_graph(gx_net* h, const Plan& P, Ctl* ctl, uint32_t* table, 
     mp.height = 1;
     cudaGraphNode_t mz, exq;
     GX_CUDA(cudaGraphAddMemsetNode(&mz, body, &ex, 1, &mp));
-    GX_CUDA(add_kernel(body, &mz, 1, P.expand_fn, dim3((unsigned)grid), dim3(kBlock), smem, args_q, &exq));
+    GX_CUDA(add_kernel(body, &mz, 1, P.ks->expand_fn, dim3((unsigned)grid), dim3(kBlock), smem, args_q, &exq));
     ex = exq;
   }
   GX_CUDA(add_kernel(body, &ex, 1, reinterpret_cast<const void*>(&gxd::level_advance_kernel), dim3(1), dim3(1), 0,
@@ -533,11 +543,12 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
   // levels on the device unless asked otherwise; the partitioned path needs the host
   const bool device_loop = !o->host_loop && P.logp == 0;
   GX_CUDA(cudaEventRecord(ev0, st));
-  unsigned long long* gcache = P.gcache ? reinterpret_cast<unsigned long long*>(base + P.off_gcache) : nullptr;
+  SeenCache gcache = P.seen;
+  gcache.base = P.gcache ? base + P.off_gcache : nullptr;
   if (!device_loop) {
     GX_CUDA(cudaMemsetAsync(ctl, 0, sizeof(Ctl), st));
     GX_CUDA(cudaMemsetAsync(table, 0, 4ull * P.B * P.nb, st));
-    if (gcache) GX_CUDA(cudaMemsetAsync(gcache, 0, 8ull * P.gcache, st));
+    if (gcache.base) GX_CUDA(cudaMemsetAsync(gcache.base, 0, P.gcache_bytes, st));
   }
 
   InitArgs ia{};
@@ -565,8 +576,6 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
   ea.dl_cap = P.dl_cap;
   ea.count_states = 1;  // region passes set their own (region_pass)
   ea.gcache = gcache;
-  ea.gcache_mask = P.gcache ? P.gcache - 1 : 0;
-  for (int w = 0; w < 3; ++w) ea.gkey_shift[w] = P.gkey[w];
   uint32_t* viol = reinterpret_cast<uint32_t*>(base + P.off_viol);
   if (o->watch) {
     const uint32_t wp = o->watch_proc;
@@ -578,25 +587,42 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
     ea.viol_buf = viol;
     ea.viol_cap = P.viol_cap;
   }
-  size_t smem = 8ull * kMaxRounds;
+  cudaFuncAttributes fa{};
+  GX_CUDA(cudaFuncGetAttributes(&fa, P.ks->expand_fn));
   const size_t blob_bytes = 4ull * net.blob.size();
-  ea.stage = (smem + blob_bytes <= std::min<size_t>(dev.smem_optin, 96 * 1024)) ? 1 : 0;
-  if (ea.stage) smem += blob_bytes;
+  size_t cache_bytes = 0;
   ea.cache_log2 = 0;
   if (P.warp_log2) {
     ea.cache_log2 = (int)P.warp_log2;
     if (ea.cache_log2 > 12) return fail(GX_ERR_INVALID, "warp_cache_log2 must be at most 12");
     if (P.W == 4) ea.cache_log2 -= 1;  // 16-byte entries: the same bytes as 2^n 2-word ones
-    smem += 4ull * P.W * (kBlock / 32) * (1ull << ea.cache_log2);
-    if (smem > dev.smem_optin)
-      return fail(GX_ERR_INVALID, "warp cache of 2^" + std::to_string(ea.cache_log2) + " entries per warp needs " +
-                                      std::to_string(smem) + " bytes of shared memory per CTA, more than " +
-                                      std::to_string(dev.smem_optin));
+    cache_bytes = 4ull * P.W * (kBlock / 32) * (1ull << ea.cache_log2);
   }
-  GX_CUDA(cudaFuncSetAttribute(P.expand_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  size_t smem = 8ull * kMaxRounds + cache_bytes;
+  if (fa.sharedSizeBytes + smem > dev.smem_optin)
+    return fail(GX_ERR_INVALID, "warp cache of 2^" + std::to_string(ea.cache_log2) + " entries per warp needs " +
+                                    std::to_string(fa.sharedSizeBytes + smem) +
+                                    " bytes of shared memory per CTA, more than " + std::to_string(dev.smem_optin));
+  // the network tables are staged unless they are large or leave no room for the cache
+  ea.stage = blob_bytes + 8ull * kMaxRounds <= 96 * 1024 &&
+                     fa.sharedSizeBytes + smem + blob_bytes <= dev.smem_optin ? 1 : 0;
+  if (ea.stage) smem += blob_bytes;
+  GX_CUDA(cudaFuncSetAttribute(P.ks->expand_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
-  GX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, P.expand_fn, kBlock, smem));
+  GX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, P.ks->expand_fn, kBlock, smem));
   if (per_sm < 1) return fail(GX_ERR_INVALID, "expansion kernel does not fit on an SM");
+  // Shared memory beyond 196 KB an SM leaves the GPU-wide cache's lookups too little L1 to
+  // be in flight in (mid network, padded from 186 to 214 KB: 19 ms became 30 ms), so a
+  // network with large tables runs fewer CTAs.
+  if (gcache.base) {
+    const size_t cta = fa.sharedSizeBytes + smem + 1024, most = 196 * 1024;
+    if (cta * per_sm > most) per_sm = std::max<int>(1, (int)(most / cta));
+    GX_CUDA(cudaFuncSetAttribute(P.ks->expand_fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)std::min<size_t>(100, (cta * per_sm * 100 + 228 * 1024 - 1) / (228 * 1024))));
+  } else {
+    GX_CUDA(cudaFuncSetAttribute(P.ks->expand_fn, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                 (int)cudaSharedmemCarveoutDefault));
+  }
   if (o->ctas_per_sm) per_sm = std::min<int>(per_sm, (int)o->ctas_per_sm);
   const uint64_t max_grid = (uint64_t)dev.sms * per_sm;
 
@@ -724,12 +750,11 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
       }
     }
     if (direct) {
-      const uint64_t warps = (F + 31) / 32;
-      const uint64_t want = (warps + kBlock / 32 - 1) / (kBlock / 32);
+      const uint64_t want = (F + kBlock / 32 - 1) / (kBlock / 32);  // a warp per state while they last
       const int grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(want, max_grid));
       for (uint32_t q = 0; q < P.regions; ++q) {
         GX_CUDA(cudaMemsetAsync(&ctl->claim, 0, sizeof(unsigned long long), st));
-        GX_CUDA(P.expand(region_pass(ea, P.regions, q), grid, smem, st));
+        GX_CUDA(P.ks->expand(region_pass(ea, P.regions, q), grid, smem, st));
         ++launches;
       }
     }

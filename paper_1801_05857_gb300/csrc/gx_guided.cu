@@ -94,10 +94,9 @@ template <int W, int B>
 __device__ __forceinline__ int64_t find_slot(const uint32_t* __restrict__ table, int log2nb, int rounds,
                                              const uint64_t* __restrict__ muls, const uint32_t (&v)[W]) {
   constexpr int S = B / W;
-  const uint64_t h = vec_hash<W>(v);
-  const uint64_t b0 = bucket_of(h, muls[0], log2nb);
+  const uint64_t h = state_hash<W>(v);
   for (int k = 0; k < rounds; ++k) {
-    const uint64_t b = k == 0 ? b0 : bucket_in_span<B>(h, muls[k], log2nb, b0);
+    const uint64_t b = seq_bucket<B>(h, k, muls, log2nb);
     uint32_t s[B];
     load_words<B>(table + b * (uint64_t)B, s);
 #pragma unroll
@@ -323,9 +322,8 @@ __global__ void __launch_bounds__(32) guided_init_kernel(const GuidedArgs a) {
   for (int w = 0; w < W; ++w) v[w] = a.init_vec[w];
   uint32_t hw[4], bad = 0;
   local_hist<W>(a.blob, a.lay, v, hw, bad);
-  const Group<1> g;
   uint32_t probes = 0, err = bad ? gx::ERR_WIDE : 0u;
-  const int r = find_or_put<W, B, 1>(a.table, a.log2nb, a.rounds, muls, v, g, probes);
+  const int r = find_or_put_state<W, B>(a.table, a.log2nb, a.rounds, muls, v, probes);
   if (r != FOP_INSERTED) err |= gx::ERR_TABLE_FULL;
   else {
     a.ctl->inserted = 1;
@@ -414,7 +412,6 @@ __global__ void __launch_bounds__(gx::kBlock) guided_expand_kernel(const GuidedA
   __syncthreads();
   const NetBlobLayout& L = a.lay;
   const int lane = threadIdx.x & 31;
-  const Group<1> g;
   const unsigned long long log_base = a.ctl->log_base;
   unsigned long long trans = 0, ins = 0;
   uint32_t probes = 0, err = 0;
@@ -449,7 +446,7 @@ __global__ void __launch_bounds__(gx::kBlock) guided_expand_kernel(const GuidedA
       bool inserted = false;
       if (k < total) {
         seek_succ<W>(t, L, v, k, s);
-        const int r = find_or_put<W, B, 1>(a.table, a.log2nb, a.rounds, muls, s, g, probes);
+        const int r = find_or_put_state<W, B>(a.table, a.log2nb, a.rounds, muls, s, probes);
         if (r == FOP_FULL) err |= gx::ERR_TABLE_FULL;
         inserted = r == FOP_INSERTED;
       }
@@ -601,7 +598,6 @@ __global__ void __launch_bounds__(kFusedThreads, 2) guided_fused_kernel(const Gu
   __syncthreads();
   if (!s_ok) err |= gx::ERR_SPIN;
   const NetBlobLayout& L = a.lay;
-  const Group<1> g;
   const unsigned long long log_base = a.ctl->log_base;
   unsigned long long trans = 0, ins = 0;
   uint32_t probes = 0;
@@ -668,7 +664,7 @@ __global__ void __launch_bounds__(kFusedThreads, 2) guided_fused_kernel(const Gu
       bool inserted = false;
       if (k < total) {
         seek_succ<W>(t, L, v, k, s);
-        const int res = find_or_put<W, B, 1>(a.table, a.log2nb, a.rounds, muls, s, g, probes);
+        const int res = find_or_put_state<W, B>(a.table, a.log2nb, a.rounds, muls, s, probes);
         if (res == FOP_FULL) err |= gx::ERR_TABLE_FULL;
         inserted = res == FOP_INSERTED;
       }

@@ -52,23 +52,37 @@ struct Net {
   uint32_t init_vec[kMaxWords] = {0, 0, 0, 0};
 };
 
-// Bit offsets of words 1..3 in the 64-bit key that the GPU-wide cache of seen
-// vectors stores for a vector: each word's payload (its fields sit at the low
-// bits of the word) follows the previous word's, and a word without fields gets
-// 64 (left out).  Returns false when the fields take more than 64 bits in all,
-// so that no such key exists.
-inline bool cache_key_shifts(const Net& n, uint32_t (&s)[3]) {
+// Key of a vector in the GPU-wide cache of seen vectors: its words' payloads side
+// by side (fields sit at the low bits of a word).  Bit offsets of words 1..3 (64
+// for a word without fields) and the key's length; false when it is over 64
+// bits, so that there is no such key.
+inline bool cache_key(const Net& n, uint32_t (&at)[3], uint32_t& bits) {
   uint32_t used[kMaxWords] = {0, 0, 0, 0};
   for (uint32_t p = 0; p < n.n_procs; ++p) {
     const uint32_t end = n.field_shift[p] + n.field_bits[p];
     if (end > used[n.field_word[p]]) used[n.field_word[p]] = end;
   }
-  uint32_t off = used[0];
+  bits = used[0];
   for (int w = 1; w < 4; ++w) {
-    s[w - 1] = used[w] ? off : 64u;
-    off += used[w];
+    at[w - 1] = used[w] ? bits : 64u;
+    bits += used[w];
   }
-  return off <= 64;
+  return bits <= 64;
+}
+
+// log2 of the bytes of an entry of a cache of 2^n entries for keys of `bits`
+// bits: the bits the entry's index does not give, in 2, 4 or 8 bytes.
+inline uint32_t cache_entry_log2(uint32_t bits, uint32_t n) {
+  const uint32_t tag = bits > n ? bits - n : 0;
+  return tag <= 16 ? 1 : (tag <= 32 ? 2 : 3);
+}
+
+// Entries (log2) of the automatic GPU-wide cache: as many as fit 64 MiB of the
+// 129 MB L2, at most 2^25.
+inline uint32_t cache_auto_log2(uint32_t bits) {
+  uint32_t n = 25;
+  while (n + cache_entry_log2(bits, n) > 26) --n;
+  return n;
 }
 
 }  // namespace gx

@@ -240,11 +240,6 @@ __device__ __forceinline__ const uint32_t* stage_tables(uint32_t* sm, const gx::
   return s_tab;
 }
 
-// Offsets in a 64-bit key of the payload of words 1..3 (ExpandArgs.gkey_shift).
-struct GKey {
-  uint32_t s[3];
-};
-
 // Where find-or-put inserts and where new vectors go: one network's table and
 // frontier ring (the level being expanded starts at begin()).  Target holds
 // the values (the batched kernel loads them per network); ParamTarget reads
@@ -266,9 +261,7 @@ struct Target {
   __device__ __forceinline__ uint64_t begin() const { return cur_begin; }
   __device__ __forceinline__ uint64_t region_mask() const { return 0; }
   __device__ __forceinline__ uint64_t region_bits() const { return 0; }
-  __device__ __forceinline__ unsigned long long* gcache() const { return nullptr; }
-  __device__ __forceinline__ uint64_t gcache_mask() const { return 0; }
-  __device__ __forceinline__ GKey gkey() const { return GKey{{64u, 64u, 64u}}; }
+  __device__ __forceinline__ gx::SeenCache gcache() const { return gx::SeenCache{}; }
 };
 
 struct ParamTarget {
@@ -283,15 +276,14 @@ struct ParamTarget {
   __device__ __forceinline__ uint64_t begin() const { return range[0]; }
   __device__ __forceinline__ uint64_t region_mask() const { return a.region_mask; }
   __device__ __forceinline__ uint64_t region_bits() const { return a.region_bits; }
-  __device__ __forceinline__ unsigned long long* gcache() const { return a.gcache; }
-  __device__ __forceinline__ uint64_t gcache_mask() const { return a.gcache_mask; }
-  __device__ __forceinline__ GKey gkey() const { return GKey{{a.gkey_shift[0], a.gkey_shift[1], a.gkey_shift[2]}}; }
+  __device__ __forceinline__ const gx::SeenCache& gcache() const { return a.gcache; }
 };
 
 // Per-warp staging of new vectors in shared memory: lanes that inserted a
-// vector append it here (ballot + popc, no atomic); every 32 staged vectors
-// are written to the next level with one global atomicAdd and one coalesced
-// store.  flush() writes what is left.  All 32 lanes call push/flush together.
+// vector append it here (ballot + popc, no atomic); whenever 32 are staged the
+// last 32 are written to the next level with one global atomicAdd and one
+// coalesced store.  flush() writes what is left.  All 32 lanes call push/flush
+// together.
 constexpr int kStage = 64;  // vectors per warp (at most 31 + 32 are ever staged)
 
 struct WarpStage {
@@ -304,14 +296,15 @@ struct WarpStage {
     unsigned long long base = 0;
     if (lane == 0) base = atomicAdd(a.next_end(), (unsigned long long)m);
     base = __shfl_sync(FULLMASK, base, 0);
+    n -= m;
     if (lane < m) {
       const uint64_t pos = base + lane;
       uint32_t v[W];
-#pragma unroll
-      for (int w = 0; w < W; ++w) v[w] = buf[lane * W + w];
+      load_vec<W>(buf + (n + lane) * W, v);
       if (pos - a.begin() <= a.fmask()) store_vec<W>(a.frontier() + (pos & a.fmask()) * W, v);
       else err |= gx::ERR_FRONTIER;
     }
+    __syncwarp();
   }
 
   template <int W, class T>
@@ -319,32 +312,15 @@ struct WarpStage {
                                        uint32_t& err) {
     const int lane = threadIdx.x & 31;
     const uint32_t im = __ballot_sync(FULLMASK, ins);
-    if (ins) {
-      const int at = n + __popc(im & ((1u << lane) - 1u));
-#pragma unroll
-      for (int w = 0; w < W; ++w) buf[at * W + w] = v[w];
-    }
+    if (ins) store_vec<W>(buf + (n + __popc(im & ((1u << lane) - 1u))) * W, v);
     n += __popc(im);
-    if (n >= 32) {
-      __syncwarp();
-      write_out<W>(a, 32, err);
-      __syncwarp();
-      // move the remainder (fewer than 32) to the front
-      if (lane < n - 32) {
-#pragma unroll
-        for (int w = 0; w < W; ++w) buf[lane * W + w] = buf[(32 + lane) * W + w];
-      }
-      n -= 32;
-      __syncwarp();
-    }
+    __syncwarp();
+    if (n >= 32) write_out<W>(a, 32, err);
   }
 
   template <int W, class T>
   __device__ __forceinline__ void flush(const T& a, uint32_t& err) {
-    __syncwarp();
     if (n > 0) write_out<W>(a, n, err);
-    n = 0;
-    __syncwarp();
   }
 };
 
@@ -361,19 +337,19 @@ struct WarpCache {
   template <int W>
   __device__ __forceinline__ bool seen(uint64_t h, const uint32_t (&v)[W]) const {
     if constexpr (W == 1) {
-      uint32_t* e = base + ((uint32_t)h & mask);
+      uint32_t* e = base + ((uint32_t)(h >> 40) & mask);
       if (*e == v[0]) return true;
       *e = v[0];
       return false;
     } else if constexpr (W == 2) {
-      unsigned long long* e = reinterpret_cast<unsigned long long*>(base) + ((uint32_t)h & mask);
+      unsigned long long* e = reinterpret_cast<unsigned long long*>(base) + ((uint32_t)(h >> 40) & mask);
       const unsigned long long x = (unsigned long long)v[0] | ((unsigned long long)v[1] << 32);
       if (*e == x) return true;
       *e = x;
       return false;
     } else {
       static_assert(W == 4, "slot width");
-      uint4* e = reinterpret_cast<uint4*>(base) + ((uint32_t)h & mask);
+      uint4* e = reinterpret_cast<uint4*>(base) + ((uint32_t)(h >> 40) & mask);
       const uint4 c = *e;
       if (c.x == v[0] && c.y == v[1] && c.z == v[2] && c.w == v[3]) return true;
       *e = make_uint4(v[0], v[1], v[2], v[3]);
@@ -382,226 +358,340 @@ struct WarpCache {
   }
 };
 
-// GPU-wide cache of recently seen vectors: direct-mapped, 2^k 64-bit entries in
-// global memory (a few MB, so it stays in L2), cleared at the start of a search.
-// A vector is written into it after its find-or-put found or inserted it, so
-// every entry is a vector of the table and a hit can skip the table probe.
-// Only 1- and 2-word vectors: an aligned 64-bit load or store is one access, so
-// an entry is never seen half-written.  Successors of a level mostly lead into
-// the levels just before and after it, which were inserted or looked up
-// moments earlier by some warp of the GPU.
+// GPU-wide cache of recently seen vectors (gx::SeenCache).  A vector is written
+// into it after its find-or-put found or inserted it, so every entry is a vector
+// of the table and a hit can skip the table probe.  An aligned load or store of
+// an entry is one access, so an entry is never seen half-written.  Successors of
+// a level mostly lead into the levels just before and after it, which were
+// inserted or looked up moments earlier by some warp of the GPU.
+// What bounds the searches that use it is DRAM traffic of random lines (128
+// bytes per bucket read, entry missed in L2 or entry written back), so entries
+// are as small as the vectors allow: the 62M-state mid network (40 bits)
+// takes 2^25 entries of 16 bits in the 64 MiB that held 2^23 of 64 bits.
+struct SeenEntry {
+  uint64_t index;
+  unsigned long long content;  // 0: this vector is never cached
+};
 template <int W>
-__device__ __forceinline__ unsigned long long gcache_key(const uint32_t (&v)[W], const GKey& k) {
-  if constexpr (W == 1) {
-    return (unsigned long long)v[0];
-  } else if constexpr (W == 2) {
-    return (unsigned long long)v[0] | ((unsigned long long)v[1] << 32);
+__device__ __forceinline__ SeenEntry seen_entry(const gx::SeenCache& c, const uint32_t (&v)[W]) {
+  uint64_t y = v[0] & ~kTag;
+#pragma unroll
+  for (int w = 1; w < W; ++w)
+    if (c.word_at[w - 1] < 64) y |= (uint64_t)(v[w] & ~kTag) << c.word_at[w - 1];
+  // a bijection of the numbers below 2^bits: odd multiplications and a xor-shift
+  y = (y * 0xD6E8FEB86659FD93ull) & c.mask;
+  y ^= y >> c.half;
+  y = (y * 0x9E3779B97F4A7C15ull) & c.mask;
+  SeenEntry e;
+  e.index = c.shift < 64 ? y >> c.shift : 0ull;
+  e.content = (y & c.tag_mask) + 1;
+  if (c.log2_bytes == 1) e.content &= 0xFFFFull;  // (the one content that does not fit becomes 0)
+  else if (c.log2_bytes == 2) e.content &= 0xFFFFFFFFull;
+  return e;
+}
+__device__ __forceinline__ unsigned long long seen_get(const gx::SeenCache& c, uint64_t i) {
+  if (c.log2_bytes == 1) return __ldcg(static_cast<const unsigned short*>(c.base) + i);
+  if (c.log2_bytes == 2) return __ldcg(static_cast<const unsigned int*>(c.base) + i);
+  return __ldcg(static_cast<const unsigned long long*>(c.base) + i);
+}
+__device__ __forceinline__ void seen_put(const gx::SeenCache& c, const SeenEntry& e) {
+  if (c.log2_bytes == 1) __stcg(static_cast<unsigned short*>(c.base) + e.index, (unsigned short)e.content);
+  else if (c.log2_bytes == 2) __stcg(static_cast<unsigned int*>(c.base) + e.index, (unsigned int)e.content);
+  else __stcg(static_cast<unsigned long long*>(c.base) + e.index, e.content);
+}
+
+// One step of find-or-put for the vector x of every lane with has set: the
+// bucket, read by G lanes, that hash-constant set k gives it.  A lane whose
+// vector is settled (r >= 0) has the GPU-wide cache updated and a new vector
+// staged for the next level.  All 32 lanes call it together.
+template <int W, int B, int G, class T>
+__device__ __forceinline__ int resolve_lanes(const T& a, const uint64_t* muls, bool has, const uint32_t (&x)[W],
+                                             uint64_t h, uint32_t k, uint32_t& probes, uint32_t& err, WarpStage& st) {
+  int r = -1;
+  const uint64_t b = seq_bucket<B>(h, k, muls, a.log2nb());
+  if constexpr (G == 1) {
+    if (has) r = bucket_step<W, B>(a.table() + b * (uint64_t)B, x);
   } else {
-    // the payload bits of the words side by side (fields sit at the low bits of
-    // each word, so the words' payloads do not overlap): one key per vector
-    unsigned long long key = v[0] & ~kTag;
-#pragma unroll
-    for (int w = 1; w < W; ++w)
-      if (k.s[w - 1] < 64) key |= (unsigned long long)(v[w] & ~kTag) << k.s[w - 1];
-    return key;
+    r = bucket_step_lanes<W, B, G>(a.table(), has, b, x);
   }
-}
-// Keys of 1- and 2-word vectors carry the tag bits and are never 0 (an empty
-// entry); the one 4-word vector whose key is 0 is never cached.
-template <int W>
-__device__ __forceinline__ bool gcache_hit(const unsigned long long* c, uint64_t mask, uint64_t h,
-                                           const uint32_t (&v)[W], const GKey& k) {
-  const unsigned long long key = gcache_key<W>(v, k);
-  return (W <= 2 || key != 0ull) && __ldcg(c + ((h >> 32) & mask)) == key;
-}
-template <int W>
-__device__ __forceinline__ void gcache_put(unsigned long long* c, uint64_t mask, uint64_t h, const uint32_t (&v)[W],
-                                           const GKey& k) {
-  const unsigned long long key = gcache_key<W>(v, k);
-  if (W <= 2 || key != 0ull) __stcg(c + ((h >> 32) & mask), key);
+  probes += has;
+  if (r >= 0 && a.gcache().base) seen_put(a.gcache(), seen_entry<W>(a.gcache(), x));
+  st.push<W>(a, r == FOP_INSERTED, x, err);
+  return r;
 }
 
-// Successors each lane generates per round.  insert_lanes takes K per lane
-// (the group issues the first-bucket loads of up to four items before it
-// resolves any of them); measured on the mid network, K = 2 or 4 costs more in
-// registers and occupancy than it gains in loads in flight, so K = 1.
-template <int G>
-struct PerLane {
-  static constexpr int K = 1;
-};
+// What a warp needs of process p to generate its local successors, one 16-byte
+// shared-memory read: word, shift and mask of the field, and where the offsets
+// of its local edges start in the network tables.
+__device__ __forceinline__ uint4 proc_desc(const uint32_t* t, const NetBlobLayout& L, uint32_t p) {
+  return make_uint4(t[L.proc_word + p], t[L.proc_shift + p], t[L.proc_mask + p], L.coff + t[L.cls_base + p]);
+}
+constexpr int kMaxProcs = 124;  // gx_load_network's limit
 
-// Find-or-put of the K vectors each lane holds (has[k]: lane holds vector k),
-// G lanes per bucket.  Phase 1 issues the first-bucket loads of all G*K items
-// of the group; phase 2 resolves them in order (found in the first bucket, or
-// the full find-or-put with the CAS and further rounds).  Vectors this call
-// inserted go to the warp's staging buffer.
-// Must be called by all 32 lanes of the warp together.
-template <int W, int B, int G, int K, class T>
-__device__ __forceinline__ void insert_lanes(const T& a, const uint64_t* muls,
-                                             const Group<G>& g, const bool (&has)[K],
-                                             const uint32_t (&s)[K][W], uint32_t& probes,
-                                             uint32_t& err, WarpStage& st,
-                                             const WarpCache& cache = WarpCache{nullptr, 0}) {
-  constexpr int LW = (B / W / G) * W;
-  constexpr int NI = G * K;            // items of the group this round
-  constexpr int CH = NI < 4 ? NI : 4;  // items in flight at a time
-  bool inserted[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) inserted[k] = false;
-#pragma unroll 1
-  for (int c = 0; c < NI; c += CH) {
-    uint32_t x[CH][W];
-    uint32_t pre[CH][LW];
-    bool hv[CH];
-#pragma unroll
-    for (int j = 0; j < CH; ++j) {
-      const int i = c + j;
-      const int src = g.base + i / K;
-      hv[j] = g.template bcast<int>(has[i % K] ? 1 : 0, src) != 0;  // uniform in the group
-#pragma unroll
-      for (int w = 0; w < W; ++w) x[j][w] = g.template bcast<uint32_t>(s[i % K][w], src);
-      if (hv[j]) {
-        const uint64_t hh = vec_hash<W>(x[j]);
-        const uint64_t b = bucket_of(hh, muls[0], a.log2nb());
-        // region passes: a vector whose first bucket lies outside this pass's region is
-        // left to the pass of that region (tested before the cache, which may only hold
-        // vectors that went to find-or-put)
-        if ((b & a.region_mask()) != a.region_bits()) {
-          hv[j] = false;
-        } else if (cache.base || a.gcache()) {
-          // A vector this warp has already sent to find-or-put needs no second lookup,
-          // nor does one that any warp found or inserted moments ago.  One lane of the
-          // group reads (and writes) the caches and the group takes its answer: other
-          // warps write the GPU-wide cache at any moment, and lanes of a group are not
-          // guaranteed to read it in one instruction, so their own reads could disagree
-          // and split the group before find-or-put's group-wide votes.
-          int known = 0;
-          if (g.glane == 0)
-            known = (cache.base && cache.template seen<W>(hh, x[j])) ||
-                    (a.gcache() && gcache_hit<W>(a.gcache(), a.gcache_mask(), hh, x[j], a.gkey()));
-          if (g.template bcast<int>(known, g.base)) hv[j] = false;
-        }
-        if (hv[j]) {
-          load_words<LW>(a.table() + b * (uint64_t)B + (uint64_t)g.glane * LW, pre[j]);
-          probes += g.glane == 0;
-        }
+// Successor generation by a warp whose lanes hold one state each (lanes without
+// one hold no successors).  The warp walks the sources of successors -- the
+// processes, then the rules -- together: open() finds, per lane, how many
+// successors the current source gives its state, and emit() appends one per
+// lane that has any left to a queue in shared memory.  Every table address but
+// the per-lane edge offsets is uniform, and a state's successors are counted on
+// the way, without a pass of their own.
+template <int W>
+struct WarpGen {
+  uint32_t src;       // next source: process src, then rule src - n_procs (uniform)
+  uint32_t e, e_end;  // this lane's successors left of the current source: edges, or combinations of the rule
+  uint32_t word;      // word index of the current process (uniform); W: a rule
+  uint32_t cur;       // that word of this lane's state; a rule: its index (uniform)
+
+  template <class Desc>
+  __device__ __forceinline__ void open(const uint32_t* t, const NetBlobLayout& L, Desc& desc, bool valid,
+                                       const uint32_t (&v)[W]) {
+    if (src < L.n_procs) {
+      const uint4 d = desc(src);
+      word = d.x;
+      cur = word_at<W>(v, d.x);
+      const uint32_t* o = t + d.w + ((cur >> d.y) & d.z);
+      e = valid ? o[0] : 0u;
+      e_end = valid ? o[1] : 0u;
+    } else {
+      const uint32_t r = src - L.n_procs;
+      uint32_t prod = valid ? 1u : 0u;
+      const uint32_t j1 = t[L.rule_off + r + 1];
+      for (uint32_t j = t[L.rule_off + r]; j < j1; ++j) {
+        const uint32_t c = t[L.rule_cls + j];
+        const uint4 d = desc(t[L.cls_proc + c]);
+        const uint32_t* o = t + L.coff + t[L.cls_base + c] + ((word_at<W>(v, d.x) >> d.y) & d.z);
+        prod *= o[1] - o[0];
+        if (!__any_sync(FULLMASK, prod != 0)) break;
       }
+      word = W;
+      cur = r;
+      e = 0;
+      e_end = prod;
     }
+    ++src;
+  }
+
+  // One successor into the W words at q (a lane with e < e_end).
+  template <class Desc>
+  __device__ __forceinline__ void emit(const uint32_t* t, const NetBlobLayout& L, Desc& desc,
+                                       const uint32_t (&v)[W], uint32_t* q) {
+    if (word < (uint32_t)W) {
+      store_vec<W>(q, v);
+      q[word] = cur ^ t[L.cdelta + e];
+    } else {
+      uint32_t out[W];
 #pragma unroll
-    for (int j = 0; j < CH; ++j) {
-      if (!hv[j]) continue;
-      const int i = c + j;
-      const int r = find_or_put_from<W, B, G, true>(a.table(), a.log2nb(), a.rounds(), muls, x[j], g, probes,
-                                                    pre[j]);
-      if (r == FOP_FULL) err |= gx::ERR_TABLE_FULL;
-      else if (a.gcache() && g.glane == 0)
-        gcache_put<W>(a.gcache(), a.gcache_mask(), vec_hash<W>(x[j]), x[j], a.gkey());
-      if (g.glane == i / K && r == FOP_INSERTED) inserted[i % K] = true;
+      for (int w = 0; w < W; ++w) out[w] = v[w];
+      uint32_t x = e;
+      const uint32_t j1 = t[L.rule_off + cur + 1];
+      for (uint32_t j = t[L.rule_off + cur]; j < j1; ++j) {
+        const uint32_t c = t[L.rule_cls + j];
+        const uint4 d = desc(t[L.cls_proc + c]);
+        const uint32_t* o = t + L.coff + t[L.cls_base + c] + ((word_at<W>(v, d.x) >> d.y) & d.z);
+        const uint32_t cnt = o[1] - o[0];
+        uint32_t i = 0;
+        if (cnt > 1) {  // one matching edge is the common case: no division
+          i = x % cnt;
+          x /= cnt;
+        }
+        xor_at<W>(out, d.x, t[L.cdelta + o[0] + i]);
+      }
+      store_vec<W>(q, out);
     }
+    ++e;
   }
-#pragma unroll
-  for (int k = 0; k < K; ++k) st.push<W>(a, inserted[k], s[k], err);
-}
-
-// One lane per bucket (G = 1): find-or-put of the vector x of every lane with
-// has set (the filters of insert_lanes already passed), its new vectors staged
-// for the next level.  All 32 lanes call it together.
-template <int W, int B, class T>
-__device__ __forceinline__ void resolve_lanes(const T& a, const uint64_t* muls, bool has, const uint32_t (&x)[W],
-                                              const uint64_t hh, uint32_t& probes, uint32_t& err, WarpStage& st) {
-  constexpr int LW = (B / W) * W;
-  const Group<1> g;
-  bool inserted = false;
-  uint32_t pre[LW];
-  if (has) {
-    const uint64_t b = bucket_of(hh, muls[0], a.log2nb());
-    load_words<LW>(a.table() + b * (uint64_t)B, pre);
-    ++probes;
-    const int r = find_or_put_hashed<W, B, 1, true>(a.table(), a.log2nb(), a.rounds(), muls, x, hh, g, probes, pre);
-    if (r == FOP_FULL) err |= gx::ERR_TABLE_FULL;
-    else if (a.gcache()) gcache_put<W>(a.gcache(), a.gcache_mask(), hh, x, a.gkey());
-    inserted = r == FOP_INSERTED;
-  }
-  st.push<W>(a, inserted, x, err);
-}
-
-// Per-warp queue of successors waiting for their find-or-put (G = 1).  The lanes
-// of a warp expand different states, whose successor counts differ: one
-// successor per lane and round leaves the lanes of the states with fewer
-// successors idle in the rounds that follow.  So each round only generates one
-// successor per lane and queues the ones the filters keep (region, per-warp
-// cache, GPU-wide cache); whenever 32 are queued, every lane resolves one, so
-// the bucket reads and compare-and-swaps run with all 32 lanes busy.
-constexpr int kQueue = 64;  // at most 31 left + 32 new
-
-template <int W>
-struct WarpQueue {
-  uint32_t* buf;             // kQueue * W words of this warp
-  unsigned long long* hash;  // kQueue hashes (vec_hash) of the queued vectors
-  int n;                     // queued vectors (uniform in the warp)
 };
 
-// Resident CTAs per SM the level kernel is compiled for (register budget).
-// A lane holds min(G, 4) first buckets in flight of B / G words each; up to
-// 8 such words fit 48 registers (5 CTAs), up to 16 fit 64 (4 CTAs), more get
-// 85 (3 CTAs); 4-word slots with 4 or more lanes per bucket also get 3.
-// (Checked with -Xptxas -v: at most a few bytes spill; the queued kernel for
-// 4-word slots in 8-word buckets spills 48 bytes and is still the fastest
-// there: 3.50 s on the memory-scaled network against 3.76 s at 4 CTAs and 64
-// registers.  4-word slots in 16-word buckets spill 48 bytes at 48 registers
-// and ran slower.)  The level kernel is latency-bound, so the extra CTA pays: 4-word
-// slots in 8-word buckets explore the memory-scaled network in 4.49 s at 5
-// CTAs, 4.94 s at 4 (plain kernel).
+// The two queues a warp keeps in shared memory, used as stacks (the last
+// entries are taken, so nothing is ever moved):
+//   raw   successors as generated.  A source gives the 32 states of a warp
+//         different numbers of successors, so generation runs with part of the
+//         lanes; hashing and the filters (region, caches) then run on a batch of
+//         32 or 64 successors, so that a lane's cache lookups are in flight
+//         together.
+//   kept  successors that passed the filters, with their hashes and the
+//         hash-constant set to try.  32 of them at a time read one bucket each;
+//         those that met a full one go back with the next set, so a lane in a
+//         crowded part of the table holds up no other.
+// Successors filtered at a time.  4-word vectors: one per lane, because shared
+// memory beyond 196 KB an SM leaves so little L1 that it limits the loads in
+// flight (irregular 1.08e8-state network: 42.1 ms with batches of 32, 68.0 ms
+// with 64, the same instructions otherwise).
+template <int W>
+constexpr int kBatch = W == 4 ? 32 : 64;
+
+template <int W, int Batch = kBatch<W>>
+struct WarpQueues {
+  static constexpr int kSlots = Batch + 32;  // at most 31 left of a batch of 32, or Batch - 1, before the next come in
+  uint32_t raw[kSlots * W];
+  uint32_t kept[kSlots * W];
+  unsigned long long hash[kSlots];  // state_hash of the kept vectors | hash-constant set
+};
+
+// Resident CTAs per SM the level kernel is compiled for (register budget): a
+// lane holds a bucket of B words (one lane per bucket), or its share of the
+// buckets in flight (bucket_step_lanes).
 template <int W, int B, int G>
 struct ExpandOcc {
-  static constexpr int inflight = (G < 4 ? G : 4) * (B / G);
-  static constexpr int min_ctas =
-      (inflight <= 8 && (W <= 2 || G == 1)) ? 5 : ((inflight <= 16 && !(W == 4 && G >= 4)) ? 4 : 3);
+  static constexpr int words = G == 1 ? B : kLanesInFlight<W, B, G> * (B / G) + 8;
+  static constexpr int min_ctas = words <= 8 ? 5 : (words <= 16 ? 4 : 3);
 };
 
-// Q: the per-warp successor queue.  Generation rounds append the successors that
-// pass the filters (region, caches) to a queue in shared memory, and find-or-put
-// runs 32 queued successors at a time with every lane busy.  Built by default
-// for 1- and 2-word vectors with one lane per bucket; for 4-word vectors in 4-
-// and 8-word buckets it is a second kernel, chosen when region passes discard
-// most successors (memory-scaled network, 2 passes: 3.52 s queued against 4.48 s;
-// the 1.08e8-state irregular network in 4 GiB, 1 pass: 57.8 ms queued against
-// 49.4 ms).
-template <int W, int B, int G, bool Q = (G == 1 && W <= 2)>
+// The expansion of a warp's share of one level: generate successors of its
+// states until a batch is queued, filter it, and resolve what is kept 32 at a
+// time -- one loop with one copy of each step (a second copy of find-or-put
+// costs registers).
+//   next(pos, m)   the warp's next m <= 32 states, at absolute frontier
+//                  positions pos.. (m = 0: none are left)
+//   desc(p)        the process descriptors (proc_desc)
+//   seen(v)        a lane's state, once, when it is taken
+//   done(v, n)     a lane's state and the number of its successors
+//   keep(b, h, x)  the filters before the GPU-wide cache: first bucket, hash,
+//                  successor
+// All 32 lanes call it together; returns with the queues empty.
+template <int W, int B, int G, int Batch, class T, class Desc, class Next, class Seen, class Done, class Keep>
+__device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls, const uint32_t* t,
+                                              const NetBlobLayout& L, WarpQueues<W, Batch>& q, WarpStage& st,
+                                              uint32_t& probes, uint32_t& err, Desc desc, Next next, Seen seen,
+                                              Done done, Keep keep) {
+  const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1u;
+  const uint32_t n_src = L.n_procs + L.n_rules;
+  int n_raw = 0, n_kept = 0;  // queued (uniform in the warp)
+  uint32_t m = 0;             // states the warp holds (lanes 0..m-1)
+  uint32_t v[W];
+#pragma unroll
+  for (int w = 0; w < W; ++w) v[w] = 0;
+  uint32_t cnt = 0;  // successors of this lane's state
+  WarpGen<W> gen;
+  gen.src = n_src;
+  gen.e = gen.e_end = gen.cur = gen.word = 0;
+  bool more = true;  // states may be left for this warp
+  while (true) {
+    while (n_raw < Batch) {
+      const uint32_t act = __ballot_sync(FULLMASK, gen.e < gen.e_end);
+      if (act != 0) {
+        if ((act >> lane) & 1u) gen.emit(t, L, desc, v, q.raw + (n_raw + __popc(act & below)) * W);
+        n_raw += __popc(act);
+      } else if (gen.src < n_src) {
+        gen.open(t, L, desc, lane < m, v);
+        cnt += gen.e_end - gen.e;
+      } else {
+        if (!more) break;
+        if (lane < m) done(v, cnt);
+        uint64_t pos = 0;
+        next(pos, m);
+        more = m != 0;
+        if (!more) break;
+        if (lane < m) {
+          load_vec<W>(tg.frontier() + ((pos + lane) & tg.fmask()) * W, v);
+          seen(v);
+        }
+        cnt = 0;
+        gen.src = 0;
+      }
+    }
+    __syncwarp();
+    {
+      const int k = n_raw < Batch ? n_raw : Batch;
+      n_raw -= k;
+      constexpr int K = Batch / 32;
+      bool on[K];
+      uint32_t x[K][W];
+      uint64_t hh[K];
+#pragma unroll
+      for (int i = 0; i < K; ++i) {
+        const int at = (int)lane + 32 * i;
+        load_vec<W>(q.raw + (n_raw + at) * W, x[i]);  // (past the k-th entry: not used)
+        hh[i] = state_hash<W>(x[i]);
+        on[i] = at < k && keep(bucket_of(hh[i], muls[0], tg.log2nb()), hh[i], x[i]);
+      }
+      if (tg.gcache().base) {
+        SeenEntry e[K];
+        unsigned long long c[K];
+#pragma unroll
+        for (int i = 0; i < K; ++i) {
+          e[i] = seen_entry<W>(tg.gcache(), x[i]);
+          c[i] = on[i] ? seen_get(tg.gcache(), e[i].index) : 0ull;
+        }
+#pragma unroll
+        for (int i = 0; i < K; ++i) on[i] = on[i] && (c[i] != e[i].content || c[i] == 0);
+      }
+#pragma unroll
+      for (int i = 0; i < K; ++i) {
+        const uint32_t km = __ballot_sync(FULLMASK, on[i]);
+        if (on[i]) {
+          const int at = n_kept + __popc(km & below);
+          store_vec<W>(q.kept + at * W, x[i]);
+          q.hash[at] = hh[i];
+        }
+        n_kept += __popc(km);
+      }
+    }
+    const bool last = !more && n_raw == 0;
+    while (n_kept >= 32 || (last && n_kept > 0)) {
+      __syncwarp();
+      const int k = n_kept < 32 ? n_kept : 32;
+      n_kept -= k;
+      const bool has = (int)lane < k;
+      uint32_t x[W];
+      load_vec<W>(q.kept + (n_kept + lane) * W, x);  // (past the k-th entry: not used)
+      const uint64_t hn = q.hash[n_kept + lane];
+      const uint32_t n = (uint32_t)(hn & kSeqMask);
+      bool again = resolve_lanes<W, B, G>(tg, muls, has, x, hn & ~kSeqMask, n, probes, err, st) < 0 && has;
+      if (again && n + 1 == (uint32_t)tg.rounds()) {
+        err |= gx::ERR_TABLE_FULL;
+        again = false;
+      }
+      const uint32_t am = __ballot_sync(FULLMASK, again);
+      if (again) {  // (the warp has read its entries: resolve_lanes synchronises it)
+        const int at = n_kept + __popc(am & below);
+        store_vec<W>(q.kept + at * W, x);
+        q.hash[at] = hn + 1;
+      }
+      n_kept += __popc(am);
+    }
+    if (last) break;
+    __syncwarp();
+  }
+}
+
+template <int W, int B, int G>
 __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expand_kernel(const gx::ExpandArgs a) {
-  static_assert(!Q || G == 1, "the successor queue needs one lane per bucket");
+  constexpr uint32_t kWarps = gx::kBlock / 32;
   extern __shared__ __align__(16) uint32_t sm[];
   // the level being expanded: from the parameters, or (device-driven level
   // loop) from the control block the previous level's advance step wrote.
   // Kept in shared memory, not registers, for the inner loop's sake.
   __shared__ unsigned long long s_range[2];
-  if (a.dev_range) {
-    const uint64_t b0 = a.ctl->cur_begin, e0 = a.ctl->cur_end;
-    // a fixed full-size grid: CTAs beyond the level's first chunks leave at once
-    const uint64_t per_cta = 32ull * (gx::kBlock / 32);
-    if ((uint64_t)blockIdx.x * per_cta >= e0 - b0) return;
+  const uint32_t nwarps = gridDim.x * kWarps;
+  uint32_t unit;  // states a warp takes at a time
+  {
+    const uint64_t b0 = a.dev_range ? a.ctl->cur_begin : a.cur_begin;
+    const uint64_t e0 = a.dev_range ? a.ctl->cur_end : a.cur_end;
+    // a level of fewer states than lanes is spread over all warps: its time is
+    // the latency of one warp's share, not throughput
+    const uint64_t full = 32ull * nwarps;
+    unit = e0 - b0 >= full ? 32u : ((uint32_t)(e0 - b0) + nwarps - 1) / nwarps;
+    // a fixed full-size grid: CTAs beyond the level's states leave at once
+    if ((uint64_t)blockIdx.x * kWarps * unit >= e0 - b0) return;
     if (threadIdx.x == 0) {
       s_range[0] = b0;
       s_range[1] = e0;
     }
-  } else if (threadIdx.x == 0) {
-    s_range[0] = a.cur_begin;
-    s_range[1] = a.cur_end;
   }
   const uint64_t* muls;
   const uint32_t* t = stage_tables(sm, a.muls, a.rounds, a.blob, a.blob_words, a.stage, muls);
+  __shared__ uint4 descs[kMaxProcs];
   __syncthreads();
   const NetBlobLayout& L = a.lay;
-  const int lane = threadIdx.x & 31;
-  const Group<G> g;
+  for (uint32_t p = threadIdx.x; p < L.n_procs; p += blockDim.x) descs[p] = proc_desc(t, L, p);
+  __syncthreads();
+  const uint32_t lane = threadIdx.x & 31;
   uint32_t trans = 0;  // per thread and launch: far below 2^32
   uint32_t probes = 0, err = 0;
-  __shared__ uint32_t stage_mem[gx::kBlock / 32][kStage * W];
+  __shared__ __align__(16) uint32_t stage_mem[kWarps][kStage * W];
+  __shared__ __align__(16) WarpQueues<W> queue_mem[kWarps];
   WarpStage st{stage_mem[threadIdx.x >> 5], 0};
-  constexpr bool kQueued = Q;
-  __shared__ uint32_t queue_mem[kQueued ? gx::kBlock / 32 : 1][kQueued ? kQueue * W : 1];
-  __shared__ unsigned long long queue_hash[kQueued ? gx::kBlock / 32 : 1][kQueued ? kQueue : 1];
-  WarpQueue<W> wq{queue_mem[kQueued ? threadIdx.x >> 5 : 0], queue_hash[kQueued ? threadIdx.x >> 5 : 0], 0};
   const ParamTarget tg{a, s_range};
   WarpCache cache{nullptr, 0};
   if (a.cache_log2 > 0) {
@@ -612,106 +702,53 @@ __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expa
     for (uint32_t i = lane; i < per_warp; i += 32) cache.base[i] = 0u;  // 0 is never a stored vector
     __syncwarp();
   }
-
-  while (true) {
-    unsigned long long chunk = 0;
-    if (lane == 0) chunk = atomicAdd(&a.ctl->claim, 32ull);
-    chunk = __shfl_sync(FULLMASK, chunk, 0);
-    const uint64_t start = s_range[0] + chunk;
-    if (start >= s_range[1]) break;
-    const uint64_t idx = start + lane;
-    const bool valid = idx < s_range[1];
-    uint32_t v[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) v[w] = 0;
-    if (valid) load_vec<W>(a.frontier + (idx & a.fmask) * W, v);
-    uint32_t remaining = valid ? count_succ<W>(t, L, v) : 0u;
-    // with region passes, the level's states are accounted for in the first pass only
-    const bool acct = valid && a.count_states;
-    if (acct) trans += remaining;
-    if (acct && remaining == 0) {
-      const uint64_t h = state_digest<W>(t, L, v);
-      const unsigned long long di = atomicAdd(&a.ctl->dl_count, 1ull);
-      atomicAdd(&a.ctl->dl_sum, (unsigned long long)h);
-      atomicXor(&a.ctl->dl_xor, (unsigned long long)h);
-      if (di < a.dl_cap) store_vec<W>(a.dl_buf + di * W, v);
-    }
-    if (a.watch && acct) check_watch<W>(a, t, L, v);
-    SuccIter it;
-    it.init();
-    if constexpr (kQueued) {
-      while (__any_sync(FULLMASK, remaining != 0)) {
-        uint32_t x[W];
-        uint64_t hh = 0;
-        bool keep = remaining != 0;
-        if (keep) {
-          next_succ<W>(it, t, L, v, x);
-          --remaining;
-          hh = vec_hash<W>(x);
-          const uint64_t b = bucket_of(hh, muls[0], a.log2nb);
-          // the filters of insert_lanes: region, per-warp cache, GPU-wide cache
-          if ((b & a.region_mask) != a.region_bits) keep = false;
-          else if (cache.base && cache.template seen<W>(hh, x)) keep = false;
-          else if (a.gcache && gcache_hit<W>(a.gcache, a.gcache_mask, hh, x, tg.gkey())) keep = false;
+  bool first = true;
+  expand_states<W, B, G, kBatch<W>>(
+      tg, muls, t, L, queue_mem[threadIdx.x >> 5], st, probes, err, [&](uint32_t p) { return descs[p]; },
+      [&](uint64_t& pos, uint32_t& m) {
+        // the first states of every warp are fixed by its index, a large level's
+        // further ones are claimed
+        m = 0;
+        if (first) {
+          pos = s_range[0] + (uint64_t)(blockIdx.x * kWarps + (threadIdx.x >> 5)) * unit;
+          first = false;
+        } else {
+          if (unit < 32) return;
+          unsigned long long c = 0;
+          if (lane == 0) c = atomicAdd(&a.ctl->claim, 32ull);
+          pos = s_range[0] + 32ull * nwarps + __shfl_sync(FULLMASK, c, 0);
         }
-        const uint32_t km = __ballot_sync(FULLMASK, keep);
-        if (keep) {
-          const int at = wq.n + __popc(km & ((1u << lane) - 1u));
-#pragma unroll
-          for (int w = 0; w < W; ++w) wq.buf[at * W + w] = x[w];
-          wq.hash[at] = hh;
+        if (pos < s_range[1]) m = s_range[1] - pos < unit ? (uint32_t)(s_range[1] - pos) : unit;
+      },
+      [&](const uint32_t(&v)[W]) {
+        if (a.watch && a.count_states) check_watch<W>(a, t, L, v);
+      },
+      [&](const uint32_t(&v)[W], uint32_t n) {
+        // with region passes, the level's states are accounted for in the first pass only
+        if (!a.count_states) return;
+        trans += n;
+        if (n == 0) {
+          const uint64_t h = state_digest<W>(t, L, v);
+          const unsigned long long di = atomicAdd(&a.ctl->dl_count, 1ull);
+          atomicAdd(&a.ctl->dl_sum, (unsigned long long)h);
+          atomicXor(&a.ctl->dl_xor, (unsigned long long)h);
+          if (di < a.dl_cap) store_vec<W>(a.dl_buf + di * W, v);
         }
-        wq.n += __popc(km);
-        if (wq.n >= 32) {
-          __syncwarp();
-          uint32_t y[W];
-#pragma unroll
-          for (int w = 0; w < W; ++w) y[w] = wq.buf[lane * W + w];
-          resolve_lanes<W, B>(tg, muls, true, y, wq.hash[lane], probes, err, st);
-          __syncwarp();
-          if (lane < wq.n - 32) {
-#pragma unroll
-            for (int w = 0; w < W; ++w) wq.buf[lane * W + w] = wq.buf[(32 + lane) * W + w];
-            wq.hash[lane] = wq.hash[32 + lane];
-          }
-          wq.n -= 32;
-          __syncwarp();
-        }
-      }
-    } else {
-      constexpr int K = PerLane<G>::K;
-      while (__any_sync(FULLMASK, remaining != 0)) {
-        uint32_t s[K][W];
-        bool has[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-          has[k] = remaining != 0;
-          if (has[k]) {
-            next_succ<W>(it, t, L, v, s[k]);
-            --remaining;
-          } else {
-#pragma unroll
-            for (int w = 0; w < W; ++w) s[k][w] = 0;
-          }
-        }
-        insert_lanes<W, B, G, K>(tg, muls, g, has, s, probes, err, st, cache);
-      }
-    }
-  }
-  if constexpr (kQueued) {  // what is left in the queue
-    __syncwarp();
-    const bool has = lane < wq.n;
-    uint32_t y[W];
-#pragma unroll
-    for (int w = 0; w < W; ++w) y[w] = has ? wq.buf[lane * W + w] : 0u;
-    resolve_lanes<W, B>(tg, muls, has, y, has ? wq.hash[lane] : 0ull, probes, err, st);
-    wq.n = 0;
-  }
+      },
+      [&](uint64_t b, uint64_t hh, const uint32_t(&x)[W]) {
+        // region passes: a vector whose first bucket lies outside this pass's region is
+        // left to the pass of that region (tested before the caches, which may only hold
+        // vectors that went to find-or-put).  A vector this warp has already sent to
+        // find-or-put needs no second lookup, nor does one that any warp found or
+        // inserted moments ago.
+        if ((b & a.region_mask) != a.region_bits) return false;
+        return !(cache.base && cache.template seen<W>(hh, x));
+      });
   st.flush<W>(tg, err);
   // the CTA's totals, one atomic per counter: at the end of a level every warp
   // finishes at once, and per-warp atomics would queue on two addresses
-  __shared__ unsigned long long s_tot[2][gx::kBlock / 32];
-  __shared__ uint32_t s_err[gx::kBlock / 32];
+  __shared__ unsigned long long s_tot[2][kWarps];
+  __shared__ uint32_t s_err[kWarps];
   const unsigned long long trans_w = warp_sum((unsigned long long)trans);
   const unsigned long long pr = warp_sum((unsigned long long)probes);
   err = __reduce_or_sync(FULLMASK, err);
@@ -724,12 +761,12 @@ __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expa
   if (threadIdx.x < 3) {
     unsigned long long x = 0;
     if (threadIdx.x < 2)
-      for (int w = 0; w < gx::kBlock / 32; ++w) x += s_tot[threadIdx.x][w];
+      for (uint32_t w = 0; w < kWarps; ++w) x += s_tot[threadIdx.x][w];
     if (threadIdx.x == 0 && x) atomicAdd(&a.ctl->transitions, x);
     if (threadIdx.x == 1 && x) atomicAdd(&a.ctl->probes, x);
     if (threadIdx.x == 2) {
       uint32_t e = 0;
-      for (int w = 0; w < gx::kBlock / 32; ++w) e |= s_err[w];
+      for (uint32_t w = 0; w < kWarps; ++w) e |= s_err[w];
       if (e) atomicOr(&a.ctl->error, e);
     }
   }
@@ -801,7 +838,7 @@ __global__ void __launch_bounds__(gx::kBlock) part_count_kernel(const gx::Expand
     for (uint32_t k = 0; k < cnt; ++k) {
       uint32_t s[W];
       next_succ<W>(it, t, L, v, s);
-      atomicAdd(&hist[(uint32_t)((vec_hash<W>(s) * mul0) >> shift)], 1u);
+      atomicAdd(&hist[(uint32_t)((state_hash<W>(s) * mul0) >> shift)], 1u);
     }
   }
   __syncthreads();
@@ -881,7 +918,7 @@ __global__ void __launch_bounds__(gx::kBlock) part_scatter_kernel(const gx::Expa
     for (uint32_t k = 0; k < cnt; ++k) {
       uint32_t s[W];
       next_succ<W>(it, t, L, v, s);
-      const uint32_t q = (uint32_t)((vec_hash<W>(s) * mul0) >> shift);
+      const uint32_t q = (uint32_t)((state_hash<W>(s) * mul0) >> shift);
       const uint32_t pos = atomicAdd(&cur[q], 1u);
       store_vec<W>(pa.succ + (uint64_t)pos * W, s);
     }
@@ -898,9 +935,8 @@ __global__ void __launch_bounds__(gx::kBlock) part_probe_kernel(const gx::Expand
   for (int i = threadIdx.x; i < a.rounds; i += blockDim.x) muls[i] = a.muls.m[i];
   __syncthreads();
   const int lane = threadIdx.x & 31;
-  const Group<G> g;
   uint32_t probes = 0, err = 0;
-  __shared__ uint32_t stage_mem[gx::kBlock / 32][kStage * W];
+  __shared__ __align__(16) uint32_t stage_mem[gx::kBlock / 32][kStage * W];
   WarpStage st{stage_mem[threadIdx.x >> 5], 0};
   __shared__ unsigned long long s_range[2];
   if (threadIdx.x == 0) {
@@ -915,12 +951,19 @@ __global__ void __launch_bounds__(gx::kBlock) part_probe_kernel(const gx::Expand
     chunk = __shfl_sync(FULLMASK, chunk, 0);
     if (chunk >= n) break;
     const uint64_t idx = chunk + lane;
-    bool has[1] = {idx < n};
-    uint32_t s[1][W];
+    bool on = idx < n;
+    uint32_t x[W];
 #pragma unroll
-    for (int w = 0; w < W; ++w) s[0][w] = 0;
-    if (has[0]) load_vec<W>(succ + idx * W, s[0]);
-    insert_lanes<W, B, G, 1>(tg, muls, g, has, s, probes, err, st);
+    for (int w = 0; w < W; ++w) x[w] = 0;
+    if (on) load_vec<W>(succ + idx * W, x);
+    const uint64_t h = state_hash<W>(x);
+    for (uint32_t k = 0; __any_sync(FULLMASK, on); ++k) {
+      if (k == (uint32_t)a.rounds) {
+        if (on) err |= gx::ERR_TABLE_FULL;
+        break;
+      }
+      on = resolve_lanes<W, B, G>(tg, muls, on, x, h, k, probes, err, st) < 0 && on;
+    }
   }
   st.flush<W>(tg, err);
   const unsigned long long pr = warp_sum((unsigned long long)probes);
@@ -936,20 +979,16 @@ __global__ void init_kernel(const gx::InitArgs a) {
   __shared__ uint64_t muls[kMaxRounds];
   for (int i = threadIdx.x; i < a.rounds; i += blockDim.x) muls[i] = a.muls.m[i];
   __syncthreads();
-  if ((int)threadIdx.x >= G) return;
-  const Group<G> g;
+  if (threadIdx.x != 0) return;
   uint32_t v[W];
 #pragma unroll
   for (int w = 0; w < W; ++w) v[w] = a.vec[w];
   uint32_t probes = 0;
-  const int r = find_or_put<W, B, G>(a.table, a.log2nb, a.rounds, muls, v, g, probes);
-  if (g.glane == 0) {
-    if (r == FOP_INSERTED) {
-      store_vec<W>(a.frontier, v);
-      a.ctl->next_end = 1ull;
-    } else {
-      a.ctl->error |= gx::ERR_TABLE_FULL;
-    }
+  if (find_or_put_state<W, B>(a.table, a.log2nb, a.rounds, muls, v, probes) == FOP_INSERTED) {
+    store_vec<W>(a.frontier, v);
+    a.ctl->next_end = 1ull;
+  } else {
+    a.ctl->error |= gx::ERR_TABLE_FULL;
   }
 }
 
@@ -995,9 +1034,9 @@ __global__ void __launch_bounds__(gx::kBlock) fop_kernel(const gx::FopArgs a) {
 
 namespace gx {
 
-template <int W, int B, int G, bool Q = (G == 1 && W <= 2)>
+template <int W, int B, int G>
 cudaError_t launch_expand(const ExpandArgs& a, int grid, size_t smem, cudaStream_t st) {
-  gxd::expand_kernel<W, B, G, Q><<<grid, kBlock, smem, st>>>(a);
+  gxd::expand_kernel<W, B, G><<<grid, kBlock, smem, st>>>(a);
   return cudaGetLastError();
 }
 template <int W, int B, int G>
@@ -1031,23 +1070,6 @@ cudaError_t launch_part_probe(const ExpandArgs& a, const uint32_t* succ, uint64_
   return cudaGetLastError();
 }
 
-// The queued level kernel as a second choice: 4-word vectors, one lane per bucket
-// of at most 8 words (with larger buckets it measured slower than the plain one).
-template <int W, int B, int G>
-constexpr bool kSecondQueued = W == 4 && G == 1 && B <= 8;
-
-using ExpandLauncher = cudaError_t (*)(const ExpandArgs&, int, size_t, cudaStream_t);
-template <int W, int B, int G>
-ExpandLauncher queued_launcher() {
-  if constexpr (kSecondQueued<W, B, G>) return &launch_expand<W, B, G, true>;
-  else return nullptr;
-}
-template <int W, int B, int G>
-const void* queued_fn() {
-  if constexpr (kSecondQueued<W, B, G>) return reinterpret_cast<const void*>(&gxd::expand_kernel<W, B, G, true>);
-  else return nullptr;
-}
-
 template <int W, int B, int G>
 const KernelSet* kernel_set() {
   static const KernelSet ks{&launch_expand<W, B, G>,
@@ -1062,9 +1084,7 @@ const KernelSet* kernel_set() {
                             reinterpret_cast<const void*>(&gxd::part_count_kernel<W>),
                             reinterpret_cast<const void*>(&gxd::part_scatter_kernel<W>),
                             reinterpret_cast<const void*>(&gxd::part_probe_kernel<W, B, G>),
-                            reinterpret_cast<const void*>(&gxd::init_kernel<W, B, G>),
-                            queued_launcher<W, B, G>(),
-                            queued_fn<W, B, G>()};
+                            reinterpret_cast<const void*>(&gxd::init_kernel<W, B, G>)};
   return &ks;
 }
 

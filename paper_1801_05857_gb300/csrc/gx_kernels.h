@@ -41,6 +41,22 @@ struct Muls {
   uint64_t m[kMaxRounds];
 };
 
+// GPU-wide cache of recently seen vectors: 2^n direct-mapped entries in global
+// memory, cleared at the start of a search (nullptr = off).  A vector's fields
+// packed side by side are a number of `bits` <= 64 bits; a bijection mixes it,
+// its top n bits are the entry's index and the others, plus one, its content
+// (0 = empty), so an entry holds a vector exactly in 16 or 32 bits where
+// that is enough.  (cache_layout in gx_internal.h fills it in.)
+struct SeenCache {
+  void* base;
+  uint64_t mask;      // 2^bits - 1
+  uint64_t tag_mask;  // 2^shift - 1
+  uint32_t shift;     // bits - n (0 when bits <= n)
+  uint32_t half;      // (bits + 1) / 2
+  uint32_t log2_bytes;  // of an entry: 1, 2 or 3
+  uint32_t word_at[3];  // bit offset in the key of the payload of words 1, 2, 3 (64: no fields)
+};
+
 struct ExpandArgs {
   const uint32_t* blob;      // encoded network (global memory)
   uint32_t blob_words;
@@ -69,15 +85,7 @@ struct ExpandArgs {
   // gx_explore_opts.region_passes).  region_mask = 0: one pass, no filter.
   uint64_t region_mask, region_bits;
   int count_states;          // 1: this pass counts transitions, deadlocks and violations
-  // GPU-wide cache of recently seen vectors: 2^k entries of 64 bits in global
-  // memory, small enough to stay in L2; nullptr = off.  An entry holds a vector's
-  // 64-bit key: the vector itself for 1- and 2-word vectors, its payload bits
-  // packed for 4-word vectors whose fields take at most 64 bits (gkey_shift).
-  unsigned long long* gcache;
-  uint64_t gcache_mask;
-  // 4-word vectors: bit offset in the key of the payload of words 1, 2, 3
-  // (word 0 at offset 0; 64 = the word carries no field)
-  uint32_t gkey_shift[3];
+  SeenCache gcache;
 };
 
 // Partitioned expansion of one level (or one batch of it): successors are
@@ -136,10 +144,6 @@ struct KernelSet {
   const void* part_scatter_fn;
   const void* part_probe_fn;
   const void* init_fn;    // for graph kernel nodes
-  // the level kernel with the per-warp successor queue, where it is a second
-  // kernel (4-word vectors, one lane per bucket of at most 8 words); else nullptr
-  cudaError_t (*expand_queued)(const ExpandArgs&, int grid, size_t smem, cudaStream_t);
-  const void* expand_queued_fn;
 };
 
 // Kernels for slot width W, bucket words B and group lanes G; nullptr if the
@@ -158,6 +162,12 @@ cudaError_t launch_digest(int W, const DigestArgs& a, int grid, cudaStream_t st)
 
 // Hash-constant multipliers: odd 64-bit values drawn from splitmix64.
 void hash_multipliers(uint64_t* out, int n);
+
+// Layout of a GPU-wide cache of 2^log2_entries entries for a network's vectors;
+// false when they have no 64-bit key.  And the entries of the automatic one (0:
+// none).
+bool cache_layout(const Net& net, uint32_t log2_entries, SeenCache& c);
+uint32_t auto_cache_log2(const Net& net);
 
 // GX_DL_GUIDED search (gx_guided.cu).
 gx_status run_guided(gx_net* h, const gx_explore_opts* opts, void* ws, uint64_t ws_bytes, cudaStream_t st);

@@ -106,28 +106,23 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
   uint64_t fcap = 1;
   while (fcap < fwant) fcap *= 2;
   // caches of seen vectors, as gx_explore chooses them (gx_explore_opts)
+  uint32_t glog = o->global_cache_log2;
+  if (glog == 0xFFFFFFFFu)
+    glog = G == 1 && slots >= (1ull << 26) && (W <= 2 || regions == 1) ? gx::auto_cache_log2(net) : 0;
+  else if (glog > 26) return gx::fail(GX_ERR_INVALID, "global_cache_log2 must be at most 26");
+  gx::SeenCache gcache{};
   uint64_t gentries = 0;
-  uint32_t gkey[3] = {64, 64, 64};
-  const bool key_fits = W <= 2 || gx::cache_key_shifts(net, gkey);
-  if (o->global_cache_log2 == 0xFFFFFFFFu) {
-    if (W <= 2 && G == 1 && (table_bytes / (4ull * W)) >= (1ull << 26)) gentries = 1ull << 23;
-  } else if (o->global_cache_log2) {
-    if (o->global_cache_log2 > 26) return gx::fail(GX_ERR_INVALID, "global_cache_log2 must be at most 26");
-    if (key_fits) gentries = 1ull << o->global_cache_log2;
-  }
+  if (glog && gx::cache_layout(net, glog, gcache)) gentries = 1ull << glog;
+  const uint64_t gcache_bytes = gentries << gcache.log2_bytes;
   if (regions > nb) regions = (uint32_t)nb;
-  // the level kernel, as gx_explore chooses it: the queued second kernel with region passes
-  const bool queued = regions > 1 && ks->expand_queued;
-  const auto expand = queued ? ks->expand_queued : ks->expand;
-  const void* expand_fn = queued ? ks->expand_queued_fn : ks->expand_fn;
   const uint32_t warp_log2 =
-      o->warp_cache_log2 == 0xFFFFFFFFu ? (gentries ? 0u : queued ? 6u : 9u) : o->warp_cache_log2;
+      o->warp_cache_log2 == 0xFFFFFFFFu ? (gentries ? 0u : W == 4 ? 6u : 9u) : o->warp_cache_log2;
   const uint64_t off_ctl = 0;
   const uint64_t off_blob = align256(sizeof(gx::Ctl));
   const uint64_t off_front = align256(off_blob + 4ull * net.blob.size());
   const uint64_t off_table = align256(off_front + 4ull * W * fcap);
   const uint64_t off_gcache = align256(off_table + 4ull * B * nb);
-  const uint64_t total = align256(off_gcache + 8ull * gentries);
+  const uint64_t total = align256(off_gcache + gcache_bytes);
   if (total > kScratchBytes)
     return gx::fail(GX_ERR_INVALID, "gx_explore_noalloc needs " + std::to_string(total) +
                                         " bytes of scratch but its static array holds " +
@@ -152,8 +147,10 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
   NA_CUDA(cudaMemcpyAsync(blob, net.blob.data(), 4 * net.blob.size(), cudaMemcpyHostToDevice, st));
   NA_CUDA(cudaMemsetAsync(ctl, 0, sizeof(gx::Ctl), st));
   NA_CUDA(cudaMemsetAsync(table, 0, 4ull * B * nb, st));
-  unsigned long long* gcache = gentries ? reinterpret_cast<unsigned long long*>(base + off_gcache) : nullptr;
-  if (gcache) NA_CUDA(cudaMemsetAsync(gcache, 0, 8ull * gentries, st));
+  if (gentries) {
+    gcache.base = base + off_gcache;
+    NA_CUDA(cudaMemsetAsync(gcache.base, 0, gcache_bytes, st));
+  }
 
   int log2nb = 0;
   while ((1ull << log2nb) < nb) ++log2nb;
@@ -184,8 +181,6 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
   ea.dl_cap = 0;  // deadlocks are counted and digested, not stored
   ea.count_states = 1;
   ea.gcache = gcache;
-  ea.gcache_mask = gentries ? gentries - 1 : 0;
-  for (int w = 0; w < 3; ++w) ea.gkey_shift[w] = gkey[w];
   if (o->watch) {  // the safety check: violations counted and digested, not stored
     const uint32_t wp = o->watch_proc;
     ea.watch = 1;
@@ -196,26 +191,30 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
     ea.viol_buf = nullptr;
     ea.viol_cap = 0;
   }
-  size_t smem = 8ull * gx::kMaxRounds;
+  // shared memory: the same rules as gx_explore
+  cudaFuncAttributes fa{};
+  NA_CUDA(cudaFuncGetAttributes(&fa, ks->expand_fn));
   const size_t blob_bytes = 4ull * net.blob.size();
-  ea.stage = (smem + blob_bytes <= std::min<size_t>((size_t)smem_optin, 96 * 1024)) ? 1 : 0;
-  if (ea.stage) smem += blob_bytes;
-  // the per-warp cache of seen vectors lives in shared memory: same rule as gx_explore
+  size_t cache_bytes = 0;
   ea.cache_log2 = 0;
   if (warp_log2) {
     ea.cache_log2 = (int)warp_log2;
     if (ea.cache_log2 > 12) return gx::fail(GX_ERR_INVALID, "warp_cache_log2 must be at most 12");
     if (W == 4) ea.cache_log2 -= 1;  // 16-byte entries: the same bytes as 2^n 2-word ones
-    smem += 4ull * W * (gx::kBlock / 32) * (1ull << ea.cache_log2);
-    if (smem > (size_t)smem_optin)
-      return gx::fail(GX_ERR_INVALID, "warp cache of 2^" + std::to_string(ea.cache_log2) +
-                                          " entries per warp needs " + std::to_string(smem) +
-                                          " bytes of shared memory per CTA, more than " +
-                                          std::to_string(smem_optin));
+    cache_bytes = 4ull * W * (gx::kBlock / 32) * (1ull << ea.cache_log2);
   }
-  NA_CUDA(cudaFuncSetAttribute(expand_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  size_t smem = 8ull * gx::kMaxRounds + cache_bytes;
+  if (fa.sharedSizeBytes + smem > (size_t)smem_optin)
+    return gx::fail(GX_ERR_INVALID, "warp cache of 2^" + std::to_string(ea.cache_log2) +
+                                        " entries per warp needs " + std::to_string(fa.sharedSizeBytes + smem) +
+                                        " bytes of shared memory per CTA, more than " +
+                                        std::to_string(smem_optin));
+  ea.stage = blob_bytes + 8ull * gx::kMaxRounds <= 96 * 1024 &&
+                     fa.sharedSizeBytes + smem + blob_bytes <= (size_t)smem_optin ? 1 : 0;
+  if (ea.stage) smem += blob_bytes;
+  NA_CUDA(cudaFuncSetAttribute(ks->expand_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
-  NA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, expand_fn, gx::kBlock, smem));
+  NA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ks->expand_fn, gx::kBlock, smem));
   if (per_sm < 1) return gx::fail(GX_ERR_INVALID, "expansion kernel does not fit on an SM");
   if (o->ctas_per_sm) per_sm = std::min<int>(per_sm, (int)o->ctas_per_sm);
   const uint64_t max_grid = (uint64_t)sms * per_sm;
@@ -230,8 +229,7 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
   while (true) {
     ea.cur_begin = cur_begin;
     ea.cur_end = cur_end;
-    const uint64_t warps = (cur_end - cur_begin + 31) / 32;
-    const uint64_t want = (warps + gx::kBlock / 32 - 1) / (gx::kBlock / 32);
+    const uint64_t want = (cur_end - cur_begin + gx::kBlock / 32 - 1) / (gx::kBlock / 32);  // a warp per state
     const int grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(want, max_grid));
     // region passes (gx_explore_opts.region_passes): pass q probes region q of the table
     for (uint32_t q = 0; q < regions; ++q) {
@@ -240,7 +238,7 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
       eq.region_bits = (uint64_t)q << (log2nb - log2r);
       eq.count_states = q == 0 ? 1 : 0;
       NA_CUDA(cudaMemsetAsync(&ctl->claim, 0, sizeof(unsigned long long), st));
-      NA_CUDA(expand(eq, grid, smem, st));
+      NA_CUDA(ks->expand(eq, grid, smem, st));
     }
     NA_CUDA(cudaMemcpyAsync(&hc, ctl, sizeof(gx::Ctl), cudaMemcpyDeviceToHost, st));
     NA_CUDA(cudaStreamSynchronize(st));

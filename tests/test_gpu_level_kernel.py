@@ -1,0 +1,89 @@
+"""The level kernel's queues, rounds and caches at the sizes where they can go wrong,
+against the CPU oracle (bit-exact, including the digest of the visited set)."""
+import pytest
+
+import oracle
+from paper_1801_05857_gb300 import gx, inputs
+
+pytestmark = pytest.mark.gpu
+
+
+def _mostly_still(n_procs, moving, n_states=2):
+    """n_procs processes of which the first `moving` cycle through their states: n_states ** moving states."""
+    cycle = [(s, 0, (s + 1) % n_states) for s in range(n_states)]
+    return inputs.Network(1, [inputs.LTS(n_states, 0, cycle if p < moving else []) for p in range(n_procs)], [])
+
+
+NETS = {
+    1: inputs.random_network(7, 6, 8, 1, 3, 8, n_sync=2, parties=2),
+    2: inputs.random_network(1, 10, 16, 1, 3, 12, n_sync=4, parties=2, cluster=4),
+    4: inputs.random_network(1, 15, 16, 1, 3, 16, n_sync=8, parties=3, cluster=4),
+}
+_want = {}
+
+
+def _oracle(key, net):
+    if key not in _want:
+        _want[key] = oracle.explore(net)
+    return _want[key]
+
+
+def _check(key, net, **opts):
+    r = _oracle(key, net)
+    h = gx.load_network(net)
+    o = gx.default_opts(**opts)
+    ws = gx.alloc_workspace(h, o)
+    gx.explore(h, o, ws)
+    s = gx.stats(h)
+    assert (s["states"], s["transitions"], gx.levels(h)) == (r.states, r.transitions, r.levels)
+    assert (s["deadlock_count"], s["deadlock_sum"], s["deadlock_xor"]) == (r.deadlock_count, r.deadlock_sum,
+                                                                          r.deadlock_xor)
+    assert gx.set_digest(h, ws) == (r.states, r.set_sum, r.set_xor)
+    return s
+
+
+@pytest.mark.parametrize("bucket,group", [(4, 0), (8, 1), (8, 0), (16, 2), (32, 1), (32, 0)])
+@pytest.mark.parametrize("W", [1, 2, 4])
+def test_crowded_tables_take_further_hash_rounds(cuda, W, bucket, group):
+    """The smallest power-of-two table that holds the states at up to 90 % (here 62-84 %):
+    vectors that meet a full bucket go back to their warp's queue with the next
+    hash-constant set (buckets of up to four slots certainly overflow)."""
+    r = _oracle(W, NETS[W])
+    slots = 1
+    while slots < r.states / 0.9:
+        slots *= 2
+    s = _check(W, NETS[W], table_bytes=slots * 4 * W, frontier_states=slots, bucket_words=bucket,
+               group_lanes=min(group, bucket // W), hash_rounds=64, warp_cache_log2=0, global_cache_log2=0)
+    assert s["slot_words"] == W
+    assert s["probes"] > r.transitions if bucket // W <= 4 else s["probes"] >= r.transitions
+
+
+@pytest.mark.parametrize("log2", [1, 9, 16, 24, 25])
+@pytest.mark.parametrize("W", [1, 2, 4])
+def test_seen_cache_entries_of_every_width(cuda, W, log2):
+    """Keys of 18, 40 and 60 bits in caches of 2^1 to 2^25 entries: entries of 16, 32 and 64
+    bits, and indexes longer than the key."""
+    s = _check(W, NETS[W], table_bytes=1 << 25, frontier_states=1 << 21, bucket_words=8, group_lanes=1,
+               global_cache_log2=log2, warp_cache_log2=0)
+    assert s["global_cache_entries"] == 1 << log2 and s["slot_words"] == W
+
+
+@pytest.mark.parametrize("moving", [1, 2, 5, 13, 16])
+@pytest.mark.parametrize("ctas", [1, 0])
+def test_levels_below_at_and_above_one_state_per_warp(cuda, moving, ctas):
+    """Binomial level sizes from 1 to 12,870 states, on a full grid and on 1216 warps."""
+    s = _check(("still", moving), _mostly_still(20, moving), table_bytes=1 << 20, ctas_per_sm=ctas)
+    assert s["states"] == 2 ** moving
+
+
+@pytest.mark.parametrize("n_procs", [31, 32, 33, 62])
+def test_batched_networks_with_more_processes_than_lanes(cuda, n_procs):
+    nets = [_mostly_still(n_procs, 9), _mostly_still(12, 7), NETS[1]]
+    b = gx.batch_create(nets)
+    o = gx.batch_opts(table_slots=1 << 16, hash_rounds=32)
+    gx.batch_explore(b, o, gx.batch_alloc_workspace(b, o))
+    for i, net in enumerate(nets):
+        r = oracle.explore(net)
+        s = gx.batch_stats(b, i)
+        assert (s["states"], s["transitions"], gx.batch_levels(b, i)) == (r.states, r.transitions, r.levels)
+        assert (s["deadlock_count"], s["deadlock_sum"]) == (r.deadlock_count, r.deadlock_sum)
