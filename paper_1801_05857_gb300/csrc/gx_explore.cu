@@ -147,27 +147,80 @@ __global__ void level_advance_kernel(const gx::LoopArgs L) {
   cudaGraphSetConditional(L.cond, more ? 1u : 0u);
 }
 
+// Digest of the states in a table.  Bound by the table's bytes where it is nearly
+// empty and by the digest's arithmetic where it is full (about 26 instructions a
+// process and state).  A warp reads 1 KB of the table at a time, 32 bytes a lane,
+// collects the occupied slots and digests 64 at a time, two per lane (two
+// independent chains of mix64), with the process descriptors in shared memory.
+// Full table scans (before: a slot per lane, empty or not, three global table
+// reads a process): mid network, 1 GiB 46 % full 2.35 -> 0.92 ms; 4-word slots, 8 GiB
+// 62 % full 15.0 -> 7.05 ms.
 template <int W>
 __global__ void __launch_bounds__(gx::kBlock) digest_kernel(const gx::DigestArgs a) {
+  constexpr int kWarps = gx::kBlock / 32, kBatch = 64, S = 8 / W;
+  __shared__ uint4 descs[kMaxProcs];
+  __shared__ __align__(16) uint32_t queue_mem[kWarps][(kBatch + 32) * W];
+  for (uint32_t p = threadIdx.x; p < a.lay.n_procs; p += blockDim.x) descs[p] = proc_desc(a.blob, a.lay, p);
+  __syncthreads();
+  uint32_t* queue = queue_mem[threadIdx.x >> 5];
+  const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1u;
+  uint32_t n = 0;  // queued (uniform in the warp)
   unsigned long long cnt = 0, sum = 0, xr = 0;
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.slots; i += stride) {
-    uint32_t v[W];
-    load_vec<W>(a.table + i * W, v);
-    bool tagged = true;
+  auto digest = [&](uint32_t k) {  // the last k <= 64 queued
+    __syncwarp();
+    n -= k;
+    uint32_t v[2][W];
+    uint64_t h[2] = {0, 0};
 #pragma unroll
-    for (int w = 0; w < W; ++w) tagged &= (v[w] & kTag) != 0;
-    if (!tagged) continue;
-    const uint64_t h = state_digest<W>(a.blob, a.lay, v);
-    cnt += 1;
-    sum += h;
-    xr ^= h;
+    for (int i = 0; i < 2; ++i) load_vec<W>(queue + (n + lane + 32 * i) * W, v[i]);  // (past the k-th: not counted)
+    uint32_t word = 0, cur[2] = {v[0][0], v[1][0]};  // the word the current processes sit in
+    for (uint32_t p = 0; p < a.lay.n_procs; ++p) {
+      const uint4 d = descs[p];
+      if (W > 1 && d.x != word) {
+        word = d.x;
+#pragma unroll
+        for (int i = 0; i < 2; ++i) cur[i] = word_at<W>(v[i], word);
+      }
+#pragma unroll
+      for (int i = 0; i < 2; ++i) h[i] = mix64(h[i] ^ (((uint64_t)p << 32) | ((cur[i] >> d.y) & d.z)));
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      if (lane + 32 * i < k) {
+        cnt += 1;
+        sum += h[i];
+        xr ^= h[i];
+      }
+    __syncwarp();
+  };
+  // pieces of 8 words (a table has at least two buckets of four)
+  const uint64_t pieces = a.slots * W / 8, stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < pieces; i0 += stride) {
+    uint32_t s[8];
+#pragma unroll
+    for (int w = 0; w < 8; ++w) s[w] = 0;
+    if (i0 + lane < pieces) load_words<8>(a.table + (i0 + lane) * 8, s);
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+      uint32_t v[W];
+      bool tagged = true;
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        v[w] = s[i * W + w];
+        tagged &= (v[w] & kTag) != 0;
+      }
+      const uint32_t m = __ballot_sync(FULLMASK, tagged);
+      if (tagged) store_vec<W>(queue + (n + __popc(m & below)) * W, v);
+      n += __popc(m);
+      if (n >= kBatch) digest(kBatch);
+    }
   }
+  if (n > 0) digest(n);
   cnt = warp_sum(cnt);
   sum = warp_sum(sum);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) xr ^= __shfl_xor_sync(FULLMASK, xr, o);
-  if ((threadIdx.x & 31) == 0 && cnt) {
+  if (lane == 0 && cnt) {
     atomicAdd(&a.out[0], cnt);
     atomicAdd(&a.out[1], sum);
     atomicXor(&a.out[2], xr);
