@@ -114,15 +114,6 @@ __device__ __forceinline__ int64_t find_slot(const uint32_t* __restrict__ table,
   return -1;
 }
 
-template <int W>
-__device__ __forceinline__ bool slot_vec(const uint32_t* table, uint64_t i, uint32_t (&v)[W]) {
-  load_vec<W>(table + i * W, v);
-  bool tagged = true;
-#pragma unroll
-  for (int w = 0; w < W; ++w) tagged &= (v[w] & kTag) != 0;
-  return tagged;
-}
-
 // Histogram of local-state indices (each < 16, else *bad is set), 4 per word.
 template <int W>
 __device__ __forceinline__ void local_hist(const uint32_t* t, const NetBlobLayout& L, const uint32_t (&v)[W],
@@ -144,58 +135,265 @@ __device__ __forceinline__ void local_hist(const uint32_t* t, const NetBlobLayou
 
 constexpr uint32_t INF = 0xFFFFFFFFu;
 
+// Labelling works on a list of the states found: state i's slot, its distance
+// d[i], and where its successors' list indexes start in `adj` (when they are
+// kept); `index` gives the list index of a slot.
+struct LabelCtl {
+  unsigned long long states;   // states found in the table
+  unsigned long long edges;    // their successors
+  unsigned long long left[4];  // ring: states without a label after round r, at r & 3
+  unsigned long long bad;      // a local state index of 16 or more
+};
+
+struct LabelArgs {
+  const uint32_t* table;
+  const uint32_t* blob;
+  NetBlobLayout lay;
+  uint32_t staged_words;  // network tables the kernels copy to shared memory (0: none)
+  gx::Muls muls;
+  int rounds, log2nb;
+  uint64_t slots;
+  uint64_t cap;           // states the last search stored: the lists' size
+  uint64_t adj_cap;       // successors there is room for in adj (0: not kept)
+  uint32_t* index;        // [slots]
+  unsigned long long* slot_of;  // [cap]
+  uint32_t* d;            // [cap]
+  uint32_t* first;        // [cap] where a state's successors start in adj
+  uint32_t* last;         // [cap] and end
+  uint32_t* adj;          // [adj_cap]
+  uint32_t* todo[2];      // [cap] states without a label, before and after a round
+  LabelCtl* ctl;
+};
+
+// Lists the states in the table; states without successors are at distance 0,
+// the others wait for the first round.  Bound by the table's bytes: a warp reads
+// 1 KB at a time, collects the occupied slots in shared memory and lists 32 at a
+// time with one atomic per counter (8-process network, 72,000 states in 64 MiB: 42
+// us; a lane per slot took 102 us here and another 64 us to gather the examples
+// from the whole table again).
 template <int W>
-__global__ void __launch_bounds__(gx::kBlock) label_init_kernel(const uint32_t* table, uint64_t slots, const uint32_t* t,
-                                                                NetBlobLayout L, uint32_t* dist) {
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < slots; i += stride) {
+__global__ void __launch_bounds__(gx::kBlock) label_collect_kernel(const LabelArgs a) {
+  constexpr int kWarps = gx::kBlock / 32, S = 8 / W;
+  __shared__ unsigned long long queue_mem[kWarps][64];
+  unsigned long long* queue = queue_mem[threadIdx.x >> 5];
+  const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1u;
+  uint32_t n = 0;  // queued (uniform in the warp)
+  auto list = [&](uint32_t k) {  // the last k <= 32 queued
+    __syncwarp();
+    n -= k;
+    const bool has = lane < k;
+    const unsigned long long slot = has ? queue[n + lane] : 0ull;
     uint32_t v[W];
-    if (!slot_vec<W>(table, i, v)) {
-      dist[i] = INF;
-      continue;
+    load_vec<W>(a.table + slot * W, v);
+    const uint32_t cnt = has ? count_succ<W>(a.blob, a.lay, v) : 0u;
+    unsigned long long upto = cnt;  // successors of this state and the ones before it
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(FULLMASK, upto, o);
+      if ((int)lane >= o) upto += y;
     }
-    dist[i] = count_succ<W>(t, L, v) == 0 ? 0u : INF;
+    const uint32_t open = __ballot_sync(FULLMASK, cnt != 0);
+    unsigned long long at = 0;  // lane 0: states, 1: todo, 31: edges
+    if (lane == 0) at = atomicAdd(&a.ctl->states, (unsigned long long)k);
+    if (lane == 1 && open) at = atomicAdd(&a.ctl->left[0], (unsigned long long)__popc(open));
+    if (lane == 31 && open) at = atomicAdd(&a.ctl->edges, upto);
+    const unsigned long long i = __shfl_sync(FULLMASK, at, 0) + lane;
+    const unsigned long long t = __shfl_sync(FULLMASK, at, 1) + __popc(open & below);
+    const unsigned long long e = __shfl_sync(FULLMASK, at, 31) + upto - cnt;
+    // (more states than the last search stored: the host reports it, no list is used)
+    if (has && i < a.cap) {
+      a.index[slot] = (uint32_t)i;
+      a.slot_of[i] = slot;
+      a.d[i] = cnt ? INF : 0u;
+      a.first[i] = (uint32_t)e;
+      a.last[i] = (uint32_t)(e + cnt);
+      if (cnt && t < a.cap) a.todo[0][t] = (uint32_t)i;
+    }
+    __syncwarp();
+  };
+  // pieces of 8 words (a table has at least two buckets of four)
+  const uint64_t pieces = a.slots * W / 8, stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < pieces; i0 += stride) {
+    uint32_t s[8];
+#pragma unroll
+    for (int w = 0; w < 8; ++w) s[w] = 0;
+    if (i0 + lane < pieces) load_words<8>(a.table + (i0 + lane) * 8, s);
+#pragma unroll
+    for (int i = 0; i < S; ++i) {
+      bool tagged = true;
+#pragma unroll
+      for (int w = 0; w < W; ++w) tagged &= (s[i * W + w] & kTag) != 0;
+      const uint32_t m = __ballot_sync(FULLMASK, tagged);
+      if (tagged) queue[n + __popc(m & below)] = (i0 + lane) * S + i;
+      n += __popc(m);
+      if (n >= 32) list(32);
+    }
   }
+  if (n > 0) list(n);
 }
 
-template <int W, int B>
-__global__ void __launch_bounds__(gx::kBlock) label_sweep_kernel(const uint32_t* table, uint64_t slots,
-                                                                 const uint32_t* t, NetBlobLayout L, gx::Muls mm,
-                                                                 int rounds, int log2nb, uint32_t* dist, uint32_t r,
-                                                                 unsigned long long* changed) {
-  __shared__ uint64_t muls[kMaxRounds];
-  for (int i = threadIdx.x; i < rounds; i += blockDim.x) muls[i] = mm.m[i];
+// The lists hold what the last search stored, and (keep) its successors fit.
+__device__ __forceinline__ bool label_lists_ok(const LabelArgs& a, bool keep) {
+  return a.ctl->states <= a.cap && (!keep || a.ctl->edges <= a.adj_cap);
+}
+
+__device__ __forceinline__ const uint32_t* label_tables(const LabelArgs& a, uint64_t* muls, uint32_t* s_tab) {
+  for (int i = threadIdx.x; i < a.rounds; i += blockDim.x) muls[i] = a.muls.m[i];
+  for (uint32_t i = threadIdx.x; i < a.staged_words; i += blockDim.x) s_tab[i] = a.blob[i];
   __syncthreads();
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  uint32_t any = 0;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < slots; i += stride) {
-    if (dist[i] != INF) continue;
+  return a.staged_words ? s_tab : a.blob;
+}
+
+// The successors' list indexes of every state, looked up once: a lane per state.
+template <int W, int B>
+__global__ void __launch_bounds__(gx::kBlock) label_adj_kernel(const LabelArgs a) {
+  extern __shared__ __align__(16) uint32_t s_tab[];
+  __shared__ uint64_t muls[kMaxRounds];
+  if (!label_lists_ok(a, true)) return;
+  const uint32_t* t = label_tables(a, muls, s_tab);
+  const uint64_t n = a.ctl->states, stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
     uint32_t v[W];
-    if (!slot_vec<W>(table, i, v)) continue;
-    const uint32_t cnt = count_succ<W>(t, L, v);
+    load_vec<W>(a.table + a.slot_of[i] * W, v);
+    const uint32_t cnt = count_succ<W>(t, a.lay, v);
+    uint32_t* out = a.adj + a.first[i];
     SuccIter it;
     it.init();
     for (uint32_t k = 0; k < cnt; ++k) {
       uint32_t s[W];
-      next_succ<W>(it, t, L, v, s);
-      const int64_t j = find_slot<W, B>(table, log2nb, rounds, muls, s);
-      if (j >= 0 && dist[j] == r - 1) {
-        dist[i] = r;
-        any = 1;
-        break;
-      }
+      next_succ<W>(it, t, a.lay, v, s);
+      const int64_t j = find_slot<W, B>(a.table, a.log2nb, a.rounds, muls, s);
+      out[k] = j >= 0 ? a.index[j] : (uint32_t)i;  // (not stored: itself, which never is a label nearer)
     }
   }
-  if (__any_sync(FULLMASK, any != 0) && (threadIdx.x & 31) == 0) atomicAdd(changed, 1ull);
 }
 
-// Content order of the training examples: the gather appends at atomic
+// The ring of counters of round r; true when the round has nothing to do,
+// because nothing is left or the round before labelled nothing.  (This round adds
+// to left[r & 3] and reads the two before it.)
+__device__ __forceinline__ bool label_round_over(const LabelArgs& a, uint32_t r, unsigned long long n) {
+  const bool over = n == 0 || (r >= 2 && n == a.ctl->left[(r - 2) & 3]);
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    a.ctl->left[(r + 1) & 3] = 0;
+    if (over) a.ctl->left[r & 3] = n;
+  }
+  return over;
+}
+
+// Round r: the states still without a label that have a successor at distance r -
+// 1 get distance r, the others are listed for the next round.  Rounds are
+// launched one behind the other.  Here with the successors kept: 8 lanes a state,
+// no table lookup (72,000 states, 12.8 successors each: 7-12 us a round; with a
+// chain of table lookups per state 34 us; a pass over the whole table 219 us).
+constexpr int kLabelLanes = 8;
+__global__ void __launch_bounds__(gx::kBlock) label_round_kernel(const LabelArgs a, uint32_t r) {
+  constexpr uint32_t kStates = gx::kBlock / kLabelLanes;  // a CTA takes at a time
+  __shared__ uint32_t s_open[kStates];
+  __shared__ unsigned long long s_base;
+  const unsigned long long n = a.ctl->left[(r - 1) & 3];
+  if (!label_lists_ok(a, true) || label_round_over(a, r, n)) return;
+  const uint32_t lane = threadIdx.x & 31, sub = lane & (kLabelLanes - 1);
+  const uint32_t group = ((1u << kLabelLanes) - 1u) << (lane & ~(kLabelLanes - 1u));
+  static_assert(kStates == 32, "the first warp lists a CTA's states");
+  for (unsigned long long i0 = (unsigned long long)blockIdx.x * kStates; i0 < n;
+       i0 += (unsigned long long)gridDim.x * kStates) {
+    const unsigned long long i = i0 + threadIdx.x / kLabelLanes;
+    bool open = i < n;
+    uint32_t idx = 0, e = 0, end = 0;
+    if (open) {
+      idx = a.todo[(r - 1) & 1][i];
+      e = a.first[idx] + sub;
+      end = a.last[idx];
+    }
+    for (; __any_sync(FULLMASK, open && e - sub < end); e += kLabelLanes) {
+      const bool hit = open && e < end && a.d[a.adj[e]] == r - 1;
+      if (__ballot_sync(FULLMASK, hit) & group) {
+        if (open && sub == 0) a.d[idx] = r;
+        open = false;
+      }
+    }
+    // one atomic per CTA: one per warp would queue on the counter's address
+    if (sub == 0) s_open[threadIdx.x / kLabelLanes] = open ? idx : INF;
+    __syncthreads();
+    if (threadIdx.x < 32) {
+      const uint32_t mine = s_open[lane], m = __ballot_sync(FULLMASK, mine != INF);
+      if (lane == 0 && m) s_base = atomicAdd(&a.ctl->left[r & 3], (unsigned long long)__popc(m));
+      __syncwarp();
+      if (mine != INF) a.todo[r & 1][s_base + __popc(m & ((1u << lane) - 1u))] = mine;
+    }
+    __syncthreads();
+  }
+}
+
+// Round r without the successors kept (too many, or a search that was stopped
+// early): a lane per state looks them up until one is at distance r - 1.
+template <int W, int B>
+__global__ void __launch_bounds__(gx::kBlock) label_lookup_round_kernel(const LabelArgs a, uint32_t r) {
+  extern __shared__ __align__(16) uint32_t s_tab[];
+  __shared__ uint64_t muls[kMaxRounds];
+  const unsigned long long n = a.ctl->left[(r - 1) & 3];
+  if (!label_lists_ok(a, false) || label_round_over(a, r, n)) return;
+  if ((unsigned long long)blockIdx.x * blockDim.x >= n) return;
+  const uint32_t* t = label_tables(a, muls, s_tab);
+  const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1u;
+  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+  for (unsigned long long i0 = (unsigned long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < n;
+       i0 += stride) {
+    bool open = i0 + lane < n;
+    uint32_t idx = 0;
+    if (open) {
+      idx = a.todo[(r - 1) & 1][i0 + lane];
+      uint32_t v[W];
+      load_vec<W>(a.table + a.slot_of[idx] * W, v);
+      const uint32_t cnt = count_succ<W>(t, a.lay, v);
+      SuccIter it;
+      it.init();
+      for (uint32_t k = 0; k < cnt && open; ++k) {
+        uint32_t s[W];
+        next_succ<W>(it, t, a.lay, v, s);
+        const int64_t j = find_slot<W, B>(a.table, a.log2nb, a.rounds, muls, s);
+        if (j >= 0 && a.d[a.index[j]] == r - 1) {
+          a.d[idx] = r;
+          open = false;
+        }
+      }
+    }
+    const uint32_t m = __ballot_sync(FULLMASK, open);
+    unsigned long long base = 0;
+    if (lane == 0 && m) base = atomicAdd(&a.ctl->left[r & 3], (unsigned long long)__popc(m));
+    base = __shfl_sync(FULLMASK, base, 0);
+    if (open) a.todo[r & 1][base + __popc(m & below)] = idx;
+  }
+}
+
+// Example i: the histogram and the label of state i of the list.
+template <int W>
+__global__ void __launch_bounds__(gx::kBlock) label_gather_kernel(const LabelArgs a, uint32_t max_dist,
+                                                                  uint8_t* hist_out, float* label_out, uint64_t cap) {
+  if (!label_lists_ok(a, false)) return;
+  const uint64_t n = a.ctl->states, stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+    uint32_t v[W], hw[4], bad = 0;
+    load_vec<W>(a.table + a.slot_of[i] * W, v);
+    local_hist<W>(a.blob, a.lay, v, hw, bad);
+    if (bad) atomicOr(&a.ctl->bad, 1ull);
+    if (i >= cap) continue;
+    reinterpret_cast<uint4*>(hist_out)[i] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+    const uint32_t d = a.d[i] == INF ? max_dist : min(a.d[i], max_dist);
+    label_out[i] = (float)d / (float)max_dist;
+  }
+}
+
+// Content order of the training examples: the states are listed at atomic
 // positions, so the examples are sorted by their own content (the 16
 // histogram bytes, then the label's bits, compared as unsigned words) to make
 // the training set -- and everything trained from it -- the same on every run.
 // Equal keys are identical examples, so an unstable sort is enough: a bitonic
 // sort over a power-of-two buffer padded with all-ones keys (no histogram byte
-// reaches 0xFF).
+// reaches 0xFF).  Passes over distances below a tile of 2^kTileLog2 examples run
+// in shared memory, all that follow one another in one launch; the others take
+// two distances at a time, four examples per thread.  2^17 examples: 20
+// launches instead of 153.
 __device__ __forceinline__ bool ex_greater(const uint4& a, uint32_t la, const uint4& b, uint32_t lb) {
   if (a.x != b.x) return a.x > b.x;
   if (a.y != b.y) return a.y > b.y;
@@ -204,32 +402,121 @@ __device__ __forceinline__ bool ex_greater(const uint4& a, uint32_t la, const ui
   return la > lb;
 }
 
-__global__ void ex_load_kernel(const uint8_t* hist, const float* label, uint64_t n, uint64_t n2, uint4* h,
-                               uint32_t* l) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += (uint64_t)gridDim.x * blockDim.x) {
-    if (i < n) {
-      h[i] = reinterpret_cast<const uint4*>(hist)[i];
-      l[i] = __float_as_uint(label[i]);
+__device__ __forceinline__ void ex_order(uint4& a, uint32_t& la, uint4& b, uint32_t& lb, bool up) {
+  if (up != ex_greater(a, la, b, lb)) return;
+  const uint4 q = a;
+  const uint32_t l = la;
+  a = b;
+  la = lb;
+  b = q;
+  lb = l;
+}
+
+// Examples at distances 2q and q: four of them a, a + q, a + 2q, a + 3q.
+__device__ __forceinline__ void ex_order4(uint4 (&x)[4], uint32_t (&l)[4], bool up) {
+  ex_order(x[0], l[0], x[2], l[2], up);
+  ex_order(x[1], l[1], x[3], l[3], up);
+  ex_order(x[0], l[0], x[1], l[1], up);
+  ex_order(x[2], l[2], x[3], l[3], up);
+}
+
+constexpr int kTileLog2 = 11;
+constexpr int kTile = 1 << kTileLog2;
+constexpr int kTileThreads = 512;
+constexpr size_t kTileBytes = 20 * kTile;
+
+// The passes of stages k0..k1 (powers of two) at distances below the tile, on one
+// tile per CTA.  `load`: the examples come from hist and label (n of them, padded).
+__global__ void __launch_bounds__(kTileThreads) ex_tile_kernel(uint4* h, uint32_t* l, uint64_t n2, uint64_t k0,
+                                                               uint64_t k1, int load, const uint8_t* hist,
+                                                               const float* label, uint64_t n) {
+  extern __shared__ __align__(16) unsigned char tile_mem[];
+  uint4* sh = reinterpret_cast<uint4*>(tile_mem);
+  uint32_t* sl = reinterpret_cast<uint32_t*>(sh + kTile);
+  const uint64_t base = (uint64_t)blockIdx.x * kTile;
+  const int tile = n2 < (uint64_t)kTile ? (int)n2 : kTile;
+  for (int i = threadIdx.x; i < tile; i += kTileThreads) {
+    if (!load) {
+      sh[i] = h[base + i];
+      sl[i] = l[base + i];
+    } else if (base + i < n) {
+      sh[i] = reinterpret_cast<const uint4*>(hist)[base + i];
+      sl[i] = __float_as_uint(label[base + i]);
     } else {
-      h[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
-      l[i] = ~0u;
+      sh[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+      sl[i] = ~0u;
     }
+  }
+  __syncthreads();
+  // two distances at a time, four examples per thread in registers
+  for (uint64_t k = k0; k <= k1; k <<= 1) {
+    int j = k / 2 < (uint64_t)tile / 2 ? (int)(k / 2) : tile / 2;
+    while (j > 0) {
+      if (j >= 2) {
+        const int q = j / 2;
+        for (int p = threadIdx.x; p < tile / 4; p += kTileThreads) {
+          const int a = ((p & ~(q - 1)) << 2) | (p & (q - 1));
+          const bool up = ((base + a) & k) == 0;
+          uint4 x[4];
+          uint32_t lx[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            x[i] = sh[a + i * q];
+            lx[i] = sl[a + i * q];
+          }
+          ex_order4(x, lx, up);
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            sh[a + i * q] = x[i];
+            sl[a + i * q] = lx[i];
+          }
+        }
+        j >>= 2;
+      } else {
+        for (int p = threadIdx.x; p < tile / 2; p += kTileThreads) {
+          const int a = p << 1;
+          ex_order(sh[a], sl[a], sh[a + 1], sl[a + 1], ((base + a) & k) == 0);
+        }
+        j = 0;
+      }
+      __syncthreads();
+    }
+  }
+  for (int i = threadIdx.x; i < tile; i += kTileThreads) {
+    h[base + i] = sh[i];
+    l[base + i] = sl[i];
   }
 }
 
-// One compare-exchange pass of the bitonic network: stage k, distance j.
-__global__ void ex_bitonic_kernel(uint4* h, uint32_t* l, uint64_t n2, uint64_t k, uint64_t j) {
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n2; i += (uint64_t)gridDim.x * blockDim.x) {
-    const uint64_t p = i ^ j;
-    if (p <= i) continue;
-    const uint4 a = h[i], b = h[p];
-    const uint32_t la = l[i], lb = l[p];
-    const bool up = (i & k) == 0;
-    if (up == ex_greater(a, la, b, lb)) {
-      h[i] = b;
-      h[p] = a;
-      l[i] = lb;
-      l[p] = la;
+// Stage k at distances j and, when `two`, j / 2 (both at least a tile).
+__global__ void __launch_bounds__(256) ex_wide_kernel(uint4* h, uint32_t* l, uint64_t n2, uint64_t k, uint64_t j,
+                                                      int two) {
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x, q = two ? j / 2 : j;
+  for (uint64_t p = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n2 / (two ? 4 : 2); p += stride) {
+    const uint64_t a = two ? ((p & ~(q - 1)) << 2) | (p & (q - 1)) : ((p & ~(j - 1)) << 1) | (p & (j - 1));
+    const bool up = (a & k) == 0;
+    if (!two) {
+      uint4 x = h[a], y = h[a + j];
+      uint32_t lx = l[a], ly = l[a + j];
+      ex_order(x, lx, y, ly, up);
+      h[a] = x;
+      h[a + j] = y;
+      l[a] = lx;
+      l[a + j] = ly;
+    } else {
+      uint4 x[4];
+      uint32_t lx[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        x[i] = h[a + i * q];
+        lx[i] = l[a + i * q];
+      }
+      ex_order4(x, lx, up);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        h[a + i * q] = x[i];
+        l[a + i * q] = lx[i];
+      }
     }
   }
 }
@@ -238,32 +525,6 @@ __global__ void ex_store_kernel(const uint4* h, const uint32_t* l, uint64_t n, u
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
     reinterpret_cast<uint4*>(hist)[i] = h[i];
     label[i] = __uint_as_float(l[i]);
-  }
-}
-
-template <int W>
-__global__ void __launch_bounds__(gx::kBlock) label_gather_kernel(const uint32_t* table, uint64_t slots,
-                                                                  const uint32_t* t, NetBlobLayout L,
-                                                                  const uint32_t* dist, uint32_t max_dist,
-                                                                  uint8_t* hist_out, float* label_out, uint64_t cap,
-                                                                  unsigned long long* count,
-                                                                  unsigned long long* bad_flag) {
-  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < slots; i += stride) {
-    uint32_t v[W];
-    if (!slot_vec<W>(table, i, v)) continue;
-    uint32_t hw[4], bad = 0;
-    local_hist<W>(t, L, v, hw, bad);
-    if (bad) atomicOr(bad_flag, 1ull);
-    const unsigned long long pos = atomicAdd(count, 1ull);
-    if (pos >= cap) continue;
-    uint32_t* dst = reinterpret_cast<uint32_t*>(hist_out + pos * 16);
-    dst[0] = hw[0];
-    dst[1] = hw[1];
-    dst[2] = hw[2];
-    dst[3] = hw[3];
-    const uint32_t d = dist[i] == INF ? max_dist : min(dist[i], max_dist);
-    label_out[pos] = (float)d / (float)max_dist;
   }
 }
 
@@ -809,8 +1070,10 @@ namespace {
 inline uint64_t a256(uint64_t x) { return (x + 255) & ~255ull; }
 
 struct GKernels {
-  void (*sweep)(const uint32_t*, uint64_t, const uint32_t*, NetBlobLayout, Muls, int, int, uint32_t*, uint32_t,
-                unsigned long long*);
+  void (*label_collect)(gxd::LabelArgs);
+  void (*label_adj)(gxd::LabelArgs);
+  void (*label_lookup_round)(gxd::LabelArgs, uint32_t);
+  void (*label_gather)(gxd::LabelArgs, uint32_t, uint8_t*, float*, uint64_t);
   const void* init;
   const void* select;
   const void* expand;
@@ -823,7 +1086,9 @@ struct GKernels {
 
 template <int W, int B>
 GKernels gk() {
-  return GKernels{&gxd::label_sweep_kernel<W, B>, reinterpret_cast<const void*>(&gxd::guided_init_kernel<W, B>),
+  return GKernels{&gxd::label_collect_kernel<W>, &gxd::label_adj_kernel<W, B>, &gxd::label_lookup_round_kernel<W, B>,
+                  &gxd::label_gather_kernel<W>,
+                  reinterpret_cast<const void*>(&gxd::guided_init_kernel<W, B>),
                   reinterpret_cast<const void*>(&gxd::guided_select_kernel<W>),
                   reinterpret_cast<const void*>(&gxd::guided_expand_kernel<W, B>),
                   reinterpret_cast<const void*>(&gxd::guided_score_kernel<W>),
@@ -1248,67 +1513,96 @@ gx_status gx_training_set(gx_net* h, void* ws, uint64_t ws_bytes, void* stream, 
     return gx::fail(GX_ERR_INVALID, "no labelling kernel for this table layout");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* base = static_cast<char*>(ws);
-  const uint32_t* table = reinterpret_cast<const uint32_t*>(base + h->ws_off_table);
-  const uint32_t* blob = reinterpret_cast<const uint32_t*>(base + h->ws_off_blob);
-  gx::Ctl* ctl = reinterpret_cast<gx::Ctl*>(base + h->ws_off_ctl);
-  unsigned long long* flags = ctl->digest;  // [0] changed, [1] count, [2] bad
-  const uint64_t slots = S.table_slots;
-  const int W = (int)S.slot_words;
-  gx::Muls mm;
-  gx::hash_multipliers(mm.m, gx::kMaxRounds);
-  const int log2nb = gx::log2_of(slots * W / S.bucket_words);
+  const uint64_t slots = S.table_slots, states = S.states;
+  if (states >= (1ull << 32)) return gx::fail(GX_ERR_OOM, "2^32 or more states to label");
+  gxd::LabelArgs a{};
+  a.table = reinterpret_cast<const uint32_t*>(base + h->ws_off_table);
+  a.blob = reinterpret_cast<const uint32_t*>(base + h->ws_off_blob);
+  a.lay = h->net.lay;
+  a.staged_words = h->net.blob.size() <= 11 * 1024 ? (uint32_t)h->net.blob.size() : 0;
+  gx::hash_multipliers(a.muls.m, gx::kMaxRounds);
+  a.rounds = (int)S.hash_rounds;
+  a.log2nb = gx::log2_of(slots * S.slot_words / S.bucket_words);
+  a.slots = slots;
+  a.cap = states;
+  a.index = dist;
   int dev = 0, sms = 0;
   GG_CUDA(cudaGetDevice(&dev));
   GG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int grid = sms * 8;
-  if (W == 1) gxd::label_init_kernel<1><<<grid, gx::kBlock, 0, st>>>(table, slots, blob, h->net.lay, dist);
-  else if (W == 2) gxd::label_init_kernel<2><<<grid, gx::kBlock, 0, st>>>(table, slots, blob, h->net.lay, dist);
-  else gxd::label_init_kernel<4><<<grid, gx::kBlock, 0, st>>>(table, slots, blob, h->net.lay, dist);
-  GG_CUDA(cudaGetLastError());
-  for (uint32_t r = 1; r <= max_dist; ++r) {
-    GG_CUDA(cudaMemsetAsync(flags, 0, 8, st));
-    k.sweep<<<grid, gx::kBlock, 0, st>>>(table, slots, blob, h->net.lay, mm, (int)S.hash_rounds, log2nb, dist, r,
-                                         flags);
-    GG_CUDA(cudaGetLastError());
-    unsigned long long changed = 0;
-    GG_CUDA(cudaMemcpyAsync(&changed, flags, 8, cudaMemcpyDeviceToHost, st));
-    GG_CUDA(cudaStreamSynchronize(st));
-    if (!changed) break;
+  // temporary memory: the control block, the lists (28 bytes a state) and, after a complete
+  // search with at most 2^28 transitions, every state's successors (4 bytes each); the sort's
+  // buffers (20 bytes an example, a power of two of them) take their place afterwards
+  const uint64_t most = std::min<uint64_t>(states, cap);
+  uint64_t n2 = 1;
+  while (n2 < most) n2 <<= 1;
+  a.adj_cap = S.complete && S.transitions <= (1ull << 28) ? S.transitions : 0;
+  struct Temp {
+    unsigned char* p = nullptr;
+    cudaStream_t st;
+    ~Temp() {
+      if (p) cudaFreeAsync(p, st);
+    }
+  } temp{nullptr, st};
+  const uint64_t lists = gx::a256(sizeof(gxd::LabelCtl));
+  auto bytes = [&] { return lists + std::max<uint64_t>(28 * states + 4 * a.adj_cap, 20 * n2); };
+  if (cudaMallocAsync(reinterpret_cast<void**>(&temp.p), bytes(), st) != cudaSuccess) {
+    cudaGetLastError();
+    temp.p = nullptr;
+    a.adj_cap = 0;  // look the successors up in every round
+    GG_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&temp.p), bytes(), st));
   }
-  GG_CUDA(cudaMemsetAsync(flags + 1, 0, 16, st));
-  if (W == 1)
-    gxd::label_gather_kernel<1><<<grid, gx::kBlock, 0, st>>>(table, slots, blob, h->net.lay, dist, max_dist, hist_out,
-                                                              label_out, cap, flags + 1, flags + 2);
-  else if (W == 2)
-    gxd::label_gather_kernel<2><<<grid, gx::kBlock, 0, st>>>(table, slots, blob, h->net.lay, dist, max_dist, hist_out,
-                                                              label_out, cap, flags + 1, flags + 2);
-  else
-    gxd::label_gather_kernel<4><<<grid, gx::kBlock, 0, st>>>(table, slots, blob, h->net.lay, dist, max_dist, hist_out,
-                                                              label_out, cap, flags + 1, flags + 2);
+  a.ctl = reinterpret_cast<gxd::LabelCtl*>(temp.p);
+  a.slot_of = reinterpret_cast<unsigned long long*>(temp.p + lists);
+  a.d = reinterpret_cast<uint32_t*>(a.slot_of + states);
+  a.first = a.d + states;
+  a.last = a.first + states;
+  a.todo[0] = a.last + states;
+  a.todo[1] = a.todo[0] + states;
+  a.adj = a.todo[1] + states;
+  GG_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(gxd::LabelCtl), st));
+  k.label_collect<<<grid, gx::kBlock, 0, st>>>(a);
+  if (a.adj_cap) k.label_adj<<<grid, gx::kBlock, 4ull * a.staged_words, st>>>(a);
   GG_CUDA(cudaGetLastError());
-  unsigned long long res[2] = {0, 0};
-  GG_CUDA(cudaMemcpyAsync(res, flags + 1, 16, cudaMemcpyDeviceToHost, st));
+  gxd::LabelCtl hc{};
+  constexpr uint32_t kAhead = 16;  // rounds launched before the host looks whether any is needed
+  for (uint32_t r = 1; r <= max_dist; ++r) {
+    if (a.adj_cap) gxd::label_round_kernel<<<grid, gx::kBlock, 0, st>>>(a, r);
+    else k.label_lookup_round<<<grid, gx::kBlock, 4ull * a.staged_words, st>>>(a, r);
+    GG_CUDA(cudaGetLastError());
+    if (r % kAhead == 0 && r < max_dist) {
+      GG_CUDA(cudaMemcpyAsync(&hc, a.ctl, sizeof(hc), cudaMemcpyDeviceToHost, st));
+      GG_CUDA(cudaStreamSynchronize(st));
+      if (hc.states > states || hc.left[r & 3] == 0 || hc.left[r & 3] == hc.left[(r - 1) & 3]) break;
+    }
+  }
+  k.label_gather<<<grid, gx::kBlock, 0, st>>>(a, max_dist, hist_out, label_out, cap);
+  GG_CUDA(cudaGetLastError());
+  GG_CUDA(cudaMemcpyAsync(&hc, a.ctl, sizeof(hc), cudaMemcpyDeviceToHost, st));
   GG_CUDA(cudaStreamSynchronize(st));
-  if (n_out) *n_out = res[0];
-  if (res[1]) return gx::fail(GX_ERR_INVALID, "a process has a local state index of 16 or more");
-  // content order (see ex_bitonic_kernel)
-  const uint64_t m = std::min<uint64_t>(res[0], cap);
-  if (m > 1) {
-    uint64_t n2 = 1;
-    while (n2 < m) n2 <<= 1;
-    uint4* sh = nullptr;
-    uint32_t* sl = nullptr;
-    GG_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&sh), 16 * n2, st));
-    GG_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&sl), 4 * n2, st));
-    const int sgrid = sms * 8;
-    gxd::ex_load_kernel<<<sgrid, 256, 0, st>>>(hist_out, label_out, m, n2, sh, sl);
-    for (uint64_t k2 = 2; k2 <= n2; k2 <<= 1)
-      for (uint64_t j = k2 >> 1; j > 0; j >>= 1) gxd::ex_bitonic_kernel<<<sgrid, 256, 0, st>>>(sh, sl, n2, k2, j);
-    gxd::ex_store_kernel<<<sgrid, 256, 0, st>>>(sh, sl, m, hist_out, label_out);
-    const cudaError_t le = cudaGetLastError();
-    GG_CUDA(cudaFreeAsync(sh, st));
-    GG_CUDA(cudaFreeAsync(sl, st));
-    GG_CUDA(le);
+  if (hc.states != states || (a.adj_cap && hc.edges > a.adj_cap))
+    return gx::fail(GX_ERR_STATE, "the workspace does not hold the last search's table");
+  if (n_out) *n_out = states;
+  if (hc.bad) return gx::fail(GX_ERR_INVALID, "a process has a local state index of 16 or more");
+  // content order (see ex_greater)
+  if (most > 1) {
+    uint4* sh = reinterpret_cast<uint4*>(temp.p + lists);
+    uint32_t* sl = reinterpret_cast<uint32_t*>(sh + n2);
+    const int tiles = (int)std::max<uint64_t>(1, n2 / gxd::kTile);
+    const uint64_t first = std::min<uint64_t>(n2, gxd::kTile);
+    gxd::ex_tile_kernel<<<tiles, gxd::kTileThreads, gxd::kTileBytes, st>>>(sh, sl, n2, 2, first, 1, hist_out, label_out,
+                                                                         most);
+    for (uint64_t k2 = 2 * first; k2 <= n2; k2 <<= 1) {
+      uint64_t j = k2 >> 1;
+      while (j >= (uint64_t)gxd::kTile) {
+        const int two = j / 2 >= (uint64_t)gxd::kTile;
+        gxd::ex_wide_kernel<<<grid, 256, 0, st>>>(sh, sl, n2, k2, j, two);
+        j >>= two ? 2 : 1;
+      }
+      gxd::ex_tile_kernel<<<tiles, gxd::kTileThreads, gxd::kTileBytes, st>>>(sh, sl, n2, k2, k2, 0, nullptr, nullptr, 0);
+    }
+    gxd::ex_store_kernel<<<grid, 256, 0, st>>>(sh, sl, most, hist_out, label_out);
+    GG_CUDA(cudaGetLastError());
     GG_CUDA(cudaStreamSynchronize(st));
   }
   return GX_OK;
