@@ -357,8 +357,8 @@ gx_status gx_set_digest(gx_net* net, void* workspace, uint64_t workspace_bytes, 
 /* CTAs of the gradient kernel at most; each writes its own partial gradient,
  * which a second kernel sums in a fixed order (gradients are deterministic). */
 #define GX_MLP_GRAD_CTAS 256
-/* Device bytes of the optimiser state gx_mlp_train needs for a batch size:
- * Adam moments, the gradient, the partial gradients and the batch indices. */
+/* Device bytes of the optimiser state gx_mlp_train needs for a batch size (room
+ * for the Adam moments and the partial gradients and losses). */
 #define GX_MLP_STATE_BYTES(batch) \
   (4ull * ((3ull + GX_MLP_GRAD_CTAS) * GX_MLP_PARAMS + GX_MLP_GRAD_CTAS + 2ull) + 8ull * (batch))
 

@@ -49,16 +49,31 @@ constexpr int NPARAM = OFF_B3 + 1;
 static_assert(NPARAM == GX_MLP_PARAMS, "parameter count");
 constexpr int kGradCtas = GX_MLP_GRAD_CTAS;  // at most this many CTAs, one partial gradient each
 
-// g[i] = sum over the CTAs c, in order, of partial[c][i]; *loss likewise.
+// A partial gradient holds W1 and W2 transposed (a column of 128 hidden units
+// after the other), as a gradient CTA's threads, one hidden unit each, write them
+// in whole lines.
+constexpr int kPartial = NPARAM;
+
+// The parameter that element q of a partial gradient belongs to.
+__device__ __forceinline__ int partial_param(int q) {
+  if (q < OFF_B1) return OFF_W1 + (q % H) * IN + q / H;
+  if (q >= OFF_W2 && q < OFF_B2) return OFF_W2 + ((q - OFF_W2) % H) * H + (q - OFF_W2) / H;
+  return q;
+}
+
+// Element q of the gradient: the sum over the CTAs c, in order, of partial[c][q].
+__device__ __forceinline__ float partial_sum(const float* __restrict__ partial, int ctas, int q) {
+  float acc = 0.f;
+#pragma unroll 8
+  for (int c = 0; c < ctas; ++c) acc += partial[(uint64_t)c * kPartial + q];
+  return acc;
+}
+
 __global__ void reduce_kernel(const float* __restrict__ partial, const float* __restrict__ partial_loss, int ctas,
                               float* __restrict__ g, float* __restrict__ loss) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < NPARAM) {
-    float acc = 0.f;
-    for (int c = 0; c < ctas; ++c) acc += partial[(uint64_t)c * NPARAM + i];
-    g[i] = acc;
-  }
-  if (i == 0) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;
+  if (q < NPARAM) g[partial_param(q)] = partial_sum(partial, ctas, q);
+  if (q == 0) {
     float l = 0.f;
     for (int c = 0; c < ctas; ++c) l += partial_loss[c];
     *loss = l;
@@ -101,27 +116,41 @@ __global__ void __launch_bounds__(gxt::kRows) mlp_tc_forward_kernel(const gxt::T
   gxt::tc_teardown(sc);
 }
 
-// ---- Gradient on the tensor cores.  One CTA of 128 threads per tile of 128
-// examples (thread t: example t of the tile, TMEM lane t), all of TMEM (512
-// columns) per CTA.  Every product is a tcgen05 BF16 x BF16 -> FP32 MMA with
-// K-major operands in shared memory (transposed operands are written
-// transposed, so every descriptor has the same form as the scorer's):
+// ---- Gradient on the tensor cores.  One CTA of 512 threads per tile of 128
+// examples, all of TMEM (512 columns) per CTA.  Every product is a tcgen05
+// BF16 x BF16 -> FP32 MMA on operands in shared memory:
 //   A1  = X W1^T,  H = bf16(relu(A1 + b1))              (forward, as the scorer)
 //   A2  = H W2^T,  y = b3 + w3 . relu(A2 + b2)
-//   dy  = 2 (y - label) / n,  D2 = dy w3^T o (A2 + b2 > 0)        (thread-local)
+//   dy  = 2 (y - label) / n,  D2 = dy w3^T o (A2 + b2 > 0)
 //   DH  = D2 W2                                          [128 x 128]
-//   [gW2 | gb2] += D2^T [H | 1]                          N = 128 + 16 (ones rows)
+//   [gW2 | gb2] += D2^T [H | 1]                          N = 128 + 16 (ones columns)
 //   DA1 = DH o (A1 + b1 > 0)
 //   [gW1 | gb1] += DA1^T [X | 1]                         N = 16 + 16
+// X, H, D2 and DA1 are written once, an example's row as 16-byte pieces of 8
+// elements; the products that take them transposed read the same memory as
+// MN-major operands (a core matrix of 8 examples x 8 elements is either a K-major
+// piece of the matrix or an MN-major piece of its transpose).
+//
+// A step's time is a chain of latencies -- loads, five products, the epilogues
+// between them -- so the epilogues are spread over 16 warps: warp w owns rows 32 (w
+// & 3).. (its TMEM lanes) and columns 32 (w >> 2)... The dot product y keeps its
+// order of additions: the four column groups add to it one after the other.
+// Step of 1024 examples (8 tiles): 12.4 us a step; with 4 warps, transposed copies of
+// the operands and sampling, packing, reduction and Adam in launches of their
+// own 42 us.
+//
 // The gradients accumulate in TMEM over the CTA's tiles, in tile order; gw3 and
 // gb3 are summed on the CUDA cores (a fixed butterfly over each warp's lanes,
 // then the warps in order), so a CTA's partial gradient does not depend on
 // scheduling.  D2 and DA1 enter their products rounded to BF16.
+constexpr int kGradThreads = 512;
 constexpr uint32_t kTrainCols = 512;
 constexpr uint32_t kColAcc = 0, kColDH = 128, kColGW2 = 256, kColGW1 = 400;
-// instruction descriptors: M = 128 with N = 128, 144 (H^T and 16 ones rows), 32 (X^T and 16 ones rows)
-constexpr uint32_t kI128 = gxt::idesc_bf16_f32(128, 128), kI144 = gxt::idesc_bf16_f32(128, 144),
-                   kI32 = gxt::idesc_bf16_f32(128, 32);
+// K groups (8 elements) of an example's row: X and 16 ones; H and 16 ones; D2, DA1
+constexpr uint32_t kGroupsX = 4, kGroupsH = 18, kGroupsD = 16;
+// instruction descriptors: M = 128 with N = 128 (K-major operands), 144 ([H | 1]) and 32 ([X | 1], both MN-major)
+constexpr uint32_t kI128 = gxt::idesc_bf16_f32(128, 128), kI144t = gxt::idesc_bf16_f32(128, 144, 1, 1),
+                   kI32t = gxt::idesc_bf16_f32(128, 32, 1, 1);
 
 // The parameters as a training CTA holds them: the scorer's image plus W2
 // transposed (the B operand of DH = D2 W2: rows j, K = k).
@@ -132,17 +161,17 @@ struct __align__(16) TcTrainWeights {
 static_assert(sizeof(TcTrainWeights) % 16 == 0, "bulk copies move multiples of 16 bytes");
 
 struct __align__(1024) TrainSmem {
-  uint8_t x[gxt::kRows * IN * 2];      // A of layer 1: [r][i], K groups 2
-  uint8_t xto[32 * gxt::kRows * 2];    // B of gW1|gb1: rows 0-15 X^T [i][r], rows 16-31 ones; K groups 16
-  uint8_t h[gxt::kRows * H * 2];       // A of layer 2: H [r][j]; then DA1^T [j][r], A of gW1
-  uint8_t hto[(H + 16) * gxt::kRows * 2];  // B of gW2|gb2: rows 0-127 H^T [j][r], rows 128-143 ones
-  uint8_t d[gxt::kRows * H * 2];       // A of DH: D2 [r][k]
-  uint8_t dt[H * gxt::kRows * 2];      // A of gW2: D2^T [k][r]
+  uint8_t x[gxt::kRows * kGroupsX * 16];   // [X | 1]
+  uint8_t h[gxt::kRows * kGroupsH * 16];   // [H | 1]
+  uint8_t d[gxt::kRows * kGroupsD * 16];   // D2
+  uint8_t da[gxt::kRows * kGroupsD * 16];  // DA1
   TcTrainWeights wt;
-  float red[4][H];                     // per-warp sums of the gw3 terms
-  float redl[4][2];                    // per-warp loss and gb3
+  float y[gxt::kRows];
+  float lab[gxt::kRows];
+  float red[4][H];                     // per row group: sums of the gw3 terms
+  float redl[4][2];                    // per row group: loss and gb3
   uint32_t tmem_slot;
-  unsigned long long mbar, mbar_load;
+  unsigned long long mbar, mbar_load[3];  // products; W1 and biases, W2, W2^T
 };
 constexpr size_t kTrainSmemBytes = sizeof(TrainSmem) + 1024;  // + alignment slack
 static_assert(kTrainSmemBytes <= 232448, "a training CTA must fit the SM's shared memory");
@@ -171,6 +200,14 @@ __device__ __forceinline__ void st_bf16(uint8_t* base, uint32_t off, float v) {
   *reinterpret_cast<__nv_bfloat16*>(base + off) = __float2bfloat16_rn(v);
 }
 
+// Programmatic dependent launch: wait for the kernel in front (and its writes) to
+// complete; let the next kernel start.
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Two warps meet at named barrier `id`.
+__device__ __forceinline__ void pair_sync(int id) { asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory"); }
+
 // Sum of v over the warp's 32 lanes for 32 columns at once, in a fixed order
 // (recursive halving: at step h the lanes with bit h set keep the upper half of
 // their columns), so lane l ends with the sum of column l.
@@ -194,141 +231,205 @@ __device__ unsigned int g_train_error;  // a bounded wait gave up (GX_ERR_SPIN_L
 // device; calls hold g_train_mutex from packing to completion).
 __device__ TcTrainWeights g_train_packed;
 
-// CTA c takes tiles c, c + gridDim.x, ... of the n examples (example index[s]
-// for slot s when index is given) and writes its partial gradient of the mean
-// loss (inv_n = 1 / n) to partial[c], its loss to partial_loss[c].
-__global__ void __launch_bounds__(gxt::kRows, 1) grad_tc_kernel(const TcTrainWeights* __restrict__ packed,
-                                                                const uint8_t* __restrict__ hist,
-                                                                const float* __restrict__ label, uint64_t n,
-                                                                const uint64_t* __restrict__ index, float inv_n,
-                                                                float* __restrict__ partial,
-                                                                float* __restrict__ partial_loss) {
+// Mini-batch drawn by a counter-based stream: element j is example
+// mix64(start + j) mod n of the training set.
+struct Draw {
+  uint64_t n, start;
+  int on;
+};
+
+// CTA c takes tiles c, c + gridDim.x, ... of the n examples and writes its partial
+// gradient of the mean loss (inv_n = 1 / n) to partial[c], its loss to
+// partial_loss[c].
+__global__ void __launch_bounds__(kGradThreads, 1)
+    grad_tc_kernel(const TcTrainWeights* __restrict__ packed, const uint8_t* __restrict__ hist,
+                   const float* __restrict__ label, uint64_t n, const Draw draw, float inv_n,
+                   float* __restrict__ partial, float* __restrict__ partial_loss) {
   extern __shared__ __align__(16) uint8_t gsm[];
   TrainSmem* s = reinterpret_cast<TrainSmem*>((reinterpret_cast<uintptr_t>(gsm) + 1023) & ~uintptr_t(1023));
-  const int t = threadIdx.x, lane = t & 31, wid = t >> 5;
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int rg = wid & 3, c = wid >> 2;  // row group (TMEM lanes), column group
+  const int t = 32 * rg + lane;          // example of the tile
   const uint64_t tiles = (n + gxt::kRows - 1) / gxt::kRows;
   if (blockIdx.x >= tiles) return;
   using namespace gxt;
-  if (t == 0) {
+  if (tid == 0) {
     mbar_init(saddr(&s->mbar), 1);
-    mbar_init(saddr(&s->mbar_load), 1);
-    mbar_expect_tx(saddr(&s->mbar_load), (uint32_t)sizeof(TcTrainWeights));
-    bulk_g2s(saddr(&s->wt), packed, (uint32_t)sizeof(TcTrainWeights), saddr(&s->mbar_load));
+    for (int i = 0; i < 3; ++i) mbar_init(saddr(&s->mbar_load[i]), 1);
   }
-  if (t < 32) {
+  if (wid == 0) {
     __syncwarp();
     tmem_alloc(saddr(&s->tmem_slot), kTrainCols);
     tmem_relinquish();
   }
-  // the ones rows of the two stacked B operands (their products give the bias gradients)
-  for (int i = t; i < 16 * gxt::kRows; i += gxt::kRows) {
-    st_bf16(s->xto, core_offset(16 + i / gxt::kRows, i % gxt::kRows, 16), 1.f);
-    st_bf16(s->hto, core_offset(H + i / gxt::kRows, i % gxt::kRows, 16), 1.f);
+  // the ones columns of [X | 1] and [H | 1] (their products give the bias gradients)
+  if (c >= 2) {
+    constexpr uint32_t kOnes = 0x3F803F80u;  // two BF16 ones
+    const uint4 ones = make_uint4(kOnes, kOnes, kOnes, kOnes);
+    uint8_t* base = c == 2 ? s->x : s->h;
+    const uint32_t k0 = c == 2 ? IN : H, kg = c == 2 ? kGroupsX : kGroupsH;
+    *reinterpret_cast<uint4*>(base + core_offset(t, k0, kg)) = ones;
+    *reinterpret_cast<uint4*>(base + core_offset(t, k0 + 8, kg)) = ones;
   }
+  // X = bf16(hist / processes) and the labels of a tile, by the first column group
+  auto fill_x = [&](uint64_t tile) {
+    if (c != 0) return;
+    const uint64_t row = tile * kRows + t;
+    const bool valid = row < n;
+    uint64_t ex = row;
+    if (draw.on) {
+      uint64_t z = draw.start + row + 0x9E3779B97F4A7C15ull;
+      z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+      z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+      ex = (z ^ (z >> 31)) % draw.n;
+    }
+    uint32_t hw[4] = {0, 0, 0, 0};
+    if (valid) {
+      const uint8_t* src = hist + ex * IN;
+      if ((reinterpret_cast<uintptr_t>(src) & 15) == 0) {
+        const uint4 q = *reinterpret_cast<const uint4*>(src);
+        hw[0] = q.x;
+        hw[1] = q.y;
+        hw[2] = q.z;
+        hw[3] = q.w;
+      } else {
+#pragma unroll
+        for (int i = 0; i < IN; ++i) hw[i >> 2] |= (uint32_t)src[i] << ((i & 3) * 8);
+      }
+    }
+    s->lab[t] = valid ? label[ex] : 0.f;
+    const float inv = feature_scale(hw);
+    uint32_t q[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t w = hw[i >> 1], sh = (i & 1) * 16;
+      q[i] = pack_bf16x2((float)((w >> sh) & 0xFFu) * inv, (float)((w >> (sh + 8)) & 0xFFu) * inv);
+    }
+    *reinterpret_cast<uint4*>(s->x + core_offset(t, 0, kGroupsX)) = make_uint4(q[0], q[1], q[2], q[3]);
+    *reinterpret_cast<uint4*>(s->x + core_offset(t, 8, kGroupsX)) = make_uint4(q[4], q[5], q[6], q[7]);
+  };
+  fill_x(blockIdx.x);
+  fence_async_smem();
   tc_fence_before();
-  tc_sync();
+  __syncthreads();
   tc_fence_after();
-  bool ok = mbar_wait_bounded(saddr(&s->mbar_load), 0);
-  if (!ok) ok = mbar_wait_bounded(saddr(&s->mbar_load), 0);  // the copy must land before the CTA leaves
-  ok = tc_sync_or(!ok) == 0;
-  const uint32_t tm = s->tmem_slot, lb = (uint32_t)(t & ~31) << 16;
-  constexpr uint32_t i128 = kI128, i144 = kI144, i32 = kI32;
+  // everything so far needs nothing of the kernel in front; the weights do
+  grid_dependency_wait();
+  grid_dependency_launch();
+  if (tid == 0) {
+    const TcWeights* fw = &packed->fw;
+    constexpr uint32_t kW1 = sizeof(fw->w1), kW2 = sizeof(fw->w2), kRest = sizeof(TcWeights) - kW1 - kW2;
+    mbar_expect_tx(saddr(&s->mbar_load[0]), kW1 + kRest);
+    bulk_g2s(saddr(&s->wt.fw.w1), fw->w1, kW1, saddr(&s->mbar_load[0]));
+    bulk_g2s(saddr(&s->wt.fw.b1), fw->b1, kRest, saddr(&s->mbar_load[0]));
+    mbar_expect_tx(saddr(&s->mbar_load[1]), kW2);
+    bulk_g2s(saddr(&s->wt.fw.w2), fw->w2, kW2, saddr(&s->mbar_load[1]));
+    mbar_expect_tx(saddr(&s->mbar_load[2]), (uint32_t)sizeof(packed->w2t));
+    bulk_g2s(saddr(&s->wt.w2t), packed->w2t, (uint32_t)sizeof(packed->w2t), saddr(&s->mbar_load[2]));
+  }
+  const uint32_t tm = s->tmem_slot, lb = (uint32_t)(32 * rg) << 16;
   uint32_t phase = 0;
   // one commit, then every thread waits; false when any thread gave up
   auto commit_wait = [&]() -> bool {
-    if (t == 0) mma_commit(saddr(&s->mbar));
+    if (tid == 0) mma_commit(saddr(&s->mbar));
     const bool w = mbar_wait_bounded(saddr(&s->mbar), phase);
     phase ^= 1u;
-    const int bad = tc_sync_or(!w);
+    const int bad = __syncthreads_or(!w);
     tc_fence_after();
     return bad == 0;
   };
-  float gw3acc[4] = {0.f, 0.f, 0.f, 0.f}, gb3acc = 0.f, lossacc = 0.f;
+  // the copies must land before the CTA leaves, so each is waited for, twice if need be
+  auto load_wait = [&](int i) -> bool {
+    bool w = mbar_wait_bounded(saddr(&s->mbar_load[i]), 0);
+    if (!w) w = mbar_wait_bounded(saddr(&s->mbar_load[i]), 0);
+    return __syncthreads_or(!w) == 0;
+  };
+  bool ok = load_wait(0);
+  float gw3acc = 0.f, gb3acc = 0.f, lossacc = 0.f;
   uint32_t first = 1;
+  int waited = 1;  // weight copies waited for
   const TcWeights& W = s->wt.fw;
   for (uint64_t tile = blockIdx.x; ok && tile < tiles; tile += gridDim.x) {
-    const uint64_t row = tile * gxt::kRows + t;
-    const bool valid = row < n;
-    const uint64_t ex = valid ? (index ? index[row] : row) : 0;
-    // X = bf16(hist / processes), and X^T
-    uint32_t cnt[IN], tot = 0;
-#pragma unroll
-    for (int i = 0; i < IN; ++i) {
-      cnt[i] = valid ? hist[ex * IN + i] : 0u;
-      tot += cnt[i];
+    if (!first) {
+      fill_x(tile);
+      fence_async_smem();
+      __syncthreads();
     }
-    const float inv = tot ? 1.f / (float)tot : 0.f;
-    {
-      uint32_t q[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i) q[i] = pack_bf16x2((float)cnt[2 * i] * inv, (float)cnt[2 * i + 1] * inv);
-      *reinterpret_cast<uint4*>(s->x + core_offset(t, 0, 2)) = make_uint4(q[0], q[1], q[2], q[3]);
-      *reinterpret_cast<uint4*>(s->x + core_offset(t, 8, 2)) = make_uint4(q[4], q[5], q[6], q[7]);
-#pragma unroll
-      for (int i = 0; i < IN; ++i) st_bf16(s->xto, core_offset(i, t, 16), (float)cnt[i] * inv);
-    }
-    const float lab = valid ? label[ex] : 0.f;
-    fence_async_smem();
-    tc_sync();
-    if (t == 0) {
+    const bool valid = tile * kRows + t < n;
+    if (tid == 0) {
       tc_fence_after();
-      mma_bf16_i(tm + kColAcc, smem_desc(saddr(s->x), 128, 256), smem_desc(saddr(W.w1), 128, 256), i128, 0u);
+      mma_bf16_i(tm + kColAcc, smem_desc(saddr(s->x), 128, 128 * kGroupsX), smem_desc(saddr(W.w1), 128, 256), kI128, 0u);
     }
     if (!(ok = commit_wait())) break;
-    // H = bf16(relu(A1 + b1)) and H^T; the ReLU's mask of A1 kept for the backward pass
-    uint32_t mask1[4];
-#pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
+    // H = bf16(relu(A1 + b1)); the ReLU's mask of A1 kept for the backward pass
+    uint32_t mask1 = 0;
+    {
       float a[32];
       tmem_ld32(tm + lb + kColAcc + 32 * c, a);
-      uint32_t m = 0, q[16];
+      uint32_t q[16];
 #pragma unroll
       for (int e = 0; e < 32; ++e) {
         a[e] += W.b1[32 * c + e];
-        if (a[e] > 0.f) m |= 1u << e;
+        if (a[e] > 0.f) mask1 |= 1u << e;
         a[e] = fmaxf(a[e], 0.f);
       }
 #pragma unroll
       for (int e = 0; e < 16; ++e) q[e] = pack_bf16x2(a[2 * e], a[2 * e + 1]);
 #pragma unroll
       for (int g = 0; g < 4; ++g)
-        *reinterpret_cast<uint4*>(s->h + core_offset(t, 32 * c + 8 * g, 16)) =
+        *reinterpret_cast<uint4*>(s->h + core_offset(t, 32 * c + 8 * g, kGroupsH)) =
             make_uint4(q[4 * g], q[4 * g + 1], q[4 * g + 2], q[4 * g + 3]);
-#pragma unroll
-      for (int e = 0; e < 32; ++e) st_bf16(s->hto, core_offset(32 * c + e, t, 16), a[e]);
-      mask1[c] = m;
     }
     tc_fence_before();
     fence_async_smem();
-    tc_sync();
-    if (t == 0) {
+    if (first) {
+      ok = load_wait(1);
+      waited = 2;
+      if (!ok) break;
+    } else {
+      __syncthreads();
+    }
+    if (tid == 0) {
       tc_fence_after();
 #pragma unroll
       for (uint32_t kk = 0; kk < H / 16; ++kk)
-        mma_bf16_i(tm + kColAcc, smem_desc(saddr(s->h) + 256u * kk, 128, 2048),
-                   smem_desc(saddr(W.w2) + 256u * kk, 128, 2048), i128, kk > 0 ? 1u : 0u);
+        mma_bf16_i(tm + kColAcc, smem_desc(saddr(s->h) + 256u * kk, 128, 128 * kGroupsH),
+                   smem_desc(saddr(W.w2) + 256u * kk, 128, 2048), kI128, kk > 0 ? 1u : 0u);
     }
     if (!(ok = commit_wait())) break;
     // y, then dy, D2 = dy w3 o (A2 + b2 > 0) and the gw3 terms dy relu(A2 + b2)
-    float y = W.b3;
-#pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
-      float a[32];
-      tmem_ld32(tm + lb + kColAcc + 32 * c, a);
+    float a[32];
+    tmem_ld32(tm + lb + kColAcc + 32 * c, a);
 #pragma unroll
-      for (int e = 0; e < 32; ++e) y += W.w3[32 * c + e] * fmaxf(a[e] + W.b2[32 * c + e], 0.f);
+    for (int e = 0; e < 32; ++e) a[e] += W.b2[32 * c + e];
+    {
+      float w3[32];
+#pragma unroll
+      for (int e = 0; e < 32; ++e) w3[e] = W.w3[32 * c + e];
+      // the column groups of a row group in order: warp (rg, c) hands y on to (rg, c + 1)
+      float y = W.b3;
+      if (c > 0) {
+        pair_sync(1 + rg * 3 + c - 1);
+        y = s->y[t];
+      }
+#pragma unroll
+      for (int e = 0; e < 32; ++e) y += w3[e] * fmaxf(a[e], 0.f);
+      s->y[t] = y;
+      if (c < 3) pair_sync(1 + rg * 3 + c);
+      __syncthreads();
     }
-    const float dy = valid ? 2.f * (y - lab) * inv_n : 0.f;
-    if (valid) lossacc += (y - lab) * (y - lab) * inv_n;
-    gb3acc += dy;
-#pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
-      float a[32], v[32];
-      tmem_ld32(tm + lb + kColAcc + 32 * c, a);
+    {
+      const float y = s->y[t], lab = s->lab[t];
+      const float dy = valid ? 2.f * (y - lab) * inv_n : 0.f;
+      if (c == 0) {
+        if (valid) lossacc += (y - lab) * (y - lab) * inv_n;
+        gb3acc += dy;
+      }
+      float v[32];
       uint32_t q[16];
 #pragma unroll
       for (int e = 0; e < 32; ++e) {
-        const float z = a[e] + W.b2[32 * c + e];
+        const float z = a[e];
         v[e] = dy * fmaxf(z, 0.f);
         a[e] = z > 0.f ? dy * W.w3[32 * c + e] : 0.f;
       }
@@ -336,92 +437,108 @@ __global__ void __launch_bounds__(gxt::kRows, 1) grad_tc_kernel(const TcTrainWei
       for (int e = 0; e < 16; ++e) q[e] = pack_bf16x2(a[2 * e], a[2 * e + 1]);
 #pragma unroll
       for (int g = 0; g < 4; ++g)
-        *reinterpret_cast<uint4*>(s->d + core_offset(t, 32 * c + 8 * g, 16)) =
+        *reinterpret_cast<uint4*>(s->d + core_offset(t, 32 * c + 8 * g, kGroupsD)) =
             make_uint4(q[4 * g], q[4 * g + 1], q[4 * g + 2], q[4 * g + 3]);
+      tc_fence_before();
+      fence_async_smem();
+      if (first) {
+        ok = load_wait(2);
+        waited = 3;
+        if (!ok) break;
+      } else {
+        __syncthreads();
+      }
+      if (tid == 0) {
+        tc_fence_after();
 #pragma unroll
-      for (int e = 0; e < 32; ++e) st_bf16(s->dt, core_offset(32 * c + e, t, 16), a[e]);
-      gw3acc[c] += warp_column_sums(v);
+        for (uint32_t kk = 0; kk < H / 16; ++kk)
+          mma_bf16_i(tm + kColDH, smem_desc(saddr(s->d) + 256u * kk, 128, 2048),
+                     smem_desc(saddr(s->wt.w2t) + 256u * kk, 128, 2048), kI128, kk > 0 ? 1u : 0u);
+        mma_commit(saddr(&s->mbar));
+        // D2^T [H | 1]: K steps of 16 examples (two rows of core matrices); it runs behind DH's epilogue
+#pragma unroll
+        for (uint32_t kk = 0; kk < kRows / 16; ++kk)
+          mma_bf16_i(tm + kColGW2, smem_desc(saddr(s->d) + 2u * kk * 128 * kGroupsD, 128 * kGroupsD, 128),
+                     smem_desc(saddr(s->h) + 2u * kk * 128 * kGroupsH, 128 * kGroupsH, 128), kI144t,
+                     (first && kk == 0) ? 0u : 1u);
+      }
+      gw3acc += warp_column_sums(v);
     }
-    tc_fence_before();
-    fence_async_smem();
-    tc_sync();
-    if (t == 0) {
+    {
+      const bool w = mbar_wait_bounded(saddr(&s->mbar), phase);
+      phase ^= 1u;
       tc_fence_after();
-#pragma unroll
-      for (uint32_t kk = 0; kk < H / 16; ++kk)
-        mma_bf16_i(tm + kColDH, smem_desc(saddr(s->d) + 256u * kk, 128, 2048),
-                   smem_desc(saddr(s->wt.w2t) + 256u * kk, 128, 2048), i128, kk > 0 ? 1u : 0u);
-#pragma unroll
-      for (uint32_t kk = 0; kk < gxt::kRows / 16; ++kk)
-        mma_bf16_i(tm + kColGW2, smem_desc(saddr(s->dt) + 256u * kk, 128, 2048),
-                   smem_desc(saddr(s->hto) + 256u * kk, 128, 2048), i144, (first && kk == 0) ? 0u : 1u);
+      if (!(ok = __syncthreads_or(!w) == 0)) break;
     }
-    if (!(ok = commit_wait())) break;
-    // DA1 = DH o (A1 + b1 > 0), written transposed over H (free since layer 2 ran)
-#pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
-      float a[32];
+    // DA1 = DH o (A1 + b1 > 0)
+    {
       tmem_ld32(tm + lb + kColDH + 32 * c, a);
+      uint32_t q[16];
 #pragma unroll
-      for (int e = 0; e < 32; ++e)
-        st_bf16(s->h, core_offset(32 * c + e, t, 16), ((mask1[c] >> e) & 1u) ? a[e] : 0.f);
+      for (int e = 0; e < 32; ++e) a[e] = ((mask1 >> e) & 1u) ? a[e] : 0.f;
+#pragma unroll
+      for (int e = 0; e < 16; ++e) q[e] = pack_bf16x2(a[2 * e], a[2 * e + 1]);
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+        *reinterpret_cast<uint4*>(s->da + core_offset(t, 32 * c + 8 * g, kGroupsD)) =
+            make_uint4(q[4 * g], q[4 * g + 1], q[4 * g + 2], q[4 * g + 3]);
     }
     tc_fence_before();
     fence_async_smem();
-    tc_sync();
-    if (t == 0) {
+    __syncthreads();
+    if (tid == 0) {
       tc_fence_after();
 #pragma unroll
-      for (uint32_t kk = 0; kk < gxt::kRows / 16; ++kk)
-        mma_bf16_i(tm + kColGW1, smem_desc(saddr(s->h) + 256u * kk, 128, 2048),
-                   smem_desc(saddr(s->xto) + 256u * kk, 128, 2048), i32, (first && kk == 0) ? 0u : 1u);
+      for (uint32_t kk = 0; kk < kRows / 16; ++kk)
+        mma_bf16_i(tm + kColGW1, smem_desc(saddr(s->da) + 2u * kk * 128 * kGroupsD, 128 * kGroupsD, 128),
+                   smem_desc(saddr(s->x) + 2u * kk * 128 * kGroupsX, 128 * kGroupsX, 128), kI32t,
+                   (first && kk == 0) ? 0u : 1u);
     }
     if (!(ok = commit_wait())) break;
     first = 0;
   }
+  while (waited < 3) load_wait(waited++);  // after a wait that gave up
   if (ok) {
-    // thread t: row t of gW2 and gW1 (hidden unit t), gb2[t], gb1[t]
-    float* g = partial + (uint64_t)blockIdx.x * NPARAM;
-#pragma unroll 1
-    for (int c = 0; c < 4; ++c) {
-      float a[32];
-      tmem_ld32(tm + lb + kColGW2 + 32 * c, a);
+    // row t of gW2 and gW1 (hidden unit t), gb2[t], gb1[t]
+    float* g = partial + (uint64_t)blockIdx.x * kPartial;
+    float a[32];
+    tmem_ld32(tm + lb + kColGW2 + 32 * c, a);
 #pragma unroll
-      for (int e = 0; e < 32; ++e) g[OFF_W2 + t * H + 32 * c + e] = a[e];
-    }
-    {
-      float a[32];
-      tmem_ld32(tm + lb + kColGW2 + H, a);  // columns 384-415: gb2 (ones rows), then gW1
-      g[OFF_B2 + t] = a[0];
-      tmem_ld32(tm + lb + kColGW1, a);      // columns 400-431: gW1, then gb1 (ones rows)
+    for (int e = 0; e < 32; ++e) g[OFF_W2 + (32 * c + e) * H + t] = a[e];
+    if (c == 0) {
+      tmem_ld32(tm + lb + kColGW1, a);  // columns 400-431: gW1, then gb1 (ones columns)
 #pragma unroll
-      for (int i = 0; i < IN; ++i) g[OFF_W1 + t * IN + i] = a[i];
+      for (int i = 0; i < IN; ++i) g[OFF_W1 + i * H + t] = a[i];
       g[OFF_B1 + t] = a[IN];
+    } else if (c == 1) {
+      tmem_ld32(tm + lb + kColGW2 + H, a);  // columns 384-415: gb2 (ones columns), then gW1
+      g[OFF_B2 + t] = a[0];
     }
-    // gw3 and gb3, loss: the warps' sums in warp order
+    // gw3 and gb3, loss: the row groups' sums in order
+    s->red[rg][32 * c + lane] = gw3acc;
+    if (c == 0) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) s->red[wid][32 * c + lane] = gw3acc[c];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      lossacc += __shfl_xor_sync(0xFFFFFFFFu, lossacc, o);
-      gb3acc += __shfl_xor_sync(0xFFFFFFFFu, gb3acc, o);
+      for (int o = 16; o > 0; o >>= 1) {
+        lossacc += __shfl_xor_sync(0xFFFFFFFFu, lossacc, o);
+        gb3acc += __shfl_xor_sync(0xFFFFFFFFu, gb3acc, o);
+      }
+      if (lane == 0) {
+        s->redl[rg][0] = lossacc;
+        s->redl[rg][1] = gb3acc;
+      }
     }
-    if (lane == 0) {
-      s->redl[wid][0] = lossacc;
-      s->redl[wid][1] = gb3acc;
-    }
-    tc_sync();
-    g[OFF_W3 + t] = ((s->red[0][t] + s->red[1][t]) + s->red[2][t]) + s->red[3][t];
-    if (t == 0) {
+    __syncthreads();
+    if (c == 0) g[OFF_W3 + t] = ((s->red[0][t] + s->red[1][t]) + s->red[2][t]) + s->red[3][t];
+    if (tid == 0) {
       g[OFF_B3] = ((s->redl[0][1] + s->redl[1][1]) + s->redl[2][1]) + s->redl[3][1];
       partial_loss[blockIdx.x] = ((s->redl[0][0] + s->redl[1][0]) + s->redl[2][0]) + s->redl[3][0];
     }
-  } else if (t == 0) {
+  } else if (tid == 0) {
     atomicOr(&g_train_error, 1u);
   }
   tc_fence_before();
-  tc_sync();
-  if (t < 32) {
+  __syncthreads();
+  if (wid == 0) {
     tc_fence_after();
     tmem_dealloc(tm, kTrainCols);
   }
@@ -440,29 +557,54 @@ __global__ void wait_selftest_kernel(uint32_t limit) {
   if (threadIdx.x == 0) g_wait_gave_up = done ? 0u : 1u;
 }
 
-// Adam (Kingma & Ba 2015) on the FP32 master parameters; clears the gradient.
-__global__ void adam_kernel(float* __restrict__ p, float* __restrict__ m, float* __restrict__ v,
-                            float* __restrict__ g, float lr, float b1t, float b2t) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= NPARAM) return;
-  const float gi = g[i];
-  const float mi = 0.9f * m[i] + 0.1f * gi;
-  const float vi = 0.999f * v[i] + 0.001f * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  p[i] -= lr * (mi / (1.f - b1t)) / (sqrtf(vi / (1.f - b2t)) + 1e-8f);
-  g[i] = 0.f;
-}
-
-// Mini-batch indices: batch element j of step s is example mix64(seed + s * B + j) mod n.
-__global__ void sample_kernel(uint64_t* __restrict__ idx, uint32_t batch, uint64_t n, uint64_t seed,
-                              uint64_t step) {
-  const uint32_t j = blockIdx.x * blockDim.x + threadIdx.x;
-  if (j >= batch) return;
-  uint64_t z = seed + step * batch + j + 0x9E3779B97F4A7C15ull;
-  z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-  z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-  idx[j] = (z ^ (z >> 31)) % n;
+// One Adam step (Kingma & Ba 2015) on the FP32 master parameters: a thread per
+// parameter sums its partial gradients, updates it and writes it into the packed
+// weights that the next step's gradient is taken at.
+__global__ void __launch_bounds__(256) update_kernel(const float* __restrict__ partial,
+                                                     const float* __restrict__ partial_loss, int ctas,
+                                                     float* p, float* m, float* v, float lr, float b1t, float b2t,
+                                                     TcTrainWeights* __restrict__ packed, float* __restrict__ loss) {
+  const int q = blockIdx.x * blockDim.x + threadIdx.x;  // moments lie as the partial gradients do
+  const int i = partial_param(q < NPARAM ? q : 0);
+  // m, v and p were last written by the step before, which the gradient in front
+  // has waited for: only the partial gradients need the wait
+  float m0 = 0.f, v0 = 0.f, p0 = 0.f;
+  if (q < NPARAM) {
+    m0 = m[q];
+    v0 = v[q];
+    p0 = p[i];
+  }
+  grid_dependency_wait();
+  grid_dependency_launch();
+  if (q == 0) {
+    float l = 0.f;
+    for (int c = 0; c < ctas; ++c) l += partial_loss[c];
+    *loss = l;
+  }
+  if (q >= NPARAM) return;
+  const float gi = partial_sum(partial, ctas, q);
+  const float mi = 0.9f * m0 + 0.1f * gi;
+  const float vi = 0.999f * v0 + 0.001f * gi * gi;
+  m[q] = mi;
+  v[q] = vi;
+  const float x = p0 - lr * (mi / (1.f - b1t)) / (sqrtf(vi / (1.f - b2t)) + 1e-8f);
+  p[i] = x;
+  gxt::TcWeights& w = packed->fw;
+  if (i < OFF_B1) {
+    st_bf16(w.w1, gxt::core_offset(i / IN, i % IN, 2), x);
+  } else if (i < OFF_W2) {
+    w.b1[i - OFF_B1] = x;
+  } else if (i < OFF_B2) {
+    const int k = (i - OFF_W2) / H, j = (i - OFF_W2) % H;
+    st_bf16(w.w2, gxt::core_offset(k, j, 16), x);
+    st_bf16(packed->w2t, gxt::core_offset(j, k, 16), x);
+  } else if (i < OFF_W3) {
+    w.b2[i - OFF_B2] = x;
+  } else if (i < OFF_B3) {
+    w.w3[i - OFF_W3] = __bfloat162float(__float2bfloat16_rn(x));
+  } else {
+    w.b3 = x;
+  }
 }
 
 }  // namespace gxm
@@ -523,18 +665,24 @@ gx_status gx_mlp_init(float* params, uint64_t seed, void* stream) {
 static std::mutex g_forward_mutex;
 static std::mutex g_train_mutex;
 
-// The gradient at params over n examples (slot j takes example index[j] when
-// index is given) on the tensor cores: pack the weights, then one CTA per tile
-// of 128 examples, at most GX_MLP_GRAD_CTAS CTAs, each writing its partial
-// gradient; the caller sums them (reduce_kernel).  Returns the CTA count.
-int launch_grad_tc(const float* params, const uint8_t* hist, const float* label, uint64_t n, const uint64_t* index,
-                   float* partial, float* partial_loss, gxm::TcTrainWeights* packed, cudaStream_t st) {
+// The gradient over n examples (drawn from a training set when `draw` is given) at
+// the packed weights: one CTA per tile of 128 examples, at most GX_MLP_GRAD_CTAS
+// CTAs, each writing its partial gradient.
+cudaError_t launch_grad_tc(const uint8_t* hist, const float* label, uint64_t n, gxm::Draw draw, float* partial,
+                           float* partial_loss, const gxm::TcTrainWeights* packed, bool overlap, cudaStream_t st) {
   const uint64_t tiles = (n + gxt::kRows - 1) / gxt::kRows;
-  const int grid = (int)std::min<uint64_t>(tiles, gxm::kGradCtas);
-  gxm::train_pack_kernel<<<gxm::kTrainPackBlocks, 256, 0, st>>>(params, packed);
-  gxm::grad_tc_kernel<<<grid, gxt::kRows, gxm::kTrainSmemBytes, st>>>(packed, hist, label, n, index,
-                                                                       1.0f / (float)n, partial, partial_loss);
-  return grid;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)std::min<uint64_t>(tiles, gxm::kGradCtas));
+  cfg.blockDim = dim3(gxm::kGradThreads);
+  cfg.dynamicSmemBytes = gxm::kTrainSmemBytes;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = overlap ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, gxm::grad_tc_kernel, packed, hist, label, n, draw, 1.0f / (float)n, partial,
+                            partial_loss);
 }
 
 gx_status gx_mlp_forward(const float* params, const uint8_t* hist, uint64_t n, float* out, void* stream) {
@@ -592,17 +740,17 @@ gx_status gx_mlp_grad(const float* params, const uint8_t* hist, const float* lab
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   const int grid = (int)std::min<uint64_t>((n + gxt::kRows - 1) / gxt::kRows, gxm::kGradCtas);
   float* scratch = nullptr;  // one partial gradient and loss per CTA
-  GM_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&scratch), sizeof(float) * (uint64_t)grid * (gxm::NPARAM + 1), st));
+  GM_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&scratch), sizeof(float) * (uint64_t)grid * (gxm::kPartial + 1), st));
   const unsigned int zero = 0;
   GM_CUDA(cudaMemcpyToSymbolAsync(gxm::g_train_error, &zero, sizeof(zero), 0, cudaMemcpyHostToDevice, st));
   std::lock_guard<std::mutex> lock(g_train_mutex);
   gxm::TcTrainWeights* packed = nullptr;
   GM_CUDA(cudaGetSymbolAddress(reinterpret_cast<void**>(&packed), gxm::g_train_packed));
-  launch_grad_tc(params, hist, label, n, nullptr, scratch, scratch + (uint64_t)grid * gxm::NPARAM, packed, st);
-  cudaError_t e = cudaGetLastError();
+  gxm::train_pack_kernel<<<gxm::kTrainPackBlocks, 256, 0, st>>>(params, packed);
+  float* scratch_loss = scratch + (uint64_t)grid * gxm::kPartial;
+  cudaError_t e = launch_grad_tc(hist, label, n, gxm::Draw{}, scratch, scratch_loss, packed, false, st);
   if (e == cudaSuccess) {
-    gxm::reduce_kernel<<<(gxm::NPARAM + 255) / 256, 256, 0, st>>>(scratch, scratch + (uint64_t)grid * gxm::NPARAM,
-                                                                  grid, grad, loss);
+    gxm::reduce_kernel<<<(gxm::NPARAM + 255) / 256, 256, 0, st>>>(scratch, scratch_loss, grid, grad, loss);
     e = cudaGetLastError();
   }
   cudaFreeAsync(scratch, st);
@@ -622,30 +770,39 @@ gx_status gx_mlp_train(float* params, float* state, const uint8_t* hist, const f
   gx_status s = set_smem();
   if (s != GX_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  // state: m | v | g | partial gradients (GX_MLP_GRAD_CTAS x NPARAM) | partial
-  // losses (GX_MLP_GRAD_CTAS) | indices (batch, 8-byte aligned)
+  // state: m | v | partial losses | partial gradients (up to GX_MLP_GRAD_CTAS of both)
   float* m = state;
   float* v = state + gxm::NPARAM;
-  float* g = state + 2 * gxm::NPARAM;
-  float* partial = state + 3 * gxm::NPARAM;
-  float* partial_loss = partial + (uint64_t)gxm::kGradCtas * gxm::NPARAM;
-  uint64_t* idx = reinterpret_cast<uint64_t*>(partial_loss + gxm::kGradCtas + 1);
-  idx = reinterpret_cast<uint64_t*>((reinterpret_cast<uintptr_t>(idx) + 7) & ~uintptr_t(7));
-  GM_CUDA(cudaMemsetAsync(state, 0, sizeof(float) * 3 * gxm::NPARAM, st));
+  float* partial_loss = state + 2 * gxm::NPARAM;
+  float* partial = partial_loss + gxm::kGradCtas;
+  GM_CUDA(cudaMemsetAsync(state, 0, sizeof(float) * 2 * gxm::NPARAM, st));
   GM_CUDA(cudaMemsetAsync(loss, 0, sizeof(float) * steps, st));
   const unsigned int zero = 0;
   GM_CUDA(cudaMemcpyToSymbolAsync(gxm::g_train_error, &zero, sizeof(zero), 0, cudaMemcpyHostToDevice, st));
   std::lock_guard<std::mutex> lock(g_train_mutex);
   gxm::TcTrainWeights* packed = nullptr;
   GM_CUDA(cudaGetSymbolAddress(reinterpret_cast<void**>(&packed), gxm::g_train_packed));
+  gxm::train_pack_kernel<<<gxm::kTrainPackBlocks, 256, 0, st>>>(params, packed);
+  const int ctas = (int)std::min<uint64_t>(((uint64_t)batch + gxt::kRows - 1) / gxt::kRows, gxm::kGradCtas);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((gxm::NPARAM + 255) / 256);
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
   double b1t = 1.0, b2t = 1.0;
   for (uint32_t t = 0; t < steps; ++t) {
     b1t *= 0.9;
     b2t *= 0.999;
-    gxm::sample_kernel<<<(batch + 255) / 256, 256, 0, st>>>(idx, batch, n, seed, t);
-    const int grid = launch_grad_tc(params, hist, label, batch, idx, partial, partial_loss, packed, st);
-    gxm::reduce_kernel<<<(gxm::NPARAM + 255) / 256, 256, 0, st>>>(partial, partial_loss, grid, g, loss + t);
-    gxm::adam_kernel<<<(gxm::NPARAM + 255) / 256, 256, 0, st>>>(params, m, v, g, lr, (float)b1t, (float)b2t);
+    // both launches of a step start before the kernel in front of them has ended and wait for it
+    // where they need its results (the first step's gradient follows the packing in full order)
+    GM_CUDA(launch_grad_tc(hist, label, batch, gxm::Draw{n, seed + (uint64_t)t * batch, 1}, partial, partial_loss,
+                           packed, t > 0, st));
+    GM_CUDA(cudaLaunchKernelEx(&cfg, gxm::update_kernel, (const float*)partial, (const float*)partial_loss, ctas, params,
+                               m, v, lr, (float)b1t, (float)b2t, packed, loss + t));
   }
   GM_CUDA(cudaGetLastError());
   unsigned int err = 0;

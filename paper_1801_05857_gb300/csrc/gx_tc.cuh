@@ -43,10 +43,11 @@ constexpr uint32_t kSpinLimit = 1u << 22;
 static_assert(kIn == 16 && kHid == 128, "tile shapes assume a 16-128-128-1 network");
 
 // Instruction descriptor of tcgen05.mma .kind::f16: FP32 accumulator (bits
-// 4-5 = 1), BF16 A and B (bits 7-9 = 1, bits 10-12 = 1), both K-major
-// (bits 15, 16 = 0), N >> 3 in bits 17-22, M >> 4 in bits 24-28.
-constexpr uint32_t idesc_bf16_f32(uint32_t m, uint32_t n) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((n >> 3) << 17) | ((m >> 4) << 24);
+// 4-5 = 1), BF16 A and B (bits 7-9 = 1, bits 10-12 = 1), each K-major (bits 15,
+// 16 = 0) or MN-major (1: the operand's transpose lies in memory), N >> 3 in
+// bits 17-22, M >> 4 in bits 24-28.
+constexpr uint32_t idesc_bf16_f32(uint32_t m, uint32_t n, uint32_t a_mn = 0, uint32_t b_mn = 0) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (a_mn << 15) | (b_mn << 16) | ((n >> 3) << 17) | ((m >> 4) << 24);
 }
 constexpr uint32_t kIdesc = idesc_bf16_f32(128, 128);
 

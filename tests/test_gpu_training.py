@@ -1,0 +1,68 @@
+"""The training kernels at the sizes where they can go wrong: which examples a step draws, batches
+below, at and above a tile and above one tile per CTA, and histograms at odd addresses."""
+import numpy as np
+import pytest
+
+from oracle import mlp as omlp
+from paper_1801_05857_gb300 import gx
+
+pytestmark = pytest.mark.gpu
+
+
+def _data(n, seed):
+    import torch
+    rng = np.random.default_rng(seed)
+    hist = rng.multinomial(9, np.ones(16) / 16, size=n).astype(np.uint8)
+    label = rng.random(n).astype(np.float32)
+    p = torch.empty(gx.MLP_PARAMS, dtype=torch.float32, device="cuda")
+    gx.mlp_init(p, seed)
+    return hist, label, p
+
+
+def _drawn(seed, step, batch, n):
+    """Example numbers of a step: mix64(seed + step * batch + j) mod n (splitmix64)."""
+    with np.errstate(over="ignore"):
+        z = np.arange(batch, dtype=np.uint64) + np.uint64(seed + step * batch) + np.uint64(0x9E3779B97F4A7C15)
+        z = (z ^ (z >> np.uint64(30))) * np.uint64(0xBF58476D1CE4E5B9)
+        z = (z ^ (z >> np.uint64(27))) * np.uint64(0x94D049BB133111EB)
+        return ((z ^ (z >> np.uint64(31))) % np.uint64(n)).astype(np.int64)
+
+
+@pytest.mark.parametrize("batch", [1, 127, 128, 129, 1000, 256 * 128 + 5])
+def test_first_steps_losses_are_those_of_the_drawn_examples(cuda, batch):
+    """Step 0's loss at the initial weights, and step 1's at weights one Adam step on (its update
+    is lr a parameter at most, so the loss moves little for a small lr)."""
+    import torch
+    hist, label, p = _data(5000, batch)
+    p0 = p.cpu().numpy()
+    losses = gx.mlp_train(p, torch.from_numpy(hist).cuda(), torch.from_numpy(label).cuda(), batch, 2, 1e-7, 77)
+    for step in range(2):
+        idx = _drawn(77, step, batch, len(hist))
+        want, _ = omlp.loss_and_grad(p0, hist[idx], label[idx])
+        assert abs(float(losses[step]) - want) <= 1e-3 * want + 1e-6
+    moved = np.abs(p.cpu().numpy() - p0)
+    assert 0 < moved.max() <= 2.1e-7 + 2 ** -24  # at most lr a step, and FP32's rounding of parameters below 1
+
+
+def test_histograms_at_odd_addresses(cuda):
+    import torch
+    hist, label, p = _data(300, 4)
+    flat = torch.zeros(300 * 16 + 1, dtype=torch.uint8, device="cuda")
+    flat[1:] = torch.from_numpy(hist.reshape(-1)).cuda()
+    lab = torch.from_numpy(label).cuda()
+    odd = flat[1:].view(300, 16)
+    assert odd.data_ptr() % 16 == 1
+    g0, l0 = gx.mlp_grad(p, torch.from_numpy(hist).cuda(), lab)
+    g1, l1 = gx.mlp_grad(p, odd, lab)
+    assert torch.equal(g0, g1) and torch.equal(l0, l1)
+    assert torch.equal(gx.mlp_forward(p, odd), gx.mlp_forward(p, torch.from_numpy(hist).cuda()))
+
+
+def test_training_is_reproducible(cuda):
+    import torch
+    hist, label, p = _data(3000, 9)
+    h, lab = torch.from_numpy(hist).cuda(), torch.from_numpy(label).cuda()
+    a, b = p.clone(), p.clone()
+    la, lb = gx.mlp_train(a, h, lab, 700, 60, 1e-3, 5), gx.mlp_train(b, h, lab, 700, 60, 1e-3, 5)
+    assert torch.equal(a, b) and torch.equal(la, lb)
+    assert float(la[-10:].mean()) < float(la[:10].mean())
