@@ -173,7 +173,7 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
 __device__ __forceinline__ float feature_scale(const uint32_t (&hw)[4]) {
   uint32_t n = 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) n += (hw[i] & 0xFFu) + ((hw[i] >> 8) & 0xFFu) + ((hw[i] >> 16) & 0xFFu) + (hw[i] >> 24);
+  for (int i = 0; i < 4; ++i) n = __dp4a(hw[i], 0x01010101u, n);
   return n ? 1.0f / (float)n : 0.f;
 }
 
@@ -186,8 +186,8 @@ __host__ __device__ constexpr uint32_t core_offset(uint32_t row, uint32_t k, uin
 // The weights of the guide network as a scoring CTA holds them in shared
 // memory: W1 and W2 as BF16 B operands in the core-matrix layout, the FP32
 // biases, w3 rounded to BF16 (kept as FP32) and b3.  One copy per search is
-// packed in global memory by tc_pack_kernel; every CTA then fetches it with a
-// single bulk copy.
+// packed in global memory (tc_pack_kernel); every CTA then fetches it with bulk
+// copies.
 struct __align__(16) TcWeights {
   uint8_t w1[kHid * kIn * 2];     // B of layer 1 (W1 as N x K), K groups: 2
   uint8_t w2[kHid * kHid * 2];    // B of layer 2 (W2 as N x K), K groups: 16
@@ -408,6 +408,259 @@ __device__ __forceinline__ bool tc_score_tile(TcScorer& sc, const uint32_t (&hw)
   tc_fence_before();
   tc_sync();
   return true;
+}
+
+// ---- Scoring many tiles: four at a time on one CTA per SM.
+//
+// For many states in one call (gx_mlp_forward); the guided search's few hundred
+// tiles an iteration, each on its own CTA, measured the same time this way.
+// What such a call's time goes to is instructions and shared-memory wavefronts of
+// the epilogues, not products or bytes: a value that is the same in every lane
+// costs four wavefronts per 16 bytes when it is read from shared memory, and
+// reading b1, b2 and w3 that way took 79 % of the shared-memory pipe and all of the
+// time (4,000,037 examples: 318 us in the kernel, with one tile or four tiles
+// per CTA alike).  So
+//   * layer 2's bias comes out of the product: one more MMA step, of a block of
+//     ones against the bias split into three BF16 parts (24 bits: the split is
+//     exact).  Layer 1's is added in FP32: H is rounded to BF16 there, and the
+//     tensor core's own order of additions would round some of it the other way;
+//   * two columns are multiplied and added per instruction (f32x2);
+//   * a tile belongs to eight warps -- warp w of a tile owns rows 32 (w & 3).. (its
+//     TMEM lanes) and 64 of the 128 columns -- and four tiles, as many as 512 TMEM
+//     columns hold, share one copy of the weights;
+//   * a tile's next X is fetched a tile ahead and written while its second product
+//     runs, 8 of its 16 columns by each half: two barriers a tile.
+// The two halves of a score's sum are added last.
+
+// Layer 2's bias as the B operand of one K = 16 step: row k is b2[k]'s three parts
+// and zeros.
+struct __align__(16) ScoreWeights {
+  TcWeights w;
+  uint8_t b2m[kHid * kIn * 2];
+};
+static_assert(sizeof(ScoreWeights) % 16 == 0, "bulk copies move multiples of 16 bytes");
+
+constexpr int kScorePackItems = kTcPackItems + kHid;
+constexpr int kScorePackBlocks = (kScorePackItems + 255) / 256;
+// Item `item` of kScorePackItems of the packed weights for the FP32 parameters p.
+__device__ __forceinline__ void score_pack_item(const float* __restrict__ p, ScoreWeights* __restrict__ out, int item) {
+  if (item < kTcPackItems) {
+    tc_pack_item(p, &out->w, item);
+    return;
+  }
+  const int k = item - kTcPackItems;
+  const float b = p[kHid * kIn + kHid + kHid * kHid + k];
+  const float hi = __bfloat162float(__float2bfloat16_rn(b));
+  const float r1 = isfinite(b) ? b - hi : 0.f;
+  const float mid = __bfloat162float(__float2bfloat16_rn(r1));
+  *reinterpret_cast<uint4*>(out->b2m + core_offset(k, 0, 2)) = make_uint4(pack_bf16x2(hi, mid), pack_bf16x2(r1 - mid, 0.f), 0u, 0u);
+  *reinterpret_cast<uint4*>(out->b2m + core_offset(k, 8, 2)) = make_uint4(0u, 0u, 0u, 0u);
+}
+
+constexpr int kScoreSlots = 4, kScoreSlotThreads = 256, kScoreThreads = kScoreSlots * kScoreSlotThreads;
+
+struct __align__(1024) ScoreSmem {
+  uint8_t x[kScoreSlots][kRows * kIn * 2];   // A of layer 1, K groups: 2
+  uint8_t h[kScoreSlots][kRows * kHid * 2];  // A of layer 2, K groups: 16
+  uint8_t ones[kRows * kIn * 2];             // A of the bias step: three ones a row, K groups: 2
+  ScoreWeights wt;
+  float part[kScoreSlots][kRows];            // the upper columns' part of each score
+  uint32_t tmem_slot;
+  unsigned long long mbar[kScoreSlots], mbar_load;
+};
+constexpr size_t kScoreSmemBytes = sizeof(ScoreSmem) + 1024;  // + alignment slack
+static_assert(kScoreSmemBytes <= 232448, "the scoring CTA must fit the SM's shared memory");
+
+__device__ __forceinline__ unsigned long long f32x2_add(unsigned long long a, unsigned long long b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ unsigned long long f32x2_fma(unsigned long long a, unsigned long long b,
+                                                        unsigned long long c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ unsigned long long f32x2(float lo, float hi) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ float2 f32x2_parts(unsigned long long x) {
+  float2 r;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(x));
+  return r;
+}
+
+// Columns 64 HALF.. of H's row t: bf16(relu(A1 + b1)) (rounded first; relu of a pair
+// is then one instruction, and the same result).  b1(k): b1[k] and b1[k + 1].
+template <int HALF, class B1>
+__device__ __forceinline__ void score_hidden(uint8_t* h, uint32_t lb, int t, B1 b1) {
+#pragma unroll
+  for (int c0 = 64 * HALF; c0 < 64 * HALF + 64; c0 += 32) {
+    float a[32];
+    tmem_ld32(lb + c0, a);
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      uint32_t q[4];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const int k = 8 * g + 2 * e;
+        const float2 u = f32x2_parts(f32x2_add(f32x2(a[k], a[k + 1]), b1(c0 + k)));
+        q[e] = pack_bf16x2(u.x, u.y);
+        asm("max.bf16x2 %0, %0, %1;" : "+r"(q[e]) : "r"(0u));
+      }
+      *reinterpret_cast<uint4*>(h + core_offset(t, (uint32_t)(c0 + 8 * g), 16)) = make_uint4(q[0], q[1], q[2], q[3]);
+    }
+  }
+}
+
+// The part of w3 . relu(A2) of columns 64 HALF.., even and odd ones apart.  w3(k):
+// w3[k] and w3[k + 1].
+template <int HALF, class W3>
+__device__ __forceinline__ float score_sum(uint32_t lb, W3 w3) {
+  unsigned long long y = 0;
+#pragma unroll
+  for (int c0 = 64 * HALF; c0 < 64 * HALF + 64; c0 += 32) {
+    float a[32];
+    tmem_ld32(lb + c0, a);
+#pragma unroll
+    for (int e = 0; e < 32; e += 2)
+      y = f32x2_fma(w3(c0 + e), f32x2(fmaxf(a[e], 0.f), fmaxf(a[e + 1], 0.f)), y);
+  }
+  const float2 p = f32x2_parts(y);
+  return p.x + p.y;
+}
+
+// Scores n states, 128 per tile, on a grid of at most one CTA per tile (kScoreThreads
+// threads, kScoreSmemBytes of dynamic shared memory).
+//   load(row, hw)   the histogram of state row < n, 4 counts per word
+//   store(row, y)   its score (called by half of the threads)
+//   par(w)          the parameters that are the same in every lane, as an object with
+//                   b1(k) and w3(k) (entries k and k + 1) and b3(), given the staged
+//                   weights
+// False, in the threads that gave up, after a wait that timed out.
+template <class Load, class Store, class Par>
+__device__ __forceinline__ bool score_tiles(void* dyn, const ScoreWeights* __restrict__ packed, uint64_t n, Load load,
+                                            Store store, Par par_of) {
+  ScoreSmem* s = reinterpret_cast<ScoreSmem*>((reinterpret_cast<uintptr_t>(dyn) + 1023) & ~uintptr_t(1023));
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  const int slot = wid >> 3, rg = wid & 3, half = (wid >> 2) & 1;
+  const int t = 32 * rg + lane;  // state of the tile
+  const uint64_t tiles = (n + kRows - 1) / kRows;
+  // tile i goes to CTA i % grid first, so that few tiles spread over the SMs
+  uint64_t tile = blockIdx.x + (uint64_t)slot * gridDim.x;
+  const uint64_t step = (uint64_t)gridDim.x * kScoreSlots;
+  if (tid == 0) {
+    for (int i = 0; i < kScoreSlots; ++i) mbar_init(saddr(&s->mbar[i]), 1);
+    mbar_init(saddr(&s->mbar_load), 1);
+    mbar_expect_tx(saddr(&s->mbar_load), (uint32_t)sizeof(ScoreWeights));
+    bulk_g2s(saddr(&s->wt), packed, (uint32_t)sizeof(ScoreWeights), saddr(&s->mbar_load));
+  }
+  if (wid == 0) {
+    __syncwarp();
+    tmem_alloc(saddr(&s->tmem_slot), kScoreSlots * kHid);
+    tmem_relinquish();
+  }
+  if (slot == 1 && half == 0) {
+    *reinterpret_cast<uint4*>(s->ones + core_offset(t, 0, 2)) = make_uint4(0x3F803F80u, 0x00003F80u, 0u, 0u);
+    *reinterpret_cast<uint4*>(s->ones + core_offset(t, 8, 2)) = make_uint4(0u, 0u, 0u, 0u);
+    fence_async_smem();
+  }
+  uint32_t hw[4];  // the next tile's row t
+  auto fetch = [&](uint64_t tl) {
+    hw[0] = hw[1] = hw[2] = hw[3] = 0;
+    if (tl * kRows + t < n) load(tl * kRows + t, hw);
+  };
+  auto write_x = [&] {
+    const float inv = feature_scale(hw);
+    const uint32_t w0 = half == 0 ? hw[0] : hw[2], w1 = half == 0 ? hw[1] : hw[3];
+    uint32_t q[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint32_t w = i < 2 ? w0 : w1, sh = (i & 1) * 16;
+      q[i] = pack_bf16x2((float)((w >> sh) & 0xFFu) * inv, (float)((w >> (sh + 8)) & 0xFFu) * inv);
+    }
+    *reinterpret_cast<uint4*>(s->x[slot] + core_offset(t, 8 * half, 2)) = make_uint4(q[0], q[1], q[2], q[3]);
+    fence_async_smem();
+  };
+  fetch(tile);
+  write_x();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  bool loaded = mbar_wait_bounded(saddr(&s->mbar_load), 0);
+  if (!loaded) loaded = mbar_wait_bounded(saddr(&s->mbar_load), 0);  // the copy must land before the CTA leaves
+  const bool ok = __syncthreads_or(!loaded) == 0;
+  const uint32_t acc = s->tmem_slot + (uint32_t)slot * kHid, lb = acc + ((uint32_t)(32 * rg) << 16);
+  const uint32_t bar = saddr(&s->mbar[slot]);
+  const bool issuer = lane == 0 && (wid & 7) == 0;
+  uint32_t phase = 0;
+  bool gave_up = !ok;
+  auto wait = [&] {
+    if (!mbar_wait_bounded(bar, phase)) gave_up = true;
+    phase ^= 1u;
+    tc_fence_after();
+  };
+  // the tile's threads meet; true in all of them when one gave up waiting
+  auto slot_sync = [&]() -> bool {
+    int r;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t"
+        "setp.ne.b32 p, %1, 0;\n\t"
+        "bar.red.or.pred q, %2, %3, p;\n\t"
+        "selp.b32 %0, 1, 0, q;\n\t}"
+        : "=r"(r)
+        : "r"((int)gave_up), "r"(1 + slot), "n"(kScoreSlotThreads)
+        : "memory");
+    return r != 0;
+  };
+  const uint32_t ones = saddr(s->ones);
+  auto layer1 = [&] {
+    tc_fence_after();
+    mma_bf16(acc, smem_desc(saddr(s->x[slot]), 128, 256), smem_desc(saddr(s->wt.w.w1), 128, 256), 0u);
+    mma_commit(bar);
+  };
+  if (ok && tile < tiles && issuer) layer1();
+  const auto par = par_of(s->wt.w);
+  while (ok && tile < tiles) {
+    const uint64_t next = tile + step;
+    fetch(next);
+    wait();
+    if (half == 0) score_hidden<0>(s->h[slot], lb, t, [&](int k) { return par.b1(k); });
+    else score_hidden<1>(s->h[slot], lb, t, [&](int k) { return par.b1(k); });
+    tc_fence_before();
+    fence_async_smem();
+    if (slot_sync()) break;
+    if (issuer) {
+      tc_fence_after();
+      const uint32_t ha = saddr(s->h[slot]), wa = saddr(s->wt.w.w2);
+      mma_bf16(acc, smem_desc(ones, 128, 256), smem_desc(saddr(s->wt.b2m), 128, 256), 0u);
+#pragma unroll
+      for (uint32_t kk = 0; kk < kHid / 16; ++kk)
+        mma_bf16(acc, smem_desc(ha + 256u * kk, 128, 2048), smem_desc(wa + 256u * kk, 128, 2048), 1u);
+      mma_commit(bar);
+    }
+    if (next < tiles) write_x();
+    wait();
+    const float y = half == 0 ? score_sum<0>(lb, [&](int k) { return par.w3(k); })
+                              : score_sum<1>(lb, [&](int k) { return par.w3(k); });
+    if (half == 1) s->part[slot][t] = y;
+    tc_fence_before();
+    if (slot_sync()) break;
+    if (issuer && next < tiles) layer1();
+    const uint64_t row = tile * kRows + t;
+    if (half == 0 && row < n) store(row, (y + s->part[slot][t]) + par.b3());
+    tile = next;
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (wid == 0) {
+    tc_fence_after();
+    tmem_dealloc(s->tmem_slot, kScoreSlots * kHid);
+  }
+  return !gave_up;
 }
 
 }  // namespace gxt
