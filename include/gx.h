@@ -172,9 +172,9 @@ typedef struct gx_explore_opts {
                                     state cache of Fig. 2): 2^n entries per warp in shared
                                     memory (2^(n-1) for 4-word vectors, the same bytes), a hit
                                     skips find-or-put.  0 = off, 1..12 = 2^n, 0xFFFFFFFF =
-                                    automatic (gx_default_opts): 2^9 unless the GPU-wide
+                                    automatic (gx_default_opts): 2^7 unless the GPU-wide
                                     cache below is in use (together they measured slower);
-                                    2^6 for 4-word vectors, whose CTAs then still fit 5 per SM */
+                                    2^6 for 4-word vectors with region passes */
   float guided_scale;            /* GX_DL_GUIDED: score at which a state falls in the last
                                     bin (scores are predicted distances / max_dist); 0 = 1.0 */
   uint32_t watch;                /* 1 = safety check (Sec. 3: the negation of a safety property
@@ -298,7 +298,9 @@ typedef struct gx_stats_t {
   uint64_t violation_xor;
   int64_t first_violation_level; /* -1 if none */
   uint64_t kernel_launches; /* kernels the search launched (initialisation, expansion,
-                               level-advance steps) */
+                               level-advance steps).  In the device-driven loop the expansion
+                               and the advance step of a level of few states run inside one
+                               launch for many levels; each is counted as one here */
   uint64_t device_levels;   /* levels expanded by the device-driven loop */
   uint64_t global_cache_entries; /* entries of the GPU-wide cache used (0 = not used) */
 } gx_stats_t;

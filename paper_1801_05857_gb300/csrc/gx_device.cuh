@@ -172,13 +172,12 @@ __device__ __forceinline__ uint64_t seq_bucket(uint64_t h, uint32_t k, const uin
   return k == 0 ? b : bucket_in_span<B>(h, muls[k], log2nb, b);
 }
 
-// One bucket of B words read by one lane: FOP_FOUND, FOP_INSERTED, or -1 when
+// A bucket's words s, as one lane holds them: FOP_FOUND, FOP_INSERTED, or -1 when
 // it is full of other vectors.
 template <int W, int B>
-__device__ __forceinline__ int bucket_step(uint32_t* __restrict__ bucket, const uint32_t (&v)[W]) {
+__device__ __forceinline__ int bucket_claim(uint32_t* __restrict__ bucket, const uint32_t (&s)[B],
+                                            const uint32_t (&v)[W]) {
   constexpr int S = B / W;
-  uint32_t s[B];
-  load_words<B>(bucket, s);
   bool match = false;
   uint32_t cand = 0;  // slots that are empty or half-written
 #pragma unroll
@@ -205,6 +204,14 @@ __device__ __forceinline__ int bucket_step(uint32_t* __restrict__ bucket, const 
     cand &= ~(1u << j);
   }
   return -1;
+}
+
+// The same for a bucket read by the lane itself.
+template <int W, int B>
+__device__ __forceinline__ int bucket_step(uint32_t* __restrict__ bucket, const uint32_t (&v)[W]) {
+  uint32_t s[B];
+  load_words<B>(bucket, s);
+  return bucket_claim<W, B>(bucket, s, v);
 }
 
 // Find-or-put of one state by one lane, bucket after bucket; `probes` is
@@ -311,87 +318,49 @@ __device__ __forceinline__ int find_or_put_hashed(uint32_t* __restrict__ table, 
   return FOP_FULL;
 }
 
-// Buckets a group of G lanes has in flight: its items' loads are issued
-// together while a lane's share of them fits 16 registers.
-template <int W, int B, int G>
-constexpr int kLanesInFlight = 16 / (B / G) < 1 ? 1 : (16 / (B / G) < G ? 16 / (B / G) : G);
-
 // One bucket for every lane with `has` set, read by groups of G > 1 lanes; all
 // 32 lanes call it together and each gets its own vector's result (as
-// bucket_step; -1 without one).  The lanes of a group read their items' buckets
-// together, several in flight, and vote; every item's owner then claims the
-// first free slot itself, so the compare-and-swaps of a group's items overlap
-// instead of following one another.
+// bucket_step; -1 without one).  The lanes of a group read their G buckets
+// together, a request per bucket, all in flight; a butterfly over the group then
+// brings every lane its own bucket's words, and it goes on as a lane that read
+// the bucket alone.  (Broadcasting every vector to its group and voting on each
+// took twice the instructions: 8-word buckets, a lane per slot: 1.4e7-state token ring
+// of 13 nodes 8.0 ms, now 4.7; 1.7e7 states of 4 words 19.1 ms, now 9.4.)
 template <int W, int B, int G>
 __device__ __forceinline__ int bucket_step_lanes(uint32_t* __restrict__ table, bool has, uint64_t b,
                                                  const uint32_t (&v)[W]) {
-  constexpr int S = B / W;
-  static_assert(G > 1 && S % G == 0, "group size must divide the slots per bucket");
-  constexpr int SPL = S / G;
-  constexpr int LW = SPL * W;
-  constexpr int CH = kLanesInFlight<W, B, G>;
+  static_assert(G > 1 && (B / W) % G == 0, "group size must divide the slots per bucket");
+  constexpr int LW = B / G;  // words of a bucket read by one lane
   const Group<G> g;
-  bool found = false;
-  int slot = S;  // first slot of the bucket that is empty or half-written
-#pragma unroll 1
-  for (int c = 0; c < G; c += CH) {
-    uint32_t s[CH][LW];
-    bool on[CH];
+  const uint32_t on = __ballot_sync(FULLMASK, has) >> g.base;
+  uint32_t s[B];  // first: words LW glane.. of the group's buckets 0..G-1
 #pragma unroll
-    for (int j = 0; j < CH; ++j) {
-      on[j] = g.template bcast<int>(has ? 1 : 0, g.base + c + j) != 0;
-      const uint64_t bj = g.template bcast<unsigned long long>(b, g.base + c + j);
-      if (on[j]) load_words<LW>(table + bj * (uint64_t)B + (uint64_t)g.glane * LW, s[j]);
-    }
+  for (int j = 0; j < G; ++j) {
+    const uint64_t bj = __shfl_sync(FULLMASK, (unsigned long long)b, g.base + j);
+    uint32_t x[LW];
 #pragma unroll
-    for (int j = 0; j < CH; ++j) {
-      if (!on[j]) continue;  // the same in every lane of the group
-      uint32_t x[W];
+    for (int i = 0; i < LW; ++i) x[i] = 0;
+    if ((on >> j) & 1u) load_words<LW>(table + bj * (uint64_t)B + (uint64_t)g.glane * LW, x);
 #pragma unroll
-      for (int w = 0; w < W; ++w) x[w] = g.template bcast<uint32_t>(v[w], g.base + c + j);
-      bool match = false;
-      int first = -1;
+    for (int i = 0; i < LW; ++i) s[j * LW + i] = x[i];
+  }
+  // transpose: lane l's piece of bucket j becomes lane j's piece l of its own
 #pragma unroll
-      for (int i = SPL - 1; i >= 0; --i) {
-        bool eq = true, tagged = true;
+  for (int m = G / 2; m >= 1; m /= 2) {
+    const bool up = (g.glane & m) != 0;
 #pragma unroll
-        for (int w = 0; w < W; ++w) {
-          eq &= (s[j][i * W + w] == x[w]);
-          tagged &= (s[j][i * W + w] & kTag) != 0;
-        }
-        match |= eq;
-        if (!tagged) first = i;
-      }
-      const bool hit = g.any(match);
-      const uint32_t free_lanes = g.ballot(first >= 0);
-      int at = S;
-      if (free_lanes) {
-        const int leader = __ffs(free_lanes) - 1;
-        at = (leader - g.base) * SPL + g.template bcast<int>(first, leader);
-      }
-      if (g.glane == c + j) {
-        found = hit;
-        slot = at;
+    for (int j = 0; j < G; ++j) {
+      if (j & m) continue;
+#pragma unroll
+      for (int i = 0; i < LW; ++i) {
+        uint32_t &lo = s[j * LW + i], &hi = s[(j | m) * LW + i];
+        const uint32_t r = __shfl_xor_sync(FULLMASK, up ? lo : hi, m);
+        if (up) lo = r;
+        else hi = r;
       }
     }
   }
-  int r = -1;
-  if (has) {
-    if (found) r = FOP_FOUND;
-    // slots fill in order: from the first free one on, each compare-and-swap
-    // that fails tells what the slot holds -- this vector, or another one
-    for (; r < 0 && slot < S; ++slot) {
-      uint32_t old[W];
-      if (cas_slot<W>(table + b * (uint64_t)B + slot * W, v, old)) {
-        r = FOP_INSERTED;
-      } else {
-        bool eq = true;
-#pragma unroll
-        for (int w = 0; w < W; ++w) eq &= (old[w] == v[w]);
-        if (eq) r = FOP_FOUND;
-      }
-    }
-  }
+  const int r = has ? bucket_claim<W, B>(table + b * (uint64_t)B, s, v) : -1;
   __syncwarp();
   return r;
 }

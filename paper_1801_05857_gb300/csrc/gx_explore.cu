@@ -62,30 +62,11 @@ uint32_t auto_cache_log2(const Net& net) {
 
 namespace gx {
 
-// The device-driven level loop (see run_search).
-struct LoopArgs {
-  Ctl* ctl;
-  unsigned long long* lv_size;    // [cap] level sizes (level 0 = 1)
-  unsigned long long* lv_tns;     // [cap] per expanded level: device time in ns (%globaltimer)
-  unsigned long long* lv_probes;  // [cap] cumulative bucket reads after the level
-  unsigned long long* lv_trans;   // [cap] cumulative transitions after the level
-  uint32_t cap;
-  int stop_dl, stop_viol;
-  uint64_t max_levels;            // 0 = no limit
-  cudaGraphConditionalHandle cond;
-};
-
 constexpr uint32_t kLoopLevels = 4096;  // levels the device loop records before the host takes over
 
 }  // namespace gx
 
 namespace gxd {
-
-__device__ __forceinline__ unsigned long long global_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
 
 // Level 0 = {initial state}; start the loop unless the insertion failed.
 __global__ void loop_start_kernel(const gx::LoopArgs L) {
@@ -109,42 +90,16 @@ __global__ void loop_start_kernel(const gx::LoopArgs L) {
 // bookkeeping, done on the device.
 __global__ void level_advance_kernel(const gx::LoopArgs L) {
   gx::Ctl& c = *L.ctl;
-  const unsigned long long k = c.levels_done;
-  const unsigned long long t = global_ns();
-  if (k < L.cap) {
-    L.lv_tns[k] = t - c.t_prev;
-    L.lv_probes[k] = c.probes;
-    L.lv_trans[k] = c.transitions;
-  }
-  c.t_prev = t;
-  c.levels_done = k + 1;
-  c.explored += c.cur_end - c.cur_begin;
-  if (c.first_dl < 0 && c.dl_count > 0) c.first_dl = (long long)c.n_levels - 1;
-  if (c.first_viol < 0 && c.viol_count > 0) c.first_viol = (long long)c.n_levels - 1;
-  const unsigned long long next_end = c.next_end;
-  if (next_end > c.cur_end) {
-    if (c.n_levels < L.cap) L.lv_size[c.n_levels] = next_end - c.cur_end;
-    c.n_levels += 1;
-  }
-  bool more = true;
-  if (c.error) {
-    more = false;
-  } else if (next_end == c.cur_end) {
-    c.complete = 1;
-    more = false;
-  } else {
-    c.cur_begin = c.cur_end;
-    c.cur_end = next_end;
-    c.claim = 0;
-    if ((L.stop_dl && c.dl_count > 0) || (L.stop_viol && c.viol_count > 0) ||
-        (L.max_levels && c.levels_done >= L.max_levels)) {
-      more = false;
-    } else if (c.n_levels >= L.cap) {  // arrays full: the host loop continues from here
-      c.yielded = 1;
-      more = false;
-    }
-  }
+  LoopState s;
+  s.load(c);
+  const LevelEnd e = level_end(c);
+  const bool more = s.advance(L, e, c.probes, c.transitions);
+  s.store(c);
+  c.claim = 0;
+  // back to the small-level kernel once a level is well below its limit
+  const bool small = s.cur_end - s.cur_begin <= kSmallLevel / 2;
   cudaGraphSetConditional(L.cond, more ? 1u : 0u);
+  cudaGraphSetConditional(L.cond_big, more && !small ? 1u : 0u);
 }
 
 // Digest of the states in a table.  Bound by the table's bytes where it is nearly
@@ -374,8 +329,10 @@ gx_status make_plan(const Net& net, const gx_explore_opts* o, Plan& P) {
     P.gcache = 1ull << glog;
     P.gcache_bytes = P.gcache << P.seen.log2_bytes;
   }
-  // (4-word vectors: 2^6, whose 4 KiB per CTA leave room for 5 CTAs per SM beside the queues)
-  P.warp_log2 = o->warp_cache_log2 == kAutoCache ? (P.gcache ? 0u : P.W == 4 ? 6u : 9u) : o->warp_cache_log2;
+  // The per-warp one: more entries find more, but their shared memory costs CTAs and L1 (token
+  // ring of 13 nodes: 2^6 4.19 ms, 2^7 4.18, 2^8 4.24, 2^9 4.86; 1.7e7 states of 4 words in one
+  // pass: 8.83, 8.76, 9.13, 10.3); region passes of 4-word vectors 2^6
+  P.warp_log2 = o->warp_cache_log2 == kAutoCache ? (P.gcache ? 0u : P.W == 4 && P.regions > 1 ? 6u : 7u) : o->warp_cache_log2;
   P.cs = o->successor_buffer ? o->successor_buffer : std::min<uint64_t>(slots / 2, (1ull << 32) - 1);
   if (P.logp == 0) P.cs = 0;  // partitioned path off: no buffer
   if (P.cs >= (1ull << 32)) return fail(GX_ERR_INVALID, "successor_buffer must be below 2^32 vectors");
@@ -455,9 +412,10 @@ void release_loop(gx_net* h) {
 }
 
 // The device-driven search as one graph: clear the control block and the
-// table, insert the initial vector, start, then WHILE(cond) {expand; advance}.
+// table, insert the initial vector, start, then WHILE(more levels) {small levels;
+// WHILE(large levels) {expand; advance}}.
 gx_status build_loop_graph(gx_net* h, const Plan& P, Ctl* ctl, uint32_t* table, const InitArgs& ia,
-                           const ExpandArgs& eg, LoopArgs la, size_t smem, uint64_t grid) {
+                           const ExpandArgs& eg, LoopArgs la, size_t smem, uint64_t grid, size_t small_smem) {
   release_loop(h);
   h->release = &release_loop;
   cudaGraph_t g;
@@ -466,6 +424,7 @@ gx_status build_loop_graph(gx_net* h, const Plan& P, Ctl* ctl, uint32_t* table, 
   cudaGraphConditionalHandle cond;
   GX_CUDA(cudaGraphConditionalHandleCreate(&cond, g, 1, cudaGraphCondAssignDefault));
   la.cond = cond;
+  GX_CUDA(cudaGraphConditionalHandleCreate(&la.cond_big, g, 0, cudaGraphCondAssignDefault));
   std::vector<cudaGraphNode_t> clears;
   auto add_memset = [&](void* dst, uint64_t words) -> cudaError_t {
     cudaMemsetParams mp{};
@@ -503,14 +462,28 @@ gx_status build_loop_graph(gx_net* h, const Plan& P, Ctl* ctl, uint32_t* table, 
   GX_CUDA(add_kernel(g, clears.data(), clears.size(), P.ks->init_fn, dim3(1), dim3(32), 0, args_i, &init));
   GX_CUDA(add_kernel(g, &init, 1, reinterpret_cast<const void*>(&gxd::loop_start_kernel), dim3(1), dim3(1), 0,
                      args_l, &start));
-  cudaGraphNodeParams cp{};
-  cp.type = cudaGraphNodeTypeConditional;
-  cp.conditional.handle = cond;
-  cp.conditional.type = cudaGraphCondTypeWhile;
-  cp.conditional.size = 1;
-  cudaGraphNode_t cnode;
-  GX_CUDA(cudaGraphAddNode(&cnode, g, &start, nullptr, 1, &cp));
-  cudaGraph_t body = cp.conditional.phGraph_out[0];
+  auto add_while = [&](cudaGraph_t gr, const cudaGraphNode_t* dep, cudaGraphConditionalHandle hd,
+                       cudaGraph_t* inside) -> cudaError_t {
+    cudaGraphNodeParams cp{};
+    cp.type = cudaGraphNodeTypeConditional;
+    cp.conditional.handle = hd;
+    cp.conditional.type = cudaGraphCondTypeWhile;
+    cp.conditional.size = 1;
+    cudaGraphNode_t nd;
+    const cudaError_t e = cudaGraphAddNode(&nd, gr, dep, nullptr, 1, &cp);
+    if (e == cudaSuccess) *inside = cp.conditional.phGraph_out[0];
+    return e;
+  };
+  cudaGraph_t outer, body;
+  GX_CUDA(add_while(g, &start, la.cond, &outer));
+  ExpandArgs es_c = eg;  // the small-level kernel: no region passes, its CTAs stage the tables once
+  es_c.cache_log2 = 0;
+  es_c.stage = small_smem > 8ull * kMaxRounds + P.ks->small_queue_bytes ? 1 : 0;
+  void* args_s[] = {&es_c, &la};
+  cudaGraphNode_t sm;
+  GX_CUDA(add_kernel(outer, nullptr, 0, P.ks->small_fn, dim3(gxd::kSmallCtas), dim3(gxd::kSmallThreads), small_smem,
+                     args_s, &sm));
+  GX_CUDA(add_while(outer, &sm, la.cond_big, &body));
   GX_CUDA(add_kernel(body, nullptr, 0, P.ks->expand_fn, dim3((unsigned)grid), dim3(kBlock), smem, args_e, &ex));
   // region passes after the first: clear the claim counter, expand again
   for (uint32_t q = 1; q < P.regions; ++q) {
@@ -711,7 +684,11 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
     std::memcpy(key.data(), o, sizeof(gx_explore_opts));
     std::memcpy(key.data() + sizeof(gx_explore_opts), extra, sizeof(extra));
     if (!h->loop_exec || h->loop_key != key) {
-      s = build_loop_graph(h, P, ctl, table, ia, eg, la, smem, max_grid);
+      // the small-level kernel: multipliers, queues and (when they are not large) network tables
+      size_t small_smem = 8ull * kMaxRounds + P.ks->small_queue_bytes;
+      if (blob_bytes <= 64 * 1024) small_smem += blob_bytes;
+      GX_CUDA(cudaFuncSetAttribute(P.ks->small_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)small_smem));
+      s = build_loop_graph(h, P, ctl, table, ia, eg, la, smem, max_grid, small_smem);
       if (s != GX_OK) return s;
       h->loop_key = key;
     }
@@ -737,7 +714,7 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
     launches = nd * P.regions;
     dev_expand = launches;
     device_levels = nd;
-    kernel_launches = 2 + (P.regions + 1) * nd;  // init, start, then the passes + advance per level
+    kernel_launches = 2 + (P.regions + 1) * nd;  // init, start, then the passes + advance step per level
     first_dl = hc->first_dl;
     first_viol = hc->first_viol;
     complete = hc->complete != 0;

@@ -672,15 +672,50 @@ __global__ void __launch_bounds__(gx::kBlock) guided_expand_kernel(const GuidedA
   }
   __syncthreads();
   const NetBlobLayout& L = a.lay;
+  __shared__ uint4 descs[kMaxProcs];
+  __shared__ __align__(16) uint32_t queue_mem[kWarps][64 * W];
+  __shared__ uint32_t rows_mem[kWarps][64 * E], s_left[kWarps];
+  __shared__ unsigned long long s_base;
+  for (uint32_t p = threadIdx.x; p < L.n_procs; p += blockDim.x) descs[p] = proc_desc(t, L, p);
+  __syncthreads();
   const int lane = threadIdx.x & 31;
   const unsigned long long log_base = a.ctl->log_base;
   unsigned long long trans = 0, ins = 0;
   uint32_t probes = 0, err = 0;
   // One warp per state: a batch holds a few thousand states, so the time of an
-  // iteration is the latency of one state's successors; lane l takes
-  // successors l, l + 32, ... and their find-or-puts overlap.  Warp w of the
-  // grid takes states w, w + (warps of the grid), ...
+  // iteration is the latency of one state's successors.  The lanes take the
+  // state's sources of successors 32 at a time (WarpGen), queue the successors and
+  // find-or-put 32 of them at once.  Warp w of the grid takes states w, w + (warps
+  // of the grid), ...
   const unsigned long long nwarps = (unsigned long long)gridDim.x * kWarps;
+  const uint32_t n_src = L.n_procs + L.n_rules, below = (1u << lane) - 1u;
+  uint32_t* queue = queue_mem[threadIdx.x >> 5];
+  const auto desc = [&](uint32_t p) { return descs[p]; };
+  uint32_t* rows = rows_mem[threadIdx.x >> 5];
+  int staged = 0;  // new states (uniform in the warp)
+  // the last m <= 32 staged states, with their histograms, to positions base.. of the pending buffer
+  auto append = [&](int m, unsigned long long base) {
+    staged -= m;
+    if (lane < m) {
+      ins += 1;
+      const uint32_t* r = rows + (staged + lane) * E;
+      uint32_t s[W], hw[4], bad = 0;
+#pragma unroll
+      for (int w = 0; w < W; ++w) s[w] = r[w];
+      local_hist<W>(t, L, s, hw, bad);
+      if (bad) err |= gx::ERR_WIDE;
+      const unsigned long long pos = base + lane;
+      if (pos < a.pend_cap) {
+        a.pend_hist[pos] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+        uint32_t* e = a.pend + pos * E;
+#pragma unroll
+        for (int w = 0; w < E; ++w) e[w] = r[w];
+      } else {
+        err |= gx::ERR_PENDING;
+      }
+    }
+    __syncwarp();
+  };
   for (unsigned long long idx = (unsigned long long)blockIdx.x * kWarps + (threadIdx.x >> 5); idx < n;
        idx += nwarps) {
     uint32_t v[W];
@@ -693,7 +728,50 @@ __global__ void __launch_bounds__(gx::kBlock) guided_expand_kernel(const GuidedA
       for (int w = 0; w < W; ++w) le[w] = v[w];
       le[W] = a.batch[idx * E + W];
     }
-    const uint32_t total = count_succ<W>(t, L, v);  // the same in every lane
+    WarpGen<W> gen;
+    gen.src = gen.e = gen.e_end = gen.word = gen.cur = 0;
+    uint32_t total = 0;  // this lane's part of the state's successors
+    int queued = 0;
+    while (true) {
+      const uint32_t act = __ballot_sync(FULLMASK, gen.e < gen.e_end);
+      if (act != 0) {
+        if ((act >> lane) & 1u) gen.emit(t, L, desc, v, queue + (queued + __popc(act & below)) * W);
+        queued += __popc(act);
+        if (queued < 32) continue;
+      } else if (gen.src < n_src) {
+        gen.open_wide(t, L, desc, v);
+        total += gen.e_end - gen.e;
+        continue;
+      }
+      if (queued == 0) break;
+      __syncwarp();
+      const int k = queued < 32 ? queued : 32;
+      queued -= k;
+      uint32_t s[W];
+      bool inserted = false;
+      if (lane < k) {
+        load_vec<W>(queue + (queued + lane) * W, s);
+        const int r = find_or_put_state<W, B>(a.table, a.log2nb, a.rounds, muls, s, probes);
+        if (r == FOP_FULL) err |= gx::ERR_TABLE_FULL;
+        inserted = r == FOP_INSERTED;
+      }
+      // stage the new states; 32 of them are appended to the pending buffer at a time
+      const uint32_t im = __ballot_sync(FULLMASK, inserted);
+      if (inserted) {
+        uint32_t* e = rows + (staged + __popc(im & below)) * E;
+#pragma unroll
+        for (int w = 0; w < W; ++w) e[w] = s[w];
+        e[W] = (uint32_t)li;
+      }
+      staged += __popc(im);
+      __syncwarp();
+      if (staged >= 32) {
+        unsigned long long base = 0;
+        if (lane == 0) base = atomicAdd(&a.ctl->pending, 32ull);
+        append(32, __shfl_sync(FULLMASK, base, 0));
+      }
+    }
+    total = __reduce_add_sync(FULLMASK, total);
     if (lane == 0) {
       trans += total;
       if (total == 0) {
@@ -701,47 +779,29 @@ __global__ void __launch_bounds__(gx::kBlock) guided_expand_kernel(const GuidedA
         atomicAdd(&a.ctl->dl_count, 1ull);
       }
     }
-    for (uint32_t k0 = 0; k0 < total; k0 += 32) {
-      const uint32_t k = k0 + lane;
-      uint32_t s[W];
-      bool inserted = false;
-      if (k < total) {
-        seek_succ<W>(t, L, v, k, s);
-        const int r = find_or_put_state<W, B>(a.table, a.log2nb, a.rounds, muls, s, probes);
-        if (r == FOP_FULL) err |= gx::ERR_TABLE_FULL;
-        inserted = r == FOP_INSERTED;
-      }
-      uint32_t hw[4] = {0, 0, 0, 0}, bad = 0;
-      if (inserted) local_hist<W>(t, L, s, hw, bad);
-      if (bad) err |= gx::ERR_WIDE;
-      const uint32_t im = __ballot_sync(FULLMASK, inserted);
-      ins += inserted ? 1u : 0u;
-      if (im) {  // append the new states to the pending buffer, one atomic per warp
-        unsigned long long base = 0;
-        if (lane == 0) base = atomicAdd(&a.ctl->pending, (unsigned long long)__popc(im));
-        base = __shfl_sync(FULLMASK, base, 0);
-        if (inserted) {
-          const unsigned long long pos = base + __popc(im & ((1u << lane) - 1u));
-          if (pos < a.pend_cap) {
-            a.pend_hist[pos] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-            uint32_t* e = a.pend + pos * E;
-#pragma unroll
-            for (int w = 0; w < W; ++w) e[w] = s[w];
-            e[W] = (uint32_t)li;
-          } else {
-            err |= gx::ERR_PENDING;
-          }
-        }
-      }
-    }
   }
+  // what the CTA's warps have staged, with one atomic for all of them: most warps
+  // expand one or two states, and 8192 atomics on one address would take 8 us
+  const int wid = threadIdx.x >> 5;
+  if (lane == 0) s_left[wid] = (uint32_t)staged;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t sum = 0;
+    for (int w = 0; w < kWarps; ++w) {
+      const uint32_t m = s_left[w];
+      s_left[w] = sum;
+      sum += m;
+    }
+    s_base = sum ? atomicAdd(&a.ctl->pending, (unsigned long long)sum) : 0ull;
+  }
+  __syncthreads();
+  if (staged > 0) append(staged, s_base + s_left[wid]);
   // the CTA's totals, one atomic per counter (every warp's at once would queue
   // on the same addresses)
   trans = warp_sum(trans);
   ins = warp_sum(ins);
   const unsigned long long pr = warp_sum((unsigned long long)probes);
   err = __reduce_or_sync(FULLMASK, err);
-  const int wid = threadIdx.x >> 5;
   if (lane == 0) {
     s_sum[0][wid] = trans;
     s_sum[1][wid] = ins;

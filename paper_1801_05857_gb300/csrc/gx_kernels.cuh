@@ -428,19 +428,21 @@ __device__ __forceinline__ uint4 proc_desc(const uint32_t* t, const NetBlobLayou
 }
 constexpr int kMaxProcs = 124;  // gx_load_network's limit
 
-// Successor generation by a warp whose lanes hold one state each (lanes without
-// one hold no successors).  The warp walks the sources of successors -- the
-// processes, then the rules -- together: open() finds, per lane, how many
-// successors the current source gives its state, and emit() appends one per
-// lane that has any left to a queue in shared memory.  Every table address but
-// the per-lane edge offsets is uniform, and a state's successors are counted on
-// the way, without a pass of their own.
+// Successor generation by a warp.  Sources of successors are the processes, then
+// the rules.  Either the lanes hold one state each (lanes without one hold no
+// successors) and the warp walks the sources together -- open() finds, per lane, how
+// many successors the current source gives its state; every table address but the
+// edge offsets is uniform -- or all lanes hold the same state and take 32 sources
+// at a time (open_wide), which costs a few dozen instructions a state instead of
+// as many per source: what counts in a level of few states.  emit() appends one
+// successor per lane that has any left to a queue in shared memory; a state's
+// successors are counted on the way, without a pass of their own.
 template <int W>
 struct WarpGen {
   uint32_t src;       // next source: process src, then rule src - n_procs (uniform)
-  uint32_t e, e_end;  // this lane's successors left of the current source: edges, or combinations of the rule
-  uint32_t word;      // word index of the current process (uniform); W: a rule
-  uint32_t cur;       // that word of this lane's state; a rule: its index (uniform)
+  uint32_t e, e_end;  // this lane's successors left of its source: edges, or combinations of the rule
+  uint32_t word;      // word index of the source's process; W: a rule
+  uint32_t cur;       // that word of this lane's state; a rule: its index
 
   template <class Desc>
   __device__ __forceinline__ void open(const uint32_t* t, const NetBlobLayout& L, Desc& desc, bool valid,
@@ -469,6 +471,35 @@ struct WarpGen {
       e_end = prod;
     }
     ++src;
+  }
+
+  // The next 32 sources of the state v that every lane holds, one per lane.
+  template <class Desc>
+  __device__ __forceinline__ void open_wide(const uint32_t* t, const NetBlobLayout& L, Desc& desc,
+                                            const uint32_t (&v)[W]) {
+    const uint32_t s = src + (threadIdx.x & 31);
+    e = e_end = 0;
+    if (s < L.n_procs) {
+      const uint4 d = desc(s);
+      word = d.x;
+      cur = word_at<W>(v, d.x);
+      const uint32_t* o = t + d.w + ((cur >> d.y) & d.z);
+      e = o[0];
+      e_end = o[1];
+    } else if (s < L.n_procs + L.n_rules) {
+      const uint32_t r = s - L.n_procs, j1 = t[L.rule_off + r + 1];
+      uint32_t prod = 1;
+      for (uint32_t j = t[L.rule_off + r]; j < j1 && prod; ++j) {
+        const uint32_t c = t[L.rule_cls + j];
+        const uint4 d = desc(t[L.cls_proc + c]);
+        const uint32_t* o = t + L.coff + t[L.cls_base + c] + ((word_at<W>(v, d.x) >> d.y) & d.z);
+        prod *= o[1] - o[0];
+      }
+      word = W;
+      cur = r;
+      e_end = prod;
+    }
+    src += 32;
   }
 
   // One successor into the W words at q (a lane with e < e_end).
@@ -529,12 +560,10 @@ struct WarpQueues {
 };
 
 // Resident CTAs per SM the level kernel is compiled for (register budget): a
-// lane holds a bucket of B words (one lane per bucket), or its share of the
-// buckets in flight (bucket_step_lanes).
+// lane holds a bucket of B words.
 template <int W, int B, int G>
 struct ExpandOcc {
-  static constexpr int words = G == 1 ? B : kLanesInFlight<W, B, G> * (B / G) + 8;
-  static constexpr int min_ctas = words <= 8 ? 5 : (words <= 16 ? 4 : 3);
+  static constexpr int min_ctas = B <= 8 ? (G == 1 ? 5 : 4) : (B <= 16 && G == 1 ? 4 : 3);
 };
 
 // The expansion of a warp's share of one level: generate successors of its
@@ -542,7 +571,8 @@ struct ExpandOcc {
 // time -- one loop with one copy of each step (a second copy of find-or-put
 // costs registers).
 //   next(pos, m)   the warp's next m <= 32 states, at absolute frontier
-//                  positions pos.. (m = 0: none are left)
+//                  positions pos.. (m = 0: none are left); a single state is
+//                  generated from by the whole warp
 //   desc(p)        the process descriptors (proc_desc)
 //   seen(v)        a lane's state, once, when it is taken
 //   done(v, n)     a lane's state and the number of its successors
@@ -573,18 +603,20 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
         if ((act >> lane) & 1u) gen.emit(t, L, desc, v, q.raw + (n_raw + __popc(act & below)) * W);
         n_raw += __popc(act);
       } else if (gen.src < n_src) {
-        gen.open(t, L, desc, lane < m, v);
+        if (m == 1) gen.open_wide(t, L, desc, v);
+        else gen.open(t, L, desc, lane < m, v);
         cnt += gen.e_end - gen.e;
       } else {
         if (!more) break;
+        if (m == 1) cnt = __reduce_add_sync(FULLMASK, cnt);
         if (lane < m) done(v, cnt);
         uint64_t pos = 0;
         next(pos, m);
         more = m != 0;
         if (!more) break;
-        if (lane < m) {
-          load_vec<W>(tg.frontier() + ((pos + lane) & tg.fmask()) * W, v);
-          seen(v);
+        if (lane < m || m == 1) {
+          load_words<W>(tg.frontier() + ((m == 1 ? pos : pos + lane) & tg.fmask()) * W, v);
+          if (lane < m) seen(v);
         }
         cnt = 0;
         gen.src = 0;
@@ -655,6 +687,11 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
   }
 }
 
+// Up to this many states per warp are taken one by one, the whole warp generating
+// from each (token ring of 11 nodes, 22 sources: levels of 1 or 2 states a warp take
+// 15-22 us instead of 19-27; of 4 or more a warp they take longer).
+constexpr uint32_t kSingly = 2;
+
 template <int W, int B, int G>
 __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expand_kernel(const gx::ExpandArgs a) {
   constexpr uint32_t kWarps = gx::kBlock / 32;
@@ -693,8 +730,9 @@ __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expa
   __shared__ __align__(16) WarpQueues<W> queue_mem[kWarps];
   WarpStage st{stage_mem[threadIdx.x >> 5], 0};
   const ParamTarget tg{a, s_range};
+  // (a warp with a few states has no use for the cache of those it has seen)
   WarpCache cache{nullptr, 0};
-  if (a.cache_log2 > 0) {
+  if (a.cache_log2 > 0 && unit == 32) {
     uint32_t* cbase = sm + 2 * kMaxRounds + (a.stage ? a.blob_words : 0);  // 16-byte aligned
     const uint32_t per_warp = (1u << a.cache_log2) * W;
     cache.base = cbase + (threadIdx.x >> 5) * per_warp;
@@ -702,15 +740,23 @@ __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expa
     for (uint32_t i = lane; i < per_warp; i += 32) cache.base[i] = 0u;  // 0 is never a stored vector
     __syncwarp();
   }
+  uint64_t own = s_range[0] + (uint64_t)(blockIdx.x * kWarps + (threadIdx.x >> 5)) * unit;
+  const uint64_t own_end = s_range[1] - own < unit ? s_range[1] : own + unit;  // (own >= the end: no states)
   bool first = true;
   expand_states<W, B, G, kBatch<W>>(
       tg, muls, t, L, queue_mem[threadIdx.x >> 5], st, probes, err, [&](uint32_t p) { return descs[p]; },
       [&](uint64_t& pos, uint32_t& m) {
         // the first states of every warp are fixed by its index, a large level's
-        // further ones are claimed
+        // further ones are claimed; a few states are taken one by one
         m = 0;
+        if (unit <= kSingly) {
+          if (own >= s_range[1] || own >= own_end) return;
+          pos = own++;
+          m = 1;
+          return;
+        }
         if (first) {
-          pos = s_range[0] + (uint64_t)(blockIdx.x * kWarps + (threadIdx.x >> 5)) * unit;
+          pos = own;
           first = false;
         } else {
           if (unit < 32) return;
@@ -772,6 +818,201 @@ __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expa
   }
 }
 
+
+// ---- the device-driven level loop
+
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// What decides about going on, as the expansion of a level left it.
+struct LevelEnd {
+  unsigned long long next_end, dl_count, viol_count;
+  unsigned int error;
+};
+__device__ __forceinline__ LevelEnd level_end(const gx::Ctl& c) {
+  return LevelEnd{__ldcg(&c.next_end), __ldcg(&c.dl_count), __ldcg(&c.viol_count), __ldcg(&c.error)};
+}
+
+// The loop's bookkeeping of the control block, in registers.
+struct LoopState {
+  unsigned long long cur_begin, cur_end, n_levels, levels_done, explored, t_prev;
+  long long first_dl, first_viol;
+  unsigned int complete, yielded;
+  __device__ __forceinline__ void load(const gx::Ctl& c) {
+    cur_begin = c.cur_begin;
+    cur_end = c.cur_end;
+    n_levels = c.n_levels;
+    levels_done = c.levels_done;
+    explored = c.explored;
+    t_prev = c.t_prev;
+    first_dl = c.first_dl;
+    first_viol = c.first_viol;
+    complete = c.complete;
+    yielded = c.yielded;
+  }
+  __device__ __forceinline__ void store(gx::Ctl& c) const {
+    c.cur_begin = cur_begin;
+    c.cur_end = cur_end;
+    c.n_levels = n_levels;
+    c.levels_done = levels_done;
+    c.explored = explored;
+    c.t_prev = t_prev;
+    c.first_dl = first_dl;
+    c.first_viol = first_viol;
+    c.complete = complete;
+    c.yielded = yielded;
+  }
+  // Level [cur_begin, cur_end) has been expanded: whether there is another one
+  // to expand now, which is then [cur_begin, cur_end).
+  __device__ __forceinline__ bool move(const gx::LoopArgs& L, const LevelEnd& e) {
+    levels_done += 1;
+    explored += cur_end - cur_begin;
+    if (first_dl < 0 && e.dl_count > 0) first_dl = (long long)n_levels - 1;
+    if (first_viol < 0 && e.viol_count > 0) first_viol = (long long)n_levels - 1;
+    if (e.next_end > cur_end) n_levels += 1;
+    if (e.error) return false;
+    if (e.next_end == cur_end) {
+      complete = 1;
+      return false;
+    }
+    cur_begin = cur_end;
+    cur_end = e.next_end;
+    if ((L.stop_dl && e.dl_count > 0) || (L.stop_viol && e.viol_count > 0) ||
+        (L.max_levels && levels_done >= L.max_levels))
+      return false;
+    if (n_levels >= L.cap) {  // arrays full: the host loop continues from here
+      yielded = 1;
+      return false;
+    }
+    return true;
+  }
+  // The same with the level's entries in the arrays.
+  __device__ __forceinline__ bool advance(const gx::LoopArgs& L, const LevelEnd& e, unsigned long long probes,
+                                          unsigned long long transitions) {
+    const unsigned long long k = levels_done, end = cur_end, t = global_ns();
+    if (k < L.cap) {
+      L.lv_tns[k] = t - t_prev;
+      L.lv_probes[k] = probes;
+      L.lv_trans[k] = transitions;
+    }
+    t_prev = t;
+    if (e.next_end > end && n_levels < L.cap) L.lv_size[n_levels] = e.next_end - end;
+    return move(L, e);
+  }
+};
+
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+// Levels of at most kSmallLevel states, one after the other in one launch by one
+// cluster of CTAs: what such a level costs elsewhere is launches, staging the
+// tables and the loop's iteration (13-17 us a level), here two cluster barriers and
+// the latency of one or a few states per warp (640-state network: 5-6 us a
+// level).  Ends at the first larger level, which the large-level loop takes.
+constexpr int kSmallCtas = 8, kSmallThreads = 512;
+constexpr uint32_t kSmallWarps = kSmallCtas * kSmallThreads / 32;
+constexpr unsigned long long kSmallLevel = 4 * kSmallWarps;
+
+template <int W>
+struct __align__(16) SmallQueues {  // of a warp, in dynamic shared memory
+  WarpQueues<W, 32> queues;
+  uint32_t stage[kStage * W];
+};
+
+template <int W, int B>
+__global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThreads, 1)
+    small_levels_kernel(const gx::ExpandArgs a, const gx::LoopArgs LA) {
+  constexpr uint32_t kWarps = kSmallThreads / 32;
+  extern __shared__ __align__(16) uint32_t sm[];
+  __shared__ unsigned long long s_range[2];
+  __shared__ uint4 descs[kMaxProcs];
+  __shared__ unsigned long long s_tot[2];
+  __shared__ uint32_t s_err, s_go;
+  const uint64_t* muls;
+  const uint32_t* t = stage_tables(sm, a.muls, a.rounds, a.blob, a.blob_words, a.stage, muls);
+  __syncthreads();
+  const NetBlobLayout& L = a.lay;
+  for (uint32_t p = threadIdx.x; p < L.n_procs; p += blockDim.x) descs[p] = proc_desc(t, L, p);
+  const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const uint32_t gw = blockIdx.x * kWarps + wid;
+  SmallQueues<W>& q = reinterpret_cast<SmallQueues<W>*>(sm + 2 * kMaxRounds + (a.stage ? a.blob_words : 0))[wid];
+  WarpStage st{q.stage, 0};
+  const ParamTarget tg{a, s_range};
+  gx::Ctl& c = *a.ctl;
+  LoopState ls;  // thread 0 of every CTA; CTA 0's is written back
+  bool more = true;
+  if (threadIdx.x == 0) {
+    ls.load(c);
+    s_go = ls.cur_end - ls.cur_begin <= kSmallLevel;
+    s_range[0] = ls.cur_begin;
+    s_range[1] = ls.cur_end;
+    s_tot[0] = s_tot[1] = 0;
+    s_err = 0;
+  }
+  __syncthreads();
+  while (s_go) {
+    uint32_t trans = 0, probes = 0, err = 0;
+    uint64_t own = s_range[0] + gw;
+    expand_states<W, B, 1, 32>(
+        tg, muls, t, L, q.queues, st, probes, err, [&](uint32_t p) { return descs[p]; },
+        [&](uint64_t& pos, uint32_t& m) {
+          m = own < s_range[1] ? 1 : 0;
+          pos = own;
+          own += kSmallWarps;
+        },
+        [&](const uint32_t(&v)[W]) {
+          if (a.watch) check_watch<W>(a, t, L, v);
+        },
+        [&](const uint32_t(&v)[W], uint32_t n) {
+          trans += n;
+          if (n == 0) {
+            const uint64_t h = state_digest<W>(t, L, v);
+            const unsigned long long di = atomicAdd(&c.dl_count, 1ull);
+            atomicAdd(&c.dl_sum, (unsigned long long)h);
+            atomicXor(&c.dl_xor, (unsigned long long)h);
+            if (di < a.dl_cap) store_vec<W>(a.dl_buf + di * W, v);
+          }
+        },
+        [](uint64_t, uint64_t, const uint32_t(&)[W]) { return true; });
+    st.flush<W>(tg, err);
+    const unsigned long long tr = warp_sum((unsigned long long)trans), pr = warp_sum((unsigned long long)probes);
+    err = __reduce_or_sync(FULLMASK, err);
+    if (lane == 0) {
+      if (tr) atomicAdd(&s_tot[0], tr);
+      if (pr) atomicAdd(&s_tot[1], pr);
+      if (err) atomicOr(&s_err, err);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      if (s_tot[0]) atomicAdd(&c.transitions, s_tot[0]);
+      if (s_tot[1]) atomicAdd(&c.probes, s_tot[1]);
+      if (s_err) atomicOr(&c.error, s_err);
+      s_tot[0] = s_tot[1] = 0;
+      s_err = 0;
+    }
+    cluster_sync();  // the level is complete
+    if (threadIdx.x == 0) {
+      const LevelEnd e = level_end(c);
+      if (blockIdx.x == 0) more = ls.advance(LA, e, __ldcg(&c.probes), __ldcg(&c.transitions));
+      else more = ls.move(LA, e);
+      s_range[0] = ls.cur_begin;
+      s_range[1] = ls.cur_end;
+      s_go = more && ls.cur_end - ls.cur_begin <= kSmallLevel;
+    }
+    cluster_sync();  // every CTA has read what the next level's expansion changes
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    ls.store(c);
+    c.claim = 0;
+    cudaGraphSetConditional(LA.cond, more ? 1u : 0u);
+    cudaGraphSetConditional(LA.cond_big, more ? 1u : 0u);
+  }
+}
 
 // ---- partitioned expansion (see PartArgs)
 
@@ -1084,7 +1325,9 @@ const KernelSet* kernel_set() {
                             reinterpret_cast<const void*>(&gxd::part_count_kernel<W>),
                             reinterpret_cast<const void*>(&gxd::part_scatter_kernel<W>),
                             reinterpret_cast<const void*>(&gxd::part_probe_kernel<W, B, G>),
-                            reinterpret_cast<const void*>(&gxd::init_kernel<W, B, G>)};
+                            reinterpret_cast<const void*>(&gxd::init_kernel<W, B, G>),
+                            reinterpret_cast<const void*>(&gxd::small_levels_kernel<W, B>),
+                            sizeof(gxd::SmallQueues<W>) * (gxd::kSmallThreads / 32)};
   return &ks;
 }
 

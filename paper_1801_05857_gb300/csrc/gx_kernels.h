@@ -88,6 +88,19 @@ struct ExpandArgs {
   SeenCache gcache;
 };
 
+// The device-driven level loop (see run_search).
+struct LoopArgs {
+  Ctl* ctl;
+  unsigned long long* lv_size;    // [cap] level sizes (level 0 = 1)
+  unsigned long long* lv_tns;     // [cap] per expanded level: device time in ns (%globaltimer)
+  unsigned long long* lv_probes;  // [cap] cumulative bucket reads after the level
+  unsigned long long* lv_trans;   // [cap] cumulative transitions after the level
+  uint32_t cap;
+  int stop_dl, stop_viol;
+  uint64_t max_levels;            // 0 = no limit
+  cudaGraphConditionalHandle cond, cond_big;  // go on with a level / with a large one
+};
+
 // Partitioned expansion of one level (or one batch of it): successors are
 // counted per table slice, scattered slice-major into a buffer, then probed
 // slice by slice so the probed part of the table stays in L2.
@@ -144,6 +157,8 @@ struct KernelSet {
   const void* part_scatter_fn;
   const void* part_probe_fn;
   const void* init_fn;    // for graph kernel nodes
+  const void* small_fn;   // levels of few states, many in one launch
+  size_t small_queue_bytes;  // of its dynamic shared memory
 };
 
 // Kernels for slot width W, bucket words B and group lanes G; nullptr if the

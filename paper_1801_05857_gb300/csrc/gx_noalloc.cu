@@ -116,7 +116,7 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
   const uint64_t gcache_bytes = gentries << gcache.log2_bytes;
   if (regions > nb) regions = (uint32_t)nb;
   const uint32_t warp_log2 =
-      o->warp_cache_log2 == 0xFFFFFFFFu ? (gentries ? 0u : W == 4 ? 6u : 9u) : o->warp_cache_log2;
+      o->warp_cache_log2 == 0xFFFFFFFFu ? (gentries ? 0u : W == 4 && regions > 1 ? 6u : 7u) : o->warp_cache_log2;
   const uint64_t off_ctl = 0;
   const uint64_t off_blob = align256(sizeof(gx::Ctl));
   const uint64_t off_front = align256(off_blob + 4ull * net.blob.size());
