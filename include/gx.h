@@ -173,8 +173,7 @@ typedef struct gx_explore_opts {
                                     memory (2^(n-1) for 4-word vectors, the same bytes), a hit
                                     skips find-or-put.  0 = off, 1..12 = 2^n, 0xFFFFFFFF =
                                     automatic (gx_default_opts): 2^7 unless the GPU-wide
-                                    cache below is in use (together they measured slower);
-                                    2^6 for 4-word vectors with region passes */
+                                    cache below is in use (together they measured slower) */
   float guided_scale;            /* GX_DL_GUIDED: score at which a state falls in the last
                                     bin (scores are predicted distances / max_dist); 0 = 1.0 */
   uint32_t watch;                /* 1 = safety check (Sec. 3: the negation of a safety property

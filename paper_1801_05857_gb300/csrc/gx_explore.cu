@@ -331,8 +331,8 @@ gx_status make_plan(const Net& net, const gx_explore_opts* o, Plan& P) {
   }
   // The per-warp one: more entries find more, but their shared memory costs CTAs and L1 (token
   // ring of 13 nodes: 2^6 4.19 ms, 2^7 4.18, 2^8 4.24, 2^9 4.86; 1.7e7 states of 4 words in one
-  // pass: 8.83, 8.76, 9.13, 10.3); region passes of 4-word vectors 2^6
-  P.warp_log2 = o->warp_cache_log2 == kAutoCache ? (P.gcache ? 0u : P.W == 4 && P.regions > 1 ? 6u : 7u) : o->warp_cache_log2;
+  // pass: 8.83, 8.76, 9.13, 10.3; 3.4e8 of 4 words in four passes: 2^5 190, 2^6 186, 2^7 182)
+  P.warp_log2 = o->warp_cache_log2 == kAutoCache ? (P.gcache ? 0u : 7u) : o->warp_cache_log2;
   P.cs = o->successor_buffer ? o->successor_buffer : std::min<uint64_t>(slots / 2, (1ull << 32) - 1);
   if (P.logp == 0) P.cs = 0;  // partitioned path off: no buffer
   if (P.cs >= (1ull << 32)) return fail(GX_ERR_INVALID, "successor_buffer must be below 2^32 vectors");

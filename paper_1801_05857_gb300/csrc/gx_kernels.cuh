@@ -578,8 +578,10 @@ struct ExpandOcc {
 //   done(v, n)     a lane's state and the number of its successors
 //   keep(b, h, x)  the filters before the GPU-wide cache: first bucket, hash,
 //                  successor
-// All 32 lanes call it together; returns with the queues empty.
-template <int W, int B, int G, int Batch, class T, class Desc, class Next, class Seen, class Done, class Keep>
+// All 32 lanes call it together; returns with the queues empty.  Wide: whether
+// next may give a single state at all.
+template <int W, int B, int G, int Batch, bool Wide = true, class T, class Desc, class Next, class Seen, class Done,
+          class Keep>
 __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls, const uint32_t* t,
                                               const NetBlobLayout& L, WarpQueues<W, Batch>& q, WarpStage& st,
                                               uint32_t& probes, uint32_t& err, Desc desc, Next next, Seen seen,
@@ -603,19 +605,19 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
         if ((act >> lane) & 1u) gen.emit(t, L, desc, v, q.raw + (n_raw + __popc(act & below)) * W);
         n_raw += __popc(act);
       } else if (gen.src < n_src) {
-        if (m == 1) gen.open_wide(t, L, desc, v);
+        if (Wide && m == 1) gen.open_wide(t, L, desc, v);
         else gen.open(t, L, desc, lane < m, v);
         cnt += gen.e_end - gen.e;
       } else {
         if (!more) break;
-        if (m == 1) cnt = __reduce_add_sync(FULLMASK, cnt);
+        if (Wide && m == 1) cnt = __reduce_add_sync(FULLMASK, cnt);
         if (lane < m) done(v, cnt);
         uint64_t pos = 0;
         next(pos, m);
         more = m != 0;
         if (!more) break;
-        if (lane < m || m == 1) {
-          load_words<W>(tg.frontier() + ((m == 1 ? pos : pos + lane) & tg.fmask()) * W, v);
+        if (lane < m || (Wide && m == 1)) {
+          load_words<W>(tg.frontier() + ((Wide && m == 1 ? pos : pos + lane) & tg.fmask()) * W, v);
           if (lane < m) seen(v);
         }
         cnt = 0;
@@ -689,8 +691,12 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
 
 // Up to this many states per warp are taken one by one, the whole warp generating
 // from each (token ring of 11 nodes, 22 sources: levels of 1 or 2 states a warp take
-// 15-22 us instead of 19-27; of 4 or more a warp they take longer).
+// 15-22 us instead of 19-27; of 4 or more a warp they take longer).  Not with 4-word
+// vectors: the second way of generating spills registers in the loop that the large
+// levels run (3.4e8 states in four passes 192 ms, without it 186).
 constexpr uint32_t kSingly = 2;
+template <int W>
+constexpr bool kWide = W < 4;
 
 template <int W, int B, int G>
 __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expand_kernel(const gx::ExpandArgs a) {
@@ -743,13 +749,13 @@ __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expa
   uint64_t own = s_range[0] + (uint64_t)(blockIdx.x * kWarps + (threadIdx.x >> 5)) * unit;
   const uint64_t own_end = s_range[1] - own < unit ? s_range[1] : own + unit;  // (own >= the end: no states)
   bool first = true;
-  expand_states<W, B, G, kBatch<W>>(
+  expand_states<W, B, G, kBatch<W>, kWide<W>>(
       tg, muls, t, L, queue_mem[threadIdx.x >> 5], st, probes, err, [&](uint32_t p) { return descs[p]; },
       [&](uint64_t& pos, uint32_t& m) {
         // the first states of every warp are fixed by its index, a large level's
         // further ones are claimed; a few states are taken one by one
         m = 0;
-        if (unit <= kSingly) {
+        if (kWide<W> && unit <= kSingly) {
           if (own >= s_range[1] || own >= own_end) return;
           pos = own++;
           m = 1;
