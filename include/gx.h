@@ -458,27 +458,27 @@ typedef struct gx_batch_opts {
   const uint64_t* expected_states; /* optional host array, one entry per network: network i
                                gets a table of at least expected_states[i] / 0.75 slots */
   uint32_t levels_cap;      /* BFS levels kept per network; 0 = 4096 */
-  uint32_t wide_factor;     /* an iteration with at most wide_factor x (warps of the
-                               expansion grid) states, over all networks, expands one
-                               warp per state (lane l takes successors l, l + 32, ...);
-                               0 = 4; GX_BATCH_WIDE_OFF: never */
+  uint32_t wide_factor;     /* a level with at most wide_factor x (a network's share of the
+                               warps of the expansion grid) states is expanded one state per
+                               warp, whose lanes take different sources of successors, and
+                               one that gives each of those warps less than chunk_states in
+                               smaller claims; 0 = 1; GX_BATCH_WIDE_OFF: always chunk_states */
 } gx_batch_opts;
 #define GX_BATCH_WIDE_OFF 0xFFFFFFFFu
 
 /* Make a batch from encoded networks (their encodings are copied; the
  * networks may be freed afterwards).  Host-only. */
 gx_status gx_batch_create(const gx_net* const* nets, uint32_t n, gx_batch** out);
-/* Free a batch and its cached graph (NULL is a no-op); the workspace belongs
- * to the caller. */
+/* Free a batch (NULL is a no-op); the workspace belongs to the caller. */
 void gx_batch_free(gx_batch* batch);
 
 /* Device workspace bytes for gx_batch_explore with these options. */
 gx_status gx_batch_workspace_bytes(const gx_batch* batch, const gx_batch_opts* opts, uint64_t* bytes);
 
-/* Explore every network of the batch (one graph launch).  workspace: device
+/* Explore every network of the batch (one launch: levels follow one another
+ * network by network).  workspace: device
  * pointer, 256-byte aligned, at least gx_batch_workspace_bytes bytes (required).
- * The instantiated graph is cached in the batch for the same workspace and
- * options.  Per-network results via gx_batch_stats / gx_batch_levels; the first
+ * Per-network results via gx_batch_stats / gx_batch_levels; the first
  * failing network's error is returned (the others' results stay valid).
  * Synchronises `stream`. */
 gx_status gx_batch_explore(gx_batch* batch, const gx_batch_opts* opts, void* workspace,

@@ -1,19 +1,19 @@
-// Batched exploration: many independent networks in one persistent launch
-// per BFS iteration, the iterations driven on the device by a CUDA graph with
-// a conditional WHILE node (no counterpart in the paper, which explores one
-// network at a time; the per-network work is the level expansion of Sec. 3
-// with the find-or-put of Sec. 4.1).
+// Batched exploration: many independent networks in one persistent launch (no
+// counterpart in the paper, which explores one network at a time; the
+// per-network work is the level expansion of Sec. 3 with the find-or-put of
+// Sec. 4.1).
 //
-// Graph (built once per workspace / options, relaunched per call):
-//   memset(all tables) -> init (initial vector of every network) -> advance(first)
-//   -> WHILE(any network active) { expand_all ; advance }
-// advance records each network's finished level, moves its level window,
-// computes the prefix of 32-state chunks over the active networks and sets
-// the loop condition.  expand_all is persistent: every warp claims chunks of
-// any network's current level.
+//   memset(all tables) -> init (initial vector of every network) -> expand
 //
-// Workspace: per-network descriptors | chunk prefix | claim counter |
-//            network blobs | level arrays | frontier rings | tables (contiguous)
+// Levels end network by network, not all together: a level's states are taken
+// in claims by any warp, the warp that finishes a level's last claim opens the
+// next one, and warps move on to another network meanwhile.  Nothing waits for
+// a network but its own next level.  (One launch per level of all networks, on
+// a device-side loop, left 85 of the 99 levels of the 256-network workload
+// with less than one claim per warp: 3.1 of 9.8 ms.)
+//
+// Workspace: per-network descriptors | claims | counter | network blobs |
+//            level arrays | frontier rings | tables (contiguous)
 
 #include <algorithm>
 #include <cstring>
@@ -29,11 +29,11 @@ struct BNet {
   NetBlobLayout lay;
   uint32_t* table;
   int log2nb;
-  uint32_t levels_cap;
   uint32_t* frontier;
   uint64_t fmask;
-  unsigned long long* levels;
+  // the level being expanded: its states, states per claim, claims, claims done
   unsigned long long cur_begin, cur_end, next_end;
+  unsigned int unit, chunks, done;
   unsigned long long transitions, dl_count, dl_sum, dl_xor, probes;
   unsigned int error, active, n_levels;
   int first_dl;
@@ -41,20 +41,23 @@ struct BNet {
 };
 
 struct BatchArgs {
-  BNet* nets;
+  BNet* nets;  // largest table first
   int n;
   int rounds;
-  int chunk;  // states per claimed chunk
+  uint32_t chunk;             // states per claim, at most
+  uint32_t levels_cap;
+  unsigned long long* levels; // levels_cap entries per network
+  // per network: claims taken of its level, and in the upper half how many it has
+  // (0: finished, and then at least kFinished are taken)
+  unsigned long long* claims;
+  unsigned int* active;       // networks that are not finished
+  uint32_t warps;             // of the expansion's grid
+  uint32_t wide;              // a level with at most this many states per warp that falls to
+                              // its network is claimed state by state
   Muls muls;
-  unsigned long long* prefix;  // n + 1 entries
-  unsigned long long* claim;
-  unsigned long long* iters;   // iterations of the WHILE loop so far
-  unsigned long long* unit;    // states per claim this iteration: chunk, or 1 (one warp per state)
-  unsigned long long wide_states;  // iterations with at most this many states use unit 1
-  unsigned long long max_iters;
-  cudaGraphConditionalHandle cond;
 };
 
+constexpr unsigned long long kFinished = 0x80000000ull;
 constexpr unsigned int ERR_LEVELS = 8u;  // a network needed more levels than levels_cap
 
 }  // namespace gx
@@ -81,107 +84,115 @@ __global__ void __launch_bounds__(gx::kBlock) batch_init_kernel(const BatchArgs 
   b.cur_begin = 0;
   b.cur_end = 1;
   b.next_end = 1;
+  b.unit = b.chunks = 1;
+  b.done = 0;
   b.transitions = b.dl_count = b.dl_sum = b.dl_xor = 0;
   b.probes = probes;
   b.error = r == FOP_INSERTED ? 0u : gx::ERR_TABLE_FULL;
   b.active = r == FOP_INSERTED ? 1u : 0u;
   b.first_dl = -1;
   b.n_levels = 1;
-  b.levels[0] = 1;
+  a.levels[(uint64_t)net * a.levels_cap] = 1;
+  a.claims[net] = r == FOP_INSERTED ? 1ull << 32 : gx::kFinished;
+  if (r == FOP_INSERTED) atomicAdd(a.active, 1u);
 }
 
-// One CTA: finish the level just expanded for every network, then lay out the
-// next iteration's chunks.
-__global__ void __launch_bounds__(1024) batch_advance_kernel(const BatchArgs a, int first) {
-  __shared__ unsigned long long warp_tot[32];
-  __shared__ unsigned long long carry, s_unit;
-  if (threadIdx.x == 0) carry = 0;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  // 1. close the level just expanded and count the states of the next one
-  unsigned long long states = 0;
-  for (int i = threadIdx.x; i < a.n; i += blockDim.x) {
-    BNet& b = a.nets[i];
-    if (!first && b.active) {
-      const unsigned long long fresh = b.next_end - b.cur_end;
-      if (b.dl_count > 0 && b.first_dl < 0) b.first_dl = (int)b.n_levels - 1;
-      if (fresh > 0) {
-        if (b.n_levels < b.levels_cap) b.levels[b.n_levels] = fresh;
-        else b.error |= gx::ERR_LEVELS;
-        b.n_levels += 1;
-      }
-      if (b.error || fresh == 0) {
-        b.active = 0;
-      } else {
-        b.cur_begin = b.cur_end;
-        b.cur_end = b.next_end;
-      }
+// Network i has finished the level it was expanding: record the next one and
+// open it, or finish the network.  One lane, after the level's last claim.
+__device__ __forceinline__ void batch_next_level(const BatchArgs& a, int i) {
+  BNet& b = a.nets[i];
+  using gx::kFinished;
+  const unsigned long long end = __ldcg(&b.cur_end), next = __ldcg(&b.next_end), fresh = next - end;
+  unsigned int err = __ldcg(&b.error), levels = __ldcg(&b.n_levels);
+  if (__ldcg(&b.first_dl) < 0 && __ldcg(&b.dl_count) > 0) b.first_dl = (int)levels - 1;
+  if (fresh > 0) {
+    if (levels < a.levels_cap) {
+      a.levels[(uint64_t)i * a.levels_cap + levels] = fresh;
+    } else {
+      err |= gx::ERR_LEVELS;
+      b.error = err;
     }
-    if (b.active) states += b.cur_end - b.cur_begin;
+    b.n_levels = levels + 1;
   }
-  states = warp_sum(states);
-  if (lane == 0) warp_tot[wid] = states;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    unsigned long long tot = 0;
-    for (int w = 0; w < (int)(blockDim.x / 32); ++w) tot += warp_tot[w];
-    // few states in all: give each one a warp, so that its successors' lookups overlap
-    s_unit = tot <= a.wide_states ? 1ull : (unsigned long long)a.chunk;
+  if (err || fresh == 0) {
+    b.active = 0;
+    atomicSub(a.active, 1u);
+    __threadfence();
+    atomicExch(a.claims + i, gx::kFinished);
+    return;
   }
-  __syncthreads();
-  const unsigned long long unit = s_unit;
-  // 2. claims per network and their exclusive prefix sums
-  for (int base = 0; base < a.n; base += blockDim.x) {
-    const int i = base + threadIdx.x;
-    unsigned long long chunks = 0;
-    if (i < a.n) {
-      const BNet& b = a.nets[i];
-      if (b.active) chunks = (b.cur_end - b.cur_begin + unit - 1) / unit;
-    }
-    // block-wide inclusive scan of chunks
-    unsigned long long inc = chunks;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const unsigned long long y = __shfl_up_sync(FULLMASK, inc, o);
-      if (lane >= o) inc += y;
-    }
-    if (lane == 31) warp_tot[wid] = inc;
-    __syncthreads();
-    if (wid == 0) {
-      const int nw = blockDim.x / 32;
-      unsigned long long w = lane < nw ? warp_tot[lane] : 0ull;
-      unsigned long long wi = w;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_up_sync(FULLMASK, wi, o);
-        if (lane >= o) wi += y;
+  // a network's share of the warps, were all networks at work: a level that gives each
+  // of them less than a full claim is taken in smaller ones
+  const unsigned long long act = __ldcg(a.active), share = a.warps > act ? a.warps / act : 1;
+  unsigned long long unit = (fresh + fresh / 4 + share - 1) / share;
+  if (fresh <= a.wide * share) unit = 1;
+  if (unit > a.chunk || a.wide == 0) unit = a.chunk;
+  while ((fresh + unit - 1) / unit >= kFinished) unit *= 2;  // (the halves of a claims word hold them)
+  const unsigned long long chunks = (fresh + unit - 1) / unit;
+  b.cur_begin = end;
+  b.cur_end = next;
+  b.unit = (unsigned int)unit;
+  b.chunks = (unsigned int)chunks;
+  b.done = 0;
+  __threadfence();
+  atomicExch(a.claims + i, chunks << 32);
+}
+
+// A claim of any network that has one left.  False: all networks are finished (or
+// nothing was to be had for kGiveUpNs, which is reported).  base: the networks below
+// it are finished.  A warp begins the search at a place of its own, so that the
+// networks are worked on side by side: the claims words, queue ends and table lines
+// of one network take only so many accesses at a time (256 networks: 9.2 ms; all
+// warps on the first open network 12.8, on the first 8 of them 11.2, on 32 10.6).
+constexpr unsigned long long kGiveUpNs = 20ull * 1000 * 1000 * 1000;
+
+__device__ __forceinline__ unsigned long long batch_now() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+  return t;
+}
+
+__device__ __forceinline__ bool batch_claim(const BatchArgs& a, uint32_t warp, int& base, int& net, uint32_t& c) {
+  const int lane = threadIdx.x & 31;
+  unsigned long long since = 0;
+  uint32_t nap = 128;
+  while (true) {
+    int found = -1;
+    const int span = (a.n - base + 31) / 32;
+    for (int k = 0; k < span; ++k) {
+      const int w0 = base + 32 * (int)((k + warp / 32) % span);
+      const unsigned long long x = w0 + lane < a.n ? __ldcg(a.claims + w0 + lane) : gx::kFinished;
+      const bool fin = (x >> 32) == 0;
+      if (__ballot_sync(FULLMASK, fin) == FULLMASK) {
+        if (w0 == base) base += 32;
+        continue;
       }
-      if (lane < nw) warp_tot[lane] = wi - w;
+      const uint32_t open = __ballot_sync(FULLMASK, (uint32_t)x < (uint32_t)(x >> 32));
+      if (open == 0) continue;
+      found = w0 + (int)__fns(open, 0, warp % __popc(open) + 1);
+      break;
     }
-    __syncthreads();
-    const unsigned long long ex = carry + warp_tot[wid] + inc - chunks;
-    if (i < a.n) a.prefix[i] = ex;
-    __syncthreads();
-    if (threadIdx.x == blockDim.x - 1) carry = ex + chunks;
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) {
-    // iteration guard: every active network gains one level per iteration, so
-    // more than max_iters iterations cannot happen; stop the loop regardless
-    const unsigned long long it = first ? 0ull : *a.iters + 1;
-    *a.iters = it;
-    bool more = carry > 0;
-    if (more && it >= a.max_iters) {
-      for (int i = 0; i < a.n; ++i)
-        if (a.nets[i].active) {
-          a.nets[i].error |= gx::ERR_LEVELS;
-          a.nets[i].active = 0;
-        }
-      more = false;
+    if (found >= 0) {
+      unsigned long long x = 0;
+      if (lane == 0) x = atomicAdd(a.claims + found, 1ull);
+      x = __shfl_sync(FULLMASK, x, 0);
+      if ((uint32_t)x < (uint32_t)(x >> 32)) {
+        net = found;
+        c = (uint32_t)x;
+        return true;
+      }
+      continue;  // taken by others
     }
-    a.prefix[a.n] = carry;
-    *a.claim = 0;
-    *a.unit = unit;
-    cudaGraphSetConditional(a.cond, more ? 1u : 0u);
+    if (base >= a.n) return false;
+    const unsigned long long now = __shfl_sync(FULLMASK, batch_now(), 0);
+    if (since == 0) since = now;
+    if (now - since > kGiveUpNs) {
+      for (int i = base + lane; i < a.n; i += 32)
+        if ((__ldcg(a.claims + i) >> 32) != 0) atomicOr(&a.nets[i].error, gx::ERR_SPIN);
+      return false;
+    }
+    __nanosleep(nap);
+    if (nap < 2048) nap *= 2;
   }
 }
 
@@ -193,7 +204,7 @@ constexpr int kBatchCacheLog2 = 8;
 
 // The network a warp is working on, staged in shared memory when the warp
 // moves to it, so that its layout and table pointers take no registers in the
-// inner loop.
+// inner loop, with the level it is working on.
 struct WarpNet {
   NetBlobLayout lay;
   uint32_t* table;
@@ -201,6 +212,7 @@ struct WarpNet {
   uint32_t* frontier;
   uint64_t fmask, cur_begin, cur_end;
   int log2nb;
+  uint32_t unit, chunks;
 };
 
 struct SmemTarget {
@@ -244,10 +256,6 @@ struct __align__(16) BatchSmem {
 
 template <int W, int B, int G>
 __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch_expand_kernel(const BatchArgs a) {
-  // a fixed full-size grid: CTAs beyond what this iteration's claims need leave
-  // before claiming (in the batch's long tail most iterations have few)
-  const unsigned long long total = __ldcg(a.prefix + a.n);
-  if ((unsigned long long)blockIdx.x * (gx::kBlock / 32) >= total) return;
   extern __shared__ __align__(16) unsigned char bsm[];
   BatchSmem<W>& S = *reinterpret_cast<BatchSmem<W>*>(bsm);
   for (int i = threadIdx.x; i < a.rounds; i += blockDim.x) S.muls[i] = a.muls.m[i];
@@ -260,58 +268,63 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
   WarpStage st{S.stage[wid], 0};
   WarpCache cache{W <= 2 ? S.cache[wid] : nullptr, (1u << kBatchCacheLog2) - 1u};
   const SmemTarget tg{&wn, a.rounds};
-  const uint32_t unit = (uint32_t)__ldcg(a.unit);  // states per claim this iteration
   const uint32_t* t = nullptr;
-  auto claim = [&]() {
-    unsigned long long c = 0;
-    if (lane == 0) c = atomicAdd(a.claim, 1ull);
-    return __shfl_sync(FULLMASK, c, 0);
-  };
-  unsigned long long c = claim();
-  while (c < total) {
-    // the network whose claims contain c: largest i with prefix[i] <= c
-    int lo = 0, hi = a.n - 1;
-    while (lo < hi) {
-      const int mid = (lo + hi + 1) >> 1;
-      if (__ldcg(a.prefix + mid) <= c) lo = mid;
-      else hi = mid - 1;
+  int net = -1, base = 0;
+  while (true) {
+    int at_net;
+    uint32_t c;
+    if (!batch_claim(a, blockIdx.x * (gx::kBlock / 32) + wid, base, at_net, c)) break;
+    BNet& b = a.nets[at_net];
+    if (at_net != net) {
+      // stage the network; the cache holds one network's vectors at a time
+      net = at_net;
+      t = b.blob;
+      if (lane == 0) {
+        wn.lay = b.lay;
+        wn.table = b.table;
+        wn.next_end = &b.next_end;
+        wn.frontier = b.frontier;
+        wn.fmask = b.fmask;
+        wn.log2nb = b.log2nb;
+      }
+      if (W <= 2)
+        for (uint32_t i = lane; i < (uint32_t)BatchSmem<W>::kCache; i += 32) S.cache[wid][i] = 0u;
+      __syncwarp();
+      if (wn.lay.n_procs <= (uint32_t)kWarpDescs && lane < wn.lay.n_procs) descs[lane] = proc_desc(t, wn.lay, lane);
     }
-    BNet& b = a.nets[lo];
-    const unsigned long long c0 = __ldcg(a.prefix + lo), c1 = __ldcg(a.prefix + lo + 1);
-    // stage the network; the cache holds one network's vectors at a time
-    t = b.blob;
+    // the level (it cannot end before this claim is done)
+    __threadfence();
     if (lane == 0) {
-      wn.lay = b.lay;
-      wn.table = b.table;
-      wn.next_end = &b.next_end;
-      wn.frontier = b.frontier;
-      wn.fmask = b.fmask;
-      wn.cur_begin = b.cur_begin;
-      wn.cur_end = b.cur_end;
-      wn.log2nb = b.log2nb;
+      wn.cur_begin = __ldcg(&b.cur_begin);
+      wn.cur_end = __ldcg(&b.cur_end);
+      wn.unit = __ldcg(&b.unit);
+      wn.chunks = __ldcg(&b.chunks);
     }
-    if (W <= 2)
-      for (uint32_t i = lane; i < (uint32_t)BatchSmem<W>::kCache; i += 32) S.cache[wid][i] = 0u;
     __syncwarp();
     const NetBlobLayout& L = wn.lay;
     const bool staged = L.n_procs <= (uint32_t)kWarpDescs;
-    if (staged && lane < L.n_procs) descs[lane] = proc_desc(t, L, lane);
-    __syncwarp();
     uint32_t probes = 0, err = 0;
     unsigned long long trans = 0;
     uint64_t pos = 0, end = 0;  // what is left of the claim
-    bool held = true;           // c is a claim of this network that has not been started
+    bool held = true;           // c is a claim that has not been started
+    uint32_t taken = 1;
     expand_states<W, B, G, 32>(
         tg, muls, t, L, S.queues[wid], st, probes, err,
         [&](uint32_t p) { return staged ? descs[p] : proc_desc(t, L, p); },
         [&](uint64_t& at, uint32_t& m) {
           m = 0;
           if (pos == end) {
-            if (!held) c = claim();
-            held = c < c1;
-            if (!held) return;  // another network's, or none are left
-            pos = wn.cur_begin + (c - c0) * unit;
-            end = pos + unit < wn.cur_end ? pos + unit : wn.cur_end;
+            if (!held) {
+              if (lane == 0) {
+                c = (uint32_t)__ldcg(a.claims + net);
+                if (c < wn.chunks) c = (uint32_t)atomicAdd(a.claims + net, 1ull);
+              }
+              c = __shfl_sync(FULLMASK, c, 0);
+              if (c >= wn.chunks) return;
+              ++taken;
+            }
+            pos = wn.cur_begin + (uint64_t)c * wn.unit;
+            end = pos + wn.unit < wn.cur_end ? pos + wn.unit : wn.cur_end;
             held = false;
           }
           at = pos;
@@ -337,6 +350,13 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
       if (tr) atomicAdd(&b.transitions, tr);
       if (pr) atomicAdd(&b.probes, pr);
       if (err) atomicOr(&b.error, err);
+    }
+    // (the warp's last use of the level: its states, counts and new states come before)
+    __threadfence();  // before the level can be seen as done
+    __syncwarp();
+    if (lane == 0 && atomicAdd(&b.done, taken) + taken == wn.chunks) {
+      __threadfence();
+      batch_next_level(a, net);
     }
     __syncwarp();
   }
@@ -391,9 +411,10 @@ struct BatchPlan {
   int W = 0, B = 0, G = 0, rounds = 0, chunk = 0;
   uint32_t levels_cap = 0, wide = 0;
   std::vector<uint64_t> slots, fcap;
-  uint64_t off_nets = 0, off_prefix = 0, off_claim = 0, off_blobs = 0, off_levels = 0,
+  uint64_t off_nets = 0, off_claims = 0, off_active = 0, off_blobs = 0, off_levels = 0,
            off_fronts = 0, off_tables = 0, table_words = 0, total = 0;
   std::vector<uint64_t> blob_off, front_off, table_off;
+  std::vector<uint32_t> order;  // networks by decreasing table size
   BatchKernels k{};
 };
 
@@ -408,17 +429,8 @@ struct gx_batch {
   std::vector<gx::BNet> res;
   std::vector<std::vector<uint64_t>> levels;
   double gpu_ms = 0;
-  // cached graph
-  cudaGraphExec_t exec = nullptr;
-  cudaGraph_t graph = nullptr;
-  void* exec_ws = nullptr;
-  std::vector<uint64_t> exec_key;
   std::vector<uint64_t> last_plan_slots;
   uint32_t last_W = 0, last_B = 0, last_G = 0, last_rounds = 0;
-  ~gx_batch() {
-    if (exec) cudaGraphExecDestroy(exec);
-    if (graph) cudaGraphDestroy(graph);
-  }
 };
 
 namespace gx {
@@ -440,7 +452,7 @@ gx_status batch_plan(const gx_batch* h, const gx_batch_opts* o, BatchPlan& P) {
     return fail(GX_ERR_INVALID, "no batch kernel for bucket_words " + std::to_string(P.B) + ", group_lanes " +
                                     std::to_string(P.G) + " with " + std::to_string(P.W) + "-word slots");
   P.levels_cap = o->levels_cap ? o->levels_cap : 4096;
-  P.wide = o->wide_factor ? o->wide_factor : 4u;
+  P.wide = o->wide_factor ? o->wide_factor : 1u;
   P.slots.resize(n);
   P.fcap.resize(n);
   for (uint32_t i = 0; i < n; ++i) {
@@ -455,10 +467,10 @@ gx_status batch_plan(const gx_batch* h, const gx_batch_opts* o, BatchPlan& P) {
   uint64_t off = 0;
   P.off_nets = off;
   off = a256(off + sizeof(BNet) * n);
-  P.off_prefix = off;
+  P.off_claims = off;
   off = a256(off + 8ull * (n + 1));
-  P.off_claim = off;
-  off = a256(off + 24);  // claim counter, iteration counter, states per claim
+  P.off_active = off;
+  off = a256(off + 24);
   P.off_blobs = off;
   P.blob_off.resize(n);
   for (uint32_t i = 0; i < n; ++i) {
@@ -481,94 +493,10 @@ gx_status batch_plan(const gx_batch* h, const gx_batch_opts* o, BatchPlan& P) {
   }
   P.table_words = (off - P.off_tables) / 4;
   P.total = a256(off);
-  return GX_OK;
-}
-
-gx_status build_graph(gx_batch* h, const BatchPlan& P, void* ws, int sms) {
-  if (h->exec) {
-    cudaGraphExecDestroy(h->exec);
-    h->exec = nullptr;
-  }
-  if (h->graph) {
-    cudaGraphDestroy(h->graph);
-    h->graph = nullptr;
-  }
-  char* base = static_cast<char*>(ws);
-  const int n = (int)h->nets.size();
-  cudaGraph_t g;
-  GB_CUDA(cudaGraphCreate(&g, 0));
-  h->graph = g;
-  cudaGraphConditionalHandle cond;
-  GB_CUDA(cudaGraphConditionalHandleCreate(&cond, g, 1, cudaGraphCondAssignDefault));
-
-  int per_sm = 0;
-  GB_CUDA(cudaFuncSetAttribute(P.k.expand, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.k.smem));
-  GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, P.k.expand, kBlock, P.k.smem));
-  const int grid = sms * std::max(per_sm, 1);
-
-  BatchArgs a{};
-  a.nets = reinterpret_cast<BNet*>(base + P.off_nets);
-  a.n = n;
-  a.rounds = P.rounds;
-  a.chunk = P.chunk;
-  hash_multipliers(a.muls.m, kMaxRounds);
-  a.prefix = reinterpret_cast<unsigned long long*>(base + P.off_prefix);
-  a.claim = reinterpret_cast<unsigned long long*>(base + P.off_claim);
-  a.iters = a.claim + 1;
-  a.unit = a.claim + 2;
-  a.wide_states = P.wide == GX_BATCH_WIDE_OFF ? 0ull : (unsigned long long)P.wide * grid * (kBlock / 32);
-  a.max_iters = (unsigned long long)P.levels_cap + 1;
-  a.cond = cond;
-
-  // memset of every table
-  cudaGraphNode_t mset;
-  cudaMemsetParams mp{};
-  mp.dst = base + P.off_tables;
-  mp.value = 0;
-  mp.elementSize = 4;
-  mp.width = P.table_words;
-  mp.height = 1;
-  mp.pitch = 0;
-  GB_CUDA(cudaGraphAddMemsetNode(&mset, g, nullptr, 0, &mp));
-
-  auto add_kernel = [&](cudaGraph_t gr, const cudaGraphNode_t* deps, size_t nd, const void* fn,
-                        dim3 grid, dim3 block, size_t smem, void** args, cudaGraphNode_t* out) -> cudaError_t {
-    cudaKernelNodeParams kp{};
-    kp.func = const_cast<void*>(fn);
-    kp.gridDim = grid;
-    kp.blockDim = block;
-    kp.sharedMemBytes = (unsigned)smem;
-    kp.kernelParams = args;
-    return cudaGraphAddKernelNode(out, gr, deps, nd, &kp);
-  };
-  void* args_a[] = {&a};
-  int first1 = 1, first0 = 0;
-  void* args_adv1[] = {&a, &first1};
-  void* args_adv0[] = {&a, &first0};
-
-  cudaGraphNode_t init, adv1;
-  const int per_block = kBlock / 32;
-  GB_CUDA(add_kernel(g, &mset, 1, P.k.init, dim3((n + per_block - 1) / per_block), dim3(kBlock), 0, args_a, &init));
-  GB_CUDA(add_kernel(g, &init, 1, reinterpret_cast<const void*>(&gxd::batch_advance_kernel), dim3(1),
-                     dim3(1024), 0, args_adv1, &adv1));
-
-  cudaGraphNodeParams cp{};
-  cp.type = cudaGraphNodeTypeConditional;
-  cp.conditional.handle = cond;
-  cp.conditional.type = cudaGraphCondTypeWhile;
-  cp.conditional.size = 1;
-  cudaGraphNode_t cnode;
-  GB_CUDA(cudaGraphAddNode(&cnode, g, &adv1, nullptr, 1, &cp));
-  cudaGraph_t body = cp.conditional.phGraph_out[0];
-
-  cudaGraphNode_t ex, adv0;
-  GB_CUDA(add_kernel(body, nullptr, 0, P.k.expand, dim3(grid), dim3(kBlock), P.k.smem, args_a, &ex));
-  GB_CUDA(add_kernel(body, &ex, 1, reinterpret_cast<const void*>(&gxd::batch_advance_kernel), dim3(1),
-                     dim3(1024), 0, args_adv0, &adv0));
-  cudaGraphExec_t exec;
-  GB_CUDA(cudaGraphInstantiate(&exec, g, 0));
-  h->exec = exec;
-  h->exec_ws = ws;
+  // large networks first: the levels of the last one left have the GPU to themselves
+  P.order.resize(n);
+  for (uint32_t i = 0; i < n; ++i) P.order[i] = i;
+  std::stable_sort(P.order.begin(), P.order.end(), [&](uint32_t x, uint32_t y) { return P.slots[x] > P.slots[y]; });
   return GX_OK;
 }
 
@@ -586,11 +514,17 @@ gx_status run_batch(gx_batch* h, const gx_batch_opts* o, void* ws, uint64_t ws_b
   GB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   char* base = static_cast<char*>(ws);
 
+  int per_sm = 0;
+  GB_CUDA(cudaFuncSetAttribute(P.k.expand, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.k.smem));
+  GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, P.k.expand, kBlock, P.k.smem));
+  const int grid = sms * std::max(per_sm, 1);
+
   // descriptors and tables
   std::vector<BNet> bn(n);
-  for (int i = 0; i < n; ++i) {
+  for (int k = 0; k < n; ++k) {
+    const uint32_t i = P.order[k];
     const Net& net = h->nets[i];
-    BNet& b = bn[i];
+    BNet& b = bn[k];
     std::memset(&b, 0, sizeof(b));
     b.blob = reinterpret_cast<const uint32_t*>(base + P.blob_off[i]);
     b.lay = net.lay;
@@ -599,33 +533,39 @@ gx_status run_batch(gx_batch* h, const gx_batch_opts* o, void* ws, uint64_t ws_b
     int l = 0;
     while ((1ull << l) < nb) ++l;
     b.log2nb = l;
-    b.levels_cap = P.levels_cap;
     b.frontier = reinterpret_cast<uint32_t*>(base + P.front_off[i]);
     b.fmask = P.fcap[i] - 1;
-    b.levels = reinterpret_cast<unsigned long long*>(base + P.off_levels) + (uint64_t)i * P.levels_cap;
     // the initial vector, padded to the batch's slot width (padding words carry only the tag)
     for (int w = 0; w < 4; ++w) b.init_vec[w] = w < P.W ? (net.init_vec[w] | kTag) : 0u;
     GB_CUDA(cudaMemcpyAsync(base + P.blob_off[i], net.blob.data(), 4 * net.blob.size(), cudaMemcpyHostToDevice, st));
   }
   GB_CUDA(cudaMemcpyAsync(base + P.off_nets, bn.data(), sizeof(BNet) * n, cudaMemcpyHostToDevice, st));
 
-  // everything the graph holds by value: kernels, launch shapes, and where the
-  // tables it clears start and end (they move when per-network sizes change)
-  std::vector<uint64_t> key{(uint64_t)P.B, (uint64_t)P.G, (uint64_t)P.rounds, (uint64_t)P.chunk,
-                            P.levels_cap, P.total, P.off_tables, P.table_words, P.wide};
-  if (!h->exec || h->exec_ws != ws || h->exec_key != key) {
-    s = build_graph(h, P, ws, sms);
-    if (s != GX_OK) return s;
-    h->exec_key = key;
-  }
+  BatchArgs a{};
+  a.nets = reinterpret_cast<BNet*>(base + P.off_nets);
+  a.n = n;
+  a.rounds = P.rounds;
+  a.chunk = (uint32_t)P.chunk;
+  a.levels_cap = P.levels_cap;
+  a.levels = reinterpret_cast<unsigned long long*>(base + P.off_levels);
+  a.claims = reinterpret_cast<unsigned long long*>(base + P.off_claims);
+  a.active = reinterpret_cast<unsigned int*>(base + P.off_active);
+  a.warps = (uint32_t)grid * (kBlock / 32);
+  a.wide = P.wide == GX_BATCH_WIDE_OFF ? 0u : P.wide;
+  hash_multipliers(a.muls.m, kMaxRounds);
+  void* args[] = {&a};
+  const int per_block = kBlock / 32;
+
   cudaEvent_t e0, e1;
   GB_CUDA(cudaEventCreate(&e0));
   GB_CUDA(cudaEventCreate(&e1));
   GB_CUDA(cudaEventRecord(e0, st));
-  GB_CUDA(cudaGraphLaunch(h->exec, st));
+  GB_CUDA(cudaMemsetAsync(base + P.off_tables, 0, 4 * P.table_words, st));
+  GB_CUDA(cudaMemsetAsync(a.active, 0, sizeof(unsigned int), st));
+  GB_CUDA(cudaLaunchKernel(P.k.init, dim3((n + per_block - 1) / per_block), dim3(kBlock), args, 0, st));
+  GB_CUDA(cudaLaunchKernel(P.k.expand, dim3(grid), dim3(kBlock), args, P.k.smem, st));
   GB_CUDA(cudaEventRecord(e1, st));
-  h->res.resize(n);
-  GB_CUDA(cudaMemcpyAsync(h->res.data(), base + P.off_nets, sizeof(BNet) * n, cudaMemcpyDeviceToHost, st));
+  GB_CUDA(cudaMemcpyAsync(bn.data(), base + P.off_nets, sizeof(BNet) * n, cudaMemcpyDeviceToHost, st));
   GB_CUDA(cudaStreamSynchronize(st));
   float ms = 0;
   cudaEventElapsedTime(&ms, e0, e1);
@@ -635,11 +575,16 @@ gx_status run_batch(gx_batch* h, const gx_batch_opts* o, void* ws, uint64_t ws_b
   std::vector<unsigned long long> lv((uint64_t)n * P.levels_cap);
   GB_CUDA(cudaMemcpyAsync(lv.data(), base + P.off_levels, 8ull * lv.size(), cudaMemcpyDeviceToHost, st));
   GB_CUDA(cudaStreamSynchronize(st));
+  h->res.resize(n);
   h->levels.assign(n, {});
   gx_status rs = GX_OK;
+  std::vector<uint32_t> slot(n);  // where network i is on the device
+  for (int k = 0; k < n; ++k) slot[P.order[k]] = (uint32_t)k;
   for (int i = 0; i < n; ++i) {
+    h->res[i] = bn[slot[i]];
     const uint32_t k = std::min<uint32_t>(h->res[i].n_levels, P.levels_cap);
-    h->levels[i].assign(lv.begin() + (uint64_t)i * P.levels_cap, lv.begin() + (uint64_t)i * P.levels_cap + k);
+    const auto first = lv.begin() + (uint64_t)slot[i] * P.levels_cap;
+    h->levels[i].assign(first, first + k);
     if (h->res[i].error && rs == GX_OK) {
       const unsigned e = h->res[i].error;
       rs = (e & ERR_TABLE_FULL)  ? fail(GX_ERR_TABLE_FULL, "network " + std::to_string(i) + ": hash table full")

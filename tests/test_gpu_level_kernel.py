@@ -87,3 +87,24 @@ def test_batched_networks_with_more_processes_than_lanes(cuda, n_procs):
         s = gx.batch_stats(b, i)
         assert (s["states"], s["transitions"], gx.batch_levels(b, i)) == (r.states, r.transitions, r.levels)
         assert (s["deadlock_count"], s["deadlock_sum"]) == (r.deadlock_count, r.deadlock_sum)
+
+
+@pytest.mark.parametrize("wide", [0, gx.BATCH_WIDE_OFF])
+@pytest.mark.parametrize("count", [1, 32, 33, 70])
+def test_batches_of_any_number_of_networks(cuda, count, wide):
+    """Levels end network by network: one network alone, a full window of the search for
+    open networks and one more; networks of very different depth and size, large ones last."""
+    nets = [inputs.token_ring(3 + i % 6) if i % 2 else inputs.random_network(i, 4 + i % 4, 5, 0, 2, 6, n_sync=2, parties=2)
+            for i in range(count)]
+    b = gx.batch_create(nets)
+    o = gx.batch_opts(table_slots=1 << 16, hash_rounds=32, wide_factor=wide)
+    ws = gx.batch_alloc_workspace(b, o)
+    for _ in range(2):
+        gx.batch_explore(b, o, ws)
+        for i, net in enumerate(nets):
+            r = oracle.explore(net)
+            s = gx.batch_stats(b, i)
+            assert s["complete"] == 1
+            assert (s["states"], s["transitions"], s["explored"]) == (r.states, r.transitions, r.explored)
+            assert (s["deadlock_count"], s["deadlock_sum"]) == (r.deadlock_count, r.deadlock_sum)
+            assert (s["first_deadlock_level"], gx.batch_levels(b, i)) == (r.first_deadlock_level, r.levels)
