@@ -209,10 +209,10 @@ typedef struct gx_explore_opts {
   uint32_t global_cache_log2;    /* GPU-wide cache of recently seen vectors: 2^n
                                     direct-mapped entries in the workspace, cleared at the
                                     start of each search and small enough to stay in L2.
-                                    An entry holds a vector exactly: its fields packed side by
-                                    side (b <= 64 bits; no effect on vectors with more) are
-                                    mixed by a bijection, n of the bits are the entry's index
-                                    and the other b - n are stored, in 16, 32 or 64 bits.  A
+                                    An entry holds a vector exactly: of its fields packed side
+                                    by side (b <= 64 bits; no effect on vectors with more) the
+                                    low b - n bits are stored, in 16, 32 or 64 bits, and the
+                                    others, mixed with a hash of those, are its index.  A
                                     vector goes in after its find-or-put found or inserted it,
                                     so a hit is a known state and skips the table probe; most
                                     successors of a level lead into the levels just before and
@@ -222,7 +222,7 @@ typedef struct gx_explore_opts {
                                     least 2^26 slots with one lane per bucket (group_lanes 1),
                                     for 4-word vectors only in one region pass; else off.  Mid
                                     network (b = 40): 0.21 bucket reads per successor and
-                                    13.7 ms; with 2^23 entries 0.38 and 17.5 ms */
+                                    12.3 ms (2^23 entries: 0.38, 3.8 ms more) */
   uint32_t guided_fused;         /* GX_DL_GUIDED: 1 = score the states an iteration inserts
                                     inside its expansion kernel (each CTA keeps them in shared
                                     memory and scores 128 at a time on the tensor cores), 0 =

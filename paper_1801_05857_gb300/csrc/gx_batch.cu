@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
             atomicXor(&b.dl_xor, (unsigned long long)h);
           }
         },
-        [&](uint64_t, uint64_t hh, const uint32_t(&x)[W]) { return !(cache.base && cache.template seen<W>(hh, x)); });
+        [&](const uint32_t(&x)[W]) { return !(cache.base && cache.template seen<W>(x)); });
     st.flush<W>(tg, err);
     const unsigned long long tr = warp_sum(trans);
     const unsigned long long pr = warp_sum((unsigned long long)probes);

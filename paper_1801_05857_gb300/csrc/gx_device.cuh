@@ -151,9 +151,6 @@ __device__ __forceinline__ bool cas_slot(uint32_t* p, const uint32_t (&v)[W], ui
 // Hash of a state vector: two odd multiplications with the upper half folded
 // into the lower one between them (a bucket comes from one more, bucket_of, so
 // every bit of the vector reaches its top bits), without vec_hash's finaliser.
-// The low bits are left out for the hash-constant set's number; the caches of
-// seen vectors take their index from the upper half.
-constexpr uint64_t kSeqMask = kMaxRounds - 1;
 template <int W>
 __device__ __forceinline__ uint64_t state_hash(const uint32_t (&v)[W]) {
   uint64_t x = v[0];
@@ -161,8 +158,7 @@ __device__ __forceinline__ uint64_t state_hash(const uint32_t (&v)[W]) {
   if constexpr (W == 4) x += ((uint64_t)v[2] | ((uint64_t)v[3] << 32)) * 0xD6E8FEB86659FD93ull;
   x *= 0xBF58476D1CE4E5B9ull;
   x ^= x >> 32;
-  x *= 0x94D049BB133111EBull;
-  return x & ~kSeqMask;
+  return x * 0x94D049BB133111EBull;
 }
 
 // The bucket that hash-constant set k gives hash h.

@@ -46,9 +46,10 @@ bool cache_layout(const Net& net, uint32_t log2_entries, SeenCache& c) {
   uint32_t bits = 0;
   if (!cache_key(net, c.word_at, bits)) return false;
   c.shift = bits > log2_entries ? bits - log2_entries : 0;
-  c.mask = bits < 64 ? (1ull << bits) - 1 : ~0ull;
   c.tag_mask = c.shift < 64 ? (1ull << c.shift) - 1 : ~0ull;
-  c.half = (bits + 1) / 2;
+  c.mask = (uint32_t)((1ull << log2_entries) - 1);
+  c.mix_shift = log2_entries ? 32 - log2_entries : 31;  // (2^0 entries: every index is 0)
+  if (c.shift > 63) c.shift = 63;
   c.log2_bytes = cache_entry_log2(bits, log2_entries);
   return true;
 }

@@ -335,21 +335,25 @@ struct WarpCache {
   uint32_t* base;  // 2^log2 entries of W words, or nullptr
   uint32_t mask;
   template <int W>
-  __device__ __forceinline__ bool seen(uint64_t h, const uint32_t (&v)[W]) const {
+  __device__ __forceinline__ bool seen(const uint32_t (&v)[W]) const {
+    uint32_t m = v[0] * 0x9E3779B1u;
+    if constexpr (W >= 2) m += v[1] * 0x85EBCA77u;
+    if constexpr (W == 4) m += v[2] * 0xC2B2AE3Du + v[3] * 0x27D4EB2Fu;
+    const uint32_t i = (m >> 20) & mask;  // (2^12 entries at most)
     if constexpr (W == 1) {
-      uint32_t* e = base + ((uint32_t)(h >> 40) & mask);
+      uint32_t* e = base + i;
       if (*e == v[0]) return true;
       *e = v[0];
       return false;
     } else if constexpr (W == 2) {
-      unsigned long long* e = reinterpret_cast<unsigned long long*>(base) + ((uint32_t)(h >> 40) & mask);
+      unsigned long long* e = reinterpret_cast<unsigned long long*>(base) + i;
       const unsigned long long x = (unsigned long long)v[0] | ((unsigned long long)v[1] << 32);
       if (*e == x) return true;
       *e = x;
       return false;
     } else {
       static_assert(W == 4, "slot width");
-      uint4* e = reinterpret_cast<uint4*>(base) + ((uint32_t)(h >> 40) & mask);
+      uint4* e = reinterpret_cast<uint4*>(base) + i;
       const uint4 c = *e;
       if (c.x == v[0] && c.y == v[1] && c.z == v[2] && c.w == v[3]) return true;
       *e = make_uint4(v[0], v[1], v[2], v[3]);
@@ -368,8 +372,14 @@ struct WarpCache {
 // bytes per bucket read, entry missed in L2 or entry written back), so entries
 // are as small as the vectors allow: the 62M-state mid network (40 bits)
 // takes 2^25 entries of 16 bits in the 64 MiB that held 2^23 of 64 bits.
+// Every successor is looked up, four in five are found, and the instructions
+// of that are what is left: so the key is only split and one half xored with a
+// hash of the other (a bijection whatever the hash is), and the table's 64-bit hash
+// is left to those that go on to it.  Mid network 13.8 -> 12.3 ms, deadlock search of
+// 4.5e7 states 12.9 -> 11.7, random network of 1.1e8 states (64 bits) 43.1 -> 40.2.
+// A hash of one multiplication left 11 % more misses in the last (42.0 ms).
 struct SeenEntry {
-  uint64_t index;
+  uint32_t index;
   unsigned long long content;  // 0: this vector is never cached
 };
 template <int W>
@@ -378,18 +388,17 @@ __device__ __forceinline__ SeenEntry seen_entry(const gx::SeenCache& c, const ui
 #pragma unroll
   for (int w = 1; w < W; ++w)
     if (c.word_at[w - 1] < 64) y |= (uint64_t)(v[w] & ~kTag) << c.word_at[w - 1];
-  // a bijection of the numbers below 2^bits: odd multiplications and a xor-shift
-  y = (y * 0xD6E8FEB86659FD93ull) & c.mask;
-  y ^= y >> c.half;
-  y = (y * 0x9E3779B97F4A7C15ull) & c.mask;
+  const uint64_t lo = y & c.tag_mask;
+  uint32_t mix = (uint32_t)lo * 0x9E3779B1u + (uint32_t)(lo >> 32) * 0x85EBCA77u;
+  mix = (mix ^ (mix >> 15)) * 0xC2B2AE3Du;
   SeenEntry e;
-  e.index = c.shift < 64 ? y >> c.shift : 0ull;
-  e.content = (y & c.tag_mask) + 1;
+  e.index = ((uint32_t)(y >> c.shift) ^ (mix >> c.mix_shift)) & c.mask;
+  e.content = lo + 1;
   if (c.log2_bytes == 1) e.content &= 0xFFFFull;  // (the one content that does not fit becomes 0)
   else if (c.log2_bytes == 2) e.content &= 0xFFFFFFFFull;
   return e;
 }
-__device__ __forceinline__ unsigned long long seen_get(const gx::SeenCache& c, uint64_t i) {
+__device__ __forceinline__ unsigned long long seen_get(const gx::SeenCache& c, uint32_t i) {
   if (c.log2_bytes == 1) return __ldcg(static_cast<const unsigned short*>(c.base) + i);
   if (c.log2_bytes == 2) return __ldcg(static_cast<const unsigned int*>(c.base) + i);
   return __ldcg(static_cast<const unsigned long long*>(c.base) + i);
@@ -540,8 +549,8 @@ struct WarpGen {
 //         lanes; hashing and the filters (region, caches) then run on a batch of
 //         32 or 64 successors, so that a lane's cache lookups are in flight
 //         together.
-//   kept  successors that passed the filters, with their hashes and the
-//         hash-constant set to try.  32 of them at a time read one bucket each;
+//   kept  successors that passed the filters, with the hash-constant set to try;
+//         only these are hashed.  32 of them at a time read one bucket each;
 //         those that met a full one go back with the next set, so a lane in a
 //         crowded part of the table holds up no other.
 // Successors filtered at a time.  4-word vectors: one per lane, because shared
@@ -556,7 +565,7 @@ struct WarpQueues {
   static constexpr int kSlots = Batch + 32;  // at most 31 left of a batch of 32, or Batch - 1, before the next come in
   uint32_t raw[kSlots * W];
   uint32_t kept[kSlots * W];
-  unsigned long long hash[kSlots];  // state_hash of the kept vectors | hash-constant set
+  uint8_t seq[kSlots];  // hash-constant set to try for each of the kept ones
 };
 
 // Resident CTAs per SM the level kernel is compiled for (register budget): a
@@ -576,8 +585,7 @@ struct ExpandOcc {
 //   desc(p)        the process descriptors (proc_desc)
 //   seen(v)        a lane's state, once, when it is taken
 //   done(v, n)     a lane's state and the number of its successors
-//   keep(b, h, x)  the filters before the GPU-wide cache: first bucket, hash,
-//                  successor
+//   keep(x)        the filters before the GPU-wide cache, of a successor
 // All 32 lanes call it together; returns with the queues empty.  Wide: whether
 // next may give a single state at all.
 template <int W, int B, int G, int Batch, bool Wide = true, class T, class Desc, class Next, class Seen, class Done,
@@ -631,13 +639,11 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
       constexpr int K = Batch / 32;
       bool on[K];
       uint32_t x[K][W];
-      uint64_t hh[K];
 #pragma unroll
       for (int i = 0; i < K; ++i) {
         const int at = (int)lane + 32 * i;
         load_vec<W>(q.raw + (n_raw + at) * W, x[i]);  // (past the k-th entry: not used)
-        hh[i] = state_hash<W>(x[i]);
-        on[i] = at < k && keep(bucket_of(hh[i], muls[0], tg.log2nb()), hh[i], x[i]);
+        on[i] = at < k && keep(x[i]);
       }
       if (tg.gcache().base) {
         SeenEntry e[K];
@@ -656,7 +662,7 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
         if (on[i]) {
           const int at = n_kept + __popc(km & below);
           store_vec<W>(q.kept + at * W, x[i]);
-          q.hash[at] = hh[i];
+          q.seq[at] = 0;
         }
         n_kept += __popc(km);
       }
@@ -669,9 +675,8 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
       const bool has = (int)lane < k;
       uint32_t x[W];
       load_vec<W>(q.kept + (n_kept + lane) * W, x);  // (past the k-th entry: not used)
-      const uint64_t hn = q.hash[n_kept + lane];
-      const uint32_t n = (uint32_t)(hn & kSeqMask);
-      bool again = resolve_lanes<W, B, G>(tg, muls, has, x, hn & ~kSeqMask, n, probes, err, st) < 0 && has;
+      const uint32_t n = has ? q.seq[n_kept + lane] : 0u;
+      bool again = resolve_lanes<W, B, G>(tg, muls, has, x, state_hash<W>(x), n, probes, err, st) < 0 && has;
       if (again && n + 1 == (uint32_t)tg.rounds()) {
         err |= gx::ERR_TABLE_FULL;
         again = false;
@@ -680,7 +685,7 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
       if (again) {  // (the warp has read its entries: resolve_lanes synchronises it)
         const int at = n_kept + __popc(am & below);
         store_vec<W>(q.kept + at * W, x);
-        q.hash[at] = hn + 1;
+        q.seq[at] = (uint8_t)(n + 1);
       }
       n_kept += __popc(am);
     }
@@ -787,14 +792,15 @@ __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expa
           if (di < a.dl_cap) store_vec<W>(a.dl_buf + di * W, v);
         }
       },
-      [&](uint64_t b, uint64_t hh, const uint32_t(&x)[W]) {
+      [&](const uint32_t(&x)[W]) {
         // region passes: a vector whose first bucket lies outside this pass's region is
         // left to the pass of that region (tested before the caches, which may only hold
         // vectors that went to find-or-put).  A vector this warp has already sent to
         // find-or-put needs no second lookup, nor does one that any warp found or
         // inserted moments ago.
-        if ((b & a.region_mask) != a.region_bits) return false;
-        return !(cache.base && cache.template seen<W>(hh, x));
+        if (a.region_mask && (bucket_of(state_hash<W>(x), muls[0], a.log2nb) & a.region_mask) != a.region_bits)
+          return false;
+        return !(cache.base && cache.template seen<W>(x));
       });
   st.flush<W>(tg, err);
   // the CTA's totals, one atomic per counter: at the end of a level every warp
@@ -984,7 +990,7 @@ __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThrea
             if (di < a.dl_cap) store_vec<W>(a.dl_buf + di * W, v);
           }
         },
-        [](uint64_t, uint64_t, const uint32_t(&)[W]) { return true; });
+        [](const uint32_t(&)[W]) { return true; });
     st.flush<W>(tg, err);
     const unsigned long long tr = warp_sum((unsigned long long)trans), pr = warp_sum((unsigned long long)probes);
     err = __reduce_or_sync(FULLMASK, err);

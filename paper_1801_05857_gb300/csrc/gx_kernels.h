@@ -43,16 +43,17 @@ struct Muls {
 
 // GPU-wide cache of recently seen vectors: 2^n direct-mapped entries in global
 // memory, cleared at the start of a search (nullptr = off).  A vector's fields
-// packed side by side are a number of `bits` <= 64 bits; a bijection mixes it,
-// its top n bits are the entry's index and the others, plus one, its content
-// (0 = empty), so an entry holds a vector exactly in 16 or 32 bits where
-// that is enough.  (cache_layout in gx_internal.h fills it in.)
+// packed side by side are a number of at most 64 bits.  Its low bits, plus one,
+// are an entry's content (0 = empty); the n bits above them, mixed with a hash of
+// the low ones, are the entry's index, which therefore gives them back: an entry
+// holds a vector exactly, in 16 or 32 bits where that is enough.
+// (cache_layout in gx_explore.cu fills it in.)
 struct SeenCache {
   void* base;
-  uint64_t mask;      // 2^bits - 1
-  uint64_t tag_mask;  // 2^shift - 1
+  uint64_t tag_mask;  // the low bits: 2^shift - 1
   uint32_t shift;     // bits - n (0 when bits <= n)
-  uint32_t half;      // (bits + 1) / 2
+  uint32_t mask;      // 2^n - 1
+  uint32_t mix_shift; // 32 - n
   uint32_t log2_bytes;  // of an entry: 1, 2 or 3
   uint32_t word_at[3];  // bit offset in the key of the payload of words 1, 2, 3 (64: no fields)
 };
