@@ -238,10 +238,8 @@ struct BatchOcc {
   static constexpr int min_ctas = ExpandOcc<W, B, G>::min_ctas < 4 ? ExpandOcc<W, B, G>::min_ctas : 4;
 };
 
-constexpr int kWarpDescs = 32;  // processes whose descriptors a warp keeps in shared memory
-
 // Dynamic shared memory of the batched kernel, per warp: queues, staging, the
-// cache of seen vectors, the network and its processes' descriptors.
+// cache of seen vectors, the network and descriptors of its edge classes.
 template <int W>
 struct __align__(16) BatchSmem {
   static constexpr int kWarps = gx::kBlock / 32;
@@ -249,7 +247,7 @@ struct __align__(16) BatchSmem {
   WarpQueues<W, 32> queues[kWarps];
   uint32_t stage[kWarps][kStage * W];
   uint32_t cache[kWarps][kCache];
-  uint4 descs[kWarps][kWarpDescs];
+  uint4 descs[kWarps][32];  // of the first edge classes, one per lane to fetch
   WarpNet net[kWarps];
   unsigned long long muls[kMaxRounds];
 };
@@ -290,7 +288,7 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
       if (W <= 2)
         for (uint32_t i = lane; i < (uint32_t)BatchSmem<W>::kCache; i += 32) S.cache[wid][i] = 0u;
       __syncwarp();
-      if (wn.lay.n_procs <= (uint32_t)kWarpDescs && lane < wn.lay.n_procs) descs[lane] = proc_desc(t, wn.lay, lane);
+      if (lane < wn.lay.n_classes) descs[lane] = class_desc(t, wn.lay, lane);
     }
     // the level (it cannot end before this claim is done)
     __threadfence();
@@ -302,7 +300,6 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
     }
     __syncwarp();
     const NetBlobLayout& L = wn.lay;
-    const bool staged = L.n_procs <= (uint32_t)kWarpDescs;
     uint32_t probes = 0, err = 0;
     unsigned long long trans = 0;
     uint64_t pos = 0, end = 0;  // what is left of the claim
@@ -310,7 +307,7 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
     uint32_t taken = 1;
     expand_states<W, B, G, 32>(
         tg, muls, t, L, S.queues[wid], st, probes, err,
-        [&](uint32_t p) { return staged ? descs[p] : proc_desc(t, L, p); },
+        ClassDescs{descs, L.n_classes < 32u ? L.n_classes : 32u},
         [&](uint64_t& at, uint32_t& m) {
           m = 0;
           if (pos == end) {

@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(gx::kBlock) digest_kernel(const gx::DigestArgs
   constexpr int kWarps = gx::kBlock / 32, kBatch = 64, S = 8 / W;
   __shared__ uint4 descs[kMaxProcs];
   __shared__ __align__(16) uint32_t queue_mem[kWarps][(kBatch + 32) * W];
-  for (uint32_t p = threadIdx.x; p < a.lay.n_procs; p += blockDim.x) descs[p] = proc_desc(a.blob, a.lay, p);
+  for (uint32_t p = threadIdx.x; p < a.lay.n_procs; p += blockDim.x) descs[p] = class_desc(a.blob, a.lay, p);
   __syncthreads();
   uint32_t* queue = queue_mem[threadIdx.x >> 5];
   const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1u;

@@ -676,7 +676,7 @@ __global__ void __launch_bounds__(gx::kBlock) guided_expand_kernel(const GuidedA
   __shared__ __align__(16) uint32_t queue_mem[kWarps][64 * W];
   __shared__ uint32_t rows_mem[kWarps][64 * E], s_left[kWarps];
   __shared__ unsigned long long s_base;
-  for (uint32_t p = threadIdx.x; p < L.n_procs; p += blockDim.x) descs[p] = proc_desc(t, L, p);
+  const ProcDescs desc = stage_descs(t, L, descs);
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const unsigned long long log_base = a.ctl->log_base;
@@ -690,7 +690,6 @@ __global__ void __launch_bounds__(gx::kBlock) guided_expand_kernel(const GuidedA
   const unsigned long long nwarps = (unsigned long long)gridDim.x * kWarps;
   const uint32_t n_src = L.n_procs + L.n_rules, below = (1u << lane) - 1u;
   uint32_t* queue = queue_mem[threadIdx.x >> 5];
-  const auto desc = [&](uint32_t p) { return descs[p]; };
   uint32_t* rows = rows_mem[threadIdx.x >> 5];
   int staged = 0;  // new states (uniform in the warp)
   // the last m <= 32 staged states, with their histograms, to positions base.. of the pending buffer

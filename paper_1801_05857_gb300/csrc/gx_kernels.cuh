@@ -429,13 +429,44 @@ __device__ __forceinline__ int resolve_lanes(const T& a, const uint64_t* muls, b
   return r;
 }
 
-// What a warp needs of process p to generate its local successors, one 16-byte
-// shared-memory read: word, shift and mask of the field, and where the offsets
-// of its local edges start in the network tables.
-__device__ __forceinline__ uint4 proc_desc(const uint32_t* t, const NetBlobLayout& L, uint32_t p) {
-  return make_uint4(t[L.proc_word + p], t[L.proc_shift + p], t[L.proc_mask + p], L.coff + t[L.cls_base + p]);
+// What a warp needs of edge class c (class p < n_procs: the local edges of process
+// p), one 16-byte shared-memory read: word, shift and mask of its process's field,
+// and where the offsets of its edges start in the network tables.
+__device__ __forceinline__ uint4 class_desc(const uint32_t* t, const NetBlobLayout& L, uint32_t c) {
+  const uint32_t p = t[L.cls_proc + c];
+  return make_uint4(t[L.proc_word + p], t[L.proc_shift + p], t[L.proc_mask + p], L.coff + t[L.cls_base + c]);
 }
 constexpr int kMaxProcs = 124;  // gx_load_network's limit
+
+// The processes' descriptors in shared memory; a rule's class takes its process's.
+struct ProcDescs {
+  const uint4* staged;
+  __device__ __forceinline__ uint4 proc(const uint32_t*, const NetBlobLayout&, uint32_t p) const { return staged[p]; }
+  __device__ __forceinline__ uint4 cls(const uint32_t* t, const NetBlobLayout& L, uint32_t c) const {
+    uint4 d = staged[t[L.cls_proc + c]];
+    d.w = L.coff + t[L.cls_base + c];
+    return d;
+  }
+};
+// All threads of a CTA fill descs (kMaxProcs entries); the caller synchronises.
+__device__ __forceinline__ ProcDescs stage_descs(const uint32_t* t, const NetBlobLayout& L, uint4* descs) {
+  for (uint32_t p = threadIdx.x; p < L.n_procs; p += blockDim.x) descs[p] = class_desc(t, L, p);
+  return ProcDescs{descs};
+}
+
+// The first n classes' descriptors in shared memory, the others from the tables.  For
+// kernels whose network tables stay in global memory (256 networks: 9.1 ms with the
+// processes' alone, 8.5 so); with the tables in shared memory it makes no difference.
+struct ClassDescs {
+  const uint4* staged;
+  uint32_t n;
+  __device__ __forceinline__ uint4 cls(const uint32_t* t, const NetBlobLayout& L, uint32_t c) const {
+    return c < n ? staged[c] : class_desc(t, L, c);
+  }
+  __device__ __forceinline__ uint4 proc(const uint32_t* t, const NetBlobLayout& L, uint32_t p) const {
+    return cls(t, L, p);
+  }
+};
 
 // Successor generation by a warp.  Sources of successors are the processes, then
 // the rules.  Either the lanes hold one state each (lanes without one hold no
@@ -457,7 +488,7 @@ struct WarpGen {
   __device__ __forceinline__ void open(const uint32_t* t, const NetBlobLayout& L, Desc& desc, bool valid,
                                        const uint32_t (&v)[W]) {
     if (src < L.n_procs) {
-      const uint4 d = desc(src);
+      const uint4 d = desc.proc(t, L, src);
       word = d.x;
       cur = word_at<W>(v, d.x);
       const uint32_t* o = t + d.w + ((cur >> d.y) & d.z);
@@ -469,8 +500,8 @@ struct WarpGen {
       const uint32_t j1 = t[L.rule_off + r + 1];
       for (uint32_t j = t[L.rule_off + r]; j < j1; ++j) {
         const uint32_t c = t[L.rule_cls + j];
-        const uint4 d = desc(t[L.cls_proc + c]);
-        const uint32_t* o = t + L.coff + t[L.cls_base + c] + ((word_at<W>(v, d.x) >> d.y) & d.z);
+        const uint4 d = desc.cls(t, L, c);
+        const uint32_t* o = t + d.w + ((word_at<W>(v, d.x) >> d.y) & d.z);
         prod *= o[1] - o[0];
         if (!__any_sync(FULLMASK, prod != 0)) break;
       }
@@ -489,7 +520,7 @@ struct WarpGen {
     const uint32_t s = src + (threadIdx.x & 31);
     e = e_end = 0;
     if (s < L.n_procs) {
-      const uint4 d = desc(s);
+      const uint4 d = desc.proc(t, L, s);
       word = d.x;
       cur = word_at<W>(v, d.x);
       const uint32_t* o = t + d.w + ((cur >> d.y) & d.z);
@@ -500,8 +531,8 @@ struct WarpGen {
       uint32_t prod = 1;
       for (uint32_t j = t[L.rule_off + r]; j < j1 && prod; ++j) {
         const uint32_t c = t[L.rule_cls + j];
-        const uint4 d = desc(t[L.cls_proc + c]);
-        const uint32_t* o = t + L.coff + t[L.cls_base + c] + ((word_at<W>(v, d.x) >> d.y) & d.z);
+        const uint4 d = desc.cls(t, L, c);
+        const uint32_t* o = t + d.w + ((word_at<W>(v, d.x) >> d.y) & d.z);
         prod *= o[1] - o[0];
       }
       word = W;
@@ -526,8 +557,8 @@ struct WarpGen {
       const uint32_t j1 = t[L.rule_off + cur + 1];
       for (uint32_t j = t[L.rule_off + cur]; j < j1; ++j) {
         const uint32_t c = t[L.rule_cls + j];
-        const uint4 d = desc(t[L.cls_proc + c]);
-        const uint32_t* o = t + L.coff + t[L.cls_base + c] + ((word_at<W>(v, d.x) >> d.y) & d.z);
+        const uint4 d = desc.cls(t, L, c);
+        const uint32_t* o = t + d.w + ((word_at<W>(v, d.x) >> d.y) & d.z);
         const uint32_t cnt = o[1] - o[0];
         uint32_t i = 0;
         if (cnt > 1) {  // one matching edge is the common case: no division
@@ -582,7 +613,7 @@ struct ExpandOcc {
 //   next(pos, m)   the warp's next m <= 32 states, at absolute frontier
 //                  positions pos.. (m = 0: none are left); a single state is
 //                  generated from by the whole warp
-//   desc(p)        the process descriptors (proc_desc)
+//   desc           the descriptors of processes and classes (ProcDescs, ClassDescs)
 //   seen(v)        a lane's state, once, when it is taken
 //   done(v, n)     a lane's state and the number of its successors
 //   keep(x)        the filters before the GPU-wide cache, of a successor
@@ -732,7 +763,7 @@ __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expa
   __shared__ uint4 descs[kMaxProcs];
   __syncthreads();
   const NetBlobLayout& L = a.lay;
-  for (uint32_t p = threadIdx.x; p < L.n_procs; p += blockDim.x) descs[p] = proc_desc(t, L, p);
+  const ProcDescs desc = stage_descs(t, L, descs);
   __syncthreads();
   const uint32_t lane = threadIdx.x & 31;
   uint32_t trans = 0;  // per thread and launch: far below 2^32
@@ -755,7 +786,7 @@ __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expa
   const uint64_t own_end = s_range[1] - own < unit ? s_range[1] : own + unit;  // (own >= the end: no states)
   bool first = true;
   expand_states<W, B, G, kBatch<W>, kWide<W>>(
-      tg, muls, t, L, queue_mem[threadIdx.x >> 5], st, probes, err, [&](uint32_t p) { return descs[p]; },
+      tg, muls, t, L, queue_mem[threadIdx.x >> 5], st, probes, err, desc,
       [&](uint64_t& pos, uint32_t& m) {
         // the first states of every warp are fixed by its index, a large level's
         // further ones are claimed; a few states are taken one by one
@@ -949,7 +980,7 @@ __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThrea
   const uint32_t* t = stage_tables(sm, a.muls, a.rounds, a.blob, a.blob_words, a.stage, muls);
   __syncthreads();
   const NetBlobLayout& L = a.lay;
-  for (uint32_t p = threadIdx.x; p < L.n_procs; p += blockDim.x) descs[p] = proc_desc(t, L, p);
+  const ProcDescs desc = stage_descs(t, L, descs);
   const uint32_t lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const uint32_t gw = blockIdx.x * kWarps + wid;
   SmallQueues<W>& q = reinterpret_cast<SmallQueues<W>*>(sm + 2 * kMaxRounds + (a.stage ? a.blob_words : 0))[wid];
@@ -971,7 +1002,7 @@ __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThrea
     uint32_t trans = 0, probes = 0, err = 0;
     uint64_t own = s_range[0] + gw;
     expand_states<W, B, 1, 32>(
-        tg, muls, t, L, q.queues, st, probes, err, [&](uint32_t p) { return descs[p]; },
+        tg, muls, t, L, q.queues, st, probes, err, desc,
         [&](uint64_t& pos, uint32_t& m) {
           m = own < s_range[1] ? 1 : 0;
           pos = own;
