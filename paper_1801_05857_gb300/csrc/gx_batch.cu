@@ -46,7 +46,7 @@ struct BatchArgs {
   int rounds;
   uint32_t chunk;             // states per claim, at most
   uint32_t levels_cap;
-  unsigned long long* levels; // levels_cap entries per network
+  unsigned long long* levels; // level sizes: entry [level * n + network]
   // per network: claims taken of its level, and in the upper half how many it has
   // (0: finished, and then at least kFinished are taken)
   unsigned long long* claims;
@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(gx::kBlock) batch_init_kernel(const BatchArgs 
   b.active = r == FOP_INSERTED ? 1u : 0u;
   b.first_dl = -1;
   b.n_levels = 1;
-  a.levels[(uint64_t)net * a.levels_cap] = 1;
+  a.levels[net] = 1;
   a.claims[net] = r == FOP_INSERTED ? 1ull << 32 : gx::kFinished;
   if (r == FOP_INSERTED) atomicAdd(a.active, 1u);
 }
@@ -107,7 +107,7 @@ __device__ __forceinline__ void batch_next_level(const BatchArgs& a, int i) {
   if (__ldcg(&b.first_dl) < 0 && __ldcg(&b.dl_count) > 0) b.first_dl = (int)levels - 1;
   if (fresh > 0) {
     if (levels < a.levels_cap) {
-      a.levels[(uint64_t)i * a.levels_cap + levels] = fresh;
+      a.levels[(uint64_t)levels * a.n + i] = fresh;
     } else {
       err |= gx::ERR_LEVELS;
       b.error = err;
@@ -516,13 +516,14 @@ gx_status run_batch(gx_batch* h, const gx_batch_opts* o, void* ws, uint64_t ws_b
   GB_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, P.k.expand, kBlock, P.k.smem));
   const int grid = sms * std::max(per_sm, 1);
 
-  // descriptors and tables
-  std::vector<BNet> bn(n);
+  // the descriptors, and behind them the networks' encodings, as one copy (256 networks: 257
+  // copies took 1.5 ms)
+  std::vector<char> up(P.off_levels - P.off_nets, 0);
+  BNet* const bn = reinterpret_cast<BNet*>(up.data());
   for (int k = 0; k < n; ++k) {
     const uint32_t i = P.order[k];
     const Net& net = h->nets[i];
     BNet& b = bn[k];
-    std::memset(&b, 0, sizeof(b));
     b.blob = reinterpret_cast<const uint32_t*>(base + P.blob_off[i]);
     b.lay = net.lay;
     b.table = reinterpret_cast<uint32_t*>(base + P.table_off[i]);
@@ -534,9 +535,9 @@ gx_status run_batch(gx_batch* h, const gx_batch_opts* o, void* ws, uint64_t ws_b
     b.fmask = P.fcap[i] - 1;
     // the initial vector, padded to the batch's slot width (padding words carry only the tag)
     for (int w = 0; w < 4; ++w) b.init_vec[w] = w < P.W ? (net.init_vec[w] | kTag) : 0u;
-    GB_CUDA(cudaMemcpyAsync(base + P.blob_off[i], net.blob.data(), 4 * net.blob.size(), cudaMemcpyHostToDevice, st));
+    std::memcpy(up.data() + (P.blob_off[i] - P.off_nets), net.blob.data(), 4 * net.blob.size());
   }
-  GB_CUDA(cudaMemcpyAsync(base + P.off_nets, bn.data(), sizeof(BNet) * n, cudaMemcpyHostToDevice, st));
+  GB_CUDA(cudaMemcpyAsync(base + P.off_nets, up.data(), up.size(), cudaMemcpyHostToDevice, st));
 
   BatchArgs a{};
   a.nets = reinterpret_cast<BNet*>(base + P.off_nets);
@@ -558,18 +559,20 @@ gx_status run_batch(gx_batch* h, const gx_batch_opts* o, void* ws, uint64_t ws_b
   GB_CUDA(cudaEventCreate(&e1));
   GB_CUDA(cudaEventRecord(e0, st));
   GB_CUDA(cudaMemsetAsync(base + P.off_tables, 0, 4 * P.table_words, st));
-  GB_CUDA(cudaMemsetAsync(a.active, 0, sizeof(unsigned int), st));
   GB_CUDA(cudaLaunchKernel(P.k.init, dim3((n + per_block - 1) / per_block), dim3(kBlock), args, 0, st));
   GB_CUDA(cudaLaunchKernel(P.k.expand, dim3(grid), dim3(kBlock), args, P.k.smem, st));
   GB_CUDA(cudaEventRecord(e1, st));
-  GB_CUDA(cudaMemcpyAsync(bn.data(), base + P.off_nets, sizeof(BNet) * n, cudaMemcpyDeviceToHost, st));
+  GB_CUDA(cudaMemcpyAsync(bn, base + P.off_nets, sizeof(BNet) * n, cudaMemcpyDeviceToHost, st));
   GB_CUDA(cudaStreamSynchronize(st));
   float ms = 0;
   cudaEventElapsedTime(&ms, e0, e1);
   cudaEventDestroy(e0);
   cudaEventDestroy(e1);
   h->gpu_ms = ms;
-  std::vector<unsigned long long> lv((uint64_t)n * P.levels_cap);
+  // as many levels as the deepest network has
+  uint32_t deepest = 0;
+  for (int k = 0; k < n; ++k) deepest = std::max(deepest, std::min<uint32_t>(bn[k].n_levels, P.levels_cap));
+  std::vector<unsigned long long> lv((uint64_t)n * deepest);
   GB_CUDA(cudaMemcpyAsync(lv.data(), base + P.off_levels, 8ull * lv.size(), cudaMemcpyDeviceToHost, st));
   GB_CUDA(cudaStreamSynchronize(st));
   h->res.resize(n);
@@ -580,8 +583,8 @@ gx_status run_batch(gx_batch* h, const gx_batch_opts* o, void* ws, uint64_t ws_b
   for (int i = 0; i < n; ++i) {
     h->res[i] = bn[slot[i]];
     const uint32_t k = std::min<uint32_t>(h->res[i].n_levels, P.levels_cap);
-    const auto first = lv.begin() + (uint64_t)slot[i] * P.levels_cap;
-    h->levels[i].assign(first, first + k);
+    h->levels[i].resize(k);
+    for (uint32_t l = 0; l < k; ++l) h->levels[i][l] = lv[(uint64_t)l * n + slot[i]];
     if (h->res[i].error && rs == GX_OK) {
       const unsigned e = h->res[i].error;
       rs = (e & ERR_TABLE_FULL)  ? fail(GX_ERR_TABLE_FULL, "network " + std::to_string(i) + ": hash table full")

@@ -384,13 +384,15 @@ gx_status device_info(Device& d) {
   return GX_OK;
 }
 
-// Pinned host copies of the control block and of the per-CTA successor
-// totals of the partitioned path, one set per thread.
+// Pinned host copies of the control block, of the device-driven loop's records and
+// of the per-CTA successor totals of the partitioned path, one set per thread.
 struct HostCtl {
   Ctl* p = nullptr;
+  unsigned long long* loop = nullptr;
   uint32_t* tot = nullptr;
   ~HostCtl() {
     if (p) cudaFreeHost(p);
+    if (loop) cudaFreeHost(loop);
     if (tot) cudaFreeHost(tot);
   }
 };
@@ -695,13 +697,15 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
     }
     GX_CUDA(cudaGraphLaunch(static_cast<cudaGraphExec_t>(h->loop_exec), st));
     GX_CUDA(cudaMemcpyAsync(hc, ctl, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
-    std::vector<unsigned long long> hl(4ull * kLoopLevels);
-    GX_CUDA(cudaMemcpyAsync(hl.data(), lv, 8ull * hl.size(), cudaMemcpyDeviceToHost, st));
+    constexpr size_t kRecords = 8ull * 4 * kLoopLevels;
+    if (!g_hctl.loop) GX_CUDA(cudaMallocHost(reinterpret_cast<void**>(&g_hctl.loop), kRecords));
+    const unsigned long long* hl = g_hctl.loop;
+    GX_CUDA(cudaMemcpyAsync(g_hctl.loop, lv, kRecords, cudaMemcpyDeviceToHost, st));
     GX_CUDA(cudaStreamSynchronize(st));
-    d2h_loop = sizeof(Ctl) + 8ull * hl.size();
+    d2h_loop = sizeof(Ctl) + kRecords;
     const uint64_t nd = hc->levels_done;
     const uint64_t nl = std::min<uint64_t>(hc->n_levels, kLoopLevels);
-    levels.assign(hl.begin(), hl.begin() + nl);
+    levels.assign(hl, hl + nl);
     for (uint64_t k = 0; k < nd && k < kLoopLevels; ++k) {
       lv_ms.push_back(1e-6 * (double)hl[kLoopLevels + k]);
       lv_probes.push_back(hl[2 * kLoopLevels + k] - prev_probes);

@@ -11,6 +11,7 @@ from __future__ import annotations
 import ctypes
 import os
 import re
+import struct
 
 import numpy as np
 
@@ -85,6 +86,16 @@ class gx_stats_t(ctypes.Structure):
                 ("violation_count", u64), ("violation_sum", u64), ("violation_xor", u64),
                 ("first_violation_level", ctypes.c_int64), ("kernel_launches", u64),
                 ("device_levels", u64), ("global_cache_entries", u64)]
+
+
+# All fields at once: a ctypes attribute read takes as long as unpacking the whole structure.
+_STATS_NAMES = [name for name, _ in gx_stats_t._fields_]
+_STATS_FORMAT = struct.Struct("@" + "".join({u64: "Q", u32: "I", i64: "q", ctypes.c_double: "d"}[t]
+                                            for _, t in gx_stats_t._fields_))
+
+
+def _stats_dict(s: gx_stats_t) -> dict:
+    return dict(zip(_STATS_NAMES, _STATS_FORMAT.unpack_from(s)))
 
 
 class gx_batch_opts(ctypes.Structure):
@@ -341,15 +352,15 @@ def find_deadlocks(net: Net, mode: int, opts: gx_explore_opts | None = None, wor
 def stats(net: Net) -> dict:
     s = gx_stats_t()
     _check(lib().gx_stats(net.handle, ctypes.byref(s)))
-    return {name: getattr(s, name) for name, _ in gx_stats_t._fields_ }
+    return _stats_dict(s)
 
 
 def levels(net: Net) -> list:
     n = u32()
     _check(lib().gx_levels(net.handle, None, 0, ctypes.byref(n)))
-    out = np.zeros(max(int(n.value), 1), dtype=np.uint64)
-    _check(lib().gx_levels(net.handle, out.ctypes.data_as(P(u64)), int(n.value), ctypes.byref(n)))
-    return [int(x) for x in out[:int(n.value)]]
+    out = (u64 * max(n.value, 1))()
+    _check(lib().gx_levels(net.handle, out, n.value, ctypes.byref(n)))
+    return out[:n.value]
 
 
 def level_profile(net: Net) -> dict:
@@ -397,7 +408,7 @@ def explore_noalloc(net: Net, opts: gx_explore_opts | None = None, stream=None,
     _check(lib().gx_explore_noalloc(net.handle, ctypes.byref(opts) if opts else None,
                                     _stream(stream), ctypes.byref(s), lv.ctypes.data_as(P(u64)),
                                     levels_cap, ctypes.byref(n)))
-    stats_d = {name: getattr(s, name) for name, _ in gx_stats_t._fields_ }
+    stats_d = _stats_dict(s)
     return stats_d, [int(x) for x in lv[:min(int(n.value), levels_cap)]]
 
 
@@ -532,15 +543,15 @@ def batch_explore(b: Batch, opts: gx_batch_opts | None, workspace, stream=None) 
 def batch_stats(b: Batch, i: int) -> dict:
     s = gx_stats_t()
     _check(lib().gx_batch_stats(b.handle, i, ctypes.byref(s)))
-    return {name: getattr(s, name) for name, _ in gx_stats_t._fields_ }
+    return _stats_dict(s)
 
 
 def batch_levels(b: Batch, i: int) -> list:
     n = u32()
     _check(lib().gx_batch_levels(b.handle, i, None, 0, ctypes.byref(n)))
-    out = np.zeros(max(int(n.value), 1), dtype=np.uint64)
-    _check(lib().gx_batch_levels(b.handle, i, out.ctypes.data_as(P(u64)), int(n.value), ctypes.byref(n)))
-    return [int(x) for x in out[:int(n.value)]]
+    out = (u64 * max(n.value, 1))()
+    _check(lib().gx_batch_levels(b.handle, i, out, n.value, ctypes.byref(n)))
+    return out[:n.value]
 
 
 def batch_autotune(b: Batch, opts: gx_batch_opts, workspace, stream=None) -> float:
