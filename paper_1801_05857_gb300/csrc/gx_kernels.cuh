@@ -1276,38 +1276,106 @@ __global__ void init_kernel(const gx::InitArgs a) {
   }
 }
 
-// Sec. 5.1: every group of G lanes takes one key at a time.
+// Sec. 5.1: find-or-put of a warp's keys, a key per lane.
+// G == 1: key after key.  Bound by random 128-byte lines read and written back; a lane
+// that took its next key while others of its warp read further buckets made it no
+// faster (1.5e8 keys, 1e8 of them new, 8-word buckets: 4.75 ms, with that 4.92).
+struct LaneFop {
+  uint32_t ins = 0, fnd = 0, fail = 0;
+  __device__ __forceinline__ void count(const gx::FopArgs& a, uint64_t i, int r) {
+    if (a.result) a.result[i] = (uint8_t)(r == FOP_INSERTED ? 1 : (r == FOP_FOUND ? 0 : 2));
+    ins += r == FOP_INSERTED;
+    fnd += r == FOP_FOUND;
+    fail += r < 0;
+  }
+};
+template <int W, int B>
+__device__ __forceinline__ void fop_lanes(const gx::FopArgs& a, const uint64_t* muls, LaneFop& n) {
+  const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += step) {
+    uint32_t v[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) v[w] = a.keys[i * W + w] | kTag;
+    const uint64_t h = vec_hash<W>(v);
+    int r = -1;
+    for (int k = 0; k < a.rounds && r < 0; ++k)
+      r = bucket_step<W, B>(a.table + seq_bucket<B>(h, k, muls, a.log2nb) * (uint64_t)B, v);
+    n.count(a, i, r);
+  }
+}
+
+// G > 1: the lanes read their buckets together (bucket_step_lanes), so a lane that is
+// done takes its next key at once.  (With a group of lanes per key, which voted on every
+// bucket, the same keys took 10.5 ms with a lane per slot of 8-word buckets, 22.6 of
+// 32-word ones; now 4.8 and 5.6.)
+template <int W, int B, int G>
+__device__ __forceinline__ void fop_groups(const gx::FopArgs& a, const uint64_t* muls, LaneFop& n) {
+  const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1u;
+  // the warp's keys: consecutive ones, of which 64 are held (base.., pos of them taken)
+  const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x / 32);
+  const uint64_t len = (a.n + warps - 1) / warps;
+  uint64_t base = ((uint64_t)blockIdx.x * (blockDim.x / 32) + (threadIdx.x >> 5)) * len;
+  const uint64_t end = base + len < a.n ? base + len : a.n;
+  uint32_t pos = 0, cur[W], nxt[W];
+  auto fetch = [&](uint64_t i, uint32_t(&x)[W]) {
+#pragma unroll
+    for (int w = 0; w < W; ++w) x[w] = i < end ? a.keys[i * W + w] : 0u;
+  };
+  fetch(base + lane, cur);
+  fetch(base + 32 + lane, nxt);
+  bool has = false;
+  uint32_t v[W], k = 0;
+  uint64_t h = 0, at = 0;
+#pragma unroll
+  for (int w = 0; w < W; ++w) v[w] = 0;
+  while (true) {
+    const uint32_t need = __ballot_sync(FULLMASK, !has);
+    if (need != 0 && base + pos < end) {
+      const uint32_t src = pos + __popc(need & below);
+      uint32_t x[W];
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        const uint32_t c = __shfl_sync(FULLMASK, cur[w], src & 31), d = __shfl_sync(FULLMASK, nxt[w], src & 31);
+        x[w] = src < 32 ? c : d;
+      }
+      if (!has && base + src < end) {
+#pragma unroll
+        for (int w = 0; w < W; ++w) v[w] = x[w] | kTag;
+        h = vec_hash<W>(v);
+        at = base + src;
+        k = 0;
+        has = true;
+      }
+      pos += __popc(need);
+      if (pos >= 32) {
+        pos -= 32;
+        base += 32;
+#pragma unroll
+        for (int w = 0; w < W; ++w) cur[w] = nxt[w];
+        fetch(base + 32 + lane, nxt);
+      }
+    }
+    if (!__any_sync(FULLMASK, has)) break;
+    const int r = bucket_step_lanes<W, B, G>(a.table, has, seq_bucket<B>(h, k, muls, a.log2nb), v);
+    if (has && (r >= 0 || ++k == (uint32_t)a.rounds)) {
+      n.count(a, at, r);
+      has = false;
+    }
+  }
+}
+
 template <int W, int B, int G>
 __global__ void __launch_bounds__(gx::kBlock) fop_kernel(const gx::FopArgs a) {
   __shared__ uint64_t muls[kMaxRounds];
   for (int i = threadIdx.x; i < a.rounds; i += blockDim.x) muls[i] = a.muls.m[i];
   __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const Group<G> g;
-  const uint64_t groups = (uint64_t)gridDim.x * blockDim.x / G;
-  uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
-  uint32_t probes = 0;
-  unsigned long long ins = 0, fnd = 0, fail = 0;
-  // the loop bound is uniform per warp: all groups of a warp leave together
-  const uint64_t warp_first = ((uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u)) / G;
-  for (uint64_t wi = warp_first; wi < a.n; wi += groups, i += groups) {
-    if (i < a.n) {
-      uint32_t v[W];
-#pragma unroll
-      for (int w = 0; w < W; ++w) v[w] = a.keys[i * W + w] | kTag;
-      const int r = find_or_put<W, B, G>(a.table, a.log2nb, a.rounds, muls, v, g, probes);
-      if (g.glane == 0) {
-        if (a.result) a.result[i] = (uint8_t)(r == FOP_INSERTED ? 1 : (r == FOP_FOUND ? 0 : 2));
-        ins += r == FOP_INSERTED;
-        fnd += r == FOP_FOUND;
-        fail += r == FOP_FULL;
-      }
-    }
-  }
-  ins = warp_sum(ins);
-  fnd = warp_sum(fnd);
-  fail = warp_sum(fail);
-  if (lane == 0) {
+  LaneFop n;
+  if constexpr (G == 1) fop_lanes<W, B>(a, muls, n);
+  else fop_groups<W, B, G>(a, muls, n);
+  const unsigned long long ins = warp_sum((unsigned long long)n.ins);
+  const unsigned long long fnd = warp_sum((unsigned long long)n.fnd);
+  const unsigned long long fail = warp_sum((unsigned long long)n.fail);
+  if ((threadIdx.x & 31) == 0) {
     if (ins) atomicAdd(&a.counters[0], ins);
     if (fnd) atomicAdd(&a.counters[1], fnd);
     if (fail) atomicAdd(&a.counters[2], fail);

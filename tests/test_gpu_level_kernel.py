@@ -108,3 +108,32 @@ def test_batches_of_any_number_of_networks(cuda, count, wide):
             assert (s["states"], s["transitions"], s["explored"]) == (r.states, r.transitions, r.explored)
             assert (s["deadlock_count"], s["deadlock_sum"]) == (r.deadlock_count, r.deadlock_sum)
             assert (s["first_deadlock_level"], gx.batch_levels(b, i)) == (r.first_deadlock_level, r.levels)
+
+
+@pytest.mark.parametrize("words,bucket,group", [(1, 8, 8), (1, 8, 2), (1, 32, 32), (2, 16, 4), (4, 16, 4)])
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 63, 64, 65, 100_003])
+def test_find_or_put_of_any_number_of_keys(cuda, n, words, bucket, group):
+    """The lanes of a warp take its keys as they become free: remainders of the 64 it holds,
+    keys that occur twice, and (one hash-constant set, nearly full buckets) keys with no place."""
+    import torch
+    g = torch.Generator().manual_seed(n)
+    some = torch.randint(0, 1 << 30, ((n + 1) // 2, words), generator=g, dtype=torch.int32)
+    keys = torch.cat([some, some])[torch.randperm(2 * len(some), generator=g)][:n].contiguous()
+    distinct = torch.unique(keys, dim=0)
+    for rounds, slots in ((32, 4 * n), (1, n // 2)):
+        table_words = max(2 * bucket, 1 << (slots * words - 1).bit_length())
+        table = torch.zeros(table_words, dtype=torch.int32, device="cuda")
+        counters = torch.zeros(3, dtype=torch.int64, device="cuda")
+        result = torch.full((n,), 9, dtype=torch.uint8, device="cuda")
+        gx.find_or_put(keys.cuda(), words, table, counters, result, bucket, group, rounds)
+        ins, fnd, full = counters.tolist()
+        got = torch.bincount(result.cpu().long(), minlength=3).tolist()
+        assert got == [fnd, ins, full] and ins + fnd + full == n
+        # the table holds the inserted keys, each once, and every key that was placed
+        rows = table.cpu().view(-1, words)
+        held = rows[(rows != 0).all(1)] & 0x7FFFFFFF
+        assert len(held) == ins == len(torch.unique(held, dim=0))
+        placed = torch.unique(keys[result.cpu() != 2], dim=0)
+        assert torch.equal(torch.unique(held, dim=0), placed)
+        if rounds == 32:
+            assert (ins, fnd, full) == (len(distinct), n - len(distinct), 0)
