@@ -738,7 +738,7 @@ __global__ void __launch_bounds__(gx::kBlock) guided_expand_kernel(const GuidedA
         queued += __popc(act);
         if (queued < 32) continue;
       } else if (gen.src < n_src) {
-        gen.open_wide(t, L, desc, v);
+        gen.open_wide(t, L, desc, true, v, 5);
         total += gen.e_end - gen.e;
         continue;
       }

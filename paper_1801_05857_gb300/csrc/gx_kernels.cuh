@@ -513,13 +513,14 @@ struct WarpGen {
     ++src;
   }
 
-  // The next 32 sources of the state v that every lane holds, one per lane.
+  // The next 2^sh sources of the state v that 2^sh neighbouring lanes hold, one per lane.
   template <class Desc>
-  __device__ __forceinline__ void open_wide(const uint32_t* t, const NetBlobLayout& L, Desc& desc,
-                                            const uint32_t (&v)[W]) {
-    const uint32_t s = src + (threadIdx.x & 31);
+  __device__ __forceinline__ void open_wide(const uint32_t* t, const NetBlobLayout& L, Desc& desc, bool valid,
+                                            const uint32_t (&v)[W], uint32_t sh) {
+    const uint32_t s = src + (threadIdx.x & ((1u << sh) - 1u));
     e = e_end = 0;
-    if (s < L.n_procs) {
+    if (!valid) {
+    } else if (s < L.n_procs) {
       const uint4 d = desc.proc(t, L, s);
       word = d.x;
       cur = word_at<W>(v, d.x);
@@ -539,7 +540,7 @@ struct WarpGen {
       cur = r;
       e_end = prod;
     }
-    src += 32;
+    src += 1u << sh;
   }
 
   // One successor into the W words at q (a lane with e < e_end).
@@ -606,19 +607,26 @@ struct ExpandOcc {
   static constexpr int min_ctas = B <= 8 ? (G == 1 ? 5 : 4) : (B <= 16 && G == 1 ? 4 : 3);
 };
 
+// Up to this many states per warp are generated from by several lanes each, which take
+// different sources of successors.  Token ring of 11 nodes, 22 sources: levels of 4 or 5
+// states a warp 18 us instead of 26-28, the search 1.61 -> 1.33 ms.  (16 states: the same
+// there; levels of 8 to 16 states a warp of the mid network 30 instead of 33 us, others
+// up to 2 % slower.)
+constexpr uint32_t kWideStates = 8;
+
 // The expansion of a warp's share of one level: generate successors of its
 // states until a batch is queued, filter it, and resolve what is kept 32 at a
 // time -- one loop with one copy of each step (a second copy of find-or-put
 // costs registers).
 //   next(pos, m)   the warp's next m <= 32 states, at absolute frontier
-//                  positions pos.. (m = 0: none are left); a single state is
-//                  generated from by the whole warp
+//                  positions pos.. (m = 0: none are left); up to kWideStates
+//                  are generated from by several lanes each
 //   desc           the descriptors of processes and classes (ProcDescs, ClassDescs)
 //   seen(v)        a lane's state, once, when it is taken
 //   done(v, n)     a lane's state and the number of its successors
 //   keep(x)        the filters before the GPU-wide cache, of a successor
 // All 32 lanes call it together; returns with the queues empty.  Wide: whether
-// next may give a single state at all.
+// few states are treated so at all.
 template <int W, int B, int G, int Batch, bool Wide = true, class T, class Desc, class Next, class Seen, class Done,
           class Keep>
 __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls, const uint32_t* t,
@@ -632,7 +640,8 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
   uint32_t v[W];
 #pragma unroll
   for (int w = 0; w < W; ++w) v[w] = 0;
-  uint32_t cnt = 0;  // successors of this lane's state
+  uint32_t sh = 0;    // 2^sh lanes hold the same state (uniform)
+  uint32_t cnt = 0;   // successors this lane has found of its state
   WarpGen<W> gen;
   gen.src = n_src;
   gen.e = gen.e_end = gen.cur = gen.word = 0;
@@ -644,20 +653,30 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
         if ((act >> lane) & 1u) gen.emit(t, L, desc, v, q.raw + (n_raw + __popc(act & below)) * W);
         n_raw += __popc(act);
       } else if (gen.src < n_src) {
-        if (Wide && m == 1) gen.open_wide(t, L, desc, v);
+        if (Wide && sh != 0) gen.open_wide(t, L, desc, (lane >> sh) < m, v, sh);
         else gen.open(t, L, desc, lane < m, v);
         cnt += gen.e_end - gen.e;
       } else {
         if (!more) break;
-        if (Wide && m == 1) cnt = __reduce_add_sync(FULLMASK, cnt);
-        if (lane < m) done(v, cnt);
+        if constexpr (Wide) {
+          for (uint32_t o = 1u << sh; o > 1; o >>= 1) cnt += __shfl_xor_sync(FULLMASK, cnt, o >> 1);
+          if ((lane >> sh) < m && (lane & ((1u << sh) - 1u)) == 0) done(v, cnt);
+        } else {
+          if (lane < m) done(v, cnt);
+        }
         uint64_t pos = 0;
         next(pos, m);
         more = m != 0;
         if (!more) break;
-        if (lane < m || (Wide && m == 1)) {
-          load_words<W>(tg.frontier() + ((Wide && m == 1 ? pos : pos + lane) & tg.fmask()) * W, v);
-          if (lane < m) seen(v);
+        if constexpr (Wide) {
+          sh = m <= kWideStates ? (uint32_t)__clz(m - 1) - 27u : 0u;
+          if ((lane >> sh) < m) {
+            load_words<W>(tg.frontier() + ((pos + (lane >> sh)) & tg.fmask()) * W, v);
+            if ((lane & ((1u << sh) - 1u)) == 0) seen(v);
+          }
+        } else if (lane < m) {
+          load_words<W>(tg.frontier() + ((pos + lane) & tg.fmask()) * W, v);
+          seen(v);
         }
         cnt = 0;
         gen.src = 0;
@@ -725,12 +744,9 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
   }
 }
 
-// Up to this many states per warp are taken one by one, the whole warp generating
-// from each (token ring of 11 nodes, 22 sources: levels of 1 or 2 states a warp take
-// 15-22 us instead of 19-27; of 4 or more a warp they take longer).  Not with 4-word
-// vectors: the second way of generating spills registers in the loop that the large
-// levels run (3.4e8 states in four passes 192 ms, without it 186).
-constexpr uint32_t kSingly = 2;
+// Whether the level kernel does so: not with 4-word vectors, where the second way of
+// generating spills registers in the loop that the large levels run (3.4e8 states in
+// two passes 188 ms, without it 183).
 template <int W>
 constexpr bool kWide = W < 4;
 
@@ -782,21 +798,14 @@ __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expa
     for (uint32_t i = lane; i < per_warp; i += 32) cache.base[i] = 0u;  // 0 is never a stored vector
     __syncwarp();
   }
-  uint64_t own = s_range[0] + (uint64_t)(blockIdx.x * kWarps + (threadIdx.x >> 5)) * unit;
-  const uint64_t own_end = s_range[1] - own < unit ? s_range[1] : own + unit;  // (own >= the end: no states)
+  const uint64_t own = s_range[0] + (uint64_t)(blockIdx.x * kWarps + (threadIdx.x >> 5)) * unit;
   bool first = true;
   expand_states<W, B, G, kBatch<W>, kWide<W>>(
       tg, muls, t, L, queue_mem[threadIdx.x >> 5], st, probes, err, desc,
       [&](uint64_t& pos, uint32_t& m) {
         // the first states of every warp are fixed by its index, a large level's
-        // further ones are claimed; a few states are taken one by one
+        // further ones are claimed
         m = 0;
-        if (kWide<W> && unit <= kSingly) {
-          if (own >= s_range[1] || own >= own_end) return;
-          pos = own++;
-          m = 1;
-          return;
-        }
         if (first) {
           pos = own;
           first = false;
@@ -1000,13 +1009,15 @@ __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThrea
   __syncthreads();
   while (s_go) {
     uint32_t trans = 0, probes = 0, err = 0;
-    uint64_t own = s_range[0] + gw;
+    // (at most 4 states a warp)
+    const uint32_t unit = ((uint32_t)(s_range[1] - s_range[0]) + kSmallWarps - 1) / kSmallWarps;
+    uint64_t own = s_range[0] + (uint64_t)gw * unit;
     expand_states<W, B, 1, 32>(
         tg, muls, t, L, q.queues, st, probes, err, desc,
         [&](uint64_t& pos, uint32_t& m) {
-          m = own < s_range[1] ? 1 : 0;
+          m = own >= s_range[1] ? 0u : s_range[1] - own < unit ? (uint32_t)(s_range[1] - own) : unit;
           pos = own;
-          own += kSmallWarps;
+          own = s_range[1];
         },
         [&](const uint32_t(&v)[W]) {
           if (a.watch) check_watch<W>(a, t, L, v);

@@ -76,6 +76,15 @@ def test_levels_below_at_and_above_one_state_per_warp(cuda, moving, ctas):
     assert s["states"] == 2 ** moving
 
 
+@pytest.mark.parametrize("n_procs", [40, 70])
+@pytest.mark.parametrize("ctas", [1, 0])
+def test_levels_of_a_few_states_per_warp(cuda, n_procs, ctas):
+    """The same levels with 2- and 4-word vectors: up to 11 states a warp, of which 1 to 8 are
+    shared out among 32 to 4 lanes each."""
+    s = _check(("few", n_procs), _mostly_still(n_procs, 16), table_bytes=1 << 22, ctas_per_sm=ctas)
+    assert s["slot_words"] == (2 if n_procs == 40 else 4)
+
+
 @pytest.mark.parametrize("n_procs", [31, 32, 33, 62])
 def test_batched_networks_with_more_processes_than_lanes(cuda, n_procs):
     nets = [_mostly_still(n_procs, 9), _mostly_still(12, 7), NETS[1]]
