@@ -225,6 +225,95 @@ __device__ __forceinline__ int find_or_put_state(uint32_t* __restrict__ table, i
   return FOP_FULL;
 }
 
+template <int G>
+struct Group {
+  uint32_t mask;  // lanes of this group within the warp
+  int base;       // first lane of the group
+  int glane;      // lane index within the group
+  __device__ __forceinline__ Group() {
+    const int lane = threadIdx.x & 31;
+    base = lane & ~(G - 1);
+    glane = lane - base;
+    mask = (G == 32) ? FULLMASK : (((1u << G) - 1u) << base);
+  }
+  __device__ __forceinline__ bool any(bool p) const {
+    if constexpr (G == 1) return p;
+    else return __any_sync(mask, p);
+  }
+  __device__ __forceinline__ uint32_t ballot(bool p) const {
+    if constexpr (G == 1) return p ? (1u << (threadIdx.x & 31)) : 0u;
+    else return __ballot_sync(mask, p);
+  }
+  template <typename T>
+  __device__ __forceinline__ T bcast(T x, int src_lane) const {
+    if constexpr (G == 1) return x;
+    else return __shfl_sync(mask, x, src_lane);
+  }
+};
+
+// Find-or-put of vector v (identical in every lane of the group).  All G lanes
+// of the group must call it together.  Returns FOP_FOUND, FOP_INSERTED or
+// FOP_FULL (no free slot under any of the `rounds` hash-constant sets), the
+// same value in every lane of the group.  `probes` of the group's first lane
+// is increased by the number of buckets read (once per bucket, not per lane).
+// find_or_put_hashed takes h = vec_hash(v) from the caller.
+template <int W, int B, int G>
+__device__ __forceinline__ int find_or_put_hashed(uint32_t* __restrict__ table, int log2nb, int rounds,
+                                                  const uint64_t* __restrict__ muls,
+                                                  const uint32_t (&v)[W], const uint64_t h, const Group<G>& g,
+                                                  uint32_t& probes) {
+  constexpr int S = B / W;
+  static_assert(S >= 1 && S % G == 0, "group size must divide the slots per bucket");
+  constexpr int SPL = S / G;
+  constexpr int LW = SPL * W;
+  const uint64_t b0 = bucket_of(h, muls[0], log2nb);
+  for (int k = 0; k < rounds; ++k) {
+    const uint64_t b = k == 0 ? b0 : bucket_in_span<B>(h, muls[k], log2nb, b0);
+    uint32_t* lane_slots = table + b * (uint64_t)B + (uint64_t)g.glane * LW;
+    uint32_t s[LW];
+    load_words<LW>(lane_slots, s);
+    probes += g.glane == 0;
+    bool match = false;
+    uint32_t cand = 0;  // slots that are empty or half-written
+#pragma unroll
+    for (int j = 0; j < SPL; ++j) {
+      bool eq = true, tagged = true;
+#pragma unroll
+      for (int w = 0; w < W; ++w) {
+        eq &= (s[j * W + w] == v[w]);
+        tagged &= (s[j * W + w] & kTag) != 0;
+      }
+      match |= eq;
+      if (!tagged) cand |= 1u << j;
+    }
+    if (g.any(match)) return FOP_FOUND;
+    // Claim the first candidate slot of the group; on failure the CAS tells
+    // what the slot holds: our vector (found) or another one (try the next).
+    while (true) {
+      const uint32_t want = g.ballot(cand != 0);
+      if (want == 0) break;
+      const int leader = __ffs(want) - 1;
+      int res = -1;
+      if ((int)(threadIdx.x & 31) == leader) {
+        const int j = __ffs(cand) - 1;
+        uint32_t old[W];
+        if (cas_slot<W>(lane_slots + j * W, v, old)) {
+          res = FOP_INSERTED;
+        } else {
+          bool eq = true;
+#pragma unroll
+          for (int w = 0; w < W; ++w) eq &= (old[w] == v[w]);
+          if (eq) res = FOP_FOUND;
+          cand &= ~(1u << j);
+        }
+      }
+      res = g.bcast(res, leader);
+      if (res >= 0) return res;
+    }
+  }
+  return FOP_FULL;
+}
+
 // One bucket for every lane with `has` set, read by groups of G > 1 lanes; all
 // 32 lanes call it together and each gets its own vector's result (as
 // bucket_step; -1 without one).  The lanes of a group read their G buckets
@@ -270,6 +359,14 @@ __device__ __forceinline__ int bucket_step_lanes(uint32_t* __restrict__ table, b
   const int r = has ? bucket_claim<W, B>(table + b * (uint64_t)B, s, v) : -1;
   __syncwarp();
   return r;
+}
+
+template <int W, int B, int G>
+__device__ __forceinline__ int find_or_put(uint32_t* __restrict__ table, int log2nb, int rounds,
+                                           const uint64_t* __restrict__ muls,
+                                           const uint32_t (&v)[W], const Group<G>& g,
+                                           uint32_t& probes) {
+  return find_or_put_hashed<W, B, G>(table, log2nb, rounds, muls, v, vec_hash<W>(v), g, probes);
 }
 
 // ---- vector fields

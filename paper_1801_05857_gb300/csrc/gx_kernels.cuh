@@ -1288,30 +1288,33 @@ __global__ void init_kernel(const gx::InitArgs a) {
 }
 
 // Sec. 5.1: find-or-put of a warp's keys, a key per lane.
-// G == 1: key after key.  Bound by random 128-byte lines read and written back; a lane
+// G == 1: key after key (find_or_put).  Bound by random 128-byte lines read and written back; a lane
 // that took its next key while others of its warp read further buckets made it no
 // faster (1.5e8 keys, 1e8 of them new, 8-word buckets: 4.75 ms, with that 4.92).
 struct LaneFop {
-  uint32_t ins = 0, fnd = 0, fail = 0;
+  unsigned long long ins = 0, fnd = 0, fail = 0;
   __device__ __forceinline__ void count(const gx::FopArgs& a, uint64_t i, int r) {
     if (a.result) a.result[i] = (uint8_t)(r == FOP_INSERTED ? 1 : (r == FOP_FOUND ? 0 : 2));
     ins += r == FOP_INSERTED;
     fnd += r == FOP_FOUND;
-    fail += r < 0;
+    fail += r != FOP_INSERTED && r != FOP_FOUND;
   }
 };
 template <int W, int B>
 __device__ __forceinline__ void fop_lanes(const gx::FopArgs& a, const uint64_t* muls, LaneFop& n) {
+  const Group<1> g;
   const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
-  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += step) {
-    uint32_t v[W];
+  uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  uint32_t probes = 0;
+  // the loop bound is uniform per warp: all lanes of a warp leave together
+  const uint64_t warp_first = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
+  for (uint64_t wi = warp_first; wi < a.n; wi += step, i += step) {
+    if (i < a.n) {
+      uint32_t v[W];
 #pragma unroll
-    for (int w = 0; w < W; ++w) v[w] = a.keys[i * W + w] | kTag;
-    const uint64_t h = vec_hash<W>(v);
-    int r = -1;
-    for (int k = 0; k < a.rounds && r < 0; ++k)
-      r = bucket_step<W, B>(a.table + seq_bucket<B>(h, k, muls, a.log2nb) * (uint64_t)B, v);
-    n.count(a, i, r);
+      for (int w = 0; w < W; ++w) v[w] = a.keys[i * W + w] | kTag;
+      n.count(a, i, find_or_put<W, B, 1>(a.table, a.log2nb, a.rounds, muls, v, g, probes));
+    }
   }
 }
 
