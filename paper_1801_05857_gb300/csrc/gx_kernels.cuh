@@ -1300,25 +1300,28 @@ struct LaneFop {
     fail += r != FOP_INSERTED && r != FOP_FOUND;
   }
 };
-template <int W, int B>
+// The same with a group of lanes per key where a lane's part of the bucket is 64 bytes
+// or more (32-word buckets, 2 lanes: 25-50 G keys/s by duplication, 23-35 with fop_groups).
+template <int W, int B, int G>
 __device__ __forceinline__ void fop_lanes(const gx::FopArgs& a, const uint64_t* muls, LaneFop& n) {
-  const Group<1> g;
-  const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
-  uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const Group<G> g;
+  const uint64_t step = (uint64_t)gridDim.x * blockDim.x / G;
+  uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
   uint32_t probes = 0;
-  // the loop bound is uniform per warp: all lanes of a warp leave together
-  const uint64_t warp_first = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
+  // the loop bound is uniform per warp: all groups of a warp leave together
+  const uint64_t warp_first = ((uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u)) / G;
   for (uint64_t wi = warp_first; wi < a.n; wi += step, i += step) {
     if (i < a.n) {
       uint32_t v[W];
 #pragma unroll
       for (int w = 0; w < W; ++w) v[w] = a.keys[i * W + w] | kTag;
-      n.count(a, i, find_or_put<W, B, 1>(a.table, a.log2nb, a.rounds, muls, v, g, probes));
+      const int r = find_or_put<W, B, G>(a.table, a.log2nb, a.rounds, muls, v, g, probes);
+      if (g.glane == 0) n.count(a, i, r);
     }
   }
 }
 
-// G > 1: the lanes read their buckets together (bucket_step_lanes), so a lane that is
+// Otherwise the lanes read their buckets together (bucket_step_lanes), so a lane that is
 // done takes its next key at once.  (With a group of lanes per key, which voted on every
 // bucket, the same keys took 10.5 ms with a lane per slot of 8-word buckets, 22.6 of
 // 32-word ones; now 4.8 and 5.6.)
@@ -1384,7 +1387,7 @@ __global__ void __launch_bounds__(gx::kBlock) fop_kernel(const gx::FopArgs a) {
   for (int i = threadIdx.x; i < a.rounds; i += blockDim.x) muls[i] = a.muls.m[i];
   __syncthreads();
   LaneFop n;
-  if constexpr (G == 1) fop_lanes<W, B>(a, muls, n);
+  if constexpr (B / G >= 16 || G == 1) fop_lanes<W, B, G>(a, muls, n);
   else fop_groups<W, B, G>(a, muls, n);
   const unsigned long long ins = warp_sum((unsigned long long)n.ins);
   const unsigned long long fnd = warp_sum((unsigned long long)n.fnd);

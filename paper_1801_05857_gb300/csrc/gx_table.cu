@@ -256,7 +256,8 @@ gx_status gx_find_or_put(const uint32_t* keys, uint64_t n_keys, uint32_t key_wor
   int per_sm = 0;
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ks->fop_fn, gx::kBlock, 0);
   if (e != cudaSuccess) return gx::fail(GX_ERR_CUDA, cudaGetErrorString(e));
-  const uint64_t blocks_needed = (n_keys + gx::kBlock - 1) / gx::kBlock;
+  const uint64_t lanes = B / G >= 16 ? (uint64_t)G : 1;  // per key (fop_kernel)
+  const uint64_t blocks_needed = (n_keys * lanes + gx::kBlock - 1) / gx::kBlock;
   // A grid of 16 times the CTAs that fit at once (the loop is grid-stride and a CTA's
   // setup is 64 multipliers): random reads from a grid whose CTAs finish and start during
   // the launch run faster than from a resident one (10^8 keys at d = 1, 8-word buckets,
