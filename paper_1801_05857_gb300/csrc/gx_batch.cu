@@ -339,7 +339,10 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
             atomicXor(&b.dl_xor, (unsigned long long)h);
           }
         },
-        [&](const uint32_t(&x)[W]) { return !(cache.base && cache.template seen<W>(x)); });
+        [&](bool on, const uint32_t(&x)[W]) {
+          const bool known = cache.base && cache.template seen<W>(on, x);
+          return on && !known;
+        });
     st.flush<W>(tg, err);
     const unsigned long long tr = warp_sum(trans);
     const unsigned long long pr = warp_sum((unsigned long long)probes);

@@ -326,26 +326,33 @@ struct WarpStage {
 
 // Per-warp cache of recently seen vectors (the block-local state cache of
 // Fig. 2, in shared memory, per warp): direct-mapped, overwritten on a miss,
-// never cleared.  Every vector written into it is passed to find-or-put by the
-// lane that wrote it, so a hit means the vector is in the table or being put
-// there by this warp, and its find-or-put can be skipped.  Only for 1- and
-// 2-word vectors, whose entries are read and written by single aligned
-// shared-memory accesses (a torn entry could otherwise fake a hit).
+// never cleared.  A vector written into it goes on to this warp's find-or-put
+// (or was found in the GPU-wide cache), so a hit means the vector is in the table
+// or will be put there by this warp, and its find-or-put can be skipped.
+// A torn entry -- words of two vectors -- could equal a third one and drop it, so
+// an entry must be read and written whole.  1- and 2-word entries are one 32- or
+// 64-bit access.  A 16-byte access is several accesses in no fixed order: for
+// 4-word entries the warp's reads, the choice of one writer per entry and the
+// writes are kept apart.
 struct WarpCache {
   uint32_t* base;  // 2^log2 entries of W words, or nullptr
   uint32_t mask;
+  // For every lane with `on` set: whether v is in the cache; else it is written.  All
+  // 32 lanes call it together.
   template <int W>
-  __device__ __forceinline__ bool seen(const uint32_t (&v)[W]) const {
+  __device__ __forceinline__ bool seen(bool on, const uint32_t (&v)[W]) const {
     uint32_t m = v[0] * 0x9E3779B1u;
     if constexpr (W >= 2) m += v[1] * 0x85EBCA77u;
     if constexpr (W == 4) m += v[2] * 0xC2B2AE3Du + v[3] * 0x27D4EB2Fu;
     const uint32_t i = (m >> 20) & mask;  // (2^12 entries at most)
     if constexpr (W == 1) {
+      if (!on) return false;
       uint32_t* e = base + i;
       if (*e == v[0]) return true;
       *e = v[0];
       return false;
     } else if constexpr (W == 2) {
+      if (!on) return false;
       unsigned long long* e = reinterpret_cast<unsigned long long*>(base) + i;
       const unsigned long long x = (unsigned long long)v[0] | ((unsigned long long)v[1] << 32);
       if (*e == x) return true;
@@ -353,11 +360,17 @@ struct WarpCache {
       return false;
     } else {
       static_assert(W == 4, "slot width");
+      const uint32_t lane = threadIdx.x & 31;
       uint4* e = reinterpret_cast<uint4*>(base) + i;
       const uint4 c = *e;
-      if (c.x == v[0] && c.y == v[1] && c.z == v[2] && c.w == v[3]) return true;
-      *e = make_uint4(v[0], v[1], v[2], v[3]);
-      return false;
+      const bool hit = on && c.x == v[0] && c.y == v[1] && c.z == v[2] && c.w == v[3];
+      const bool miss = on && !hit;
+      __syncwarp();
+      if (miss) e->x = lane;  // (no tag: never a stored vector's first word)
+      __syncwarp();
+      if (miss && e->x == lane) *e = make_uint4(v[0], v[1], v[2], v[3]);
+      __syncwarp();
+      return hit;
     }
   }
 };
@@ -624,7 +637,8 @@ constexpr uint32_t kWideStates = 8;
 //   desc           the descriptors of processes and classes (ProcDescs, ClassDescs)
 //   seen(v)        a lane's state, once, when it is taken
 //   done(v, n)     a lane's state and the number of its successors
-//   keep(x)        the filters before the GPU-wide cache, of a successor
+//   keep(on, x)    the filters before the GPU-wide cache: whether a lane's successor x
+//                  (if on) passes them; all 32 lanes call it together
 // All 32 lanes call it together; returns with the queues empty.  Wide: whether
 // few states are treated so at all.
 template <int W, int B, int G, int Batch, bool Wide = true, class T, class Desc, class Next, class Seen, class Done,
@@ -693,7 +707,7 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
       for (int i = 0; i < K; ++i) {
         const int at = (int)lane + 32 * i;
         load_vec<W>(q.raw + (n_raw + at) * W, x[i]);  // (past the k-th entry: not used)
-        on[i] = at < k && keep(x[i]);
+        on[i] = keep(at < k, x[i]);
       }
       if (tg.gcache().base) {
         SeenEntry e[K];
@@ -832,15 +846,16 @@ __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expa
           if (di < a.dl_cap) store_vec<W>(a.dl_buf + di * W, v);
         }
       },
-      [&](const uint32_t(&x)[W]) {
+      [&](bool on, const uint32_t(&x)[W]) {
         // region passes: a vector whose first bucket lies outside this pass's region is
         // left to the pass of that region (tested before the caches, which may only hold
         // vectors that went to find-or-put).  A vector this warp has already sent to
         // find-or-put needs no second lookup, nor does one that any warp found or
         // inserted moments ago.
         if (a.region_mask && (bucket_of(state_hash<W>(x), muls[0], a.log2nb) & a.region_mask) != a.region_bits)
-          return false;
-        return !(cache.base && cache.template seen<W>(x));
+          on = false;
+        const bool known = cache.base && cache.template seen<W>(on, x);
+        return on && !known;
       });
   st.flush<W>(tg, err);
   // the CTA's totals, one atomic per counter: at the end of a level every warp
@@ -1032,7 +1047,7 @@ __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThrea
             if (di < a.dl_cap) store_vec<W>(a.dl_buf + di * W, v);
           }
         },
-        [](const uint32_t(&)[W]) { return true; });
+        [](bool on, const uint32_t(&)[W]) { return on; });
     st.flush<W>(tg, err);
     const unsigned long long tr = warp_sum((unsigned long long)trans), pr = warp_sum((unsigned long long)probes);
     err = __reduce_or_sync(FULLMASK, err);

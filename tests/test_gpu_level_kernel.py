@@ -146,3 +146,14 @@ def test_find_or_put_of_any_number_of_keys(cuda, n, words, bucket, group):
         assert torch.equal(torch.unique(held, dim=0), placed)
         if rounds == 32:
             assert (ins, fnd, full) == (len(distinct), n - len(distinct), 0)
+
+
+@pytest.mark.parametrize("passes", [1, 2])
+@pytest.mark.parametrize("log2", [2, 3, 7])
+def test_small_warp_caches_of_4_word_vectors_lose_no_state(cuda, log2, passes):
+    """16-byte entries of the per-warp cache: with two or four of them every batch has many
+    lanes that miss on the same entry, and only one of them may write it.  An entry made of
+    two vectors could equal a third, which would then never be stored."""
+    s = _check(4, NETS[4], table_bytes=1 << 24, bucket_words=8, group_lanes=1, hash_rounds=32, host_loop=1,
+               region_passes=passes, warp_cache_log2=log2, global_cache_log2=0)
+    assert s["slot_words"] == 4 and s["region_passes"] == passes and s["global_cache_entries"] == 0
