@@ -971,9 +971,11 @@ struct LoopState {
   }
 };
 
+// (Not the .aligned forms: those want a warp whose lanes arrive together, and one lane
+// keeps the books of a level just before.)
 __device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
 }
 
 // Levels of at most kSmallLevel states, one after the other in one launch by one

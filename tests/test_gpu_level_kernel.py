@@ -157,3 +157,17 @@ def test_small_warp_caches_of_4_word_vectors_lose_no_state(cuda, log2, passes):
     s = _check(4, NETS[4], table_bytes=1 << 24, bucket_words=8, group_lanes=1, hash_rounds=32, host_loop=1,
                region_passes=passes, warp_cache_log2=log2, global_cache_log2=0)
     assert s["slot_words"] == 4 and s["region_passes"] == passes and s["global_cache_entries"] == 0
+
+
+@pytest.mark.parametrize("passes", [1, 2])
+@pytest.mark.parametrize("n", [6, 7])
+def test_few_state_levels_hand_over_in_a_stopped_search(cuda, n, passes):
+    """A search whose levels grow past the few-state kernel's limit (512 states) stops at its
+    first deadlock: what that kernel did before the hand-over, the large levels after it
+    (one or two region passes) and the stop give the oracle's results."""
+    net = inputs.random_network(8, n, 8, 0, 3, 8, n_sync=n - 1, parties=2)
+    r = _want[("stopped", n)] = oracle.explore(net, stop_at_first_deadlock=True)
+    assert max(r.levels) > 512 and r.deadlock_count and not r.complete
+    s = _check(("stopped", n), net, table_bytes=1 << 24, bucket_words=8, group_lanes=1, hash_rounds=32,
+               region_passes=passes, stop_at_first_deadlock=1)
+    assert s["complete"] == 0 and s["first_deadlock_level"] == r.first_deadlock_level
