@@ -170,7 +170,8 @@ typedef struct gx_explore_opts {
   uint32_t guided_bins;          /* GX_DL_GUIDED: priority bins; 0 = 32 */
   uint32_t warp_cache_log2;      /* per-warp cache of recently seen vectors (the block-local
                                     state cache of Fig. 2): 2^n entries per warp in shared
-                                    memory (2^(n-1) for 4-word vectors, the same bytes), a hit
+                                    memory (2^(n-1) for 4-word vectors with more than 64 field
+                                    bits), a hit
                                     skips find-or-put.  0 = off, 1..12 = 2^n, 0xFFFFFFFF =
                                     automatic (gx_default_opts): 2^7 unless the GPU-wide
                                     cache below is in use (together they measured slower) */

@@ -265,7 +265,7 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
   WarpNet& wn = S.net[wid];
   uint4* descs = S.descs[wid];
   WarpStage st{S.stage[wid], 0};
-  WarpCache cache{W <= 2 ? S.cache[wid] : nullptr, (1u << kBatchCacheLog2) - 1u};
+  WarpCache cache{W <= 2 ? S.cache[wid] : nullptr, (1u << kBatchCacheLog2) - 1u, nullptr};
   const SmemTarget tg{&wn, a.rounds};
   const uint32_t* t = nullptr;
   int net = -1, base = 0;

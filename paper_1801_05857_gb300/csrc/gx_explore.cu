@@ -59,6 +59,26 @@ uint32_t auto_cache_log2(const Net& net) {
   return cache_key(net, at, bits) ? cache_auto_log2(bits) : 0;
 }
 
+gx_status warp_cache_layout(const Net& net, uint32_t warp_log2, ExpandArgs& a, size_t& bytes) {
+  a.cache_log2 = a.cache_key64 = 0;
+  bytes = 0;
+  if (warp_log2 == 0) return GX_OK;
+  if (warp_log2 > 12) return fail(GX_ERR_INVALID, "warp_cache_log2 must be at most 12");
+  a.cache_log2 = (int)warp_log2;
+  uint32_t bits = 0;
+  size_t entry = 4ull * net.slot_words;
+  if (net.slot_words == 4) {
+    if (cache_key(net, a.gcache.word_at, bits)) {
+      a.cache_key64 = 1;
+      entry = 8;
+    } else {
+      a.cache_log2 -= 1;  // 16-byte entries: the same bytes
+    }
+  }
+  bytes = entry * (kBlock / 32) << a.cache_log2;
+  return GX_OK;
+}
+
 }  // namespace gx
 
 namespace gx {
@@ -620,13 +640,7 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
   GX_CUDA(cudaFuncGetAttributes(&fa, P.ks->expand_fn));
   const size_t blob_bytes = 4ull * net.blob.size();
   size_t cache_bytes = 0;
-  ea.cache_log2 = 0;
-  if (P.warp_log2) {
-    ea.cache_log2 = (int)P.warp_log2;
-    if (ea.cache_log2 > 12) return fail(GX_ERR_INVALID, "warp_cache_log2 must be at most 12");
-    if (P.W == 4) ea.cache_log2 -= 1;  // 16-byte entries: the same bytes as 2^n 2-word ones
-    cache_bytes = 4ull * P.W * (kBlock / 32) * (1ull << ea.cache_log2);
-  }
+  if ((s = warp_cache_layout(net, P.warp_log2, ea, cache_bytes)) != GX_OK) return s;
   size_t smem = 8ull * kMaxRounds + cache_bytes;
   if (fa.sharedSizeBytes + smem > dev.smem_optin)
     return fail(GX_ERR_INVALID, "warp cache of 2^" + std::to_string(ea.cache_log2) + " entries per warp needs " +

@@ -55,7 +55,8 @@ struct SeenCache {
   uint32_t mask;      // 2^n - 1
   uint32_t mix_shift; // 32 - n
   uint32_t log2_bytes;  // of an entry: 1, 2 or 3
-  uint32_t word_at[3];  // bit offset in the key of the payload of words 1, 2, 3 (64: no fields)
+  uint32_t word_at[3];  // bit offset in the key of the payload of words 1, 2, 3 (64: no fields;
+                        // set without a cache too, for the per-warp one)
 };
 
 struct ExpandArgs {
@@ -74,6 +75,7 @@ struct ExpandArgs {
   uint32_t* dl_buf;          // deadlock vectors, W words each
   uint32_t dl_cap;
   int cache_log2;            // per-warp cache of recently seen vectors: 2^cache_log2 entries (0 = off)
+  int cache_key64;           // its entries are 64-bit keys (4-word vectors whose fields fit)
   // safety check: a state whose field (word, shift, mask) equals watch_value violates
   int watch;
   uint32_t watch_word, watch_shift, watch_mask, watch_value;
@@ -184,6 +186,10 @@ void hash_multipliers(uint64_t* out, int n);
 // none).
 bool cache_layout(const Net& net, uint32_t log2_entries, SeenCache& c);
 uint32_t auto_cache_log2(const Net& net);
+
+// Per-warp cache of 2^warp_log2 entries (gx_explore_opts.warp_cache_log2): fills in
+// a's and the bytes it takes in a CTA.  GX_ERR_INVALID above 2^12.
+gx_status warp_cache_layout(const Net& net, uint32_t warp_log2, ExpandArgs& a, size_t& bytes);
 
 // GX_DL_GUIDED search (gx_guided.cu).
 gx_status run_guided(gx_net* h, const gx_explore_opts* opts, void* ws, uint64_t ws_bytes, cudaStream_t st);

@@ -196,13 +196,7 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
   NA_CUDA(cudaFuncGetAttributes(&fa, ks->expand_fn));
   const size_t blob_bytes = 4ull * net.blob.size();
   size_t cache_bytes = 0;
-  ea.cache_log2 = 0;
-  if (warp_log2) {
-    ea.cache_log2 = (int)warp_log2;
-    if (ea.cache_log2 > 12) return gx::fail(GX_ERR_INVALID, "warp_cache_log2 must be at most 12");
-    if (W == 4) ea.cache_log2 -= 1;  // 16-byte entries: the same bytes as 2^n 2-word ones
-    cache_bytes = 4ull * W * (gx::kBlock / 32) * (1ull << ea.cache_log2);
-  }
+  if ((s = gx::warp_cache_layout(net, warp_log2, ea, cache_bytes)) != GX_OK) return s;
   size_t smem = 8ull * gx::kMaxRounds + cache_bytes;
   if (fa.sharedSizeBytes + smem > (size_t)smem_optin)
     return gx::fail(GX_ERR_INVALID, "warp cache of 2^" + std::to_string(ea.cache_log2) +

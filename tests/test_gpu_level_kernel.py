@@ -148,13 +148,26 @@ def test_find_or_put_of_any_number_of_keys(cuda, n, words, bucket, group):
             assert (ins, fnd, full) == (len(distinct), n - len(distinct), 0)
 
 
+# 4-word vectors of 60, 64 (the longest 64-bit cache key, all ones reached) and 65 field bits
+WIDE_NETS = {
+    60: NETS[4],
+    64: _mostly_still(16, 4, 16),
+    65: inputs.Network(1, _mostly_still(16, 4, 16).procs + _mostly_still(1, 1).procs, []),
+}
+WIDE_NETS[64].procs[4:] = [inputs.LTS(16, 15, [])] * 12
+
+
 @pytest.mark.parametrize("passes", [1, 2])
-@pytest.mark.parametrize("log2", [2, 3, 7])
-def test_small_warp_caches_of_4_word_vectors_lose_no_state(cuda, log2, passes):
-    """16-byte entries of the per-warp cache: with two or four of them every batch has many
-    lanes that miss on the same entry, and only one of them may write it.  An entry made of
-    two vectors could equal a third, which would then never be stored."""
-    s = _check(4, NETS[4], table_bytes=1 << 24, bucket_words=8, group_lanes=1, hash_rounds=32, host_loop=1,
+@pytest.mark.parametrize("log2", [1, 2, 3, 7])
+@pytest.mark.parametrize("bits", [60, 64, 65])
+def test_small_warp_caches_of_4_word_vectors_lose_no_state(cuda, bits, log2, passes):
+    """The per-warp cache of 4-word vectors, entries of 8 bytes up to 64 field bits and of 16
+    above: with a few of them every batch has many lanes that miss on the same entry, and
+    only one of them may write it.  An entry made of two vectors could equal a third, which
+    would then never be stored."""
+    net = WIDE_NETS[bits]
+    assert gx.layout(gx.load_network(net))["field_bits"].sum() == bits
+    s = _check(("wide", bits), net, table_bytes=1 << 24, bucket_words=8, group_lanes=1, hash_rounds=32, host_loop=1,
                region_passes=passes, warp_cache_log2=log2, global_cache_log2=0)
     assert s["slot_words"] == 4 and s["region_passes"] == passes and s["global_cache_entries"] == 0
 
