@@ -63,10 +63,12 @@ __device__ __forceinline__ uint32_t saddr(const void* p) { return (uint32_t)__cv
 
 // The scoring threads (warps 0-3 of the CTA, TMEM lanes 0-127) synchronise on
 // named barrier 1 among themselves, so a larger CTA whose other warps do
-// something else can score tiles too.
+// something else can score tiles too.  (barrier.sync, not bar.sync, here and below: the
+// latter wants a warp's lanes to arrive together, and they come out of polling loops
+// and branches that one lane takes.)
 constexpr int kTcBarrier = 1;
 __device__ __forceinline__ void tc_sync() {
-  asm volatile("bar.sync %0, %1;" ::"n"(kTcBarrier), "n"(kRows) : "memory");
+  asm volatile("barrier.sync %0, %1;" ::"n"(kTcBarrier), "n"(kRows) : "memory");
 }
 // OR of pred over the scoring threads, in every one of them.
 __device__ __forceinline__ int tc_sync_or(int pred) {
@@ -74,7 +76,7 @@ __device__ __forceinline__ int tc_sync_or(int pred) {
   asm volatile(
       "{\n\t.reg .pred p, q;\n\t"
       "setp.ne.b32 p, %1, 0;\n\t"
-      "bar.red.or.pred q, %2, %3, p;\n\t"
+      "barrier.red.or.pred q, %2, %3, p;\n\t"
       "selp.b32 %0, 1, 0, q;\n\t}"
       : "=r"(r)
       : "r"(pred), "n"(kTcBarrier), "n"(kRows)
@@ -149,6 +151,7 @@ __device__ __forceinline__ void mma_commit(uint32_t mbar) {
 // 32 w .. 32 w + 31); waits for the load before returning.
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float (&v)[32]) {
   uint32_t r[32];
+  __syncwarp();  // a warp-wide instruction: the lanes may come from a polling loop
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
       "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
@@ -609,7 +612,7 @@ __device__ __forceinline__ bool score_tiles(void* dyn, const ScoreWeights* __res
     asm volatile(
         "{\n\t.reg .pred p, q;\n\t"
         "setp.ne.b32 p, %1, 0;\n\t"
-        "bar.red.or.pred q, %2, %3, p;\n\t"
+        "barrier.red.or.pred q, %2, %3, p;\n\t"
         "selp.b32 %0, 1, 0, q;\n\t}"
         : "=r"(r)
         : "r"((int)gave_up), "r"(1 + slot), "n"(kScoreSlotThreads)
