@@ -588,14 +588,8 @@ __global__ void __launch_bounds__(256) update_kernel(const float* __restrict__ p
                                                      TcTrainWeights* __restrict__ packed, float* __restrict__ loss) {
   const int q = blockIdx.x * blockDim.x + threadIdx.x;  // moments lie as the partial gradients do
   const int i = partial_param(q < NPARAM ? q : 0);
-  // m, v and p were last written by the step before, which the gradient in front
-  // has waited for: only the partial gradients need the wait
-  float m0 = 0.f, v0 = 0.f, p0 = 0.f;
-  if (q < NPARAM) {
-    m0 = m[q];
-    v0 = v[q];
-    p0 = p[i];
-  }
+  // (m, v and p too, which the step before wrote: only the wait makes another grid's
+  // writes visible, although the gradient in front has waited for that step)
   grid_dependency_wait();
   grid_dependency_launch();
   if (q == 0) {
@@ -604,9 +598,12 @@ __global__ void __launch_bounds__(256) update_kernel(const float* __restrict__ p
     *loss = l;
   }
   if (q >= NPARAM) return;
+  const float m0 = m[q], v0 = v[q], p0 = p[i];
   const float gi = partial_sum(partial, ctas, q);
-  const float mi = 0.9f * m0 + 0.1f * gi;
-  const float vi = 0.999f * v0 + 0.001f * gi * gi;
+  // (which product is fused with the sum is written out: left to the compiler it has
+  // changed with the order of the loads, and the trained bits with it)
+  const float mi = __fmaf_rn(0.1f, gi, __fmul_rn(0.9f, m0));
+  const float vi = __fmaf_rn(__fmul_rn(0.001f, gi), gi, __fmul_rn(0.999f, v0));
   m[q] = mi;
   v[q] = vi;
   const float x = p0 - lr * (mi / (1.f - b1t)) / (sqrtf(vi / (1.f - b2t)) + 1e-8f);

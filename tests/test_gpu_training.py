@@ -66,3 +66,41 @@ def test_training_is_reproducible(cuda):
     la, lb = gx.mlp_train(a, h, lab, 700, 60, 1e-3, 5), gx.mlp_train(b, h, lab, 700, 60, 1e-3, 5)
     assert torch.equal(a, b) and torch.equal(la, lb)
     assert float(la[-10:].mean()) < float(la[:10].mean())
+
+
+@pytest.mark.parametrize("batch", [1, 300, 256 * 128 + 5])
+def test_every_step_is_an_adam_step_at_the_weights_before_it(cuda, batch):
+    """Steps 0..4 one by one: the parameters after step k are those before it moved by an Adam
+    step whose gradient mlp_grad takes at them, over the examples that step draws, and the
+    step's loss is mlp_grad's.  mlp_grad packs the FP32 parameters by a kernel of its own, so
+    a weight, bias or transposed copy that the update left stale shows in the next step.
+
+    Tolerance: the gradients are the same sums in the same order, so what differs is FP32
+    rounding in the update (under 20 roundings of 2^-24 relative, on an update of a few lr)
+    and the rounding of the parameter itself."""
+    import torch
+    hist, label, p0 = _data(5000, batch)
+    dh, dl = torch.from_numpy(hist).cuda(), torch.from_numpy(label).cuda()
+    lr, seed, steps = 1e-3, 31, 5
+    f = lambda x: float(np.float32(x))
+    m = np.zeros(gx.MLP_PARAMS)
+    v = np.zeros(gx.MLP_PARAMS)
+    b1t = b2t = 1.0
+    before = p0.clone()
+    for k in range(steps):
+        idx = torch.from_numpy(_drawn(seed, k, batch, len(hist))).cuda()
+        g, loss = gx.mlp_grad(before, dh[idx].contiguous(), dl[idx].contiguous())
+        after = p0.clone()
+        losses = gx.mlp_train(after, dh, dl, batch, k + 1, lr, seed)
+        assert abs(float(losses[k]) - float(loss)) <= 1e-6 * float(loss)
+        g = g.cpu().numpy().astype(np.float64)
+        m = f(0.9) * m + f(0.1) * g
+        v = f(0.999) * v + f(0.001) * g * g
+        b1t, b2t = b1t * 0.9, b2t * 0.999
+        c1, c2 = f(np.float32(1) - np.float32(b1t)), f(np.float32(1) - np.float32(b2t))
+        move = f(lr) * (m / c1) / (np.sqrt(v / c2) + f(1e-8))
+        p = before.cpu().numpy().astype(np.float64)
+        got = after.cpu().numpy().astype(np.float64)
+        assert (np.abs(got - (p - move)) <= 20 * 2.0 ** -24 * np.abs(move) + 2.0 ** -23 * np.abs(p) + 1e-12).all()
+        assert np.abs(got - p).max() > 0.1 * lr
+        before = after
