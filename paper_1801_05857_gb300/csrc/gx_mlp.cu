@@ -198,9 +198,14 @@ struct __align__(1024) TrainSmem {
 constexpr size_t kTrainSmemBytes = sizeof(TrainSmem) + 1024;  // + alignment slack
 static_assert(kTrainSmemBytes <= 232448, "a training CTA must fit the SM's shared memory");
 
-// W2^T in the core-matrix layout: item (row j, K group g) packs W2[8g .. 8g+7][j].
+__device__ unsigned int g_train_error;  // a bounded wait gave up (GX_ERR_SPIN_LIMIT)
+
+// The first kernel of a call: clears the error flag (under the call's lock, like all that
+// reads or sets it) and packs the parameters.  W2^T in the core-matrix layout: item (row j,
+// K group g) packs W2[8g .. 8g+7][j].
 constexpr int kTrainPackItems = gxt::kTcPackItems + H * 16;
 __global__ void train_pack_kernel(const float* __restrict__ p, TcTrainWeights* __restrict__ out) {
+  if (blockIdx.x == 0 && threadIdx.x == 0) g_train_error = 0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kTrainPackItems; i += gridDim.x * blockDim.x) {
     if (i < gxt::kTcPackItems) {
       gxt::tc_pack_item(p, &out->fw, i);
@@ -248,7 +253,6 @@ __device__ __forceinline__ float warp_column_sums(float (&v)[32]) {
   return v[0];
 }
 
-__device__ unsigned int g_train_error;  // a bounded wait gave up (GX_ERR_SPIN_LIMIT)
 // The weights a gradient is taken at, packed for the tensor cores (one copy per
 // device; calls hold g_train_mutex from packing to completion).
 __device__ TcTrainWeights g_train_packed;
@@ -758,8 +762,6 @@ gx_status gx_mlp_grad(const float* params, const uint8_t* hist, const float* lab
   const int grid = (int)std::min<uint64_t>((n + gxt::kRows - 1) / gxt::kRows, gxm::kGradCtas);
   float* scratch = nullptr;  // one partial gradient and loss per CTA
   GM_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&scratch), sizeof(float) * (uint64_t)grid * (gxm::kPartial + 1), st));
-  const unsigned int zero = 0;
-  GM_CUDA(cudaMemcpyToSymbolAsync(gxm::g_train_error, &zero, sizeof(zero), 0, cudaMemcpyHostToDevice, st));
   std::lock_guard<std::mutex> lock(g_train_mutex);
   gxm::TcTrainWeights* packed = nullptr;
   GM_CUDA(cudaGetSymbolAddress(reinterpret_cast<void**>(&packed), gxm::g_train_packed));
@@ -794,8 +796,6 @@ gx_status gx_mlp_train(float* params, float* state, const uint8_t* hist, const f
   float* partial = partial_loss + gxm::kGradCtas;
   GM_CUDA(cudaMemsetAsync(state, 0, sizeof(float) * 2 * gxm::NPARAM, st));
   GM_CUDA(cudaMemsetAsync(loss, 0, sizeof(float) * steps, st));
-  const unsigned int zero = 0;
-  GM_CUDA(cudaMemcpyToSymbolAsync(gxm::g_train_error, &zero, sizeof(zero), 0, cudaMemcpyHostToDevice, st));
   std::lock_guard<std::mutex> lock(g_train_mutex);
   gxm::TcTrainWeights* packed = nullptr;
   GM_CUDA(cudaGetSymbolAddress(reinterpret_cast<void**>(&packed), gxm::g_train_packed));
