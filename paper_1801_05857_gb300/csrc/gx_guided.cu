@@ -366,6 +366,24 @@ __global__ void __launch_bounds__(gx::kBlock) label_lookup_round_kernel(const La
   }
 }
 
+// Histogram i of the caller's array, whose address need not be a multiple of 16.
+__device__ __forceinline__ uint4 hist_load(const uint8_t* hist, uint64_t i) {
+  if ((reinterpret_cast<uintptr_t>(hist) & 15) == 0) return reinterpret_cast<const uint4*>(hist)[i];
+  uint32_t w[4] = {0, 0, 0, 0};
+#pragma unroll
+  for (int k = 0; k < 16; ++k) w[k >> 2] |= (uint32_t)hist[i * 16 + k] << ((k & 3) * 8);
+  return make_uint4(w[0], w[1], w[2], w[3]);
+}
+__device__ __forceinline__ void hist_store(uint8_t* hist, uint64_t i, const uint4& q) {
+  if ((reinterpret_cast<uintptr_t>(hist) & 15) == 0) {
+    reinterpret_cast<uint4*>(hist)[i] = q;
+    return;
+  }
+  const uint32_t w[4] = {q.x, q.y, q.z, q.w};
+#pragma unroll
+  for (int k = 0; k < 16; ++k) hist[i * 16 + k] = (uint8_t)(w[k >> 2] >> ((k & 3) * 8));
+}
+
 // Example i: the histogram and the label of state i of the list.
 template <int W>
 __global__ void __launch_bounds__(gx::kBlock) label_gather_kernel(const LabelArgs a, uint32_t max_dist,
@@ -378,7 +396,7 @@ __global__ void __launch_bounds__(gx::kBlock) label_gather_kernel(const LabelArg
     local_hist<W>(a.blob, a.lay, v, hw, bad);
     if (bad) atomicOr(&a.ctl->bad, 1ull);
     if (i >= cap) continue;
-    reinterpret_cast<uint4*>(hist_out)[i] = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+    hist_store(hist_out, i, make_uint4(hw[0], hw[1], hw[2], hw[3]));
     const uint32_t d = a.d[i] == INF ? max_dist : min(a.d[i], max_dist);
     label_out[i] = (float)d / (float)max_dist;
   }
@@ -440,7 +458,7 @@ __global__ void __launch_bounds__(kTileThreads) ex_tile_kernel(uint4* h, uint32_
       sh[i] = h[base + i];
       sl[i] = l[base + i];
     } else if (base + i < n) {
-      sh[i] = reinterpret_cast<const uint4*>(hist)[base + i];
+      sh[i] = hist_load(hist, base + i);
       sl[i] = __float_as_uint(label[base + i]);
     } else {
       sh[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
@@ -523,7 +541,7 @@ __global__ void __launch_bounds__(256) ex_wide_kernel(uint4* h, uint32_t* l, uin
 
 __global__ void ex_store_kernel(const uint4* h, const uint32_t* l, uint64_t n, uint8_t* hist, float* label) {
   for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x) {
-    reinterpret_cast<uint4*>(hist)[i] = h[i];
+    hist_store(hist, i, h[i]);
     label[i] = __uint_as_float(l[i]);
   }
 }

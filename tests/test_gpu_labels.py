@@ -82,3 +82,33 @@ def test_examples_come_sorted_at_every_size(cuda, cap):
     keys = [tuple(w) + (float(x),) for w, x in zip(words.tolist(), label)]
     assert keys == sorted(keys)
     assert hist.sum(1).tolist() == [7] * n  # every row is a state's histogram
+
+
+@pytest.mark.parametrize("offset", [1, 4, 8])
+@pytest.mark.parametrize("cap", [1, 2, 2049, 10206])
+def test_examples_at_odd_addresses(cuda, cap, offset):
+    """The histograms' address need not be a multiple of 16: the same examples as at one (with
+    cap below the states found, which ones are written is open: they are sorted histograms)."""
+    import torch
+    net = inputs.token_ring(7)  # 10,206 states
+    h = gx.load_network(net)
+    o = gx.default_opts(table_bytes=1 << 20, hash_rounds=32)
+    ws = gx.alloc_workspace(h, o)
+    gx.explore(h, o, ws)
+    s = gx.stats(h)
+    dist = torch.empty(s["table_slots"], dtype=torch.int32, device="cuda")
+    flat = torch.full((16 * cap + offset + 16,), 0xA5, dtype=torch.uint8, device="cuda")
+    assert flat.data_ptr() % 16 == 0
+    label = torch.zeros(cap, dtype=torch.float32, device="cuda")
+    n = ctypes.c_uint64()
+    gx._check(gx.lib().gx_training_set(h.handle, ws.data_ptr(), ws.numel(), None, dist.data_ptr(), 16,
+                                       flat.data_ptr() + offset, label.data_ptr(), cap, ctypes.byref(n)))
+    assert n.value == s["states"]
+    got = flat.cpu().numpy()
+    assert (got[:offset] == 0xA5).all() and (got[offset + 16 * cap:] == 0xA5).all()
+    hist = got[offset:offset + 16 * cap].reshape(cap, 16)
+    keys = [tuple(w) + (float(x),) for w, x in zip(np.ascontiguousarray(hist).view("<u4").tolist(), label.cpu())]
+    assert keys == sorted(keys) and (hist.sum(1) == 7).all()
+    if cap >= s["states"]:
+        want_hist, want_label = gx.training_set(h, ws, 16)
+        assert (want_hist.cpu().numpy() == hist).all() and torch.equal(want_label, label)
