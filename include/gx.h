@@ -374,12 +374,13 @@ gx_status gx_set_digest(gx_net* net, void* workspace, uint64_t workspace_bytes, 
  * uint32 per table slot (gx_stats table_slots).  *n_out = states found (may
  * exceed cap).  The examples come sorted by content (the 16 histogram bytes,
  * then the label's bits, as unsigned words), so with cap >= *n_out the output
- * is the same on every run.  Temporary device memory (cudaMallocAsync on
- * `stream`): 28 bytes per state and, after a complete search of at most 2^28
- * transitions, 4 per transition (left out when there is no room), or the
- * sort's 20 bytes per example, the count rounded up to a power of two, if that
- * is more.  GX_ERR_INVALID if a process has more than 16 local states;
- * GX_ERR_STATE if the workspace no longer holds the search's table. */
+ * is the same on every run.  The states are those the workspace's table holds
+ * now.  Temporary device memory (cudaMallocAsync on `stream`) that must be had:
+ * the sort's 20 bytes per example written, the count rounded up to a power of
+ * two (none for fewer than two).  Where there is room, and below 2^32 states,
+ * the call also takes 28 bytes per state and, after a complete search of at
+ * most 2^28 transitions, 4 per transition, first, and is several times faster
+ * for it.  GX_ERR_INVALID if a process has more than 16 local states. */
 gx_status gx_training_set(gx_net* net, void* workspace, uint64_t workspace_bytes, void* stream,
                           uint32_t* dist_scratch, uint32_t max_dist, uint8_t* hist_out,
                           float* label_out, uint64_t cap, uint64_t* n_out);

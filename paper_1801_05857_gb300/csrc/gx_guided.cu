@@ -155,7 +155,7 @@ struct LabelArgs {
   uint64_t slots;
   uint64_t cap;           // states the last search stored: the lists' size
   uint64_t adj_cap;       // successors there is room for in adj (0: not kept)
-  uint32_t* index;        // [slots]
+  uint32_t* index;        // [slots] (without lists: a slot's distance)
   unsigned long long* slot_of;  // [cap]
   uint32_t* d;            // [cap]
   uint32_t* first;        // [cap] where a state's successors start in adj
@@ -399,6 +399,83 @@ __global__ void __launch_bounds__(gx::kBlock) label_gather_kernel(const LabelArg
     hist_store(hist_out, i, make_uint4(hw[0], hw[1], hw[2], hw[3]));
     const uint32_t d = a.d[i] == INF ? max_dist : min(a.d[i], max_dist);
     label_out[i] = (float)d / (float)max_dist;
+  }
+}
+
+// ---- labelling without lists, in the caller's scratch alone (dist: a distance per
+// slot): for tables of 2^32 or more states, for lack of memory, and for a table that
+// is not the one the last search left.  Every round passes over the whole table.
+
+template <int W>
+__device__ __forceinline__ bool slot_vec(const uint32_t* table, uint64_t i, uint32_t (&v)[W]) {
+  load_vec<W>(table + i * W, v);
+  bool tagged = true;
+#pragma unroll
+  for (int w = 0; w < W; ++w) tagged &= (v[w] & kTag) != 0;
+  return tagged;
+}
+
+template <int W>
+__global__ void __launch_bounds__(gx::kBlock) slot_init_kernel(const LabelArgs a) {
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.slots; i += stride) {
+    uint32_t v[W];
+    a.index[i] = slot_vec<W>(a.table, i, v) && count_succ<W>(a.blob, a.lay, v) == 0 ? 0u : INF;
+  }
+}
+
+// Round r: sets *changed when a slot was labelled.
+template <int W, int B>
+__global__ void __launch_bounds__(gx::kBlock) slot_round_kernel(const LabelArgs a, uint32_t r,
+                                                                unsigned long long* changed) {
+  extern __shared__ __align__(16) uint32_t s_tab[];
+  __shared__ uint64_t muls[kMaxRounds];
+  const uint32_t* t = label_tables(a, muls, s_tab);
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  bool any = false;
+  for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.slots; i += stride) {
+    uint32_t v[W];
+    if (a.index[i] != INF || !slot_vec<W>(a.table, i, v)) continue;
+    const uint32_t cnt = count_succ<W>(t, a.lay, v);
+    SuccIter it;
+    it.init();
+    for (uint32_t k = 0; k < cnt; ++k) {
+      uint32_t s[W];
+      next_succ<W>(it, t, a.lay, v, s);
+      const int64_t j = find_slot<W, B>(a.table, a.log2nb, a.rounds, muls, s);
+      if (j >= 0 && a.index[j] == r - 1) {
+        a.index[i] = r;
+        any = true;
+        break;
+      }
+    }
+  }
+  if (any) *changed = 1;
+}
+
+// Examples of the occupied slots, at positions counted in out[0]; out[1]: a local state
+// index of 16 or more.
+template <int W>
+__global__ void __launch_bounds__(gx::kBlock) slot_gather_kernel(const LabelArgs a, uint32_t max_dist,
+                                                                 uint8_t* hist_out, float* label_out, uint64_t cap,
+                                                                 unsigned long long* out) {
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t stride = (uint64_t)gridDim.x * blockDim.x;
+  for (uint64_t i0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); i0 < a.slots; i0 += stride) {
+    uint32_t v[W], hw[4], bad = 0;
+    const uint64_t i = i0 + lane;
+    const bool has = i < a.slots && slot_vec<W>(a.table, i, v);
+    const uint32_t m = __ballot_sync(FULLMASK, has);
+    unsigned long long base = 0;
+    if (lane == 0 && m) base = atomicAdd(out, (unsigned long long)__popc(m));
+    const unsigned long long pos = __shfl_sync(FULLMASK, base, 0) + __popc(m & ((1u << lane) - 1u));
+    if (!has) continue;
+    local_hist<W>(a.blob, a.lay, v, hw, bad);
+    if (bad) out[1] = 1;
+    if (pos >= cap) continue;
+    hist_store(hist_out, pos, make_uint4(hw[0], hw[1], hw[2], hw[3]));
+    const uint32_t d = min(a.index[i], max_dist);  // (INF: max_dist)
+    label_out[pos] = (float)d / (float)max_dist;
   }
 }
 
@@ -1146,11 +1223,39 @@ namespace {
 
 inline uint64_t a256(uint64_t x) { return (x + 255) & ~255ull; }
 
+// Temporary device memory of one call, stream-ordered; given back at the end.
+struct TempMem {
+  cudaStream_t st;
+  unsigned char* p = nullptr;
+  uint64_t bytes = 0;
+  explicit TempMem(cudaStream_t s) : st(s) {}
+  TempMem(const TempMem&) = delete;
+  TempMem& operator=(const TempMem&) = delete;
+  bool alloc(uint64_t n) {
+    if (cudaMallocAsync(reinterpret_cast<void**>(&p), n, st) == cudaSuccess) {
+      bytes = n;
+      return true;
+    }
+    cudaGetLastError();
+    p = nullptr;
+    return false;
+  }
+  void release() {
+    if (p) cudaFreeAsync(p, st);
+    p = nullptr;
+    bytes = 0;
+  }
+  ~TempMem() { release(); }
+};
+
 struct GKernels {
   void (*label_collect)(gxd::LabelArgs);
   void (*label_adj)(gxd::LabelArgs);
   void (*label_lookup_round)(gxd::LabelArgs, uint32_t);
   void (*label_gather)(gxd::LabelArgs, uint32_t, uint8_t*, float*, uint64_t);
+  void (*slot_init)(gxd::LabelArgs);
+  void (*slot_round)(gxd::LabelArgs, uint32_t, unsigned long long*);
+  void (*slot_gather)(gxd::LabelArgs, uint32_t, uint8_t*, float*, uint64_t, unsigned long long*);
   const void* init;
   const void* select;
   const void* expand;
@@ -1164,7 +1269,8 @@ struct GKernels {
 template <int W, int B>
 GKernels gk() {
   return GKernels{&gxd::label_collect_kernel<W>, &gxd::label_adj_kernel<W, B>, &gxd::label_lookup_round_kernel<W, B>,
-                  &gxd::label_gather_kernel<W>,
+                  &gxd::label_gather_kernel<W>, &gxd::slot_init_kernel<W>, &gxd::slot_round_kernel<W, B>,
+                  &gxd::slot_gather_kernel<W>,
                   reinterpret_cast<const void*>(&gxd::guided_init_kernel<W, B>),
                   reinterpret_cast<const void*>(&gxd::guided_select_kernel<W>),
                   reinterpret_cast<const void*>(&gxd::guided_expand_kernel<W, B>),
@@ -1591,7 +1697,6 @@ gx_status gx_training_set(gx_net* h, void* ws, uint64_t ws_bytes, void* stream, 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   char* base = static_cast<char*>(ws);
   const uint64_t slots = S.table_slots, states = S.states;
-  if (states >= (1ull << 32)) return gx::fail(GX_ERR_OOM, "2^32 or more states to label");
   gxd::LabelArgs a{};
   a.table = reinterpret_cast<const uint32_t*>(base + h->ws_off_table);
   a.blob = reinterpret_cast<const uint32_t*>(base + h->ws_off_blob);
@@ -1607,68 +1712,96 @@ gx_status gx_training_set(gx_net* h, void* ws, uint64_t ws_bytes, void* stream, 
   GG_CUDA(cudaGetDevice(&dev));
   GG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int grid = sms * 8;
-  // temporary memory: the control block, the lists (28 bytes a state) and, after a complete
-  // search with at most 2^28 transitions, every state's successors (4 bytes each); the sort's
-  // buffers (20 bytes an example, a power of two of them) take their place afterwards
-  const uint64_t most = std::min<uint64_t>(states, cap);
-  uint64_t n2 = 1;
-  while (n2 < most) n2 <<= 1;
-  a.adj_cap = S.complete && S.transitions <= (1ull << 28) ? S.transitions : 0;
-  struct Temp {
-    unsigned char* p = nullptr;
-    cudaStream_t st;
-    ~Temp() {
-      if (p) cudaFreeAsync(p, st);
-    }
-  } temp{nullptr, st};
+  const size_t smem = 4ull * a.staged_words;
+  gx::TempMem temp{st};
+  uint64_t n = 0, bad = 0;  // states found
+  // With lists: temporary memory for the control block, the lists (28 bytes a state) and, after
+  // a complete search with at most 2^28 transitions, every state's successors (4 bytes each).
+  // Less when there is no room, and no lists at all when there is none for them either.
   const uint64_t lists = gx::a256(sizeof(gxd::LabelCtl));
-  auto bytes = [&] { return lists + std::max<uint64_t>(28 * states + 4 * a.adj_cap, 20 * n2); };
-  if (cudaMallocAsync(reinterpret_cast<void**>(&temp.p), bytes(), st) != cudaSuccess) {
-    cudaGetLastError();
-    temp.p = nullptr;
-    a.adj_cap = 0;  // look the successors up in every round
-    GG_CUDA(cudaMallocAsync(reinterpret_cast<void**>(&temp.p), bytes(), st));
-  }
-  a.ctl = reinterpret_cast<gxd::LabelCtl*>(temp.p);
-  a.slot_of = reinterpret_cast<unsigned long long*>(temp.p + lists);
-  a.d = reinterpret_cast<uint32_t*>(a.slot_of + states);
-  a.first = a.d + states;
-  a.last = a.first + states;
-  a.todo[0] = a.last + states;
-  a.todo[1] = a.todo[0] + states;
-  a.adj = a.todo[1] + states;
-  GG_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(gxd::LabelCtl), st));
-  k.label_collect<<<grid, gx::kBlock, 0, st>>>(a);
-  if (a.adj_cap) k.label_adj<<<grid, gx::kBlock, 4ull * a.staged_words, st>>>(a);
-  GG_CUDA(cudaGetLastError());
-  gxd::LabelCtl hc{};
-  constexpr uint32_t kAhead = 16;  // rounds launched before the host looks whether any is needed
-  for (uint32_t r = 1; r <= max_dist; ++r) {
-    if (a.adj_cap) gxd::label_round_kernel<<<grid, gx::kBlock, 0, st>>>(a, r);
-    else k.label_lookup_round<<<grid, gx::kBlock, 4ull * a.staged_words, st>>>(a, r);
-    GG_CUDA(cudaGetLastError());
-    if (r % kAhead == 0 && r < max_dist) {
-      GG_CUDA(cudaMemcpyAsync(&hc, a.ctl, sizeof(hc), cudaMemcpyDeviceToHost, st));
-      GG_CUDA(cudaStreamSynchronize(st));
-      if (hc.states > states || hc.left[r & 3] == 0 || hc.left[r & 3] == hc.left[(r - 1) & 3]) break;
+  if (states < (1ull << 32)) {
+    a.adj_cap = S.complete && S.transitions <= (1ull << 28) ? S.transitions : 0;
+    if (!temp.alloc(lists + 28 * states + 4 * a.adj_cap) && a.adj_cap) {
+      a.adj_cap = 0;  // look the successors up in every round
+      temp.alloc(lists + 28 * states);
     }
   }
-  k.label_gather<<<grid, gx::kBlock, 0, st>>>(a, max_dist, hist_out, label_out, cap);
-  GG_CUDA(cudaGetLastError());
-  GG_CUDA(cudaMemcpyAsync(&hc, a.ctl, sizeof(hc), cudaMemcpyDeviceToHost, st));
-  GG_CUDA(cudaStreamSynchronize(st));
-  if (hc.states != states || (a.adj_cap && hc.edges > a.adj_cap))
-    return gx::fail(GX_ERR_STATE, "the workspace does not hold the last search's table");
-  if (n_out) *n_out = states;
-  if (hc.bad) return gx::fail(GX_ERR_INVALID, "a process has a local state index of 16 or more");
-  // content order (see ex_greater)
-  if (most > 1) {
-    uint4* sh = reinterpret_cast<uint4*>(temp.p + lists);
+  bool listed = temp.p != nullptr;
+  if (listed) {
+    a.ctl = reinterpret_cast<gxd::LabelCtl*>(temp.p);
+    a.slot_of = reinterpret_cast<unsigned long long*>(temp.p + lists);
+    a.d = reinterpret_cast<uint32_t*>(a.slot_of + states);
+    a.first = a.d + states;
+    a.last = a.first + states;
+    a.todo[0] = a.last + states;
+    a.todo[1] = a.todo[0] + states;
+    a.adj = a.todo[1] + states;
+    GG_CUDA(cudaMemsetAsync(a.ctl, 0, sizeof(gxd::LabelCtl), st));
+    k.label_collect<<<grid, gx::kBlock, 0, st>>>(a);
+    if (a.adj_cap) k.label_adj<<<grid, gx::kBlock, smem, st>>>(a);
+    GG_CUDA(cudaGetLastError());
+    gxd::LabelCtl hc{};
+    constexpr uint32_t kAhead = 16;  // rounds launched before the host looks whether any is needed
+    for (uint32_t r = 1; r <= max_dist; ++r) {
+      if (a.adj_cap) gxd::label_round_kernel<<<grid, gx::kBlock, 0, st>>>(a, r);
+      else k.label_lookup_round<<<grid, gx::kBlock, smem, st>>>(a, r);
+      GG_CUDA(cudaGetLastError());
+      if (r % kAhead == 0 && r < max_dist) {
+        GG_CUDA(cudaMemcpyAsync(&hc, a.ctl, sizeof(hc), cudaMemcpyDeviceToHost, st));
+        GG_CUDA(cudaStreamSynchronize(st));
+        if (hc.states > states || (a.adj_cap && hc.edges > a.adj_cap) || hc.left[r & 3] == 0 ||
+            hc.left[r & 3] == hc.left[(r - 1) & 3])
+          break;
+      }
+    }
+    k.label_gather<<<grid, gx::kBlock, 0, st>>>(a, max_dist, hist_out, label_out, cap);
+    GG_CUDA(cudaGetLastError());
+    GG_CUDA(cudaMemcpyAsync(&hc, a.ctl, sizeof(hc), cudaMemcpyDeviceToHost, st));
+    GG_CUDA(cudaStreamSynchronize(st));
+    n = hc.states;
+    bad = hc.bad;
+    // (a table that was written to since the search: its states and successors are not held)
+    if (hc.states > states || (a.adj_cap && hc.edges > a.adj_cap)) listed = false;
+  }
+  if (!listed) {
+    temp.release();
+    unsigned long long* flags = reinterpret_cast<gx::Ctl*>(base + h->ws_off_ctl)->digest;
+    k.slot_init<<<grid, gx::kBlock, 0, st>>>(a);
+    GG_CUDA(cudaGetLastError());
+    for (uint32_t r = 1; r <= max_dist; ++r) {
+      unsigned long long changed = 0;
+      GG_CUDA(cudaMemsetAsync(flags, 0, sizeof(changed), st));
+      k.slot_round<<<grid, gx::kBlock, smem, st>>>(a, r, flags);
+      GG_CUDA(cudaGetLastError());
+      GG_CUDA(cudaMemcpyAsync(&changed, flags, sizeof(changed), cudaMemcpyDeviceToHost, st));
+      GG_CUDA(cudaStreamSynchronize(st));
+      if (!changed) break;
+    }
+    unsigned long long res[2] = {0, 0};
+    GG_CUDA(cudaMemsetAsync(flags, 0, sizeof(res), st));
+    k.slot_gather<<<grid, gx::kBlock, 0, st>>>(a, max_dist, hist_out, label_out, cap, flags);
+    GG_CUDA(cudaGetLastError());
+    GG_CUDA(cudaMemcpyAsync(res, flags, sizeof(res), cudaMemcpyDeviceToHost, st));
+    GG_CUDA(cudaStreamSynchronize(st));
+    n = res[0];
+    bad = res[1];
+  }
+  if (n_out) *n_out = n;
+  if (bad) return gx::fail(GX_ERR_INVALID, "a process has a local state index of 16 or more");
+  // content order (see ex_greater): buffers of 20 bytes an example, a power of two of them
+  const uint64_t m = std::min<uint64_t>(n, cap);
+  if (m > 1) {
+    uint64_t n2 = 1;
+    while (n2 < m) n2 <<= 1;
+    if (temp.bytes < 20 * n2) {
+      temp.release();
+      if (!temp.alloc(20 * n2)) return gx::fail(GX_ERR_CUDA, "no device memory to sort the examples in");
+    }
+    uint4* sh = reinterpret_cast<uint4*>(temp.p);
     uint32_t* sl = reinterpret_cast<uint32_t*>(sh + n2);
     const int tiles = (int)std::max<uint64_t>(1, n2 / gxd::kTile);
     const uint64_t first = std::min<uint64_t>(n2, gxd::kTile);
-    gxd::ex_tile_kernel<<<tiles, gxd::kTileThreads, gxd::kTileBytes, st>>>(sh, sl, n2, 2, first, 1, hist_out, label_out,
-                                                                         most);
+    gxd::ex_tile_kernel<<<tiles, gxd::kTileThreads, gxd::kTileBytes, st>>>(sh, sl, n2, 2, first, 1, hist_out, label_out, m);
     for (uint64_t k2 = 2 * first; k2 <= n2; k2 <<= 1) {
       uint64_t j = k2 >> 1;
       while (j >= (uint64_t)gxd::kTile) {
@@ -1678,7 +1811,7 @@ gx_status gx_training_set(gx_net* h, void* ws, uint64_t ws_bytes, void* stream, 
       }
       gxd::ex_tile_kernel<<<tiles, gxd::kTileThreads, gxd::kTileBytes, st>>>(sh, sl, n2, k2, k2, 0, nullptr, nullptr, 0);
     }
-    gxd::ex_store_kernel<<<grid, 256, 0, st>>>(sh, sl, most, hist_out, label_out);
+    gxd::ex_store_kernel<<<grid, 256, 0, st>>>(sh, sl, m, hist_out, label_out);
     GG_CUDA(cudaGetLastError());
     GG_CUDA(cudaStreamSynchronize(st));
   }

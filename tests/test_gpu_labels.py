@@ -112,3 +112,130 @@ def test_examples_at_odd_addresses(cuda, cap, offset):
     if cap >= s["states"]:
         want_hist, want_label = gx.training_set(h, ws, 16)
         assert (want_hist.cpu().numpy() == hist).all() and torch.equal(want_label, label)
+
+
+def _examples(h, ws, max_dist, cap):
+    """gx_training_set with room for cap examples: (states found, histograms, labels)."""
+    import torch
+    dist = torch.empty(gx.stats(h)["table_slots"], dtype=torch.int32, device="cuda")
+    hist = torch.zeros((max(cap, 1), 16), dtype=torch.uint8, device="cuda")
+    label = torch.zeros(max(cap, 1), dtype=torch.float32, device="cuda")
+    n = ctypes.c_uint64()
+    gx._check(gx.lib().gx_training_set(h.handle, ws.data_ptr(), ws.numel(), None, dist.data_ptr(), max_dist,
+                                       hist.data_ptr() if cap else None, label.data_ptr() if cap else None, cap,
+                                       ctypes.byref(n)))
+    k = min(n.value, cap)
+    return n.value, hist[:k].cpu().numpy().astype(np.int64), label[:k].cpu().numpy()
+
+
+@pytest.mark.parametrize("change", ["fewer", "more"])
+@pytest.mark.parametrize("max_levels", [0, 5])
+def test_labels_of_the_table_as_it_is_now(cuda, max_levels, change):
+    """The examples are those of the states the workspace's table holds at the call: a third of
+    them taken out, or states put in that the search had not found, each in its own bucket."""
+    import torch
+    net = inputs.planted_network(1, 4, n_traps=2)
+    h = gx.load_network(net)
+    o = gx.default_opts(table_bytes=1 << 22, hash_rounds=32, max_levels=max_levels, bucket_words=8, group_lanes=1,
+                        global_cache_log2=0)
+    ws = gx.alloc_workspace(h, o)
+    gx.explore(h, o, ws)
+    s = gx.stats(h)
+    assert s["slot_words"] == 1
+    table = ws[ws.numel() - 4 * s["table_slots"]:].view(torch.int32)  # the last part of the workspace
+    at = torch.nonzero(table).flatten()
+    assert len(at) == s["states"]
+    if change == "fewer":
+        # (whole buckets' first slots only when nothing is behind them: a lookup ends at an empty slot)
+        first = at[(at % 8 == 0) & (table[(at // 8) * 8 + 1] == 0)]
+        table[first[::3]] = 0
+    else:
+        lay = gx.layout(h)
+        top = int(lay["field_bits"].sum())
+        have = set((table[at].cpu().numpy().astype(np.int64) & 0x7FFFFFFF).tolist())
+        new = [v for v in range(1 << top) if v not in have][::7][:50]
+        empty = torch.nonzero(table.view(-1, 8)[:, 0] == 0).flatten()[:len(new)]
+        table[empty * 8] = torch.tensor([v - (1 << 31) for v in new], dtype=torch.int32, device="cuda")
+    now = table[torch.nonzero(table).flatten()].cpu().numpy().astype(np.int64) & 0x7FFFFFFF
+    lay = gx.layout(h)
+    states = [tuple(int(v >> int(sh)) & ((1 << int(b)) - 1) for sh, b in zip(lay["field_offset"], lay["field_bits"]))
+              for v in now]
+    n, hist, label = _examples(h, ws, 8, len(states))
+    assert n == len(states)
+    if change == "more":  # put in at buckets of no meaning: no lookup finds them, and each is an example
+        found = {tuple(int(v >> int(sh)) & ((1 << int(b)) - 1) for sh, b in zip(lay["field_offset"], lay["field_bits"]))
+                 for v in have}
+    else:
+        found = set(states)
+    succ = {x: [tuple(t) for t in oracle.successors(net, np.array(x, dtype=np.uint32))] for x in states}
+    dist = {x: 0 for x in states if not succ[x]}
+    for r in range(1, 9):
+        near = [x for x in states if x not in dist and any(t in found and dist.get(t) == r - 1 for t in succ[x])]
+        dist.update((x, r) for x in near)
+    want = _rows(np.array([np.bincount(x, minlength=16) for x in states]),
+                 [min(dist.get(x, 8), 8) / 8 for x in states], 8)
+    assert _rows(hist, label, 8) == want
+
+
+class _PoolProps(ctypes.Structure):  # CUmemPoolProps
+    _fields_ = [("alloc_type", ctypes.c_int), ("handle_types", ctypes.c_int), ("loc_type", ctypes.c_int),
+                ("loc_id", ctypes.c_int), ("security", ctypes.c_void_p), ("max_size", ctypes.c_size_t),
+                ("usage", ctypes.c_ushort), ("reserved", ctypes.c_ubyte * 54)]
+
+
+@pytest.mark.parametrize("n_procs", [10, 11])
+def test_labels_without_room_for_lists(cuda, n_procs):
+    """A device memory pool of 32 MiB: it holds the lists of 1,080,000 states without their
+    successors, and no lists of 5,400,000 states.  The call goes without them, counts with
+    no memory at all, and writes examples of the same states."""
+    import torch
+    net = inputs.planted_network(1, n_procs, n_traps=2)
+    h = gx.load_network(net)
+    o = gx.default_opts(table_bytes=1 << 26, hash_rounds=32)
+    ws = gx.alloc_workspace(h, o)
+    gx.explore(h, o, ws)
+    states = gx.stats(h)["states"]
+    too_much = 28 * states + (4 * gx.stats(h)["transitions"] if n_procs == 10 else 0)
+    assert too_much > 2 * (32 << 20)
+    n, hist, label = _examples(h, ws, 64, states)
+    rows = lambda x, y: set(map(tuple, np.concatenate([x, np.rint(y * 64).astype(np.int64)[:, None]], 1).tolist()))
+    want = rows(hist, label)
+    cu = ctypes.CDLL("libcuda.so.1")
+    default, small = ctypes.c_void_p(), ctypes.c_void_p()
+    props = _PoolProps(alloc_type=1, loc_type=1, loc_id=torch.cuda.current_device(), max_size=32 << 20)
+    assert cu.cuDeviceGetMemPool(ctypes.byref(default), torch.cuda.current_device()) == 0
+    assert cu.cuMemPoolCreate(ctypes.byref(small), ctypes.byref(props)) == 0
+    try:
+        assert cu.cuDeviceSetMemPool(torch.cuda.current_device(), small) == 0
+        p = ctypes.c_uint64()
+        if cu.cuMemAllocFromPoolAsync(ctypes.byref(p), ctypes.c_size_t(too_much), small, None) == 0:
+            cu.cuMemFreeAsync(p, None)
+            pytest.skip("the driver does not hold the pool to its limit")
+        assert _examples(h, ws, 64, 0)[0] == states
+        n, hist, label = _examples(h, ws, 64, 1000)
+        assert n == states and len(hist) == 1000
+        assert rows(hist, label) <= want
+    finally:
+        assert cu.cuDeviceSetMemPool(torch.cuda.current_device(), default) == 0
+        torch.cuda.synchronize()
+        cu.cuMemPoolDestroy(small)
+
+
+def test_labels_of_more_than_2_32_states(cuda):
+    """The 5.37e9-state network in its 128 GiB table: counted and labelled without lists (their
+    indexes have 32 bits).  No state of it is a deadlock, so every label is 1."""
+    import torch
+    free, _ = torch.cuda.mem_get_info()
+    if free < (210 << 30):
+        pytest.skip("needs 210 GiB of free device memory")
+    h = gx.load_network(inputs.workload("scaled"))
+    o = gx.default_opts(table_bytes=4 << 35, bucket_words=8, group_lanes=1, hash_rounds=64)
+    ws = gx.alloc_workspace(h, o)
+    gx.explore(h, o, ws)
+    s = gx.stats(h)
+    assert s["states"] >= 1 << 32 and s["deadlock_count"] == 0
+    n, hist, label = _examples(h, ws, 1, 4097)
+    del ws
+    torch.cuda.empty_cache()
+    assert n == s["states"]
+    assert (hist.sum(1) == 16).all() and (label == 1.0).all()
