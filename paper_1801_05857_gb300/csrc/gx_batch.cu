@@ -98,8 +98,8 @@ __global__ void __launch_bounds__(gx::kBlock) batch_init_kernel(const BatchArgs 
 }
 
 // Network i has finished the level it was expanding: record the next one and
-// open it, or finish the network.  One lane, after the level's last claim.
-__device__ __forceinline__ void batch_next_level(const BatchArgs& a, int i) {
+// open it, or finish the network (false).  One lane, after the level's last claim.
+__device__ __forceinline__ bool batch_next_level(const BatchArgs& a, int i) {
   BNet& b = a.nets[i];
   using gx::kFinished;
   const unsigned long long end = __ldcg(&b.cur_end), next = __ldcg(&b.next_end), fresh = next - end;
@@ -119,7 +119,7 @@ __device__ __forceinline__ void batch_next_level(const BatchArgs& a, int i) {
     atomicSub(a.active, 1u);
     __threadfence();
     atomicExch(a.claims + i, gx::kFinished);
-    return;
+    return false;
   }
   // a network's share of the warps, were all networks at work: a level that gives each
   // of them less than a full claim is taken in smaller ones
@@ -136,14 +136,31 @@ __device__ __forceinline__ void batch_next_level(const BatchArgs& a, int i) {
   b.done = 0;
   __threadfence();
   atomicExch(a.claims + i, chunks << 32);
+  return true;
 }
 
-// A claim of any network that has one left.  False: all networks are finished (or
-// nothing was to be had for kGiveUpNs, which is reported).  base: the networks below
-// it are finished.  A warp begins the search at a place of its own, so that the
-// networks are worked on side by side: the claims words, queue ends and table lines
-// of one network take only so many accesses at a time (256 networks: 9.2 ms; all
-// warps on the first open network 12.8, on the first 8 of them 11.2, on 32 10.6).
+// A claim of any network that has one left, of network `first` before others if that is
+// one (the warp has just opened its next level).  False: all networks are finished (or
+// nothing was to be had for kGiveUpNs, which is reported).
+// A warp begins the search at a place of its own, so that the networks are worked on side by
+// side: the claims words, queue ends and table lines of one network take only so many
+// accesses at a time (256 networks: 9.2 ms; all warps on the first open network 12.8, on the
+// first 8 of them 11.2, on 32 10.6).
+// For the same reason warps that find nothing must not crowd the words of those that work:
+// they look at kLook groups of 32 networks, then pause, twice as long each time (from 128 ns
+// to 2 us for each of up to 8 unfinished networks), and a claim they got halves the pause.
+// Without that -- all groups, pauses of 2 us at most, none after a claim taken by others --
+// 32 networks of 640 states took 1.35 ms instead of 0.40, 32 of 118,098 5.3 instead of 2.15,
+// 256 of the workload 8.5 instead of 8.3.  (Pauses up to 8, 16, 32 us for any number of
+// networks: one network 1.6, 1.8, 2.0 ms instead of 1.39; looking at 1, 4 or 8 groups: the
+// same within 5 %.)
+struct Search {
+  int base;        // networks below it are finished
+  uint32_t place;  // the group of 32 networks to look at next
+  uint32_t nap;    // ns
+};
+constexpr int kLook = 2;
+constexpr uint32_t kShortNap = 128, kLongNap = 2048;
 constexpr unsigned long long kGiveUpNs = 20ull * 1000 * 1000 * 1000;
 
 __device__ __forceinline__ unsigned long long batch_now() {
@@ -152,25 +169,26 @@ __device__ __forceinline__ unsigned long long batch_now() {
   return t;
 }
 
-__device__ __forceinline__ bool batch_claim(const BatchArgs& a, uint32_t warp, int& base, int& net, uint32_t& c) {
+__device__ __forceinline__ bool batch_claim(const BatchArgs& a, uint32_t warp, Search& at, int first, int& net,
+                                            uint32_t& c) {
   const int lane = threadIdx.x & 31;
   unsigned long long since = 0;
-  uint32_t nap = 128;
   while (true) {
-    int found = -1;
-    const int span = (a.n - base + 31) / 32;
-    for (int k = 0; k < span; ++k) {
-      const int w0 = base + 32 * (int)((k + warp / 32) % span);
+    int found = first;
+    first = -1;
+    const int span = (a.n - at.base + 31) / 32;
+    int look = kLook;
+    for (int k = 0; found < 0 && look > 0 && k < span; ++k) {
+      const int w0 = at.base + 32 * (int)(at.place++ % span);
       const unsigned long long x = w0 + lane < a.n ? __ldcg(a.claims + w0 + lane) : gx::kFinished;
-      const bool fin = (x >> 32) == 0;
-      if (__ballot_sync(FULLMASK, fin) == FULLMASK) {
-        if (w0 == base) base += 32;
-        continue;
+      if (__all_sync(FULLMASK, (x >> 32) == 0)) {
+        if (w0 != at.base) continue;
+        at.base += 32;
+        break;
       }
+      --look;
       const uint32_t open = __ballot_sync(FULLMASK, (uint32_t)x < (uint32_t)(x >> 32));
-      if (open == 0) continue;
-      found = w0 + (int)__fns(open, 0, warp % __popc(open) + 1);
-      break;
+      if (open) found = w0 + (int)__fns(open, 0, warp % __popc(open) + 1);
     }
     if (found >= 0) {
       unsigned long long x = 0;
@@ -179,20 +197,22 @@ __device__ __forceinline__ bool batch_claim(const BatchArgs& a, uint32_t warp, i
       if ((uint32_t)x < (uint32_t)(x >> 32)) {
         net = found;
         c = (uint32_t)x;
+        at.place = warp / 32;
+        at.nap = at.nap > 2 * kShortNap ? at.nap / 2 : kShortNap;
         return true;
       }
-      continue;  // taken by others
     }
-    if (base >= a.n) return false;
+    const uint32_t active = __shfl_sync(FULLMASK, __ldcg(a.active), 0);
+    if (active == 0 || at.base >= a.n) return false;
     const unsigned long long now = __shfl_sync(FULLMASK, batch_now(), 0);
     if (since == 0) since = now;
     if (now - since > kGiveUpNs) {
-      for (int i = base + lane; i < a.n; i += 32)
+      for (int i = at.base + lane; i < a.n; i += 32)
         if ((__ldcg(a.claims + i) >> 32) != 0) atomicOr(&a.nets[i].error, gx::ERR_SPIN);
       return false;
     }
-    __nanosleep(nap);
-    if (nap < 2048) nap *= 2;
+    __nanosleep(at.nap);
+    if (at.nap < kLongNap * (active < 8 ? active : 8)) at.nap *= 2;
   }
 }
 
@@ -268,11 +288,13 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
   WarpCache cache{W <= 2 ? S.cache[wid] : nullptr, (1u << kBatchCacheLog2) - 1u, nullptr};
   const SmemTarget tg{&wn, a.rounds};
   const uint32_t* t = nullptr;
-  int net = -1, base = 0;
+  const uint32_t warp = blockIdx.x * (gx::kBlock / 32) + wid;
+  Search at{0, warp / 32, kShortNap};
+  int net = -1, first = -1;
   while (true) {
     int at_net;
     uint32_t c;
-    if (!batch_claim(a, blockIdx.x * (gx::kBlock / 32) + wid, base, at_net, c)) break;
+    if (!batch_claim(a, warp, at, first, at_net, c)) break;
     BNet& b = a.nets[at_net];
     if (at_net != net) {
       // stage the network; the cache holds one network's vectors at a time
@@ -309,7 +331,7 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
     expand_states<W, B, G, 32>(
         tg, muls, t, L, S.queues[wid], st, probes, err,
         ClassDescs{descs, L.n_classes < 32u ? L.n_classes : 32u},
-        [&](uint64_t& at, uint32_t& m) {
+        [&](uint64_t& from, uint32_t& m) {
           m = 0;
           if (pos == end) {
             if (!held) {
@@ -325,7 +347,7 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
             end = pos + wn.unit < wn.cur_end ? pos + wn.unit : wn.cur_end;
             held = false;
           }
-          at = pos;
+          from = pos;
           m = end - pos < 32 ? (uint32_t)(end - pos) : 32u;
           pos += m;
         },
@@ -355,11 +377,12 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
     // (the warp's last use of the level: its states, counts and new states come before)
     __threadfence();  // before the level can be seen as done
     __syncwarp();
+    bool opened = false;
     if (lane == 0 && atomicAdd(&b.done, taken) + taken == wn.chunks) {
       __threadfence();
-      batch_next_level(a, net);
+      opened = batch_next_level(a, net);
     }
-    __syncwarp();
+    first = __any_sync(FULLMASK, opened) ? net : -1;
   }
 }
 

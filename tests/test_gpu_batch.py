@@ -102,3 +102,20 @@ def test_batched_workload_against_stored_oracle(cuda):
         assert gx.batch_levels(b, i) == x["levels"], i
         assert (s["deadlock_count"], s["deadlock_sum"], s["deadlock_xor"]) == (
             x["deadlock_count"], x["deadlock_sum"], x["deadlock_xor"]), i
+
+
+@pytest.mark.parametrize("count", [1, 31, 32, 33, 64, 65, 300])
+def test_every_number_of_networks(cuda, count):
+    """Networks are looked for in groups of 32, of which the first are skipped once finished:
+    counts at the edges of groups, with the deep networks first, last and spread (tables
+    decide the order), so that groups finish in any order."""
+    kinds = [inputs.producer_consumers(), inputs.token_ring(6), inputs.workload("tiny"), inputs.token_ring(4)]
+    want = [oracle.explore(n) for n in kinds]
+    which = [(i * i + i // 3) % 4 for i in range(count)]
+    slots = [2 * want[k].states << (i % 3) for i, k in enumerate(which)]
+    b = gx.batch_create([kinds[k] for k in which])
+    o = gx.batch_opts(hash_rounds=32, expected_states=slots)
+    ws = gx.batch_alloc_workspace(b, o)
+    gx.batch_explore(b, o, ws)
+    for i, k in enumerate(which):
+        _check_net(b, i, want[k])
