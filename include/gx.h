@@ -474,6 +474,12 @@ gx_status gx_batch_create(const gx_net* const* nets, uint32_t n, gx_batch** out)
 /* Free a batch (NULL is a no-op); the workspace belongs to the caller. */
 void gx_batch_free(gx_batch* batch);
 
+/* Longest time in ns that a warp of a later gx_batch_explore waits for work while no
+ * level of any network ends (0 = the default, 20 s).  A warp that has waited so long
+ * leaves and the others finish the batch; a network that is left unfinished all the
+ * same is reported as GX_ERR_SPIN_LIMIT.  Host-only. */
+gx_status gx_batch_set_wait_limit(gx_batch* batch, uint64_t ns);
+
 /* Device workspace bytes for gx_batch_explore with these options. */
 gx_status gx_batch_workspace_bytes(const gx_batch* batch, const gx_batch_opts* opts, uint64_t* bytes);
 

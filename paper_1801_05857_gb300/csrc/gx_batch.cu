@@ -50,7 +50,8 @@ struct BatchArgs {
   // per network: claims taken of its level, and in the upper half how many it has
   // (0: finished, and then at least kFinished are taken)
   unsigned long long* claims;
-  unsigned int* active;       // networks that are not finished
+  unsigned int* active;       // [0] networks that are not finished, [1] levels that ended
+  unsigned long long give_up_ns;  // a warp's longest wait without either changing
   uint32_t warps;             // of the expansion's grid
   uint32_t wide;              // a level with at most this many states per warp that falls to
                               // its network is claimed state by state
@@ -58,6 +59,7 @@ struct BatchArgs {
 };
 
 constexpr unsigned long long kFinished = 0x80000000ull;
+constexpr uint64_t kGiveUpNs = 20ull * 1000 * 1000 * 1000;  // (gx_batch_set_wait_limit)
 constexpr unsigned int ERR_LEVELS = 8u;  // a network needed more levels than levels_cap
 
 }  // namespace gx
@@ -102,6 +104,7 @@ __global__ void __launch_bounds__(gx::kBlock) batch_init_kernel(const BatchArgs 
 __device__ __forceinline__ bool batch_next_level(const BatchArgs& a, int i) {
   BNet& b = a.nets[i];
   using gx::kFinished;
+  atomicAdd(a.active + 1, 1u);
   const unsigned long long end = __ldcg(&b.cur_end), next = __ldcg(&b.next_end), fresh = next - end;
   unsigned int err = __ldcg(&b.error), levels = __ldcg(&b.n_levels);
   if (__ldcg(&b.first_dl) < 0 && __ldcg(&b.dl_count) > 0) b.first_dl = (int)levels - 1;
@@ -140,8 +143,11 @@ __device__ __forceinline__ bool batch_next_level(const BatchArgs& a, int i) {
 }
 
 // A claim of any network that has one left, of network `first` before others if that is
-// one (the warp has just opened its next level).  False: all networks are finished (or
-// nothing was to be had for kGiveUpNs, which is reported).
+// one (the warp has just opened its next level).  False: all networks are finished, or this
+// warp has waited give_up_ns in which no level ended and no claim was taken before its eyes.
+// That is no error: the claims being worked on (a claim may hold up to 2^32 successors a
+// state) are finished by their warps, and the one that ends a level goes on with the next.
+// The host reports a network that was left unfinished, which only a lost claim can cause.
 // A warp begins the search at a place of its own, so that the networks are worked on side by
 // side: the claims words, queue ends and table lines of one network take only so many
 // accesses at a time (256 networks: 9.2 ms; all warps on the first open network 12.8, on the
@@ -161,8 +167,6 @@ struct Search {
 };
 constexpr int kLook = 2;
 constexpr uint32_t kShortNap = 128, kLongNap = 2048;
-constexpr unsigned long long kGiveUpNs = 20ull * 1000 * 1000 * 1000;
-
 __device__ __forceinline__ unsigned long long batch_now() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
@@ -173,6 +177,7 @@ __device__ __forceinline__ bool batch_claim(const BatchArgs& a, uint32_t warp, S
                                             uint32_t& c) {
   const int lane = threadIdx.x & 31;
   unsigned long long since = 0;
+  uint32_t ended = 0;  // levels, at the last look
   while (true) {
     int found = first;
     first = -1;
@@ -201,16 +206,17 @@ __device__ __forceinline__ bool batch_claim(const BatchArgs& a, uint32_t warp, S
         at.nap = at.nap > 2 * kShortNap ? at.nap / 2 : kShortNap;
         return true;
       }
+      since = 0;  // taken by others
     }
-    const uint32_t active = __shfl_sync(FULLMASK, __ldcg(a.active), 0);
+    const unsigned long long state = __shfl_sync(FULLMASK, __ldcg(reinterpret_cast<const unsigned long long*>(a.active)), 0);
+    const uint32_t active = (uint32_t)state;
     if (active == 0 || at.base >= a.n) return false;
     const unsigned long long now = __shfl_sync(FULLMASK, batch_now(), 0);
-    if (since == 0) since = now;
-    if (now - since > kGiveUpNs) {
-      for (int i = at.base + lane; i < a.n; i += 32)
-        if ((__ldcg(a.claims + i) >> 32) != 0) atomicOr(&a.nets[i].error, gx::ERR_SPIN);
-      return false;
+    if (since == 0 || ended != (uint32_t)(state >> 32)) {
+      since = now;
+      ended = (uint32_t)(state >> 32);
     }
+    if (now - since > a.give_up_ns) return false;
     __nanosleep(at.nap);
     if (at.nap < kLongNap * (active < 8 ? active : 8)) at.nap *= 2;
   }
@@ -454,6 +460,7 @@ struct gx_batch {
   std::vector<std::vector<uint64_t>> levels;
   double gpu_ms = 0;
   std::vector<uint64_t> last_plan_slots;
+  uint64_t give_up_ns = gx::kGiveUpNs;
   uint32_t last_W = 0, last_B = 0, last_G = 0, last_rounds = 0;
 };
 
@@ -575,6 +582,7 @@ gx_status run_batch(gx_batch* h, const gx_batch_opts* o, void* ws, uint64_t ws_b
   a.levels = reinterpret_cast<unsigned long long*>(base + P.off_levels);
   a.claims = reinterpret_cast<unsigned long long*>(base + P.off_claims);
   a.active = reinterpret_cast<unsigned int*>(base + P.off_active);
+  a.give_up_ns = h->give_up_ns;
   a.warps = (uint32_t)grid * (kBlock / 32);
   a.wide = P.wide == GX_BATCH_WIDE_OFF ? 0u : P.wide;
   hash_multipliers(a.muls.m, kMaxRounds);
@@ -609,6 +617,7 @@ gx_status run_batch(gx_batch* h, const gx_batch_opts* o, void* ws, uint64_t ws_b
   for (int k = 0; k < n; ++k) slot[P.order[k]] = (uint32_t)k;
   for (int i = 0; i < n; ++i) {
     h->res[i] = bn[slot[i]];
+    if (h->res[i].active && !h->res[i].error) h->res[i].error = ERR_SPIN;  // its warps gave up waiting
     const uint32_t k = std::min<uint32_t>(h->res[i].n_levels, P.levels_cap);
     h->levels[i].resize(k);
     for (uint32_t l = 0; l < k; ++l) h->levels[i][l] = lv[(uint64_t)l * n + slot[i]];
@@ -617,7 +626,7 @@ gx_status run_batch(gx_batch* h, const gx_batch_opts* o, void* ws, uint64_t ws_b
       rs = (e & ERR_TABLE_FULL)  ? fail(GX_ERR_TABLE_FULL, "network " + std::to_string(i) + ": hash table full")
          : (e & ERR_FRONTIER)    ? fail(GX_ERR_FRONTIER_OVERFLOW, "network " + std::to_string(i) + ": frontier overflow")
          : (e & ERR_LEVELS)      ? fail(GX_ERR_OOM, "network " + std::to_string(i) + ": more levels than levels_cap")
-                                 : fail(GX_ERR_SPIN_LIMIT, "network " + std::to_string(i) + ": device wait gave up");
+                                 : fail(GX_ERR_SPIN_LIMIT, "network " + std::to_string(i) + ": left unfinished after waits that gave up");
     }
   }
   h->have_result = true;
@@ -651,6 +660,13 @@ gx_status gx_batch_create(const gx_net* const* nets, uint32_t n, gx_batch** out)
 }
 
 void gx_batch_free(gx_batch* b) { delete b; }
+
+gx_status gx_batch_set_wait_limit(gx_batch* b, uint64_t ns) {
+  gx::clear_error();
+  if (!b) return gx::fail(GX_ERR_INVALID, "batch is NULL");
+  b->give_up_ns = ns ? ns : gx::kGiveUpNs;
+  return GX_OK;
+}
 
 gx_status gx_batch_workspace_bytes(const gx_batch* b, const gx_batch_opts* opts, uint64_t* bytes) {
   gx::clear_error();

@@ -161,6 +161,7 @@ def lib(build_if_missing: bool = True) -> ctypes.CDLL:
         "gx_batch_create": ([P(vp), u32, P(vp)], ctypes.c_int),
         "gx_batch_free": ([vp], None),
         "gx_batch_workspace_bytes": ([vp, P(gx_batch_opts), P(u64)], ctypes.c_int),
+        "gx_batch_set_wait_limit": ([vp, u64], ctypes.c_int),
         "gx_batch_explore": ([vp, P(gx_batch_opts), vp, u64, vp], ctypes.c_int),
         "gx_batch_stats": ([vp, u32, P(gx_stats_t)], ctypes.c_int),
         "gx_batch_levels": ([vp, u32, P(u64), u32, P(u32)], ctypes.c_int),
@@ -509,6 +510,10 @@ def batch_create(nets) -> Batch:
     h = ctypes.c_void_p()
     _check(lib().gx_batch_create(arr, len(handles), ctypes.byref(h)))
     return Batch(h.value, len(handles))
+
+
+def batch_set_wait_limit(b: Batch, ns: int) -> None:
+    _check(lib().gx_batch_set_wait_limit(b.handle, ns))
 
 
 def batch_opts(expected_states=None, **kw) -> gx_batch_opts:

@@ -119,3 +119,22 @@ def test_every_number_of_networks(cuda, count):
     gx.batch_explore(b, o, ws)
     for i, k in enumerate(which):
         _check_net(b, i, want[k])
+
+
+@pytest.mark.parametrize("limit_us", [1, 200, 0])
+def test_warps_that_wait_long_fail_no_batch(cuda, limit_us):
+    """A network of 20,000 levels of one state keeps one warp busy for some 100 ms while the
+    others wait.  Whatever the limit of a wait (0: the default), the batch is explored to the
+    end: a waiting warp may leave, but levels that end are progress and no error."""
+    n = 20000
+    chain = inputs.Network(1, [inputs.LTS(n, 0, [(i, 0, i + 1) for i in range(n - 1)])], [])
+    kinds = [chain, inputs.token_ring(6), inputs.workload("tiny")]
+    want = [oracle.explore(k) for k in kinds]
+    b = gx.batch_create(kinds)
+    gx.batch_set_wait_limit(b, 1000 * limit_us)
+    o = gx.batch_opts(hash_rounds=32, expected_states=[2 * r.states for r in want], levels_cap=n)
+    ws = gx.batch_alloc_workspace(b, o)
+    for _ in range(2):
+        gx.batch_explore(b, o, ws)
+        for i, r in enumerate(want):
+            _check_net(b, i, r)
