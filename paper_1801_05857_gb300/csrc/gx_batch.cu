@@ -279,7 +279,7 @@ struct __align__(16) BatchSmem {
   unsigned long long muls[kMaxRounds];
 };
 
-template <int W, int B, int G>
+template <int W, int B, int G, bool Share>
 __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch_expand_kernel(const BatchArgs a) {
   extern __shared__ __align__(16) unsigned char bsm[];
   BatchSmem<W>& S = *reinterpret_cast<BatchSmem<W>*>(bsm);
@@ -334,7 +334,7 @@ __global__ void __launch_bounds__(gx::kBlock, BatchOcc<W, B, G>::min_ctas) batch
     uint64_t pos = 0, end = 0;  // what is left of the claim
     bool held = true;           // c is a claim that has not been started
     uint32_t taken = 1;
-    expand_states<W, B, G, 32>(
+    expand_states<W, B, G, 32, true, Share>(
         tg, muls, t, L, S.queues[wid], st, probes, err,
         ClassDescs{descs, L.n_classes < 32u ? L.n_classes : 32u},
         [&](uint64_t& from, uint32_t& m) {
@@ -404,18 +404,19 @@ struct BatchKernels {
 };
 
 template <int W, int B, int G>
-BatchKernels batch_kernels() {
+BatchKernels batch_kernels(bool share) {
   return BatchKernels{reinterpret_cast<const void*>(&gxd::batch_init_kernel<W, B, G>),
-                      reinterpret_cast<const void*>(&gxd::batch_expand_kernel<W, B, G>),
+                      share ? reinterpret_cast<const void*>(&gxd::batch_expand_kernel<W, B, G, true>)
+                            : reinterpret_cast<const void*>(&gxd::batch_expand_kernel<W, B, G, false>),
                       sizeof(gxd::BatchSmem<W>)};
 }
 
 // (B, G) pairs built for batches; the autotuner picks among them.
 const int kCands[][2] = {{4, 1}, {8, 1}, {8, 2}, {16, 1}, {16, 2}, {32, 2}, {32, 4}};
 
-bool lookup(int W, int B, int G, BatchKernels& out) {
+bool lookup(int W, int B, int G, bool share, BatchKernels& out) {
 #define GX_BK(w, b, g) \
-  if (W == w && B == b && G == g) { out = batch_kernels<w, b, g>(); return true; }
+  if (W == w && B == b && G == g) { out = batch_kernels<w, b, g>(share); return true; }
   GX_BK(1, 4, 1) GX_BK(1, 8, 1) GX_BK(1, 8, 2) GX_BK(1, 16, 1) GX_BK(1, 16, 2) GX_BK(1, 32, 2) GX_BK(1, 32, 4)
   GX_BK(2, 4, 1) GX_BK(2, 8, 1) GX_BK(2, 8, 2) GX_BK(2, 16, 1) GX_BK(2, 16, 2) GX_BK(2, 32, 2) GX_BK(2, 32, 4)
   GX_BK(4, 4, 1) GX_BK(4, 8, 1) GX_BK(4, 8, 2) GX_BK(4, 16, 1) GX_BK(4, 16, 2) GX_BK(4, 32, 2) GX_BK(4, 32, 4)
@@ -479,7 +480,9 @@ gx_status batch_plan(const gx_batch* h, const gx_batch_opts* o, BatchPlan& P) {
   if (P.rounds < 1 || P.rounds > kMaxRounds) return fail(GX_ERR_INVALID, "hash_rounds must be 1..64");
   if (P.chunk < 32 || P.chunk % 32 || P.chunk > 4096)
     return fail(GX_ERR_INVALID, "chunk_states must be a multiple of 32 in 32..4096");
-  if (!lookup(P.W, P.B, P.G, P.k))
+  bool share = false;  // of a rule's combinations, between lanes (WarpGen)
+  for (const Net& net : h->nets) share |= net.lay.max_source >= gxd::kShareFrom;
+  if (!lookup(P.W, P.B, P.G, share, P.k))
     return fail(GX_ERR_INVALID, "no batch kernel for bucket_words " + std::to_string(P.B) + ", group_lanes " +
                                     std::to_string(P.G) + " with " + std::to_string(P.W) + "-word slots");
   P.levels_cap = o->levels_cap ? o->levels_cap : 4096;

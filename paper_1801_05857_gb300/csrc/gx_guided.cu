@@ -748,7 +748,7 @@ __global__ void __launch_bounds__(1024) guided_select_kernel(const GuidedArgs a)
   select_batch<W>(a);
 }
 
-template <int W, int B>
+template <int W, int B, bool Share>
 __global__ void __launch_bounds__(gx::kBlock) guided_expand_kernel(const GuidedArgs a) {
   constexpr int E = W + 1;
   constexpr int kWarps = gx::kBlock / 32;
@@ -822,13 +822,19 @@ __global__ void __launch_bounds__(gx::kBlock) guided_expand_kernel(const GuidedA
       for (int w = 0; w < W; ++w) le[w] = v[w];
       le[W] = a.batch[idx * E + W];
     }
-    WarpGen<W> gen;
+    WarpGen<W, Share> gen;
     gen.src = gen.e = gen.e_end = gen.word = gen.cur = 0;
     uint32_t total = 0;  // this lane's part of the state's successors
     int queued = 0;
     while (true) {
-      const uint32_t act = __ballot_sync(FULLMASK, gen.e < gen.e_end);
+      uint32_t act = __ballot_sync(FULLMASK, gen.e < gen.e_end);
       if (act != 0) {
+        if constexpr (Share) {
+          if (__popc(act) <= 16) {
+            gen.share(act, 5);
+            act = __ballot_sync(FULLMASK, gen.e < gen.e_end);
+          }
+        }
         if ((act >> lane) & 1u) gen.emit(t, L, desc, v, queue + (queued + __popc(act & below)) * W);
         queued += __popc(act);
         if (queued < 32) continue;
@@ -1259,6 +1265,7 @@ struct GKernels {
   const void* init;
   const void* select;
   const void* expand;
+  const void* expand_share;  // for networks with a source of kShareFrom successors or more
   const void* score;
   const void* path;
   const void* start;    // pop the first batch and start the device loop
@@ -1273,7 +1280,8 @@ GKernels gk() {
                   &gxd::slot_gather_kernel<W>,
                   reinterpret_cast<const void*>(&gxd::guided_init_kernel<W, B>),
                   reinterpret_cast<const void*>(&gxd::guided_select_kernel<W>),
-                  reinterpret_cast<const void*>(&gxd::guided_expand_kernel<W, B>),
+                  reinterpret_cast<const void*>(&gxd::guided_expand_kernel<W, B, false>),
+                  reinterpret_cast<const void*>(&gxd::guided_expand_kernel<W, B, true>),
                   reinterpret_cast<const void*>(&gxd::guided_score_kernel<W>),
                   reinterpret_cast<const void*>(&gxd::guided_path_kernel<W>),
                   reinterpret_cast<const void*>(&gxd::guided_loop_start_kernel<W>),
@@ -1314,6 +1322,7 @@ gx_status guided_plan(const Net& net, const gx_explore_opts* o, GPlan& P) {
   P.W = (int)net.slot_words;
   P.B = o->bucket_words ? (int)o->bucket_words : 8;
   if (P.B < P.W || !gk_lookup(P.W, P.B, P.k)) return fail(GX_ERR_INVALID, "unsupported bucket_words for guided search");
+  if (net.lay.max_source >= gxd::kShareFrom) P.k.expand = P.k.expand_share;
   P.rounds = o->hash_rounds ? (int)o->hash_rounds : 8;
   if (P.rounds < 1 || P.rounds > kMaxRounds) return fail(GX_ERR_INVALID, "hash_rounds must be 1..64");
   P.nbins = o->guided_bins ? (int)o->guided_bins : 32;

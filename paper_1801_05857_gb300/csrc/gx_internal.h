@@ -33,6 +33,7 @@ struct NetBlobLayout {
   uint32_t rule_off;    // [n_rules + 1] into rule_cls
   uint32_t rule_cls;    // class id of each rule participant
   uint32_t total;       // blob length in words
+  uint32_t max_source;  // most successors that one process or rule can give a state
 };
 
 struct Net {

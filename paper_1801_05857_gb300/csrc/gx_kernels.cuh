@@ -506,12 +506,21 @@ struct ClassDescs {
 // as many per source: what counts in a level of few states.  emit() appends one
 // successor per lane that has any left to a queue in shared memory; a state's
 // successors are counted on the way, without a pass of their own.
-template <int W>
+// Share: lanes whose source is exhausted take part of what is left of another lane's
+// (share), for the kernels that give a warp one or a few states: a rule of many
+// combinations would be one lane's work.  (4096 states with one rule of 729: guided
+// search 4.0 -> 0.29 ms, batch of one such network 4.4 -> 0.29.)
+// Kernels of their own, for networks with a source of kShareFrom successors or more
+// (max_source): the others gain nothing and would pay for the check and a register (256
+// networks: 8.2 ms, with it 8.4).
+constexpr uint32_t kShareFrom = 16;
+template <int W, bool Share = false>
 struct WarpGen {
   uint32_t src;       // next source: process src, then rule src - n_procs (uniform)
   uint32_t e, e_end;  // this lane's successors left of its source: edges, or combinations of the rule
   uint32_t word;      // word index of the source's process; W: a rule
   uint32_t cur;       // that word of this lane's state; a rule: its index
+  uint32_t stride;    // Share: every how many of its source's successors are this lane's
 
   template <class Desc>
   __device__ __forceinline__ void open(const uint32_t* t, const NetBlobLayout& L, Desc& desc, bool valid,
@@ -539,6 +548,7 @@ struct WarpGen {
       e = 0;
       e_end = prod;
     }
+    stride = 1;
     ++src;
   }
 
@@ -569,7 +579,33 @@ struct WarpGen {
       cur = r;
       e_end = prod;
     }
+    stride = 1;
     src += 1u << sh;
+  }
+
+  // When at most half of the 2^sh lanes that hold a state have successors left, and some
+  // lane has many: the ones that have none take every 2nd, 4th, ... of theirs.  act: the
+  // lanes with successors left.  All 32 lanes call it together.
+  __device__ __forceinline__ void share(uint32_t act, uint32_t sh) {
+    static_assert(Share, "only with strides");
+    const uint32_t lane = threadIdx.x & 31, n = 1u << sh, sub = lane & (n - 1u), first = lane - sub;
+    const uint32_t busy = (act >> first) & (0xFFFFFFFFu >> (32u - n));
+    const uint32_t k = __popc(busy);
+    // (sharing 8 successors takes about as long as the steps it saves)
+    if (!__any_sync(FULLMASK, 2 * k <= n && e < e_end && (e_end - e) / stride >= 8)) return;
+    const uint32_t log = k > 1 ? 32u - __clz(k - 1u) : 0u;  // 2^log >= k parts of the group
+    const uint32_t m = 2 * k <= n && k > 0 ? sh - log : 0u;   // 2^m lanes each
+    const uint32_t part = sub & ((1u << m) - 1u);
+    const bool has = m == 0 || (sub >> m) < k;
+    const int from = m == 0 || !has ? (int)lane : (int)(first + __fns(busy, 0, (int)(sub >> m) + 1));
+    e = __shfl_sync(FULLMASK, e, from);
+    e_end = __shfl_sync(FULLMASK, e_end, from);
+    word = __shfl_sync(FULLMASK, word, from);
+    cur = __shfl_sync(FULLMASK, cur, from);
+    stride = __shfl_sync(FULLMASK, stride, from);
+    if (!has || e_end - e <= part * stride) e = e_end;
+    else e += part * stride;
+    stride <<= m;
   }
 
   // One successor into the W words at q (a lane with e < e_end).
@@ -599,7 +635,8 @@ struct WarpGen {
       }
       store_vec<W>(q, out);
     }
-    ++e;
+    if constexpr (Share) e = e_end - e > stride ? e + stride : e_end;  // (no overflow: ranges end below 2^32)
+    else ++e;
   }
 };
 
@@ -641,7 +678,10 @@ struct ExpandOcc {
 // states a warp 18 us instead of 26-28, the search 1.61 -> 1.33 ms.  (16 states: the same
 // there; levels of 8 to 16 states a warp of the mid network 30 instead of 33 us, others
 // up to 2 % slower.)
-constexpr uint32_t kWideStates = 8;
+// With sharing, two lanes for each of 9 to 16 states still pay (16 networks of 4096 states
+// with one rule of 729: 2.4 -> 1.6 ms).
+template <bool Share>
+constexpr uint32_t kWideStates = Share ? 16 : 8;
 
 // The expansion of a warp's share of one level: generate successors of its
 // states until a batch is queued, filter it, and resolve what is kept 32 at a
@@ -656,8 +696,8 @@ constexpr uint32_t kWideStates = 8;
 //   keep(on, x)    the filters before the GPU-wide cache: whether a lane's successor x
 //                  (if on) passes them; all 32 lanes call it together
 // All 32 lanes call it together; returns with the queues empty.  Wide: whether
-// few states are treated so at all.
-template <int W, int B, int G, int Batch, bool Wide = true, class T, class Desc, class Next, class Seen, class Done,
+// few states are treated so at all; Share: see WarpGen.
+template <int W, int B, int G, int Batch, bool Wide = true, bool Share = false, class T, class Desc, class Next, class Seen, class Done,
           class Keep>
 __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls, const uint32_t* t,
                                               const NetBlobLayout& L, WarpQueues<W, Batch>& q, WarpStage& st,
@@ -672,14 +712,20 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
   for (int w = 0; w < W; ++w) v[w] = 0;
   uint32_t sh = 0;    // 2^sh lanes hold the same state (uniform)
   uint32_t cnt = 0;   // successors this lane has found of its state
-  WarpGen<W> gen;
+  WarpGen<W, Share> gen;
   gen.src = n_src;
   gen.e = gen.e_end = gen.cur = gen.word = 0;
   bool more = true;  // states may be left for this warp
   while (true) {
     while (n_raw < Batch) {
-      const uint32_t act = __ballot_sync(FULLMASK, gen.e < gen.e_end);
+      uint32_t act = __ballot_sync(FULLMASK, gen.e < gen.e_end);
       if (act != 0) {
+        if constexpr (Share) {
+          if (sh != 0 && __popc(act) <= 16) {
+            gen.share(act, sh);
+            act = __ballot_sync(FULLMASK, gen.e < gen.e_end);
+          }
+        }
         if ((act >> lane) & 1u) gen.emit(t, L, desc, v, q.raw + (n_raw + __popc(act & below)) * W);
         n_raw += __popc(act);
       } else if (gen.src < n_src) {
@@ -699,7 +745,7 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
         more = m != 0;
         if (!more) break;
         if constexpr (Wide) {
-          sh = m <= kWideStates ? (uint32_t)__clz(m - 1) - 27u : 0u;
+          sh = m <= kWideStates<Share> ? (uint32_t)__clz(m - 1) - 27u : 0u;
           if ((lane >> sh) < m) {
             load_words<W>(tg.frontier() + ((pos + (lane >> sh)) & tg.fmask()) * W, v);
             if ((lane & ((1u << sh) - 1u)) == 0) seen(v);

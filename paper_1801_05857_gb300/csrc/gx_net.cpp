@@ -176,8 +176,11 @@ static gx_status encode(const gx_net_desc* d, Net& net) {
       cls_maxdeg[c] = std::max<uint64_t>(cls_maxdeg[c], coff[cls_base[c] + s + 1] - coff[cls_base[c] + s]);
   }
   constexpr uint64_t kSuccCap = 1ull << 40;
-  uint64_t bound = 0;
-  for (uint32_t p = 0; p < n; ++p) bound += cls_maxdeg[p];
+  uint64_t bound = 0, source = 0;
+  for (uint32_t p = 0; p < n; ++p) {
+    bound += cls_maxdeg[p];
+    source = std::max(source, cls_maxdeg[p]);
+  }
   for (uint32_t r = 0; r < d->n_rules; ++r) {
     uint64_t prod = 1;
     for (uint32_t j = rule_off[r]; j < rule_off[r + 1]; ++j) {
@@ -185,10 +188,12 @@ static gx_status encode(const gx_net_desc* d, Net& net) {
       prod = (m && prod > kSuccCap / m) ? kSuccCap : prod * m;
     }
     bound = std::min(kSuccCap, bound + prod);
+    source = std::max(source, prod);
   }
   // The kernels count one state's successors, and a rule's combinations, in 32 bits.
   if (bound > 0xFFFFFFFFull) return fail(GX_ERR_INVALID, "a state can have 2^32 or more successors");
   net.max_succ = bound;
+  L.max_source = (uint32_t)source;
   std::vector<uint32_t>& B = net.blob;
   B.clear();
   auto put = [&](const std::vector<uint32_t>& v) {
