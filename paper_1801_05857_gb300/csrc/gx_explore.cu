@@ -59,6 +59,14 @@ uint32_t auto_cache_log2(const Net& net) {
   return cache_key(net, at, bits) ? cache_auto_log2(bits) : 0;
 }
 
+cudaError_t allow_smem(const void* fn, size_t smem_optin, size_t* static_bytes) {
+  cudaFuncAttributes fa{};
+  const cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+  if (e != cudaSuccess) return e;
+  if (static_bytes) *static_bytes = fa.sharedSizeBytes;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem_optin - fa.sharedSizeBytes));
+}
+
 gx_status warp_cache_layout(const Net& net, uint32_t warp_log2, ExpandArgs& a, size_t& bytes) {
   a.cache_log2 = a.cache_key64 = 0;
   bytes = 0;
@@ -438,7 +446,8 @@ void release_loop(gx_net* h) {
 // table, insert the initial vector, start, then WHILE(more levels) {small levels;
 // WHILE(large levels) {expand; advance}}.
 gx_status build_loop_graph(gx_net* h, const Plan& P, Ctl* ctl, uint32_t* table, const InitArgs& ia,
-                           const ExpandArgs& eg, LoopArgs la, size_t smem, uint64_t grid, size_t small_smem) {
+                           const ExpandArgs& eg, LoopArgs la, size_t smem, int carveout, uint64_t grid,
+                           size_t small_smem) {
   release_loop(h);
   h->release = &release_loop;
   cudaGraph_t g;
@@ -507,7 +516,15 @@ gx_status build_loop_graph(gx_net* h, const Plan& P, Ctl* ctl, uint32_t* table, 
   GX_CUDA(add_kernel(outer, nullptr, 0, P.ks->small_fn, dim3(gxd::kSmallCtas), dim3(gxd::kSmallThreads), small_smem,
                      args_s, &sm));
   GX_CUDA(add_while(outer, &sm, la.cond_big, &body));
-  GX_CUDA(add_kernel(body, nullptr, 0, P.ks->expand_fn, dim3((unsigned)grid), dim3(kBlock), smem, args_e, &ex));
+  auto add_expand = [&](const cudaGraphNode_t* dep, void** args, cudaGraphNode_t* out) -> cudaError_t {
+    cudaError_t e = add_kernel(body, dep, dep ? 1 : 0, P.ks->expand_fn, dim3((unsigned)grid), dim3(kBlock), smem, args, out);
+    cudaLaunchAttributeValue v{};
+    v.sharedMemCarveout = (unsigned)carveout;
+    if (e == cudaSuccess && carveout >= 0)
+      e = cudaGraphKernelNodeSetAttribute(*out, cudaLaunchAttributePreferredSharedMemoryCarveout, &v);
+    return e;
+  };
+  GX_CUDA(add_expand(nullptr, args_e, &ex));
   // region passes after the first: clear the claim counter, expand again
   for (uint32_t q = 1; q < P.regions; ++q) {
     ExpandArgs eq = region_pass(eg, P.regions, q);
@@ -520,7 +537,7 @@ gx_status build_loop_graph(gx_net* h, const Plan& P, Ctl* ctl, uint32_t* table, 
     mp.height = 1;
     cudaGraphNode_t mz, exq;
     GX_CUDA(cudaGraphAddMemsetNode(&mz, body, &ex, 1, &mp));
-    GX_CUDA(add_kernel(body, &mz, 1, P.ks->expand_fn, dim3((unsigned)grid), dim3(kBlock), smem, args_q, &exq));
+    GX_CUDA(add_expand(&mz, args_q, &exq));
     ex = exq;
   }
   GX_CUDA(add_kernel(body, &ex, 1, reinterpret_cast<const void*>(&gxd::level_advance_kernel), dim3(1), dim3(1), 0,
@@ -636,35 +653,31 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
     ea.viol_buf = viol;
     ea.viol_cap = P.viol_cap;
   }
-  cudaFuncAttributes fa{};
-  GX_CUDA(cudaFuncGetAttributes(&fa, P.ks->expand_fn));
+  size_t fixed = 0;  // static shared memory of the level kernel
+  GX_CUDA(allow_smem(P.ks->expand_fn, dev.smem_optin, &fixed));
   const size_t blob_bytes = 4ull * net.blob.size();
   size_t cache_bytes = 0;
   if ((s = warp_cache_layout(net, P.warp_log2, ea, cache_bytes)) != GX_OK) return s;
   size_t smem = 8ull * kMaxRounds + cache_bytes;
-  if (fa.sharedSizeBytes + smem > dev.smem_optin)
+  if (fixed + smem > dev.smem_optin)
     return fail(GX_ERR_INVALID, "warp cache of 2^" + std::to_string(ea.cache_log2) + " entries per warp needs " +
-                                    std::to_string(fa.sharedSizeBytes + smem) +
+                                    std::to_string(fixed + smem) +
                                     " bytes of shared memory per CTA, more than " + std::to_string(dev.smem_optin));
   // the network tables are staged unless they are large or leave no room for the cache
   ea.stage = blob_bytes + 8ull * kMaxRounds <= 96 * 1024 &&
-                     fa.sharedSizeBytes + smem + blob_bytes <= dev.smem_optin ? 1 : 0;
+                     fixed + smem + blob_bytes <= dev.smem_optin ? 1 : 0;
   if (ea.stage) smem += blob_bytes;
-  GX_CUDA(cudaFuncSetAttribute(P.ks->expand_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   GX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, P.ks->expand_fn, kBlock, smem));
   if (per_sm < 1) return fail(GX_ERR_INVALID, "expansion kernel does not fit on an SM");
   // Shared memory beyond 196 KB an SM leaves the GPU-wide cache's lookups too little L1 to
   // be in flight in (mid network, padded from 186 to 214 KB: 19 ms became 30 ms), so a
   // network with large tables runs fewer CTAs.
+  int carveout = -1;  // (an attribute of the launches, not of the function)
   if (gcache.base) {
-    const size_t cta = fa.sharedSizeBytes + smem + 1024, most = 196 * 1024;
+    const size_t cta = fixed + smem + 1024, most = 196 * 1024;
     if (cta * per_sm > most) per_sm = std::max<int>(1, (int)(most / cta));
-    GX_CUDA(cudaFuncSetAttribute(P.ks->expand_fn, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)std::min<size_t>(100, (cta * per_sm * 100 + 228 * 1024 - 1) / (228 * 1024))));
-  } else {
-    GX_CUDA(cudaFuncSetAttribute(P.ks->expand_fn, cudaFuncAttributePreferredSharedMemoryCarveout,
-                                 (int)cudaSharedmemCarveoutDefault));
+    carveout = (int)std::min<size_t>(100, (cta * per_sm * 100 + 228 * 1024 - 1) / (228 * 1024));
   }
   if (o->ctas_per_sm) per_sm = std::min<int>(per_sm, (int)o->ctas_per_sm);
   const uint64_t max_grid = (uint64_t)dev.sms * per_sm;
@@ -704,8 +717,8 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
       // the small-level kernel: multipliers, queues and (when they are not large) network tables
       size_t small_smem = 8ull * kMaxRounds + P.ks->small_queue_bytes;
       if (blob_bytes <= 64 * 1024) small_smem += blob_bytes;
-      GX_CUDA(cudaFuncSetAttribute(P.ks->small_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)small_smem));
-      s = build_loop_graph(h, P, ctl, table, ia, eg, la, smem, max_grid, small_smem);
+      GX_CUDA(allow_smem(P.ks->small_fn, dev.smem_optin));
+      s = build_loop_graph(h, P, ctl, table, ia, eg, la, smem, carveout, max_grid, small_smem);
       if (s != GX_OK) return s;
       h->loop_key = key;
     }
@@ -754,8 +767,8 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
     pa.succ = reinterpret_cast<uint32_t*>(base + P.off_succ);
     pa.logp = P.logp;
     psmem = 8ull * kMaxRounds + (ea.stage ? blob_bytes : 0) + (4ull << P.logp);
-    GX_CUDA(cudaFuncSetAttribute(P.ks->part_count_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem));
-    GX_CUDA(cudaFuncSetAttribute(P.ks->part_scatter_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)psmem));
+    GX_CUDA(allow_smem(P.ks->part_count_fn, dev.smem_optin));
+    GX_CUDA(allow_smem(P.ks->part_scatter_fn, dev.smem_optin));
     int pp = 0;
     GX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&pp, P.ks->part_probe_fn, kBlock, 0));
     probe_grid = dev.sms * std::max(pp, 1);
@@ -803,7 +816,7 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
       const int grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(want, max_grid));
       for (uint32_t q = 0; q < P.regions; ++q) {
         GX_CUDA(cudaMemsetAsync(&ctl->claim, 0, sizeof(unsigned long long), st));
-        GX_CUDA(P.ks->expand(region_pass(ea, P.regions, q), grid, smem, st));
+        GX_CUDA(P.ks->expand(region_pass(ea, P.regions, q), grid, smem, carveout, st));
         ++launches;
       }
     }

@@ -1505,7 +1505,7 @@ gx_status run_guided(gx_net* h, const gx_explore_opts* opts, void* ws, uint64_t 
   const size_t blob_bytes = 4ull * net.blob.size();
   a.stage = (blob_bytes <= (size_t)optin - 32 * 1024) ? 1 : 0;
   const size_t smem = a.stage ? blob_bytes : 0;
-  GG_CUDA(cudaFuncSetAttribute(P.k.expand, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  GG_CUDA(allow_smem(P.k.expand, (size_t)optin));
   GG_CUDA(cudaFuncSetAttribute(P.k.score, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gxt::kTcSmemBytes));
   GG_CUDA(cudaFuncSetAttribute(P.k.score, cudaFuncAttributePreferredSharedMemoryCarveout,
                                (int)cudaSharedmemCarveoutMaxShared));
@@ -1523,7 +1523,7 @@ gx_status run_guided(gx_net* h, const gx_explore_opts* opts, void* ws, uint64_t 
   if (fused) {
     a.stage = fused_bytes(blob_bytes) <= (size_t)optin ? 1 : 0;  // else the tables are read from global memory
     fused_smem = fused_bytes(a.stage ? blob_bytes : 0);
-    GG_CUDA(cudaFuncSetAttribute(P.k.fused, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fused_smem));
+    GG_CUDA(allow_smem(P.k.fused, (size_t)optin));
     int fp = 0;
     GG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fp, P.k.fused, gxd::kFusedThreads, fused_smem));
     fp = std::min(std::max(fp, 1), 4);  // TMEM: 128 columns per CTA, 512 per SM

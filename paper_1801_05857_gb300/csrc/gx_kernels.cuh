@@ -1483,9 +1483,18 @@ __global__ void __launch_bounds__(gx::kBlock) fop_kernel(const gx::FopArgs a) {
 namespace gx {
 
 template <int W, int B, int G>
-cudaError_t launch_expand(const ExpandArgs& a, int grid, size_t smem, cudaStream_t st) {
-  gxd::expand_kernel<W, B, G><<<grid, kBlock, smem, st>>>(a);
-  return cudaGetLastError();
+cudaError_t launch_expand(const ExpandArgs& a, int grid, size_t smem, int carveout, cudaStream_t st) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(kBlock);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  at[0].val.sharedMemCarveout = (unsigned)carveout;
+  cfg.attrs = at;
+  cfg.numAttrs = carveout >= 0 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, gxd::expand_kernel<W, B, G>, a);
 }
 template <int W, int B, int G>
 cudaError_t launch_init(const InitArgs& a, cudaStream_t st) {

@@ -147,7 +147,7 @@ struct FopArgs {
 };
 
 struct KernelSet {
-  cudaError_t (*expand)(const ExpandArgs&, int grid, size_t smem, cudaStream_t);
+  cudaError_t (*expand)(const ExpandArgs&, int grid, size_t smem, int carveout, cudaStream_t);  // carveout: percent, -1: default
   cudaError_t (*part_count)(const ExpandArgs&, const PartArgs&, size_t smem, cudaStream_t);
   cudaError_t (*part_scan)(const PartArgs&, cudaStream_t);
   cudaError_t (*part_scatter)(const ExpandArgs&, const PartArgs&, size_t smem, cudaStream_t);
@@ -175,6 +175,11 @@ inline const KernelSet* kernels_for(int W, int B, int G) {
   if (W == 4) return kernels_w4(B, G);
   return nullptr;
 }
+
+// Lets a kernel take all the dynamic shared memory its static part leaves: the same
+// value for every caller, as the attribute belongs to the function, which searches of
+// other networks launch with other sizes, from cached graphs and other threads too.
+cudaError_t allow_smem(const void* fn, size_t smem_optin, size_t* static_bytes = nullptr);
 
 cudaError_t launch_digest(int W, const DigestArgs& a, int grid, cudaStream_t st);
 

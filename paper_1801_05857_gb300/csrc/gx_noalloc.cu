@@ -192,21 +192,20 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
     ea.viol_cap = 0;
   }
   // shared memory: the same rules as gx_explore
-  cudaFuncAttributes fa{};
-  NA_CUDA(cudaFuncGetAttributes(&fa, ks->expand_fn));
+  size_t fixed = 0;  // static shared memory of the level kernel
+  NA_CUDA(gx::allow_smem(ks->expand_fn, (size_t)smem_optin, &fixed));
   const size_t blob_bytes = 4ull * net.blob.size();
   size_t cache_bytes = 0;
   if ((s = gx::warp_cache_layout(net, warp_log2, ea, cache_bytes)) != GX_OK) return s;
   size_t smem = 8ull * gx::kMaxRounds + cache_bytes;
-  if (fa.sharedSizeBytes + smem > (size_t)smem_optin)
+  if (fixed + smem > (size_t)smem_optin)
     return gx::fail(GX_ERR_INVALID, "warp cache of 2^" + std::to_string(ea.cache_log2) +
-                                        " entries per warp needs " + std::to_string(fa.sharedSizeBytes + smem) +
+                                        " entries per warp needs " + std::to_string(fixed + smem) +
                                         " bytes of shared memory per CTA, more than " +
                                         std::to_string(smem_optin));
   ea.stage = blob_bytes + 8ull * gx::kMaxRounds <= 96 * 1024 &&
-                     fa.sharedSizeBytes + smem + blob_bytes <= (size_t)smem_optin ? 1 : 0;
+                     fixed + smem + blob_bytes <= (size_t)smem_optin ? 1 : 0;
   if (ea.stage) smem += blob_bytes;
-  NA_CUDA(cudaFuncSetAttribute(ks->expand_fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   int per_sm = 0;
   NA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ks->expand_fn, gx::kBlock, smem));
   if (per_sm < 1) return gx::fail(GX_ERR_INVALID, "expansion kernel does not fit on an SM");
@@ -232,7 +231,7 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
       eq.region_bits = (uint64_t)q << (log2nb - log2r);
       eq.count_states = q == 0 ? 1 : 0;
       NA_CUDA(cudaMemsetAsync(&ctl->claim, 0, sizeof(unsigned long long), st));
-      NA_CUDA(ks->expand(eq, grid, smem, st));
+      NA_CUDA(ks->expand(eq, grid, smem, -1, st));
     }
     NA_CUDA(cudaMemcpyAsync(&hc, ctl, sizeof(gx::Ctl), cudaMemcpyDeviceToHost, st));
     NA_CUDA(cudaStreamSynchronize(st));

@@ -184,3 +184,71 @@ def test_few_state_levels_hand_over_in_a_stopped_search(cuda, n, passes):
     s = _check(("stopped", n), net, table_bytes=1 << 24, bucket_words=8, group_lanes=1, hash_rounds=32,
                region_passes=passes, stop_at_first_deadlock=1)
     assert s["complete"] == 0 and s["first_deadlock_level"] == r.first_deadlock_level
+
+
+def _star(n_states, n_procs, moving):
+    """One process that can go from its first state to any of n_states - 1 others (its tables take
+    8 n_states bytes), beside n_procs two-state processes of which `moving` cycle."""
+    net = _mostly_still(n_procs, moving)
+    net.procs.append(inputs.LTS(n_states, 0, [(0, 0, s) for s in range(1, n_states)]))
+    return net
+
+
+@pytest.mark.parametrize("loop", [0, 1])
+def test_networks_of_different_table_sizes_take_turns(cuda, loop):
+    """Kernels staged with 0.5, 56 and 40 KB of network tables and with an explicit warp cache,
+    one after the other and again on their cached graphs: what one search asks of a kernel
+    (shared memory, its split with the L1) is not changed by another's."""
+    runs = []
+    for key, net, kw in [("small", _mostly_still(70, 5), {}), ("star7000", _star(7000, 70, 2), {}),
+                         ("star5000", _star(5000, 70, 2), dict(warp_cache_log2=9)),
+                         ("small_cached", _mostly_still(70, 6), dict(global_cache_log2=16))]:
+        o = gx.default_opts(table_bytes=1 << 24, bucket_words=8, group_lanes=1, hash_rounds=32, host_loop=loop, **kw)
+        h = gx.load_network(net)
+        runs.append((key, net, h, o, gx.alloc_workspace(h, o)))
+    for order in ([0, 1, 2, 3], [1, 0, 2, 1, 3, 2, 0, 1]):
+        for i in order:
+            key, net, h, o, ws = runs[i]
+            r = _oracle(key, net)
+            gx.explore(h, o, ws)
+            s = gx.stats(h)
+            assert (s["states"], s["transitions"], gx.levels(h)) == (r.states, r.transitions, r.levels)
+            assert s["slot_words"] == 4 and gx.set_digest(h, ws) == (r.states, r.set_sum, r.set_xor)
+
+
+def test_searches_of_several_threads(cuda):
+    """Four threads, a stream and a network each, of different table sizes and caches: every
+    search takes the shared memory it needs, whatever the others ask for in between."""
+    import threading
+    import torch
+    runs = [("small", _mostly_still(70, 5), {}), ("star7000", _star(7000, 70, 2), {}),
+            ("star5000", _star(5000, 70, 2), dict(warp_cache_log2=9, host_loop=1)),
+            ("small_cached", _mostly_still(70, 6), dict(global_cache_log2=16))]
+    want = [_oracle(key, net) for key, net, _ in runs]
+    bad = []
+
+    def work(i):
+        try:
+            torch.cuda.set_device(0)
+            key, net, kw = runs[i]
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                o = gx.default_opts(table_bytes=1 << 22, bucket_words=8, group_lanes=1, hash_rounds=32, **kw)
+                for _ in range(5):  # (a handle each: its graph is built anew)
+                    h = gx.load_network(net)
+                    ws = gx.alloc_workspace(h, o)
+                    for _ in range(4):
+                        gx.explore(h, o, ws, stream)
+                        s = gx.stats(h)
+                        assert (s["states"], s["transitions"], gx.levels(h)) == (
+                            want[i].states, want[i].transitions, want[i].levels), key
+                    stream.synchronize()
+        except Exception as e:  # noqa: BLE001 -- reported by the main thread
+            bad.append((runs[i][0], repr(e)))
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(runs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not bad, bad
