@@ -42,7 +42,19 @@ void hash_multipliers(uint64_t* out, int n) {
   }
 }
 
-bool cache_layout(const Net& net, uint32_t log2_entries, SeenCache& c) {
+cudaError_t allow_smem(const void* fn, size_t smem_optin, size_t* static_bytes) {
+  cudaFuncAttributes fa{};
+  const cudaError_t e = cudaFuncGetAttributes(&fa, fn);
+  if (e != cudaSuccess) return e;
+  if (static_bytes) *static_bytes = fa.sharedSizeBytes;
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem_optin - fa.sharedSizeBytes));
+}
+
+constexpr uint32_t kAutoCache = 0xFFFFFFFFu;  // warp_cache_log2 / global_cache_log2: automatic
+
+// Layout of a GPU-wide cache of 2^log2_entries entries; false when the network's vectors
+// have no 64-bit key.
+static bool cache_layout(const Net& net, uint32_t log2_entries, SeenCache& c) {
   uint32_t bits = 0;
   if (!cache_key(net, c.word_at, bits)) return false;
   c.shift = bits > log2_entries ? bits - log2_entries : 0;
@@ -54,36 +66,79 @@ bool cache_layout(const Net& net, uint32_t log2_entries, SeenCache& c) {
   return true;
 }
 
-uint32_t auto_cache_log2(const Net& net) {
-  uint32_t at[3], bits = 0;
-  return cache_key(net, at, bits) ? cache_auto_log2(bits) : 0;
+// The automatic GPU-wide cache: in tables of at least 2^26 slots with one lane per bucket
+// (where it was measured), for vectors whose fields fit one 64-bit key; else the per-warp
+// one.  4-word vectors: only in one pass (1.08e8-state irregular network, 4 GiB: 42 ms with
+// it, 50 ms without; the memory-filling product network in two passes, 8 GiB: 231 ms with
+// it, 186 ms without).
+// The per-warp one: more entries find more, but their shared memory costs CTAs and L1 (token
+// ring of 13 nodes: 2^6 4.19 ms, 2^7 4.18, 2^8 4.24, 2^9 4.86; 1.7e7 states of 4 words in one
+// pass, 16-byte entries, half as many: 8.83, 8.76, 9.13, 10.3; 3.4e8 of 4 words in two
+// passes, 8-byte entries: 2^6 189, 2^7 185, 2^8 199).
+gx_status plan_caches(const Net& net, const gx_explore_opts& o, int lanes, uint64_t slots, uint32_t regions,
+                      CachePlan& p) {
+  uint32_t log2 = o.global_cache_log2;
+  if (log2 == kAutoCache) {
+    uint32_t at[3], bits = 0;
+    const bool use = lanes == 1 && slots >= (1ull << 26) && (net.slot_words <= 2 || regions == 1);
+    log2 = use && cache_key(net, at, bits) ? cache_auto_log2(bits) : 0;
+  } else if (log2 > 26) {
+    return fail(GX_ERR_INVALID, "global_cache_log2 must be at most 26");
+  }
+  if (log2 && cache_layout(net, log2, p.seen)) {
+    p.entries = 1ull << log2;
+    p.bytes = p.entries << p.seen.log2_bytes;
+  }
+  p.warp_log2 = o.warp_cache_log2 == kAutoCache ? (p.entries ? 0u : 7u) : o.warp_cache_log2;
+  return GX_OK;
 }
 
-cudaError_t allow_smem(const void* fn, size_t smem_optin, size_t* static_bytes) {
-  cudaFuncAttributes fa{};
-  const cudaError_t e = cudaFuncGetAttributes(&fa, fn);
-  if (e != cudaSuccess) return e;
-  if (static_bytes) *static_bytes = fa.sharedSizeBytes;
-  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(smem_optin - fa.sharedSizeBytes));
-}
-
-gx_status warp_cache_layout(const Net& net, uint32_t warp_log2, ExpandArgs& a, size_t& bytes) {
+gx_status plan_expand(const Net& net, const gx_explore_opts& o, const KernelSet& ks, uint32_t warp_log2,
+                      size_t smem_optin, ExpandArgs& a, ExpandLaunch& l) {
+  auto cuda = [](cudaError_t e, const char* what) {
+    return e == cudaSuccess ? GX_OK : fail(GX_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
+  };
+  size_t fixed = 0;  // static shared memory
+  gx_status s = cuda(allow_smem(ks.expand_fn, smem_optin, &fixed), "attributes of the level kernel");
+  if (s != GX_OK) return s;
+  // the per-warp cache: 4-word vectors take 64-bit keys as entries where their fields fit, else
+  // half as many 16-byte ones
   a.cache_log2 = a.cache_key64 = 0;
-  bytes = 0;
-  if (warp_log2 == 0) return GX_OK;
+  size_t cache_bytes = 0;
   if (warp_log2 > 12) return fail(GX_ERR_INVALID, "warp_cache_log2 must be at most 12");
-  a.cache_log2 = (int)warp_log2;
-  uint32_t bits = 0;
-  size_t entry = 4ull * net.slot_words;
-  if (net.slot_words == 4) {
-    if (cache_key(net, a.gcache.word_at, bits)) {
+  if (warp_log2) {
+    uint32_t bits = 0;
+    size_t entry = 4ull * net.slot_words;
+    a.cache_log2 = (int)warp_log2;
+    if (net.slot_words == 4 && cache_key(net, a.gcache.word_at, bits)) {
       a.cache_key64 = 1;
       entry = 8;
-    } else {
-      a.cache_log2 -= 1;  // 16-byte entries: the same bytes
+    } else if (net.slot_words == 4) {
+      a.cache_log2 -= 1;
     }
+    cache_bytes = entry * (kBlock / 32) << a.cache_log2;
   }
-  bytes = entry * (kBlock / 32) << a.cache_log2;
+  l.smem = 8ull * kMaxRounds + cache_bytes;
+  if (fixed + l.smem > smem_optin)
+    return fail(GX_ERR_INVALID, "warp cache of 2^" + std::to_string(a.cache_log2) + " entries per warp needs " +
+                                    std::to_string(fixed + l.smem) +
+                                    " bytes of shared memory per CTA, more than " + std::to_string(smem_optin));
+  // the network tables are staged unless they are large or leave no room for the cache
+  const size_t blob_bytes = 4ull * net.blob.size();
+  a.stage = blob_bytes + 8ull * kMaxRounds <= 96 * 1024 && fixed + l.smem + blob_bytes <= smem_optin ? 1 : 0;
+  if (a.stage) l.smem += blob_bytes;
+  s = cuda(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&l.per_sm, ks.expand_fn, kBlock, l.smem), "occupancy of the level kernel");
+  if (s != GX_OK) return s;
+  if (l.per_sm < 1) return fail(GX_ERR_INVALID, "expansion kernel does not fit on an SM");
+  // Shared memory beyond 196 KB an SM leaves the GPU-wide cache's lookups too little L1 to
+  // be in flight in (mid network, padded from 186 to 214 KB: 19 ms became 30 ms), so a
+  // network with large tables runs fewer CTAs.
+  if (a.gcache.base) {
+    const size_t cta = fixed + l.smem + 1024, most = 196 * 1024;
+    if (cta * l.per_sm > most) l.per_sm = std::max<int>(1, (int)(most / cta));
+    l.carveout = (int)std::min<size_t>(100, (cta * l.per_sm * 100 + 228 * 1024 - 1) / (228 * 1024));
+  }
+  if (o.ctas_per_sm) l.per_sm = std::min<int>(l.per_sm, (int)o.ctas_per_sm);
   return GX_OK;
 }
 
@@ -255,8 +310,6 @@ constexpr int kPartCtas = 1024;  // CTAs of the partitioned count/scatter passes
 // over 128 GiB (the GPU's address-translation reach); the later hash rounds of
 // a vector stay inside the same 64 GiB span as its first (bucket_in_span).
 constexpr uint64_t kAutoRegionBytes = 1ull << gxd::kSpanLog2Bytes;
-constexpr uint32_t kAutoCache = 0xFFFFFFFFu;  // warp_cache_log2 / global_cache_log2: automatic
-
 // Arguments of pass q of `passes` region passes over a table of 2^log2nb buckets.
 inline ExpandArgs region_pass(const ExpandArgs& a, uint32_t passes, uint32_t q) {
   ExpandArgs r = a;
@@ -279,10 +332,7 @@ struct Plan {
   uint64_t cs = 0;         // successor buffer capacity (vectors)
   uint64_t part_min = 0;   // smallest level that may use the partitioned path
   uint32_t regions = 1;    // passes per level of the direct path (region passes)
-  uint64_t gcache = 0;     // entries of the GPU-wide cache of seen vectors (0 = off)
-  uint64_t gcache_bytes = 0;
-  SeenCache seen{};        // its layout (base left out)
-  uint32_t warp_log2 = 0;  // per-warp cache of seen vectors: 2^warp_log2 entries (0 = off)
+  CachePlan cache;         // of seen vectors
   uint64_t off_ctl = 0, off_blob = 0, off_dl = 0, off_viol = 0, off_loop = 0, off_front = 0, off_table = 0;
   uint64_t off_hist = 0, off_off = 0, off_ptot = 0, off_tot = 0, off_succ = 0, off_gcache = 0;
   uint64_t total = 0;
@@ -345,23 +395,8 @@ gx_status make_plan(const Net& net, const gx_explore_opts* o, Plan& P) {
     while (P.regions < 16 && tbytes / P.regions > kAutoRegionBytes) P.regions *= 2;
   }
   if (P.regions > P.nb) P.regions = (uint32_t)P.nb;
-  // the caches of seen vectors: auto = the GPU-wide one in tables of at least 2^26 slots
-  // with one lane per bucket (where it was measured), for vectors whose fields fit one
-  // 64-bit key, else the per-warp one (2^9).  4-word vectors: only in one pass (1.08e8-state
-  // irregular network, 4 GiB: 42 ms with it, 50 ms without; the memory-filling product
-  // network in two passes, 8 GiB: 231 ms with it, 186 ms without)
-  uint32_t glog = o->global_cache_log2;
-  if (glog == kAutoCache)
-    glog = P.G == 1 && slots >= (1ull << 26) && (P.W <= 2 || P.regions == 1) ? auto_cache_log2(net) : 0;
-  else if (glog > 26) return fail(GX_ERR_INVALID, "global_cache_log2 must be at most 26");
-  if (glog && cache_layout(net, glog, P.seen)) {
-    P.gcache = 1ull << glog;
-    P.gcache_bytes = P.gcache << P.seen.log2_bytes;
-  }
-  // The per-warp one: more entries find more, but their shared memory costs CTAs and L1 (token
-  // ring of 13 nodes: 2^6 4.19 ms, 2^7 4.18, 2^8 4.24, 2^9 4.86; 1.7e7 states of 4 words in one
-  // pass: 8.83, 8.76, 9.13, 10.3; 3.4e8 of 4 words in four passes: 2^5 190, 2^6 186, 2^7 182)
-  P.warp_log2 = o->warp_cache_log2 == kAutoCache ? (P.gcache ? 0u : 7u) : o->warp_cache_log2;
+  const gx_status cs = plan_caches(net, *o, P.G, slots, P.regions, P.cache);
+  if (cs != GX_OK) return cs;
   P.cs = o->successor_buffer ? o->successor_buffer : std::min<uint64_t>(slots / 2, (1ull << 32) - 1);
   if (P.logp == 0) P.cs = 0;  // partitioned path off: no buffer
   if (P.cs >= (1ull << 32)) return fail(GX_ERR_INVALID, "successor_buffer must be below 2^32 vectors");
@@ -392,7 +427,7 @@ gx_status make_plan(const Net& net, const gx_explore_opts* o, Plan& P) {
   P.off_succ = off;
   off = align_up(off + 4ull * P.W * P.cs);
   P.off_gcache = off;
-  off = align_up(off + P.gcache_bytes);
+  off = align_up(off + P.cache.bytes);
   P.total = off;
   return GX_OK;
 }
@@ -474,7 +509,7 @@ gx_status build_loop_graph(gx_net* h, const Plan& P, Ctl* ctl, uint32_t* table, 
   const uint64_t words = (uint64_t)P.B * P.nb;
   constexpr uint64_t kPiece = 1ull << 30;  // words per memset node
   for (uint64_t w0 = 0; w0 < words; w0 += kPiece) GX_CUDA(add_memset(table + w0, std::min(kPiece, words - w0)));
-  if (eg.gcache.base) GX_CUDA(add_memset(eg.gcache.base, (P.gcache_bytes + 3) / 4));
+  if (eg.gcache.base) GX_CUDA(add_memset(eg.gcache.base, (P.cache.bytes + 3) / 4));
   auto add_kernel = [&](cudaGraph_t gr, const cudaGraphNode_t* deps, size_t nd, const void* fn, dim3 gd, dim3 bd,
                         size_t sh, void** args, cudaGraphNode_t* out) -> cudaError_t {
     cudaKernelNodeParams kp{};
@@ -609,12 +644,12 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
   // levels on the device unless asked otherwise; the partitioned path needs the host
   const bool device_loop = !o->host_loop && P.logp == 0;
   GX_CUDA(cudaEventRecord(ev0, st));
-  SeenCache gcache = P.seen;
-  gcache.base = P.gcache ? base + P.off_gcache : nullptr;
+  SeenCache gcache = P.cache.seen;
+  gcache.base = P.cache.entries ? base + P.off_gcache : nullptr;
   if (!device_loop) {
     GX_CUDA(cudaMemsetAsync(ctl, 0, sizeof(Ctl), st));
     GX_CUDA(cudaMemsetAsync(table, 0, 4ull * P.B * P.nb, st));
-    if (gcache.base) GX_CUDA(cudaMemsetAsync(gcache.base, 0, P.gcache_bytes, st));
+    if (gcache.base) GX_CUDA(cudaMemsetAsync(gcache.base, 0, P.cache.bytes, st));
   }
 
   InitArgs ia{};
@@ -653,34 +688,11 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
     ea.viol_buf = viol;
     ea.viol_cap = P.viol_cap;
   }
-  size_t fixed = 0;  // static shared memory of the level kernel
-  GX_CUDA(allow_smem(P.ks->expand_fn, dev.smem_optin, &fixed));
-  const size_t blob_bytes = 4ull * net.blob.size();
-  size_t cache_bytes = 0;
-  if ((s = warp_cache_layout(net, P.warp_log2, ea, cache_bytes)) != GX_OK) return s;
-  size_t smem = 8ull * kMaxRounds + cache_bytes;
-  if (fixed + smem > dev.smem_optin)
-    return fail(GX_ERR_INVALID, "warp cache of 2^" + std::to_string(ea.cache_log2) + " entries per warp needs " +
-                                    std::to_string(fixed + smem) +
-                                    " bytes of shared memory per CTA, more than " + std::to_string(dev.smem_optin));
-  // the network tables are staged unless they are large or leave no room for the cache
-  ea.stage = blob_bytes + 8ull * kMaxRounds <= 96 * 1024 &&
-                     fixed + smem + blob_bytes <= dev.smem_optin ? 1 : 0;
-  if (ea.stage) smem += blob_bytes;
-  int per_sm = 0;
-  GX_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, P.ks->expand_fn, kBlock, smem));
-  if (per_sm < 1) return fail(GX_ERR_INVALID, "expansion kernel does not fit on an SM");
-  // Shared memory beyond 196 KB an SM leaves the GPU-wide cache's lookups too little L1 to
-  // be in flight in (mid network, padded from 186 to 214 KB: 19 ms became 30 ms), so a
-  // network with large tables runs fewer CTAs.
-  int carveout = -1;  // (an attribute of the launches, not of the function)
-  if (gcache.base) {
-    const size_t cta = fixed + smem + 1024, most = 196 * 1024;
-    if (cta * per_sm > most) per_sm = std::max<int>(1, (int)(most / cta));
-    carveout = (int)std::min<size_t>(100, (cta * per_sm * 100 + 228 * 1024 - 1) / (228 * 1024));
-  }
-  if (o->ctas_per_sm) per_sm = std::min<int>(per_sm, (int)o->ctas_per_sm);
-  const uint64_t max_grid = (uint64_t)dev.sms * per_sm;
+  ExpandLaunch el;
+  if ((s = plan_expand(net, *o, *P.ks, P.cache.warp_log2, dev.smem_optin, ea, el)) != GX_OK) return s;
+  const size_t smem = el.smem, blob_bytes = 4ull * net.blob.size();
+  const int carveout = el.carveout;
+  const uint64_t max_grid = (uint64_t)dev.sms * el.per_sm;
 
   std::vector<uint64_t> levels{1};
   uint64_t cur_begin = 0, cur_end = 1, explored = 0;
@@ -909,7 +921,7 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
   S.expand_launches = launches;
   S.kernel_launches = kernel_launches + (launches - dev_expand);
   S.region_passes = P.regions;
-  S.global_cache_entries = P.gcache;
+  S.global_cache_entries = P.cache.entries;
   S.device_levels = device_levels;
   S.probes = hc->probes;
   S.partitioned_levels = part_levels;

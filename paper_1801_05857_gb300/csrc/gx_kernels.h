@@ -186,15 +186,26 @@ cudaError_t launch_digest(int W, const DigestArgs& a, int grid, cudaStream_t st)
 // Hash-constant multipliers: odd 64-bit values drawn from splitmix64.
 void hash_multipliers(uint64_t* out, int n);
 
-// Layout of a GPU-wide cache of 2^log2_entries entries for a network's vectors;
-// false when they have no 64-bit key.  And the entries of the automatic one (0:
-// none).
-bool cache_layout(const Net& net, uint32_t log2_entries, SeenCache& c);
-uint32_t auto_cache_log2(const Net& net);
+// The caches of seen vectors of a search, as its options and its table decide
+// (gx_explore_opts): for every entry point that runs the level kernel.
+struct CachePlan {
+  uint64_t entries = 0;   // of the GPU-wide one (0 = off), and its bytes
+  uint64_t bytes = 0;
+  SeenCache seen{};       // its layout (base left out)
+  uint32_t warp_log2 = 0; // per-warp one: 2^warp_log2 entries (0 = off)
+};
+gx_status plan_caches(const Net& net, const gx_explore_opts& o, int lanes, uint64_t slots, uint32_t regions,
+                      CachePlan& p);
 
-// Per-warp cache of 2^warp_log2 entries (gx_explore_opts.warp_cache_log2): fills in
-// a's and the bytes it takes in a CTA.  GX_ERR_INVALID above 2^12.
-gx_status warp_cache_layout(const Net& net, uint32_t warp_log2, ExpandArgs& a, size_t& bytes);
+// How the level kernel is launched: the shared memory of a CTA, CTAs per SM and the
+// split with the L1.  Fills in a's stage and per-warp cache; a's gcache must be set.
+struct ExpandLaunch {
+  size_t smem = 0;
+  int per_sm = 0;
+  int carveout = -1;  // percent of shared memory, -1: default
+};
+gx_status plan_expand(const Net& net, const gx_explore_opts& o, const KernelSet& ks, uint32_t warp_log2,
+                      size_t smem_optin, ExpandArgs& a, ExpandLaunch& l);
 
 // GX_DL_GUIDED search (gx_guided.cu).
 gx_status run_guided(gx_net* h, const gx_explore_opts* opts, void* ws, uint64_t ws_bytes, cudaStream_t st);

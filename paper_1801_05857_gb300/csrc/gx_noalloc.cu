@@ -105,24 +105,16 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
   const uint64_t fwant = o->frontier_states ? o->frontier_states : std::max<uint64_t>(4096, slots / 4);
   uint64_t fcap = 1;
   while (fcap < fwant) fcap *= 2;
-  // caches of seen vectors, as gx_explore chooses them (gx_explore_opts)
-  uint32_t glog = o->global_cache_log2;
-  if (glog == 0xFFFFFFFFu)
-    glog = G == 1 && slots >= (1ull << 26) && (W <= 2 || regions == 1) ? gx::auto_cache_log2(net) : 0;
-  else if (glog > 26) return gx::fail(GX_ERR_INVALID, "global_cache_log2 must be at most 26");
-  gx::SeenCache gcache{};
-  uint64_t gentries = 0;
-  if (glog && gx::cache_layout(net, glog, gcache)) gentries = 1ull << glog;
-  const uint64_t gcache_bytes = gentries << gcache.log2_bytes;
   if (regions > nb) regions = (uint32_t)nb;
-  const uint32_t warp_log2 =
-      o->warp_cache_log2 == 0xFFFFFFFFu ? (gentries ? 0u : W == 4 && regions > 1 ? 6u : 7u) : o->warp_cache_log2;
+  gx::CachePlan cache;
+  gx_status s = gx::plan_caches(net, *o, G, slots, regions, cache);
+  if (s != GX_OK) return s;
   const uint64_t off_ctl = 0;
   const uint64_t off_blob = align256(sizeof(gx::Ctl));
   const uint64_t off_front = align256(off_blob + 4ull * net.blob.size());
   const uint64_t off_table = align256(off_front + 4ull * W * fcap);
   const uint64_t off_gcache = align256(off_table + 4ull * B * nb);
-  const uint64_t total = align256(off_gcache + gcache_bytes);
+  const uint64_t total = align256(off_gcache + cache.bytes);
   if (total > kScratchBytes)
     return gx::fail(GX_ERR_INVALID, "gx_explore_noalloc needs " + std::to_string(total) +
                                         " bytes of scratch but its static array holds " +
@@ -130,7 +122,7 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
                                         "; lower table_bytes / frontier_states or use gx_explore");
 
   unsigned char* base = nullptr;
-  gx_status s = scratch_for_current_device(base);
+  s = scratch_for_current_device(base);
   if (s != GX_OK) return s;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int dev = 0, sms = 0, smem_optin = 0;
@@ -147,10 +139,9 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
   NA_CUDA(cudaMemcpyAsync(blob, net.blob.data(), 4 * net.blob.size(), cudaMemcpyHostToDevice, st));
   NA_CUDA(cudaMemsetAsync(ctl, 0, sizeof(gx::Ctl), st));
   NA_CUDA(cudaMemsetAsync(table, 0, 4ull * B * nb, st));
-  if (gentries) {
-    gcache.base = base + off_gcache;
-    NA_CUDA(cudaMemsetAsync(gcache.base, 0, gcache_bytes, st));
-  }
+  gx::SeenCache gcache = cache.seen;
+  gcache.base = cache.entries ? base + off_gcache : nullptr;
+  if (gcache.base) NA_CUDA(cudaMemsetAsync(gcache.base, 0, cache.bytes, st));
 
   int log2nb = 0;
   while ((1ull << log2nb) < nb) ++log2nb;
@@ -191,26 +182,9 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
     ea.viol_buf = nullptr;
     ea.viol_cap = 0;
   }
-  // shared memory: the same rules as gx_explore
-  size_t fixed = 0;  // static shared memory of the level kernel
-  NA_CUDA(gx::allow_smem(ks->expand_fn, (size_t)smem_optin, &fixed));
-  const size_t blob_bytes = 4ull * net.blob.size();
-  size_t cache_bytes = 0;
-  if ((s = gx::warp_cache_layout(net, warp_log2, ea, cache_bytes)) != GX_OK) return s;
-  size_t smem = 8ull * gx::kMaxRounds + cache_bytes;
-  if (fixed + smem > (size_t)smem_optin)
-    return gx::fail(GX_ERR_INVALID, "warp cache of 2^" + std::to_string(ea.cache_log2) +
-                                        " entries per warp needs " + std::to_string(fixed + smem) +
-                                        " bytes of shared memory per CTA, more than " +
-                                        std::to_string(smem_optin));
-  ea.stage = blob_bytes + 8ull * gx::kMaxRounds <= 96 * 1024 &&
-                     fixed + smem + blob_bytes <= (size_t)smem_optin ? 1 : 0;
-  if (ea.stage) smem += blob_bytes;
-  int per_sm = 0;
-  NA_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ks->expand_fn, gx::kBlock, smem));
-  if (per_sm < 1) return gx::fail(GX_ERR_INVALID, "expansion kernel does not fit on an SM");
-  if (o->ctas_per_sm) per_sm = std::min<int>(per_sm, (int)o->ctas_per_sm);
-  const uint64_t max_grid = (uint64_t)sms * per_sm;
+  gx::ExpandLaunch el;
+  if ((s = gx::plan_expand(net, *o, *ks, cache.warp_log2, (size_t)smem_optin, ea, el)) != GX_OK) return s;
+  const uint64_t max_grid = (uint64_t)sms * el.per_sm;
 
   gx::Ctl hc;  // pageable copy of the control block
   uint64_t cur_begin = 0, cur_end = 1, explored = 0, launches = 0;
@@ -231,7 +205,7 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
       eq.region_bits = (uint64_t)q << (log2nb - log2r);
       eq.count_states = q == 0 ? 1 : 0;
       NA_CUDA(cudaMemsetAsync(&ctl->claim, 0, sizeof(unsigned long long), st));
-      NA_CUDA(ks->expand(eq, grid, smem, -1, st));
+      NA_CUDA(ks->expand(eq, grid, el.smem, el.carveout, st));
     }
     NA_CUDA(cudaMemcpyAsync(&hc, ctl, sizeof(gx::Ctl), cudaMemcpyDeviceToHost, st));
     NA_CUDA(cudaStreamSynchronize(st));
@@ -279,7 +253,7 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
   S2.fill = (double)S2.states / (double)slots;
   S2.expand_launches = launches * regions;
   S2.region_passes = regions;
-  S2.global_cache_entries = gentries;
+  S2.global_cache_entries = cache.entries;
   S2.probes = hc.probes;
   S2.h2d_bytes = 4ull * net.blob.size();
   S2.d2h_bytes = sizeof(gx::Ctl) * launches;

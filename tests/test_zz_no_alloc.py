@@ -112,3 +112,20 @@ def test_noalloc_rejects_what_it_cannot_do(cuda):
     # still usable afterwards
     s, lv = gx.explore_noalloc(h, gx.default_opts(table_bytes=1 << 20))
     assert s["states"] == 2 * 6 * 3 ** 5 and sum(lv) == s["states"]
+
+
+@pytest.mark.parametrize("passes", [1, 2, 4])
+def test_noalloc_chooses_the_caches_that_explore_chooses(cuda, passes):
+    """The automatic per-warp cache of 4-word vectors is the same with and without region passes
+    as in gx_explore: the same share of the successors needs a bucket read.  (One CTA per SM, so
+    that levels fill the warps; which warp takes which state moves the count by under 0.5 %.)"""
+    net = inputs.product_network(1, 16, 16, [2] * 12 + [3] * 4)
+    h = gx.load_network(net)
+    o = gx.default_opts(table_bytes=1 << 25, bucket_words=8, group_lanes=1, hash_rounds=64, region_passes=passes,
+                        host_loop=1, ctas_per_sm=1, frontier_states=1 << 20)
+    ws = gx.alloc_workspace(h, o)
+    gx.explore(h, o, ws)
+    want = gx.stats(h)
+    got, _ = gx.explore_noalloc(h, o)
+    assert got["states"] == want["states"] and want["probes"] < 0.85 * want["transitions"]
+    assert abs(got["probes"] - want["probes"]) <= 0.015 * want["probes"]
