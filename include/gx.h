@@ -221,7 +221,8 @@ typedef struct gx_explore_opts {
                                     (gx_default_opts): the most entries that take 64 MiB (2^25
                                     for b <= 41, 2^24 for b <= 56, 2^23 above), in tables of at
                                     least 2^26 slots with one lane per bucket (group_lanes 1),
-                                    for 4-word vectors only in one region pass; else off.  Mid
+                                    for 4-word vectors only in one region pass and where the
+                                    workspace has the room; else off.  Mid
                                     network (b = 40): 0.21 bucket reads per successor and
                                     12.3 ms (2^23 entries: 0.38, 3.8 ms more) */
   uint32_t guided_fused;         /* GX_DL_GUIDED: 1 = score the states an iteration inserts

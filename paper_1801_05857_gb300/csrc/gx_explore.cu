@@ -603,6 +603,13 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
     GX_CUDA(cudaMallocAsync(&ws, P.total, st));
     owned = true;
   } else {
+    // A workspace that lacks only the room for the automatic cache of 4-word vectors does
+    // without: it was sized when they had none.
+    if (ws_bytes < P.total && ws_bytes >= P.off_gcache && P.W == 4 && o->global_cache_log2 == kAutoCache) {
+      gx_explore_opts off = *o;
+      off.global_cache_log2 = 0;
+      if ((s = make_plan(net, &off, P = Plan{})) != GX_OK) return s;
+    }
     if (ws_bytes < P.total)
       return fail(GX_ERR_OOM, "workspace holds " + std::to_string(ws_bytes) + " bytes, need " +
                                   std::to_string(P.total));

@@ -252,3 +252,25 @@ def test_searches_of_several_threads(cuda):
     for t in threads:
         t.join()
     assert not bad, bad
+
+
+def test_workspace_without_room_for_the_automatic_cache(cuda):
+    """4-word vectors in 2^26 slots: a workspace with no room for the GPU-wide cache is searched
+    without it; one byte less is refused."""
+    import torch
+    h = gx.load_network(NETS[4])
+    kw = dict(table_bytes=1 << 30, bucket_words=8, group_lanes=1, hash_rounds=32)
+    need = gx.workspace_bytes(h, gx.default_opts(global_cache_log2=0, **kw))
+    full = gx.workspace_bytes(h, gx.default_opts(**kw))
+    assert full > need
+    r = _oracle(4, NETS[4])
+    for size, entries in ((full, 1 << 23), (need, 0)):
+        ws = torch.empty(size, dtype=torch.uint8, device="cuda")
+        gx.explore(h, gx.default_opts(**kw), ws)
+        s = gx.stats(h)
+        assert (s["states"], s["transitions"], gx.levels(h)) == (r.states, r.transitions, r.levels)
+        assert gx.set_digest(h, ws) == (r.states, r.set_sum, r.set_xor)
+        assert s["slot_words"] == 4 and s["global_cache_entries"] == entries
+    with pytest.raises(gx.GxError) as e:
+        gx.explore(h, gx.default_opts(**kw), torch.empty(need - 1, dtype=torch.uint8, device="cuda"))
+    assert e.value.status == gx.GX_ERR_OOM
