@@ -289,7 +289,9 @@ typedef struct gx_stats_t {
   double fill;              /* states / table_slots */
   double gpu_ms;            /* device time of the search (CUDA events around it) */
   double expand_ms;         /* summed device time of the level-expansion kernels */
-  uint64_t expand_launches; /* level-expansion kernel launches */
+  uint64_t expand_launches; /* level expansions, one per region pass (guided: iterations).
+                               Each is a launch, except that in the device-driven loop the
+                               expansions of levels of few states share launches */
   uint64_t probes;          /* buckets read by find-or-put during the search */
   uint64_t h2d_bytes;       /* host-to-device bytes the search copied (network tables) */
   uint64_t d2h_bytes;       /* device-to-host bytes it copied (progress, deadlock states) */
@@ -298,10 +300,10 @@ typedef struct gx_stats_t {
   uint64_t violation_sum;   /* order-free digest of the violation set, as for deadlocks */
   uint64_t violation_xor;
   int64_t first_violation_level; /* -1 if none */
-  uint64_t kernel_launches; /* kernels the search launched (initialisation, expansion,
-                               level-advance steps).  In the device-driven loop the expansion
-                               and the advance step of a level of few states run inside one
-                               launch for many levels; each is counted as one here */
+  uint64_t kernel_launches; /* steps of a breadth-first search (initialisation, expansions,
+                               level-advance steps).  Launches are fewer in the device-driven
+                               loop, where those of levels of few states share one:
+                               gx_launch_count */
   uint64_t device_levels;   /* levels expanded by the device-driven loop */
   uint64_t global_cache_entries; /* entries of the GPU-wide cache used (0 = not used) */
 } gx_stats_t;
@@ -309,6 +311,10 @@ typedef struct gx_stats_t {
 /* Copy the statistics of the last search on `net` into *out (host memory).
  * GX_ERR_STATE if no search has run on it yet.  Host-only. */
 gx_status gx_stats(const gx_net* net, gx_stats_t* out);
+
+/* Kernels that the last breadth-first search on `net` launched (0 after a guided one):
+ * every launch counted once, however many levels of few states it expands.  Host-only. */
+gx_status gx_launch_count(const gx_net* net, uint64_t* n);
 
 /* Level sizes of the last search: out[k] = number of states at BFS depth k.
  * Writes min(cap, n_levels) entries; *n_levels gets the total. */

@@ -180,6 +180,7 @@ __global__ void level_advance_kernel(const gx::LoopArgs L) {
   const bool more = s.advance(L, e, c.probes, c.transitions);
   s.store(c);
   c.claim = 0;
+  c.large_levels += 1;
   // back to the small-level kernel once a level is well below its limit
   const bool small = s.cur_end - s.cur_begin <= kSmallLevel / 2;
   cudaGraphSetConditional(L.cond, more ? 1u : 0u);
@@ -712,6 +713,7 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
   std::vector<uint64_t> lv_probes, lv_trans;
   uint64_t prev_probes = 0, prev_trans = 0;
   bool complete = false, finished = false;
+  uint64_t launched = 0;  // by the device-driven loop, each launch counted once
   uint64_t kernel_launches = device_loop ? 0 : 1, device_levels = 0, d2h_loop = 0, dev_expand = 0;
   if (device_loop) {
     LoopArgs la{};
@@ -766,6 +768,7 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
     dev_expand = launches;
     device_levels = nd;
     kernel_launches = 2 + (P.regions + 1) * nd;  // init, start, then the passes + advance step per level
+    launched = 2 + hc->small_launches + (uint64_t)(P.regions + 1) * hc->large_levels;
     first_dl = hc->first_dl;
     first_viol = hc->first_viol;
     complete = hc->complete != 0;
@@ -927,6 +930,7 @@ gx_status run_search(gx_net* h, const gx_explore_opts* opts, bool stop_first, vo
   S.expand_ms = expand_ms;
   S.expand_launches = launches;
   S.kernel_launches = kernel_launches + (launches - dev_expand);
+  h->launches = device_loop ? launched + (launches - dev_expand) : S.kernel_launches;
   S.region_passes = P.regions;
   S.global_cache_entries = P.cache.entries;
   S.device_levels = device_levels;
@@ -1002,6 +1006,14 @@ gx_status gx_stats(const gx_net* h, gx_stats_t* out) {
   if (!h || !out) return gx::fail(GX_ERR_INVALID, "net or out is NULL");
   if (!h->have_result) return gx::fail(GX_ERR_STATE, "no search has run on this network");
   *out = h->stats;
+  return GX_OK;
+}
+
+gx_status gx_launch_count(const gx_net* h, uint64_t* n) {
+  gx::clear_error();
+  if (!h || !n) return gx::fail(GX_ERR_INVALID, "net or n is NULL");
+  if (!h->have_result) return gx::fail(GX_ERR_STATE, "no search has run on this network");
+  *n = h->launches;
   return GX_OK;
 }
 

@@ -1627,6 +1627,7 @@ gx_status run_guided(gx_net* h, const gx_explore_opts* opts, void* ws, uint64_t 
     for (const auto& st2 : path) h->guided_trace.insert(h->guided_trace.end(), st2.begin(), st2.end());
     h->deadlocks = path.back();
   }
+  h->launches = 0;
   gx_stats_t& S = h->stats;
   std::memset(&S, 0, sizeof(S));
   S.states = hc.inserted;

@@ -93,6 +93,7 @@ struct gx_net {
   gx::Net net;
   bool have_result = false;
   gx_stats_t stats{};
+  uint64_t launches = 0;  // kernels the last breadth-first search launched (gx_launch_count)
   std::vector<uint64_t> levels;
   // per expanded level: device time, buckets read, transitions
   std::vector<double> level_ms;

@@ -1142,6 +1142,7 @@ __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThrea
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     ls.store(c);
     c.claim = 0;
+    c.small_launches += 1;
     cudaGraphSetConditional(LA.cond, more ? 1u : 0u);
     cudaGraphSetConditional(LA.cond_big, more ? 1u : 0u);
   }

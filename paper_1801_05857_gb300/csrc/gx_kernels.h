@@ -33,6 +33,7 @@ struct Ctl {
   unsigned long long t_prev;        // %globaltimer (ns) at the end of the previous level
   long long first_dl, first_viol;   // level of the first deadlock / violation, -1 if none
   unsigned int complete, yielded;   // the frontier ran empty / the level arrays filled up
+  unsigned int small_launches, large_levels;  // launches of the few-state kernel; levels beside it
 };
 static_assert(sizeof(Ctl) <= 256, "control block");
 

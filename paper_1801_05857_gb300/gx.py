@@ -138,6 +138,7 @@ def lib(build_if_missing: bool = True) -> ctypes.CDLL:
         "gx_find_deadlocks": ([vp, P(gx_explore_opts), u32, vp, u64, vp, P(u32), u32, P(u64)],
                               ctypes.c_int),
         "gx_stats": ([vp, P(gx_stats_t)], ctypes.c_int),
+        "gx_launch_count": ([vp, P(u64)], ctypes.c_int),
         "gx_levels": ([vp, P(u64), u32, P(u32)], ctypes.c_int),
         "gx_deadlocks": ([vp, P(u32), u32, P(u32)], ctypes.c_int),
         "gx_violations": ([vp, P(u32), u32, P(u32)], ctypes.c_int),
@@ -354,6 +355,12 @@ def stats(net: Net) -> dict:
     s = gx_stats_t()
     _check(lib().gx_stats(net.handle, ctypes.byref(s)))
     return _stats_dict(s)
+
+
+def launch_count(net: Net) -> int:
+    n = u64()
+    _check(lib().gx_launch_count(net.handle, ctypes.byref(n)))
+    return n.value
 
 
 def levels(net: Net) -> list:

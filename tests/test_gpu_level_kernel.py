@@ -274,3 +274,28 @@ def test_workspace_without_room_for_the_automatic_cache(cuda):
     with pytest.raises(gx.GxError) as e:
         gx.explore(h, gx.default_opts(**kw), torch.empty(need - 1, dtype=torch.uint8, device="cuda"))
     assert e.value.status == gx.GX_ERR_OOM
+
+
+@pytest.mark.parametrize("passes", [1, 2])
+@pytest.mark.parametrize("net", [inputs.workload("tiny"), inputs.token_ring(8), NETS[4]], ids=lambda n: n.name or "net")
+def test_launch_count_counts_a_launch_once(cuda, net, passes):
+    """The few-state kernel is launched at the start and whenever a level falls to 256 states, and
+    takes levels of up to 512; every other level is an expansion per region pass and an advance
+    step.  With levels driven by the host each expansion is a launch."""
+    h = gx.load_network(net)
+    o = gx.default_opts(table_bytes=1 << 24, hash_rounds=32, region_passes=passes)
+    gx.explore(h, o, gx.alloc_workspace(h, o))
+    sizes, n, i = gx.levels(h), 2, 0  # initialisation, start
+    while i < len(sizes):
+        n += 1
+        while i < len(sizes) and sizes[i] <= 512:
+            i += 1
+        while i < len(sizes):
+            n += passes + 1
+            i += 1
+            if i < len(sizes) and sizes[i] <= 256:
+                break
+    assert gx.launch_count(h) == n
+    o = gx.default_opts(table_bytes=1 << 24, hash_rounds=32, region_passes=passes, host_loop=1)
+    gx.explore(h, o, gx.alloc_workspace(h, o))
+    assert gx.launch_count(h) == 1 + passes * len(sizes)
