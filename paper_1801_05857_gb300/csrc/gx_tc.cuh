@@ -453,9 +453,11 @@ __device__ __forceinline__ void score_pack_item(const float* __restrict__ p, Sco
   }
   const int k = item - kTcPackItems;
   const float b = p[kHid * kIn + kHid + kHid * kHid + k];
-  const float hi = __bfloat162float(__float2bfloat16_rn(b));
+  // (parts rounded towards zero: to nearest, a finite bias next to the largest would become
+  // infinite minus infinite)
+  const float hi = __bfloat162float(__float2bfloat16_rz(b));
   const float r1 = isfinite(b) ? b - hi : 0.f;
-  const float mid = __bfloat162float(__float2bfloat16_rn(r1));
+  const float mid = __bfloat162float(__float2bfloat16_rz(r1));
   *reinterpret_cast<uint4*>(out->b2m + core_offset(k, 0, 2)) = make_uint4(pack_bf16x2(hi, mid), pack_bf16x2(r1 - mid, 0.f), 0u, 0u);
   *reinterpret_cast<uint4*>(out->b2m + core_offset(k, 8, 2)) = make_uint4(0u, 0u, 0u, 0u);
 }

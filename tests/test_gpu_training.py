@@ -104,3 +104,36 @@ def test_every_step_is_an_adam_step_at_the_weights_before_it(cuda, batch):
         assert (np.abs(got - (p - move)) <= 20 * 2.0 ** -24 * np.abs(move) + 2.0 ** -23 * np.abs(p) + 1e-12).all()
         assert np.abs(got - p).max() > 0.1 * lr
         before = after
+
+
+def test_scores_with_extreme_biases(cuda):
+    """Second-layer biases up to the largest floats (their three BF16 parts must stay finite),
+    down to 1e-37, infinite and NaN: the scores are those of the network with the bias added
+    to a unit's sum.  w3 scales each unit's part to about 1, exactly (a power of two)."""
+    import torch
+    hist, _, p = _data(300, 2)
+    W1, b1, W2, b2, w3, b3 = omlp.unpack(p.cpu().numpy())
+    big = float(np.finfo(np.float32).max)
+    for bias in (big, np.nextafter(np.float32(big), np.float32(0)), 3.3895e38, 3.39e38, 1e38, -big, 1.0, 1 / 3, 1e-30,
+                 -1e-37, np.inf, -np.inf, np.nan):
+        q = p.cpu().numpy().copy()
+        b2at = 128 * 16 + 128 + 128 * 128
+        q[b2at:b2at + 128] = 0
+        q[b2at + 5] = bias
+        q[b2at + 128:b2at + 256] = 0
+        scale = 2.0 ** -int(np.floor(np.log2(abs(bias)))) if np.isfinite(bias) else 1.0
+        q[b2at + 128 + 5] = min(max(scale, 2.0 ** -126), 2.0 ** 120)
+        y = gx.mlp_forward(torch.from_numpy(q).cuda(), torch.from_numpy(hist).cuda()).cpu().numpy().astype(np.float64)
+        with np.errstate(invalid="ignore"):
+            want = omlp.forward(q, hist)
+        if np.isnan(bias):
+            continue  # (max(NaN, 0) is the hardware's choice; it must only not hang or poison others)
+        if np.isinf(bias):
+            assert (y == want).all()
+            continue
+        assert np.isfinite(y).all(), bias
+        # (a hidden value of up to 1 may round to the other BF16 neighbour, 2^-9 away: times a weight
+        # of at most 128 ** -0.5 and w3 of up to 4, 7e-4)
+        assert (np.abs(y - want) <= 1e-3 * np.maximum(1, np.abs(want))).all(), bias
+    y0 = gx.mlp_forward(p, torch.from_numpy(hist).cuda()).cpu().numpy()
+    assert np.isfinite(y0).all()
