@@ -602,7 +602,8 @@ def guided_part(torch, gx, inputs, guide) -> dict:
             torch.cuda.empty_cache()
 
     # five seeds per size; BFS in a 24 GiB table up to 14 processes and a 128 GiB one at 16
-    rows, summary = [], []
+    # (only the medians are returned: with every run's record the bench's one line was 33 KB)
+    summary = []
     for n, k in ((12, 2), (13, 2), (14, 2), (16, 3)):
         per = []
         for seed in range(5):
@@ -614,7 +615,6 @@ def guided_part(torch, gx, inputs, guide) -> dict:
             per.append({"network": net.name, "guided_runs": runs, "fused_runs": fused_runs,
                         "untrained": guided(net, untrained),
                         "bfs": bfs(net, 24 if n <= 14 else 128)})
-        rows.extend(per)
 
         def med(vals):
             v = sorted(vals)
@@ -640,7 +640,7 @@ def guided_part(torch, gx, inputs, guide) -> dict:
                       "ms_per_adam_step": round((t2 - t1) * 1e3 / 4000, 4), "batch": 1024,
                       "loss_first": round(float(lo[:10].mean()), 4), "loss_last": round(float(lo[-50:].mean()), 4)},
             "scoring": scoring_rate(torch, gx, params),
-            "summary": summary, "instances": rows}
+            "summary": summary}
 
 
 def scoring_rate(torch, gx, params, n=1 << 22) -> dict:

@@ -59,3 +59,40 @@ def test_traffic_captures_match_the_kernel_code():
         with open(path, "w") as f:
             f.write("int a = 1;\nint b = 3;\n")
         assert bench.kernel_code_digest([rel]) != base
+
+
+def test_guided_part_adds_a_summary_not_every_run():
+    """The bench prints one line, which must stay short enough to be read back: 200 guided
+    searches, 20 breadth-first ones and their networks add no more than their medians (on
+    stand-ins for the GPU library and torch)."""
+    from types import SimpleNamespace as NS
+
+    import numpy as np
+    bench = _bench_module()
+    runs = []
+
+    class Array(list):
+        def cpu(self):
+            return self
+
+        def numpy(self):
+            return np.array(self)
+
+    def stats(_):
+        return {"explored": 164441 + len(runs), "states": 2730458, "gpu_ms": 1.921, "expand_launches": 33,
+                "first_deadlock_level": 32, "fill": 0.7561, "n_levels": 19}
+
+    gx = NS(load_network=lambda n: n, guided_set_weights=lambda h, p: None, default_opts=lambda **k: k,
+            guided_alloc_workspace=lambda h, o: None, alloc_workspace=lambda h, o: None, GX_DL_GUIDED=2, GX_DL_BFS_FIRST=0,
+            find_deadlocks=lambda *a: runs.append(a) or (1, None), stats=stats, guided_trace=lambda h: [0] * 33,
+            GxError=RuntimeError, MLP_PARAMS=1, mlp_init=lambda p, s: None, mlp_forward=lambda p, h: None)
+    event = NS(record=lambda s: None, elapsed_time=lambda o: 2.0)
+    torch = NS(cuda=NS(synchronize=lambda: None, empty_cache=lambda: None, current_stream=lambda: None,
+                       Event=lambda enable_timing: event),
+               empty=lambda *a, **k: None, randint=lambda *a, **k: None, float32=0, uint8=0)
+    guide = NS(collect_examples=lambda nets, d: (np.zeros((5, 16)), None), train=lambda h, l, steps, lr: (None, Array([0.1] * 99)))
+    inputs = NS(planted_network=lambda seed, n, n_traps=1: NS(name=f"planted_s{seed}_n{n}_k{n_traps}"))
+    part = bench.guided_part(torch, gx, inputs, guide)
+    assert len(runs) == 4 * 5 * (5 + 5 + 1 + 1)
+    assert [s["guided_found"] for s in part["summary"]] == [25] * 4 and part["summary"][0]["bfs_median_ms"] == 1.921
+    assert len(json.dumps(part)) < 4096
