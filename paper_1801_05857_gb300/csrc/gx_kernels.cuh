@@ -1367,46 +1367,22 @@ __global__ void init_kernel(const gx::InitArgs a) {
   }
 }
 
-// Sec. 5.1: find-or-put of a warp's keys, a key per lane.
-// G == 1: key after key (find_or_put).  Bound by random 128-byte lines read and written back; a lane
-// that took its next key while others of its warp read further buckets made it no
-// faster (1.5e8 keys, 1e8 of them new, 8-word buckets: 4.75 ms, with that 4.92).
-struct LaneFop {
-  unsigned long long ins = 0, fnd = 0, fail = 0;
-  __device__ __forceinline__ void count(const gx::FopArgs& a, uint64_t i, int r) {
-    if (a.result) a.result[i] = (uint8_t)(r == FOP_INSERTED ? 1 : (r == FOP_FOUND ? 0 : 2));
-    ins += r == FOP_INSERTED;
-    fnd += r == FOP_FOUND;
-    fail += r != FOP_INSERTED && r != FOP_FOUND;
-  }
-};
-// The same with a group of lanes per key where a lane's part of the bucket is 64 bytes
-// or more (32-word buckets, 2 lanes: 25-50 G keys/s by duplication, 23-35 with fop_groups).
-template <int W, int B, int G>
-__device__ __forceinline__ void fop_lanes(const gx::FopArgs& a, const uint64_t* muls, LaneFop& n) {
-  const Group<G> g;
-  const uint64_t step = (uint64_t)gridDim.x * blockDim.x / G;
-  uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
-  uint32_t probes = 0;
-  // the loop bound is uniform per warp: all groups of a warp leave together
-  const uint64_t warp_first = ((uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u)) / G;
-  for (uint64_t wi = warp_first; wi < a.n; wi += step, i += step) {
-    if (i < a.n) {
-      uint32_t v[W];
-#pragma unroll
-      for (int w = 0; w < W; ++w) v[w] = a.keys[i * W + w] | kTag;
-      const int r = find_or_put<W, B, G>(a.table, a.log2nb, a.rounds, muls, v, g, probes);
-      if (g.glane == 0) n.count(a, i, r);
-    }
-  }
+// Sec. 5.1: key i of the sequence has result r.
+__device__ __forceinline__ void fop_count(const gx::FopArgs& a, uint64_t i, int r, unsigned long long& ins,
+                                          unsigned long long& fnd, unsigned long long& fail) {
+  if (a.result) a.result[i] = (uint8_t)(r == FOP_INSERTED ? 1 : (r == FOP_FOUND ? 0 : 2));
+  ins += r == FOP_INSERTED;
+  fnd += r == FOP_FOUND;
+  fail += r == FOP_FULL;
 }
 
-// Otherwise the lanes read their buckets together (bucket_step_lanes), so a lane that is
-// done takes its next key at once.  (With a group of lanes per key, which voted on every
+// The lanes of a warp take their own keys and read their buckets together
+// (bucket_step_lanes), so a lane that is done takes its next key at once.  (With a group of lanes per key, which voted on every
 // bucket, the same keys took 10.5 ms with a lane per slot of 8-word buckets, 22.6 of
 // 32-word ones; now 4.8 and 5.6.)
 template <int W, int B, int G>
-__device__ __forceinline__ void fop_groups(const gx::FopArgs& a, const uint64_t* muls, LaneFop& n) {
+__device__ __forceinline__ void fop_groups(const gx::FopArgs& a, const uint64_t* muls, unsigned long long& ins,
+                                           unsigned long long& fnd, unsigned long long& fail) {
   const uint32_t lane = threadIdx.x & 31, below = (1u << lane) - 1u;
   // the warp's keys: consecutive ones, of which 64 are held (base.., pos of them taken)
   const uint64_t warps = (uint64_t)gridDim.x * (blockDim.x / 32);
@@ -1455,24 +1431,49 @@ __device__ __forceinline__ void fop_groups(const gx::FopArgs& a, const uint64_t*
     if (!__any_sync(FULLMASK, has)) break;
     const int r = bucket_step_lanes<W, B, G>(a.table, has, seq_bucket<B>(h, k, muls, a.log2nb), v);
     if (has && (r >= 0 || ++k == (uint32_t)a.rounds)) {
-      n.count(a, at, r);
+      fop_count(a, at, r >= 0 ? r : FOP_FULL, ins, fnd, fail);
       has = false;
     }
   }
 }
 
+// A key per lane (G == 1), or per group of lanes where a lane's part of the bucket is 64 bytes
+// or more (32-word buckets, 2 lanes: 25-50 G keys/s by duplication, 23-35 with fop_groups),
+// key after key.  Bound by random 128-byte lines read and written back; a lane that took its
+// next key while others of its warp read further buckets made it no faster (1.5e8 keys, 1e8
+// of them new, 8-word buckets, G = 1: 4.75 ms, with that 4.92).  The loop stands here and
+// not in a function: as one it took 46 registers for <2, 32, 2> instead of 40, a CTA an SM
+// less (2e7 keys, each five times: 0.57 ms instead of 0.54).
 template <int W, int B, int G>
 __global__ void __launch_bounds__(gx::kBlock) fop_kernel(const gx::FopArgs a) {
   __shared__ uint64_t muls[kMaxRounds];
   for (int i = threadIdx.x; i < a.rounds; i += blockDim.x) muls[i] = a.muls.m[i];
   __syncthreads();
-  LaneFop n;
-  if constexpr (B / G >= 16 || G == 1) fop_lanes<W, B, G>(a, muls, n);
-  else fop_groups<W, B, G>(a, muls, n);
-  const unsigned long long ins = warp_sum((unsigned long long)n.ins);
-  const unsigned long long fnd = warp_sum((unsigned long long)n.fnd);
-  const unsigned long long fail = warp_sum((unsigned long long)n.fail);
-  if ((threadIdx.x & 31) == 0) {
+  const int lane = threadIdx.x & 31;
+  unsigned long long ins = 0, fnd = 0, fail = 0;
+  if constexpr (G == 1 || B / G >= 16) {
+    const Group<G> g;
+    const uint64_t groups = (uint64_t)gridDim.x * blockDim.x / G;
+    uint64_t i = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) / G;
+    uint32_t probes = 0;
+    // the loop bound is uniform per warp: all groups of a warp leave together
+    const uint64_t warp_first = ((uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u)) / G;
+    for (uint64_t wi = warp_first; wi < a.n; wi += groups, i += groups) {
+      if (i < a.n) {
+        uint32_t v[W];
+#pragma unroll
+        for (int w = 0; w < W; ++w) v[w] = a.keys[i * W + w] | kTag;
+        const int r = find_or_put<W, B, G>(a.table, a.log2nb, a.rounds, muls, v, g, probes);
+        if (g.glane == 0) fop_count(a, i, r, ins, fnd, fail);
+      }
+    }
+  } else {
+    fop_groups<W, B, G>(a, muls, ins, fnd, fail);
+  }
+  ins = warp_sum(ins);
+  fnd = warp_sum(fnd);
+  fail = warp_sum(fail);
+  if (lane == 0) {
     if (ins) atomicAdd(&a.counters[0], ins);
     if (fnd) atomicAdd(&a.counters[1], fnd);
     if (fail) atomicAdd(&a.counters[2], fail);

@@ -2,6 +2,7 @@
 // Sec. 4.1 compares against, and of the random-access probes that give the
 // table its roofline.
 
+#include <algorithm>
 #include <string>
 
 #include "gx_kernels.cuh"
@@ -257,12 +258,18 @@ gx_status gx_find_or_put(const uint32_t* keys, uint64_t n_keys, uint32_t key_wor
   e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ks->fop_fn, gx::kBlock, 0);
   if (e != cudaSuccess) return gx::fail(GX_ERR_CUDA, cudaGetErrorString(e));
   const uint64_t lanes = B / G >= 16 ? (uint64_t)G : 1;  // per key (fop_kernel)
-  const uint64_t blocks_needed = (n_keys * lanes + gx::kBlock - 1) / gx::kBlock;
+  uint64_t blocks_needed = (n_keys * lanes + gx::kBlock - 1) / gx::kBlock;
+  const uint64_t resident = (uint64_t)sm_count() * (per_sm > 0 ? per_sm : 1);
+  // Warps that take keys one after the other (fop_groups) get 256 each, but not so many that
+  // the GPU is not full, nor fewer than 32 (3e6 new keys, 8-word buckets, 8 lanes: 0.23 ms
+  // with 32 keys a warp, 0.10 with 128, 0.09 with 256; 1e5 keys: 0.023, 0.031, 0.038).
+  if (G > 1 && lanes == 1)
+    blocks_needed = std::min(blocks_needed, std::max(resident, (n_keys + 8 * gx::kBlock - 1) / (8 * gx::kBlock)));
   // A grid of 16 times the CTAs that fit at once (the loop is grid-stride and a CTA's
   // setup is 64 multipliers): random reads from a grid whose CTAs finish and start during
   // the launch run faster than from a resident one (10^8 keys at d = 1, 8-word buckets,
   // one lane per bucket: 27.3 against 23.8 G keys/s; at d = 21: 56.2 against 50.3).
-  const uint64_t cap = (uint64_t)sm_count() * (per_sm > 0 ? per_sm : 1) * 16;
+  const uint64_t cap = resident * 16;
   const int grid = (int)(blocks_needed < cap ? blocks_needed : cap);
   e = ks->fop(a, grid > 0 ? grid : 1, st);
   if (e != cudaSuccess) return gx::fail(GX_ERR_CUDA, cudaGetErrorString(e));

@@ -137,3 +137,24 @@ def test_probe_kernels_run(cuda):
         gx.probe_random(1, buf, 1 << 16, nbytes, 2, sink)
     torch.cuda.synchronize()
     assert int((buf != 0).sum().item()) > 0
+
+
+@pytest.mark.parametrize("W,B,G", [(1, 8, 8), (1, 32, 32), (2, 16, 4), (4, 8, 2)])
+@pytest.mark.parametrize("n", [1, 31, 33, 255, 257, 2049, 300_001, 3_000_001])
+def test_every_key_is_taken_once_at_every_share_of_a_warp(cuda, W, B, G, n):
+    """Groups of lanes: 32 to 256 keys a warp by the number of keys, the last warp's share ragged.
+    Every key gets a result, each distinct one is inserted exactly once."""
+    import torch
+    keys = torch.from_numpy(np.ascontiguousarray(inputs.key_sequence(n, 1, words=W)).view(np.int32)).cuda()
+    keys = torch.cat([keys.reshape(n, W), keys.reshape(n, W)[: n // 2]]).contiguous()
+    m = len(keys)
+    slots = 64
+    while slots < n / 0.6:
+        slots *= 2
+    table = torch.zeros(slots * W, dtype=torch.int32, device="cuda")
+    counters = torch.zeros(3, dtype=torch.int64, device="cuda")
+    result = torch.full((m,), 7, dtype=torch.uint8, device="cuda")
+    gx.find_or_put(keys, W, table, counters, result=result, bucket_words=B, group_lanes=G, hash_rounds=64)
+    torch.cuda.synchronize()
+    assert counters.tolist() == [n, m - n, 0]
+    assert (result == 1).sum().item() == n and (result == 0).sum().item() == m - n
