@@ -358,7 +358,7 @@ gx_status make_plan(const Net& net, const gx_explore_opts* o, Plan& P) {
                                     std::to_string(S) + ")");
   P.rounds = o->hash_rounds ? (int)o->hash_rounds : 8;
   if (P.rounds < 1 || P.rounds > kMaxRounds) return fail(GX_ERR_INVALID, "hash_rounds must be 1..64");
-  P.ks = kernels_for(P.W, P.B, P.G);
+  P.ks = kernels_for(net, P.B, P.G);
   if (!P.ks) return fail(GX_ERR_INVALID, "no kernel built for this (slot, bucket, group) size");
   const uint64_t table_bytes = o->table_bytes ? o->table_bytes : (1ull << 30);
   const uint64_t bucket_bytes = 4ull * P.B;

@@ -507,13 +507,14 @@ struct ClassDescs {
 // successor per lane that has any left to a queue in shared memory; a state's
 // successors are counted on the way, without a pass of their own.
 // Share: lanes whose source is exhausted take part of what is left of another lane's
-// (share), for the kernels that give a warp one or a few states: a rule of many
-// combinations would be one lane's work.  (4096 states with one rule of 729: guided
-// search 4.0 -> 0.29 ms, batch of one such network 4.4 -> 0.29.)
+// (share), where a warp has one or a few states: a rule of many combinations would be
+// one lane's work.  (4096 states with one rule of 729: guided search 4.0 -> 0.29 ms,
+// batch of one such network 4.4 -> 0.29, exploration 3.8 -> 0.32; 65,536 states with one of
+// 6561: exploration 57 -> 16.7.)
 // Kernels of their own, for networks with a source of kShareFrom successors or more
 // (max_source): the others gain nothing and would pay for the check and a register (256
-// networks: 8.2 ms, with it 8.4).
-constexpr uint32_t kShareFrom = 16;
+// networks: 8.2 ms, with it 8.4; mid network 12.4, 12.7).
+using gx::kShareFrom;
 template <int W, bool Share = false>
 struct WarpGen {
   uint32_t src;       // next source: process src, then rule src - n_procs (uniform)
@@ -823,10 +824,11 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
 // Whether the level kernel does so: not with 4-word vectors, where the second way of
 // generating spills registers in the loop that the large levels run (3.4e8 states in
 // two passes 188 ms, without it 183).
-template <int W>
-constexpr bool kWide = W < 4;
+// (Not so where lanes share: there the levels of few states count.)
+template <int W, bool Share>
+constexpr bool kWide = Share || W < 4;
 
-template <int W, int B, int G>
+template <int W, int B, int G, bool Share>
 __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expand_kernel(const gx::ExpandArgs a) {
   constexpr uint32_t kWarps = gx::kBlock / 32;
   extern __shared__ __align__(16) uint32_t sm[];
@@ -876,7 +878,7 @@ __global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expa
   }
   const uint64_t own = s_range[0] + (uint64_t)(blockIdx.x * kWarps + (threadIdx.x >> 5)) * unit;
   bool first = true;
-  expand_states<W, B, G, kBatch<W>, kWide<W>>(
+  expand_states<W, B, G, kBatch<W>, kWide<W, Share>, Share>(
       tg, muls, t, L, queue_mem[threadIdx.x >> 5], st, probes, err, desc,
       [&](uint64_t& pos, uint32_t& m) {
         // the first states of every warp are fixed by its index, a large level's
@@ -1055,7 +1057,7 @@ struct __align__(16) SmallQueues {  // of a warp, in dynamic shared memory
   uint32_t stage[kStage * W];
 };
 
-template <int W, int B>
+template <int W, int B, bool Share>
 __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThreads, 1)
     small_levels_kernel(const gx::ExpandArgs a, const gx::LoopArgs LA) {
   constexpr uint32_t kWarps = kSmallThreads / 32;
@@ -1091,7 +1093,7 @@ __global__ void __cluster_dims__(kSmallCtas, 1, 1) __launch_bounds__(kSmallThrea
     // (at most 4 states a warp)
     const uint32_t unit = ((uint32_t)(s_range[1] - s_range[0]) + kSmallWarps - 1) / kSmallWarps;
     uint64_t own = s_range[0] + (uint64_t)gw * unit;
-    expand_states<W, B, 1, 32>(
+    expand_states<W, B, 1, 32, true, Share>(
         tg, muls, t, L, q.queues, st, probes, err, desc,
         [&](uint64_t& pos, uint32_t& m) {
           m = own >= s_range[1] ? 0u : s_range[1] - own < unit ? (uint32_t)(s_range[1] - own) : unit;
@@ -1484,7 +1486,7 @@ __global__ void __launch_bounds__(gx::kBlock) fop_kernel(const gx::FopArgs a) {
 
 namespace gx {
 
-template <int W, int B, int G>
+template <int W, int B, int G, bool Share>
 cudaError_t launch_expand(const ExpandArgs& a, int grid, size_t smem, int carveout, cudaStream_t st) {
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)grid);
@@ -1496,7 +1498,7 @@ cudaError_t launch_expand(const ExpandArgs& a, int grid, size_t smem, int carveo
   at[0].val.sharedMemCarveout = (unsigned)carveout;
   cfg.attrs = at;
   cfg.numAttrs = carveout >= 0 ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, gxd::expand_kernel<W, B, G>, a);
+  return cudaLaunchKernelEx(&cfg, gxd::expand_kernel<W, B, G, Share>, a);
 }
 template <int W, int B, int G>
 cudaError_t launch_init(const InitArgs& a, cudaStream_t st) {
@@ -1529,23 +1531,26 @@ cudaError_t launch_part_probe(const ExpandArgs& a, const uint32_t* succ, uint64_
   return cudaGetLastError();
 }
 
-template <int W, int B, int G>
+template <int W, int B, int G, bool Share = false>
 const KernelSet* kernel_set() {
-  static const KernelSet ks{&launch_expand<W, B, G>,
+  const KernelSet* sharing = nullptr;
+  if constexpr (!Share) sharing = kernel_set<W, B, G, true>();
+  static const KernelSet ks{&launch_expand<W, B, G, Share>,
                             &launch_part_count<W>,
                             &launch_part_scan,
                             &launch_part_scatter<W>,
                             &launch_part_probe<W, B, G>,
                             &launch_init<W, B, G>,
                             &launch_fop<W, B, G>,
-                            reinterpret_cast<const void*>(&gxd::expand_kernel<W, B, G>),
+                            reinterpret_cast<const void*>(&gxd::expand_kernel<W, B, G, Share>),
                             reinterpret_cast<const void*>(&gxd::fop_kernel<W, B, G>),
                             reinterpret_cast<const void*>(&gxd::part_count_kernel<W>),
                             reinterpret_cast<const void*>(&gxd::part_scatter_kernel<W>),
                             reinterpret_cast<const void*>(&gxd::part_probe_kernel<W, B, G>),
                             reinterpret_cast<const void*>(&gxd::init_kernel<W, B, G>),
-                            reinterpret_cast<const void*>(&gxd::small_levels_kernel<W, B>),
-                            sizeof(gxd::SmallQueues<W>) * (gxd::kSmallThreads / 32)};
+                            reinterpret_cast<const void*>(&gxd::small_levels_kernel<W, B, Share>),
+                            sizeof(gxd::SmallQueues<W>) * (gxd::kSmallThreads / 32),
+                            sharing};
   return &ks;
 }
 

@@ -163,7 +163,11 @@ struct KernelSet {
   const void* init_fn;    // for graph kernel nodes
   const void* small_fn;   // levels of few states, many in one launch
   size_t small_queue_bytes;  // of its dynamic shared memory
+  // the set for networks with a source of kShareFrom successors or more, whose lanes
+  // share a rule's combinations (nullptr: this is that set)
+  const KernelSet* sharing;
 };
+constexpr uint32_t kShareFrom = 16;
 
 // Kernels for slot width W, bucket words B and group lanes G; nullptr if the
 // combination is not built.
@@ -175,6 +179,10 @@ inline const KernelSet* kernels_for(int W, int B, int G) {
   if (W == 2) return kernels_w2(B, G);
   if (W == 4) return kernels_w4(B, G);
   return nullptr;
+}
+inline const KernelSet* kernels_for(const Net& net, int B, int G) {
+  const KernelSet* ks = kernels_for((int)net.slot_words, B, G);
+  return ks && net.lay.max_source >= kShareFrom ? ks->sharing : ks;
 }
 
 // Lets a kernel take all the dynamic shared memory its static part leaves: the same

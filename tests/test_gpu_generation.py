@@ -56,6 +56,26 @@ def test_batches_of_networks_with_many_combinations(cuda, name, count):
         assert gx.batch_levels(b, i) == r.levels
 
 
+@pytest.mark.parametrize("opts", [dict(), dict(bucket_words=16, group_lanes=1), dict(host_loop=1, group_lanes=1),
+                                  dict(region_passes=2), dict(watch=1, watch_proc=0, watch_state=1)], ids=str)
+@pytest.mark.parametrize("name", NETS)
+def test_exploration_of_networks_with_many_combinations(cuda, name, opts):
+    net = NETS[name]
+    r = oracle.explore(net, watch=(0, 1))
+    h = gx.load_network(net)
+    o = gx.default_opts(table_bytes=1 << 24, hash_rounds=64, **opts)
+    ws = gx.alloc_workspace(h, o)
+    gx.explore(h, o, ws)
+    s = gx.stats(h)
+    assert (s["states"], s["transitions"], gx.levels(h)) == (r.states, r.transitions, r.levels)
+    assert gx.set_digest(h, ws) == (r.states, r.set_sum, r.set_xor)
+    if opts.get("watch"):
+        assert (s["violation_count"], s["violation_xor"]) == (r.violation_count, r.violation_xor)
+    if not opts:
+        n, levels = gx.explore_noalloc(h, o)
+        assert (n["states"], n["transitions"], levels) == (r.states, r.transitions, r.levels)
+
+
 @pytest.mark.parametrize("name", NETS)
 def test_guided_search_of_networks_with_many_combinations(cuda, name):
     import torch
