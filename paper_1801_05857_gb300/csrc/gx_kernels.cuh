@@ -1333,6 +1333,10 @@ __global__ void __launch_bounds__(gx::kBlock) part_probe_kernel(const gx::Expand
 #pragma unroll
     for (int w = 0; w < W; ++w) x[w] = 0;
     if (on) load_vec<W>(succ + idx * W, x);
+    if (on && a.gcache.base) {  // the filter that the level kernel applies as it generates
+      const SeenEntry e = seen_entry<W>(a.gcache, x);
+      on = e.content == 0 || seen_get(a.gcache, e.index) != e.content;
+    }
     const uint64_t h = state_hash<W>(x);
     for (uint32_t k = 0; __any_sync(FULLMASK, on); ++k) {
       if (k == (uint32_t)a.rounds) {

@@ -299,3 +299,17 @@ def test_launch_count_counts_a_launch_once(cuda, net, passes):
     o = gx.default_opts(table_bytes=1 << 24, hash_rounds=32, region_passes=passes, host_loop=1)
     gx.explore(h, o, gx.alloc_workspace(h, o))
     assert gx.launch_count(h) == 1 + passes * len(sizes)
+
+
+@pytest.mark.parametrize("W", [1, 2, 4])
+def test_partitioned_levels_ask_the_gpu_wide_cache(cuda, W):
+    """Levels expanded by the partitioned path leave out the bucket reads of vectors that the
+    GPU-wide cache holds, as the level kernel does; without the cache every successor reads."""
+    kw = dict(table_bytes=1 << 26, hash_rounds=32, bucket_words=8, group_lanes=1, partition_min_states=1,
+              warp_cache_log2=0)
+    r = _oracle(W, NETS[W])
+    s = _check(W, NETS[W], global_cache_log2=0, **kw)
+    assert s["partitioned_levels"] == s["n_levels"] and s["probes"] >= r.transitions
+    s = _check(W, NETS[W], global_cache_log2=20, **kw)
+    assert s["partitioned_levels"] == s["n_levels"] and s["global_cache_entries"] == 1 << 20
+    assert s["probes"] < 0.8 * r.transitions
