@@ -358,13 +358,13 @@ gx_status make_plan(const Net& net, const gx_explore_opts* o, Plan& P) {
                                     std::to_string(S) + ")");
   P.rounds = o->hash_rounds ? (int)o->hash_rounds : 8;
   if (P.rounds < 1 || P.rounds > kMaxRounds) return fail(GX_ERR_INVALID, "hash_rounds must be 1..64");
-  P.ks = kernels_for(net, P.B, P.G);
-  if (!P.ks) return fail(GX_ERR_INVALID, "no kernel built for this (slot, bucket, group) size");
+  if (!kernels_for(P.W, P.B, P.G)) return fail(GX_ERR_INVALID, "no kernel built for this (slot, bucket, group) size");
   const uint64_t table_bytes = o->table_bytes ? o->table_bytes : (1ull << 30);
   const uint64_t bucket_bytes = 4ull * P.B;
   if (table_bytes < 2 * bucket_bytes) return fail(GX_ERR_INVALID, "table_bytes is smaller than two buckets");
   P.nb = pow2_floor(table_bytes / bucket_bytes);
   const uint64_t slots = P.nb * (uint64_t)S;
+  P.ks = kernels_for(net, P.B, P.G, slots);
   P.fcap = pow2_ceil(o->frontier_states ? o->frontier_states : std::max<uint64_t>(4096, slots / 4));
   P.dl_cap = o->deadlock_cap ? o->deadlock_cap : 1024;
   if (o->watch) {

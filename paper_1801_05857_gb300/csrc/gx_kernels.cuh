@@ -669,9 +669,11 @@ struct WarpQueues {
 
 // Resident CTAs per SM the level kernel is compiled for (register budget): a
 // lane holds a bucket of B words.
-template <int W, int B, int G>
+// (A sharing lane holds more: 4-word slots in 4-word buckets would spill 58 bytes with 5 CTAs,
+// 3.8e6 states 3.38 ms, with 4 CTAs 2.47.)
+template <int W, int B, int G, bool Share = false>
 struct ExpandOcc {
-  static constexpr int min_ctas = B <= 8 ? (G == 1 ? 5 : 4) : (B <= 16 && G == 1 ? 4 : 3);
+  static constexpr int min_ctas = Share && W == 4 && B == 4 ? 4 : B <= 8 ? (G == 1 ? 5 : 4) : (B <= 16 && G == 1 ? 4 : 3);
 };
 
 // Up to this many states per warp are generated from by several lanes each, which take
@@ -824,12 +826,12 @@ __device__ __forceinline__ void expand_states(const T& tg, const uint64_t* muls,
 // Whether the level kernel does so: not with 4-word vectors, where the second way of
 // generating spills registers in the loop that the large levels run (3.4e8 states in
 // two passes 188 ms, without it 183).
-// (Not so where lanes share: there the levels of few states count.)
+// (The sharing set does, for tables whose levels are small: kernels_for.)
 template <int W, bool Share>
 constexpr bool kWide = Share || W < 4;
 
 template <int W, int B, int G, bool Share>
-__global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G>::min_ctas) expand_kernel(const gx::ExpandArgs a) {
+__global__ void __launch_bounds__(gx::kBlock, ExpandOcc<W, B, G, Share>::min_ctas) expand_kernel(const gx::ExpandArgs a) {
   constexpr uint32_t kWarps = gx::kBlock / 32;
   extern __shared__ __align__(16) uint32_t sm[];
   // the level being expanded: from the parameters, or (device-driven level

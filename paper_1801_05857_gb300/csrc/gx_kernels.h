@@ -163,8 +163,8 @@ struct KernelSet {
   const void* init_fn;    // for graph kernel nodes
   const void* small_fn;   // levels of few states, many in one launch
   size_t small_queue_bytes;  // of its dynamic shared memory
-  // the set for networks with a source of kShareFrom successors or more, whose lanes
-  // share a rule's combinations (nullptr: this is that set)
+  // the set whose lanes share a state's sources and a rule's combinations (nullptr: this is
+  // that set; kernels_for)
   const KernelSet* sharing;
 };
 constexpr uint32_t kShareFrom = 16;
@@ -180,9 +180,17 @@ inline const KernelSet* kernels_for(int W, int B, int G) {
   if (W == 4) return kernels_w4(B, G);
   return nullptr;
 }
-inline const KernelSet* kernels_for(const Net& net, int B, int G) {
+// The kernels for a network and a table of `slots` slots: the sharing set for networks with a
+// source of kShareFrom successors or more, and for 4-word vectors in tables below 2^26
+// slots.  Large levels of these lose 1-5 % with it (1.08e8 states 40.2 -> 40.7 ms, 3.4e8 in two
+// passes 185 -> 195), levels of few states a warp gain as much as half (20,736 states, one
+// pass 0.38 -> 0.31 ms, four 0.88 -> 0.54; 2^18 states of 124 processes in four passes 3.09
+// -> 1.16, where the kernels before the staged ones took 2.19); 2^26 slots hold some 4e7
+// states, whose levels are still mostly of the second kind.
+inline const KernelSet* kernels_for(const Net& net, int B, int G, uint64_t slots) {
   const KernelSet* ks = kernels_for((int)net.slot_words, B, G);
-  return ks && net.lay.max_source >= kShareFrom ? ks->sharing : ks;
+  const bool share = net.lay.max_source >= kShareFrom || (net.slot_words == 4 && slots < (1ull << 26));
+  return ks && share ? ks->sharing : ks;
 }
 
 // Lets a kernel take all the dynamic shared memory its static part leaves: the same

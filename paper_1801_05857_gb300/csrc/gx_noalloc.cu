@@ -92,8 +92,7 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
   const int G = o->group_lanes ? (int)o->group_lanes : std::min(S, 32);
   const int rounds = o->hash_rounds ? (int)o->hash_rounds : 8;
   if (rounds < 1 || rounds > gx::kMaxRounds) return gx::fail(GX_ERR_INVALID, "hash_rounds must be 1..64");
-  const gx::KernelSet* ks = gx::kernels_for(net, B, G);
-  if (!ks) return gx::fail(GX_ERR_INVALID, "group_lanes must be a power of two dividing bucket_words / slot words");
+  if (!gx::kernels_for(W, B, G)) return gx::fail(GX_ERR_INVALID, "group_lanes must be a power of two dividing bucket_words / slot words");
   uint32_t regions = o->region_passes ? o->region_passes : 1;  // tables here are far below 64 GiB
   if (regions > 16 || (regions & (regions - 1)))
     return gx::fail(GX_ERR_INVALID, "region_passes must be a power of two from 1 to 16");
@@ -102,6 +101,7 @@ gx_status gx_explore_noalloc(const gx_net* h, const gx_explore_opts* opts, void*
   while (nb * 2 * 4ull * B <= table_bytes) nb *= 2;
   if (nb < 2) return gx::fail(GX_ERR_INVALID, "table_bytes is smaller than two buckets");
   const uint64_t slots = nb * (uint64_t)S;
+  const gx::KernelSet* ks = gx::kernels_for(net, B, G, slots);
   const uint64_t fwant = o->frontier_states ? o->frontier_states : std::max<uint64_t>(4096, slots / 4);
   uint64_t fcap = 1;
   while (fcap < fwant) fcap *= 2;

@@ -313,3 +313,15 @@ def test_partitioned_levels_ask_the_gpu_wide_cache(cuda, W):
     s = _check(W, NETS[W], global_cache_log2=20, **kw)
     assert s["partitioned_levels"] == s["n_levels"] and s["global_cache_entries"] == 1 << 20
     assert s["probes"] < 0.8 * r.transitions
+
+
+@pytest.mark.parametrize("opts", [dict(), dict(global_cache_log2=0), dict(region_passes=2), dict(host_loop=1, region_passes=4),
+                                  dict(warp_cache_log2=2, global_cache_log2=0, group_lanes=2)], ids=str)
+@pytest.mark.parametrize("bits", [60, 64, 65])
+def test_4_word_vectors_in_large_tables(cuda, bits, opts):
+    """Tables of 2^26 slots and more run level kernels of their own for 4-word vectors (one state
+    per lane in every level): the same networks as in the small tables above."""
+    kw = dict(table_bytes=1 << 30, hash_rounds=32, bucket_words=8, group_lanes=1)
+    kw.update(opts)
+    s = _check(("wide", bits), WIDE_NETS[bits], **kw)
+    assert s["slot_words"] == 4 and s["table_slots"] == 1 << 26
