@@ -496,7 +496,7 @@ def table_slots_for(states: int) -> int:
 
 
 def batched_part(torch, gx, inputs, steps: int = 5) -> dict:
-    """The 256-network batched workload: one graph launch (autotuned) vs one gx_explore
+    """The 256-network batched workload: one batched call (autotuned) vs one gx_explore
     per network in sequence.  A sizing pass with 2^21-slot tables counts each network's
     states; the measured runs give every network a table at <= 75 % fill."""
     nets = inputs.batch_workload()

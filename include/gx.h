@@ -449,10 +449,8 @@ gx_status gx_guided_trace(const gx_net* net, uint32_t* out, uint32_t cap, uint32
 /* ------------------------------------------------------------------------------------------
  * Batched exploration of many independent networks (no counterpart in the
  * paper, which explores one network per run; each network is explored exactly
- * as by gx_explore).  All networks advance one BFS level per iteration inside
- * one persistent kernel launch; the iterations run on the device as a CUDA
- * graph with a conditional WHILE node, so one graph launch explores the whole
- * batch.  Narrower vectors are padded to the batch's widest slot.
+ * as by gx_explore), in one persistent kernel launch: levels follow one another
+ * network by network.  Narrower vectors are padded to the batch's widest slot.
  * ---------------------------------------------------------------------------------------- */
 typedef struct gx_batch gx_batch;
 

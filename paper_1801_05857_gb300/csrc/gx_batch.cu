@@ -251,8 +251,6 @@ struct SmemTarget {
   __device__ __forceinline__ uint32_t* frontier() const { return w->frontier; }
   __device__ __forceinline__ uint64_t fmask() const { return w->fmask; }
   __device__ __forceinline__ uint64_t begin() const { return w->cur_begin; }
-  __device__ __forceinline__ uint64_t region_mask() const { return 0; }
-  __device__ __forceinline__ uint64_t region_bits() const { return 0; }
   __device__ __forceinline__ gx::SeenCache gcache() const { return gx::SeenCache{}; }
 };
 
@@ -745,7 +743,7 @@ gx_status gx_batch_autotune(gx_batch* b, gx_batch_opts* io, void* ws, uint64_t w
       o.chunk_states = ch;
       gx::BatchPlan P;
       if (gx::batch_plan(b, &o, P) != GX_OK || P.total > ws_bytes) continue;
-      // one warm-up (graph build), then the median of three timed runs
+      // one warm-up, then the median of three timed runs
       gx_status s = gx::run_batch(b, &o, ws, ws_bytes, st);
       if (s != GX_OK) continue;
       double t[3];

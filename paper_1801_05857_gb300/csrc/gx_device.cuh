@@ -21,7 +21,9 @@
 //     candidate for the CAS, whose return value is the slot's true content,
 //     so no read ever has to wait for another writer;
 //   * the hash-constant sets of Sec. 4.1 are multiply-shift multipliers
-//     (Dietzfelbinger et al. 1997) over a splitmix64-mixed vector.
+//     (Dietzfelbinger et al. 1997) over a hash of the vector: vec_hash (a
+//     splitmix64 finaliser) in the isolated table, state_hash (two odd
+//     multiplications) in the searches.
 #pragma once
 
 #include <cstdint>

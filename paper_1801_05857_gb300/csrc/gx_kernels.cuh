@@ -1,10 +1,11 @@
 // Templated kernels of the exploration path, instantiated per slot width W in
 // gx_kernels_w{1,2,4}.cu.
 //
-//   expand_kernel  one BFS level (Sec. 3): claim open vectors, count and
-//                  generate successors from the staged network tables,
-//                  find-or-put each successor (Sec. 4.1), append the new ones
-//                  to the next level, count transitions, record deadlocks.
+//   expand_kernel  one BFS level (Sec. 3): claim open vectors, generate their
+//                  successors from the staged network tables, find-or-put each
+//                  (Sec. 4.1), append the new ones to the next level, count
+//                  transitions, record deadlocks.
+//   small_levels_kernel  levels of few states, many in one launch.
 //   init_kernel    inserts the initial vector (level 0).
 //   fop_kernel     the isolated hash-table experiment of Sec. 5.1.
 #pragma once
@@ -241,29 +242,9 @@ __device__ __forceinline__ const uint32_t* stage_tables(uint32_t* sm, const gx::
 }
 
 // Where find-or-put inserts and where new vectors go: one network's table and
-// frontier ring (the level being expanded starts at begin()).  Target holds
-// the values (the batched kernel loads them per network); ParamTarget reads
-// them from the single-network kernel's parameters, which live in the
-// constant bank and so take no registers in the inner loop.
-struct Target {
-  uint32_t* tab;
-  int l2nb, nrounds;
-  unsigned long long* nend;
-  uint32_t* front;
-  uint64_t fm;
-  uint64_t cur_begin;
-  __device__ __forceinline__ uint32_t* table() const { return tab; }
-  __device__ __forceinline__ int log2nb() const { return l2nb; }
-  __device__ __forceinline__ int rounds() const { return nrounds; }
-  __device__ __forceinline__ unsigned long long* next_end() const { return nend; }
-  __device__ __forceinline__ uint32_t* frontier() const { return front; }
-  __device__ __forceinline__ uint64_t fmask() const { return fm; }
-  __device__ __forceinline__ uint64_t begin() const { return cur_begin; }
-  __device__ __forceinline__ uint64_t region_mask() const { return 0; }
-  __device__ __forceinline__ uint64_t region_bits() const { return 0; }
-  __device__ __forceinline__ gx::SeenCache gcache() const { return gx::SeenCache{}; }
-};
-
+// frontier ring (the level being expanded starts at begin()).  Read from the
+// kernel's parameters, which live in the constant bank and so take no registers in
+// the inner loop; the batched kernel has its own (SmemTarget).
 struct ParamTarget {
   const gx::ExpandArgs& a;
   const unsigned long long* range;  // [begin, end) of the level, in shared memory
@@ -274,8 +255,6 @@ struct ParamTarget {
   __device__ __forceinline__ uint32_t* frontier() const { return a.frontier; }
   __device__ __forceinline__ uint64_t fmask() const { return a.fmask; }
   __device__ __forceinline__ uint64_t begin() const { return range[0]; }
-  __device__ __forceinline__ uint64_t region_mask() const { return a.region_mask; }
-  __device__ __forceinline__ uint64_t region_bits() const { return a.region_bits; }
   __device__ __forceinline__ const gx::SeenCache& gcache() const { return a.gcache; }
 };
 
